@@ -187,7 +187,7 @@ def tolerance(case):
         return {"rel": 1.3e-5, "max": 5e-5}
     if case["dtype"] == "f32":                                # fp32 sums throughout
         return {"rel": 1e-5, "max": 1e-4, "differ": 0.01}
-    return {"rel": 8e-4, "max": 0.032, "differ": 0.01}        # activations as bf16 pairs, bf16 caches: 2e-4, one bf16 step
+    return {"rel": 1.2e-3, "max": 0.032, "differ": 0.01}      # activations as bf16 pairs, bf16 caches: 3e-4, one bf16 step
 
 
 # ---- states ------------------------------------------------------------------------------------------------------
