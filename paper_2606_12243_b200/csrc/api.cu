@@ -68,7 +68,7 @@ size_t carve(const viasd_config &c, char *base, Workspace *ws) {
         w.a_head = cv.take<void>(R * c.d_model * 4);
         w.ssq_head = cv.take<float>((size_t)(c.d_model / 128 + 1) * 4 * R * 4);
         w.attn_counters = cv.take<int>(attn_counter_count(c.max_batch, c.n_kv_heads) * sizeof(int));
-        w.n_counters = widest / 128 + 8;
+        w.n_counters = widest / 64 + 8;                      // (a tile of the pair kernel's gate/up launch has 64 features)
         w.gemm_counters = cv.take<int>(w.n_counters * 4);
     }
     if (ws) *ws = w;
@@ -187,7 +187,7 @@ int forward_sweep(viasd_model *m, const viasd_cache *cache, const viasd_draft *d
     const int B = d->batch, M = d->n_nodes + 1 + replay, rows = B * M;
     const int qd = c.n_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
     const size_t R = m->ws.rows_alloc;
-    const bool dual = mode == 2;
+    const bool dual = mode == 2, wide = rows >= TC_WIDE_MIN_ROWS;
     int rc;
     // layers this sweep visits, and for each whether the slim stream takes part
     const int n_run = mode == 1 ? m->n_routed : c.n_layers;
@@ -199,8 +199,11 @@ int forward_sweep(viasd_model *m, const viasd_cache *cache, const viasd_draft *d
     };
     auto gemm = [&](TcLaunch L, const ActMaps &xm, int nrows) -> int {
         return timed(m, VIASD_T_GEMM, st, [&]() -> int {
-            for (int row0 = 0; row0 < nrows; row0 += 128) {
-                const int nr = nrows - row0 < 128 ? nrows - row0 : 128, nt = tc_pick_nt(nr, true);
+            // launches of 128 rows; the pair kernel's, up to 256 rows, of equal height
+            const int launches = (nrows + TC_WIDE_ROWS - 1) / TC_WIDE_ROWS;
+            const int step = wide ? ((nrows + launches - 1) / launches + 15) / 16 * 16 : 128;
+            for (int row0 = 0; row0 < nrows; row0 += step) {
+                const int nr = nrows - row0 < step ? nrows - row0 : step, nt = wide ? tc_wide_th(nr) : tc_pick_nt(nr, true);
                 const int ni = nt / 8 - 1;
                 L.map_x = &xm.map[ni]; L.x_box_rows = xm.box_rows[ni];
                 L.has_lo = 1; L.lo_row_offset = (int)R;
@@ -211,7 +214,7 @@ int forward_sweep(viasd_model *m, const viasd_cache *cache, const viasd_draft *d
                 L.run_flag = m->run_flag;
                 L.ssq_stride = (int)R; L.inv_d = 1.0f / (float)c.d_model; L.eps = c.rms_eps;
                 L.split_row = dual ? rows : 0;
-                int r2 = launch_gemm_tc(L, st);
+                int r2 = wide ? launch_gemm_wide(L, st) : launch_gemm_tc(L, st);
                 if (r2) return r2;
             }
             return (int)VIASD_OK;
@@ -265,7 +268,7 @@ int forward_sweep(viasd_model *m, const viasd_cache *cache, const viasd_draft *d
         }
         {   // gate / up with SwiGLU
             TcLaunch L; memset(&L, 0, sizeof(L));
-            wseg(L, 0, lm.wg, c.d_ff); wseg(L, 1, lm.wu, c.d_ff); L.n_seg = 2;
+            wseg(L, 0, wide ? lm.wg64 : lm.wg, c.d_ff); wseg(L, 1, wide ? lm.wu64 : lm.wu, c.d_ff); L.n_seg = 2;
             L.k = c.d_model; L.epi = EPI_SWIGLU; L.out_act = m->ws.act; L.act_plane = R * c.d_ff; L.ld_out = c.d_ff;
             L.ssq_in = m->ws.ssq; L.ssq_in_n = ssq_n;
             if ((rc = gemm(L, m->maps_a, nrows))) return rc;
@@ -423,8 +426,8 @@ int viasd_init_model(const viasd_config *cfg, const viasd_weights *w, const unsi
         const uint64_t d = cfg->d_model, qd = (uint64_t)cfg->n_heads * cfg->head_dim,
                        kvd = (uint64_t)cfg->n_kv_heads * cfg->head_dim, ff = cfg->d_ff, R = m->ws.rows_alloc;
         m->lmaps = new (std::nothrow) LayerMaps[L];
-        auto wm = [&](WMap &o, const void *base, uint64_t n, uint64_t k) {
-            o.box_rows = tc_box_rows(n, 128);
+        auto wm = [&](WMap &o, const void *base, uint64_t n, uint64_t k, uint32_t box = 128) {
+            o.box_rows = tc_box_rows(n, box);
             return tc_make_map(&o.map, base, n, k, o.box_rows);
         };
         rc = m->lmaps ? VIASD_OK : VIASD_EINVAL;
@@ -432,7 +435,7 @@ int viasd_init_model(const viasd_config *cfg, const viasd_weights *w, const unsi
             LayerMaps &lm = m->lmaps[l];
             if ((rc = wm(lm.wq, m->wq[l], qd, d)) || (rc = wm(lm.wk, m->wk[l], kvd, d)) || (rc = wm(lm.wv, m->wv[l], kvd, d)) ||
                 (rc = wm(lm.wo, m->wo[l], d, qd)) || (rc = wm(lm.wg, m->wg[l], ff, d)) || (rc = wm(lm.wu, m->wu[l], ff, d)) ||
-                (rc = wm(lm.wd, m->wd[l], d, ff))) break;
+                (rc = wm(lm.wd, m->wd[l], d, ff)) || (rc = wm(lm.wg64, m->wg[l], ff, d, 64)) || (rc = wm(lm.wu64, m->wu[l], ff, d, 64))) break;
         }
         if (!rc) rc = wm(m->head_map, m->lm_head, cfg->vocab, d);
         auto am = [&](ActMaps &o, const void *base, uint64_t k) {
@@ -594,9 +597,11 @@ int viasd_verify_step(viasd_model *m, viasd_cache *cache, const viasd_draft *dra
     if ((rc = check_params(params))) return rc;
     if (params->policy == 1) return verify_step_routed(m, cache, draft, params, slim_logits, full_logits, result, stream);
     // Both verifiers in one sweep over the layers (routed layers' weights are read once for both) while the two
-    // row streams together fit one launch (128 token rows: an MMA of 256 columns with the hi/lo planes); beyond
+    // row streams together fit one launch (128 token rows, 256 where the pair kernel runs the pass); beyond
     // that a sweep would stream every routed layer twice anyway, and the passes run one after the other.
-    if (m && m->fused && draft && 2 * draft->batch * (draft->n_nodes + 1) <= m->opt.dual_max_rows) {
+    const int block_rows = draft ? draft->batch * (draft->n_nodes + 1) : 0;
+    const int dual_max = !m ? 0 : m->opt.dual_max_rows == 128 && block_rows >= TC_WIDE_MIN_ROWS ? TC_WIDE_ROWS : m->opt.dual_max_rows;
+    if (m && m->fused && draft && 2 * block_rows <= dual_max) {
         if ((rc = check_draft(m, draft)) || (rc = check_cache(cache))) return rc;
         if ((rc = forward_sweep(m, cache, draft, 2, full_logits, slim_logits, (cudaStream_t)stream))) return rc;
         if ((rc = tier_accept_impl(m, draft, params, slim_logits, full_logits, 3, result, true, stream))) return rc;

@@ -66,7 +66,7 @@ struct Workspace {                      // pointers into the caller's workspace 
 
 struct WMap { CUtensorMap map; uint32_t box_rows; };        // TMA view of one weight matrix
 struct ActMaps { CUtensorMap map[16]; uint32_t box_rows[16]; }; // TMA views of an activation buffer, NT = 8, 16, ..., 128
-struct LayerMaps { WMap wq, wk, wv, wo, wg, wu, wd; };
+struct LayerMaps { WMap wq, wk, wv, wo, wg, wu, wd, wg64, wu64; };   // (wg64 / wu64: 64-row boxes, for the pair kernel)
 struct CacheMaps { CUtensorMap k, v; const void *k_ptr, *v_ptr; };   // TMA views of one model's KV cache
 
 // Optional CUDA-event record (measurement only).  A run of consecutive launches of one class shares one pair of

@@ -29,6 +29,7 @@ struct TcParams {                       // kernel argument block
     float *q_out; __nv_bfloat16 *kc, *vc; const float *cosv, *sinv; const int *len_eff, *depth;
     int rope_M, rope_H, rope_Hkv, max_batch, max_ctx, layer_ord;
     int tree_stride;                    // ints between the depth tables of consecutive sequences
+    int tt, slot_rows, out_vec4, x_stages;   // pair kernel: token sub-tiles, rows of a partial slot, 16-byte output stores, activation slots
     // two row streams in one launch (full verifier rows first, slim verifier rows from split_row on)
     int split_row, layer_ord2; float *out_f32_2; const float *next_gain2; __nv_bfloat16 *kc2, *vc2;
     const int *run_flag;                // null, or a device flag: the kernel leaves at once when it is zero
@@ -71,6 +72,16 @@ uint32_t tc_box_rows(uint64_t tensor_rows, uint32_t want);
 size_t tc_scratch_floats(int sm_count, int nt, bool dual);
 int tc_tiles(int n);
 int launch_gemm_tc(const TcLaunch &L, cudaStream_t st);
+// gemm_wide.cu: pairs of CTAs, up to 256 token rows; L.nt = tc_wide_th(rows), gate/up maps with 64-row boxes
+constexpr int TC_WIDE_ROWS = 256;
+// Token rows of one verifier from which a pass runs on the pair kernel (the choice may not depend on whether the other
+// verifier's rows ride along, or the one-sweep step and its pieces would differ in the last bit).  8B shapes, one-CTA /
+// pair kernel, us: 54 rows QKV 16.0 / 18.0, O 13.7 / 15.7, gate-up 45.7 / 45.5, down 29 / 30; 108 rows 19.8 / 20.1,
+// 17.0 / 17.2, 63 / 56, 36 / 32.  Whole steps: 13B batch 8 (56 rows, 112 in routed layers) 6.94 -> 6.70 ms with it, 8B
+// batch 1 (27 and 54 rows) 4.33 -> 4.51 ms.
+constexpr int TC_WIDE_MIN_ROWS = 48;
+int tc_wide_th(int rows);
+int launch_gemm_wide(const TcLaunch &L, cudaStream_t st);
 
 void tc_fill_params(const TcLaunch &L, TcParams &p);
 

@@ -93,6 +93,29 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
+// ---- the same for a whole warp in step ---------------------------------------------------------
+// Loops that feed TMA and the tensor cores, run by all lanes of their warp with the instruction itself predicated to one
+// lane.  Inside an `if (lane == 0)` the compiler keeps addresses, coordinates and descriptors in per-thread registers and
+// moves each of them over to the uniform registers these instructions take: about 60 cycles per tcgen05.mma of the pair
+// kernel, 500 for a box of four, where a uniform loop takes 300.  (The one-CTA kernel, two boxes per stage, gains nothing.)
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    int spins = 0;
+    while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+        if ((++spins & 255) == 0) {
+            const bool late = clock64() - t0 > WAIT_LIMIT_CYCLES;
+            if (late && (threadIdx.x & 31) == 0) { *abort_flag = 1; atomicExch(status, VIASD_EDEVICE); }
+            if (__any_sync(0xffffffffu, late || *abort_flag)) return false;
+        }
+    }
+    return true;
+}
+__device__ __forceinline__ void mbar_expect_tx_if(uint32_t on, uint32_t bar, uint32_t bytes) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t"
+                 "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%1], %2;\n\t}" ::"r"(on), "r"(bar), "r"(bytes) : "memory");
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
