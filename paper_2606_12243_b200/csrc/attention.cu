@@ -1,3 +1,4 @@
+// Choice of the attention kernel, and the CUDA-core kernel for fp32 models and head_dim 64.
 // KV-append attention over a drafted block: each of the M query rows of a sequence attends to the
 // committed cache rows 0..n-1 and to the block rows on its own root path (causal mask for a chain,
 // ancestor mask for a tree).  Split-KV: a CTA handles one (sequence, kv head, key range, group of
@@ -223,10 +224,14 @@ static int mma_attention(viasd_model *m, const void *kc, const void *vc, bool sl
     // shape at batch 1, 264 tiles, attention 1.78 -> 1.61 ms per step)
     int use = kind == 3 ? (hpi && tiles_total * subs >= (subs > 1 ? 2LL : QRi > 16 ? 1LL : 8LL) * m->sm_count ? 2 : 0) : kind;
     if (use == 2 && !hpi) use = 0;
+    // more than 128 query rows per kv head are more than the mma.sync kernel's eight query tiles: the rows-on-lanes kernel
+    // takes them in items of at most 128, whose MMAs are then full (8 sequences x 8 kv heads x 256 rows against 1000 keys:
+    // 816 us on the CUDA cores, 55 us)
+    if (use == 0 && QR > 128) use = 1;
     const int reps = use == 1 ? attention_tc_replicas(QR) : 1;
-    const int nsplit = mma_nsplit(m, batch, M, streams, use != 0, reps, use == 2 ? subs : 1, use == 2 ? QRi : 0);
+    const int nsplit = mma_nsplit(m, batch, M, streams, use != 0, reps, use == 2 ? subs : use == 1 ? attention_tc_items(QR) : 1, use == 2 ? QRi : 0);
     const int n_part = nsplit * reps;        // key ranges per (row, head) that have to be merged
-    const bool fuse = n_part > 1 && n_part <= 32 && (use == 2 ? QRi : QR) * n_part <= 160;
+    const bool fuse = n_part > 1 && n_part <= 32 && (use == 2 ? QRi : QR) * n_part <= 160 && attention_tc_items(QR) <= VIASD_ATTN_ITEMS_PER_KV_HEAD;
     int rc;
     if (use == 2) {
         // The keys-on-lanes kernel deals tiles, not key ranges, evenly to the CTAs (nsplit 0) when the partial buffer
@@ -251,7 +256,7 @@ static int mma_attention(viasd_model *m, const void *kc, const void *vc, bool sl
 int launch_attention(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, int batch, int M,
                      cudaStream_t st) {
     const viasd_config &c = m->cfg;
-    if (attention_mma_supported(m, M)) {
+    if (attention_tensor_supported(m)) {
         return mma_attention(m, kc, vc, slim, layer_ord, nullptr, nullptr, 0, 1, batch, M, st);
     }
     int nsplit = attention_nsplit(m, batch, M);

@@ -537,6 +537,7 @@ attention_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
 }  // namespace
 
 // tensor maps over the caches are rebuilt only when the caller's pointers change
+int attention_tensor_supported(const viasd_model *m) { return m->cfg.dtype == 1 && m->cfg.head_dim == HD && m->use_tc; }
 int attention_mma_supported(const viasd_model *m, int M) {
     const viasd_config &c = m->cfg;
     return c.dtype == 1 && c.head_dim == HD && (c.n_heads / c.n_kv_heads) * M <= 128 && m->use_tc;

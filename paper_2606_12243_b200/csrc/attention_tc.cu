@@ -1,7 +1,7 @@
 // Block attention on the 5th-generation tensor cores (tcgen05 + TMEM), bf16 caches, head_dim 128.
 //
-// Same work as attention_mma.cu - the M block rows of a sequence (all query heads of one kv head packed into one
-// query tile, at most 128 rows) against the committed context plus the block's own rows under the ancestor
+// Same work as attention_mma.cu - the M block rows of a sequence (all query heads of one kv head, dealt to items of at
+// most 128 rows: a prompt chunk of 64 rows under 4 query heads per kv head is two) against the committed context plus the block's own rows under the ancestor
 // mask, split over key ranges - but with both contractions on tcgen05:
 //
 //   S[rows, 128 keys] = Q K^T      A = Q (shared memory, K-major, hi and lo planes: two MMAs into one S)
@@ -52,7 +52,8 @@ struct AttnTcArgs {
     int M, H, Hkv, max_batch, max_ctx, layer_ord, nsplit;
     int batch, layer_ord2;      // second row stream: rows batch*M.., its own cache and layer ordinal
     int streams, n_items, items_per_cta, fuse_merge, nstage;
-    int qrows8;                 // query rows per kv head rounded up to 8
+    int subs, rows_sub;         // items per kv head and the query rows of each (whole rows of 8 but for the last)
+    int qrows8;                 // query rows of an item rounded up to 8
     int reps, rows_per_rep;     // R replicas of the query rows, 128 / R lanes each
     uint32_t qoff[4];           // byte offsets of the staged query regions: hi dims 0..63, hi 64..127, lo 0..63, lo 64..127
     uint32_t q_bytes;           // staged queries in all; the ring follows
@@ -60,14 +61,16 @@ struct AttnTcArgs {
     float scale;                // log2(e) / sqrt(hd)
 };
 
-struct Item { int be, b, g, stream, split, n_ctx, k_begin, k_end, n_tiles, row_base; };
+struct Item { int be, b, g, row0, rows, stream, split, n_ctx, k_begin, k_end, n_tiles, row_base; };   // rows row0 .. of kv head g / subs
 
 __device__ __forceinline__ Item decode_item(const AttnTcArgs &a, int item) {
     Item it;
     it.split = item % a.nsplit;
     const int bg = item / a.nsplit;
-    it.g = bg % a.Hkv;
-    it.be = bg / a.Hkv;
+    it.g = bg % (a.Hkv * a.subs);
+    it.be = bg / (a.Hkv * a.subs);
+    it.row0 = (it.g % a.subs) * a.rows_sub;
+    it.rows = min(a.rows_sub, a.H / a.Hkv * a.M - it.row0);
     it.stream = it.be / a.batch;
     it.b = it.be - it.stream * a.batch;
     it.n_ctx = a.len_eff[it.b];
@@ -77,7 +80,7 @@ __device__ __forceinline__ Item decode_item(const AttnTcArgs &a, int item) {
     it.k_begin = it.split * chunk;
     it.k_end = min(Tk, it.k_begin + chunk);
     it.n_tiles = it.k_end > it.k_begin ? (it.k_end - it.k_begin + TKEYS - 1) / TKEYS : 0;
-    it.row_base = (((it.stream ? a.layer_ord2 : a.layer_ord) * a.max_batch + it.b) * a.Hkv + it.g) * a.max_ctx;
+    it.row_base = (((it.stream ? a.layer_ord2 : a.layer_ord) * a.max_batch + it.b) * a.Hkv + it.g / a.subs) * a.max_ctx;
     return it;
 }
 
@@ -163,7 +166,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     PDL_TRIGGER();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int NSTAGE = a.nstage;
-    const int grp = a.H / a.Hkv, QR = grp * a.M;
+    const int grp = a.H / a.Hkv;
     // staged queries first (the MMA reads 128 rows from each chunk: what lies behind the live rows is the ring)
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t qsm = base, ring = base + a.q_bytes;
@@ -284,7 +287,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         // ---------------- softmax / epilogue (warps 2..5 <-> TMEM lane quarters 2,3,0,1): one thread, one query row ----------------
         const int quarter = warp & 3, trow = quarter * 32 + lane, et = threadIdx.x - 64;
         const int rep = trow / a.rows_per_rep, row = trow - rep * a.rows_per_rep;     // replica, query row
-        const bool live = row < QR, warp_live = (quarter * 32) % a.rows_per_rep < QR;
         const int KR = TKEYS / a.reps, key0 = rep * KR;                                // this replica's keys of a tile
         const uint32_t tlane = tmem + ((uint32_t)(quarter * 32) << 16);
         PDL_WAIT();
@@ -299,32 +301,32 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         for (int item = i0; item < i1 && ok; ++item) {
             const Item it = decode_item(a, item);
             if (it.be != q_be || it.g != q_g) {
-                // stage the query rows of this (sequence, kv head) as bf16 hi / lo planes, pre-scaled, in the K-major
-                // 128-byte-swizzled layout the MMA reads; four elements per thread at a time, loads first
-                const int n_el = a.qrows8 * (HD / 2);
-                for (int idx0 = et; idx0 < n_el; idx0 += 4 * 128) {
-                    float2 v[4];
+                // stage the item's query rows as bf16 hi / lo planes, pre-scaled, in the K-major 128-byte-swizzled layout
+                // the MMA reads; a warp takes whole rows, eight 16-byte loads per thread in flight
+                for (int rb = warp - 2; rb < a.qrows8; rb += 8 * 4) {
+                    float4 v[8];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int idx = idx0 + q * 128, r = idx / (HD / 2), d2 = (idx % (HD / 2)) * 2;
-                        v[q] = make_float2(0.f, 0.f);
-                        if (idx < n_el && r < QR) {
-                            const int h = it.g * grp + r / a.M, i = r % a.M;
-                            v[q] = __ldcg(reinterpret_cast<const float2 *>(a.q + ((size_t)(it.be * a.M + i) * a.H + h) * HD + d2));
+                    for (int q = 0; q < 8; ++q) {
+                        const int r = rb + q * 4;
+                        v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (r < it.rows) {
+                            const int gr = it.row0 + r, h = (it.g / a.subs) * grp + gr / a.M, i = gr % a.M;
+                            v[q] = __ldcg(reinterpret_cast<const float4 *>(a.q + ((size_t)(it.be * a.M + i) * a.H + h) * HD + 4 * lane));
                         }
                     }
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int idx = idx0 + q * 128, r = idx / (HD / 2), d2 = (idx % (HD / 2)) * 2;
-                        if (idx >= n_el) continue;
-                        uint32_t hi, lo;
-                        split_pair(v[q].x * a.scale, v[q].y * a.scale, hi, lo);
-                        const int dc = d2 & 63;                                    // dim inside its 64-dim chunk
+                    for (int q = 0; q < 8; ++q) {
+                        const int r = rb + q * 4, d4 = 4 * lane;
+                        if (r >= a.qrows8) continue;
+                        uint2 hi, lo;
+                        split_pair(v[q].x * a.scale, v[q].y * a.scale, hi.x, lo.x);
+                        split_pair(v[q].z * a.scale, v[q].w * a.scale, hi.y, lo.y);
+                        const int dc = d4 & 63;                                    // dim inside its 64-dim chunk
                         for (int rp = 0; rp < a.reps; ++rp) {                      // one copy per replica's block of lanes
                             const uint32_t rr = (uint32_t)(rp * a.rows_per_rep + r);
                             const uint32_t off = rr * 128u + ((((uint32_t)dc >> 3) ^ (rr & 7u)) << 4) + ((uint32_t)dc & 7u) * 2u;
-                            *reinterpret_cast<uint32_t *>(q_gen + a.qoff[d2 >> 6] + off) = hi;
-                            *reinterpret_cast<uint32_t *>(q_gen + a.qoff[2 + (d2 >> 6)] + off) = lo;
+                            *reinterpret_cast<uint2 *>(q_gen + a.qoff[d4 >> 6] + off) = hi;
+                            *reinterpret_cast<uint2 *>(q_gen + a.qoff[2 + (d4 >> 6)] + off) = lo;
                         }
                     }
                 }
@@ -333,7 +335,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 if (lane == 0) mbar_arrive(qfull_bar);
                 q_be = it.be; q_g = it.g;
             }
-            const int h = it.g * grp + row / a.M, node = row % a.M;
+            const bool live = row < it.rows, warp_live = (quarter * 32) % a.rows_per_rep < it.rows;
+            const int h = (it.g / a.subs) * grp + (it.row0 + row) / a.M, node = (it.row0 + row) % a.M;
             const unsigned long long anc = live ? a.tree[it.b].anc[node] : 0ull;
             float m_run = -INFINITY, l_run = 0.f;
 
@@ -469,15 +472,16 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 __threadfence();
                 if (!(ok = wg_sync())) break;
                 if (et == 0) {
-                    const int old = atomicAdd(&a.counters[it.be * a.Hkv + it.g], 1);
+                    int *ctr = a.counters + it.be * a.Hkv * a.subs + it.g;
+                    const int old = atomicAdd(ctr, 1);
                     last_sh = old == a.nsplit - 1;
-                    if (last_sh) a.counters[it.be * a.Hkv + it.g] = 0;
+                    if (last_sh) *ctr = 0;
                 }
                 if (!(ok = wg_sync())) break;
                 if (last_sh) {
                     __threadfence();
-                    for (int r = warp - 2; r < QR; r += 4) {
-                        const int hh = it.g * grp + r / a.M, i = r % a.M;
+                    for (int r = warp - 2; r < it.rows; r += 4) {
+                        const int hh = (it.g / a.subs) * grp + (it.row0 + r) / a.M, i = (it.row0 + r) % a.M;
                         const float *src = a.part + (((size_t)it.be * a.H + hh) * a.M + i) * (size_t)n_part * ROWF;
                         // lane s holds range s's (max, sum); the weights go round by shuffle (at most 32 ranges when fused)
                         float ms = -INFINITY, ls = 0.f;
@@ -531,8 +535,13 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 
 }  // namespace
 
-// Replicas of the query rows across the 128 TMEM lanes (each takes a share of every tile's keys)
-int attention_tc_replicas(int query_rows) { return query_rows <= 32 ? 4 : query_rows <= 64 ? 2 : 1; }
+// Items per kv head (at most 128 query rows each)
+int attention_tc_items(int query_rows) { return (query_rows + 127) / 128; }
+// Replicas of an item's query rows across the 128 TMEM lanes (each takes a share of every tile's keys)
+int attention_tc_replicas(int query_rows) {
+    query_rows = (query_rows + attention_tc_items(query_rows) - 1) / attention_tc_items(query_rows);
+    return query_rows <= 32 ? 4 : query_rows <= 64 ? 2 : 1;
+}
 
 // tensor maps over the caches are rebuilt only when the caller's pointers change
 static int cache_maps_tc(viasd_model *m, CacheMaps &cm, const void *kc, const void *vc, int n_layers) {
@@ -560,9 +569,12 @@ int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool sli
         cm2 = &m->cmaps_slim;
         if ((rc = cache_maps_tc(m, *cm2, kc2, vc2, m->n_routed))) return rc;
     }
-    const int grp = c.n_heads / c.n_kv_heads, QR = grp * M;
-    if (QR > 128) return VIASD_EINVAL;
+    const int QR = c.n_heads / c.n_kv_heads * M;
     AttnTcArgs a;
+    a.subs = attention_tc_items(QR);
+    a.rows_sub = a.subs == 1 ? QR : ((QR + a.subs - 1) / a.subs + 7) / 8 * 8;
+    a.subs = (QR + a.rows_sub - 1) / a.rows_sub;
+    if (fuse_merge && a.subs > VIASD_ATTN_ITEMS_PER_KV_HEAD) return VIASD_EINVAL;
     a.q = m->ws.q; a.part = m->ws.part; a.out = (__nv_bfloat16 *)m->ws.attn;
     a.out_plane = m->ws.rows_alloc * (size_t)c.n_heads * HD;
     a.len_eff = m->ws.len_eff; a.tree = m->ws.tree; a.status = &m->ws.stats->device_status; a.run_flag = m->run_flag;
@@ -571,7 +583,7 @@ int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool sli
     a.batch = batch; a.layer_ord2 = layer_ord2; a.streams = streams;
     a.counters = m->ws.attn_counters;
     a.fuse_merge = fuse_merge;
-    a.qrows8 = (QR + 7) / 8 * 8;
+    a.qrows8 = (a.rows_sub + 7) / 8 * 8;
     a.reps = attention_tc_replicas(QR);
     a.rows_per_rep = 128 / a.reps;
     {
@@ -583,7 +595,7 @@ int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool sli
             a.qoff[k] = a.reps == 1 ? k * slot : (k / per_period) * 16384u + (k % per_period) * slot;
         a.q_bytes = a.qoff[3] + (uint32_t)(a.reps - 1) * period + slot;
     }
-    a.n_items = streams * batch * c.n_kv_heads * nsplit;
+    a.n_items = streams * batch * c.n_kv_heads * a.subs * nsplit;
     int grid = a.n_items < m->sm_count ? a.n_items : m->sm_count;
     a.items_per_cta = (a.n_items + grid - 1) / grid;
     grid = (a.n_items + a.items_per_cta - 1) / a.items_per_cta;

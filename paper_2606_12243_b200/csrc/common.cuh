@@ -218,6 +218,8 @@ int launch_attention_mma(viasd_model *m, const void *kc, const void *vc, bool sl
                          const void *vc2, int layer_ord2, int streams, int batch, int M, int nsplit, int fuse_merge,
                          cudaStream_t st);
 int attention_tc_replicas(int query_rows);
+int attention_tc_items(int query_rows);
+int attention_tensor_supported(const viasd_model *m);
 int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, const void *kc2,
                          const void *vc2, int layer_ord2, int streams, int batch, int M, int nsplit, int fuse_merge,
                          cudaStream_t st);

@@ -141,6 +141,10 @@ def test_forward_with_many_rows(name, batch, nodes):
     base = W.get(name)
     wl = replace(base, batch=batch, ctx=70, parent=W.chain(nodes),
                  shape=replace(base.shape, n_layers=2, d_ff=base.shape.d_ff + 8, vocab=base.shape.vocab + 2), n_routed=1)
+    _check_rows(wl)
+
+
+def _check_rows(wl):
     vb = _vb()
     eng, st, si, model = _prepare(wl)
     rows = step.block_rows(st.pending, si.draft_tok)
@@ -156,6 +160,16 @@ def test_forward_with_many_rows(name, batch, nodes):
         assert rel.max() <= PU.TOL["bf16"]["rel_l2"] and (err.max(axis=2) / rms).max() <= 7.0, (rel.max(), (err.max(axis=2) / rms).max())
     assert vb.get_stats(eng.model).device_status == 0
     assert eng.guards_intact()
+
+
+# Attention of a block with more than 128 query rows per kv head: items of at most 128 rows
+@pytest.mark.parametrize("name,batch,nodes,ctx", [("mini_8b_tree", 1, 32, 700), ("mini_8b_tree", 2, 63, 0), ("mini_32b", 1, 25, 517),
+                                                  ("mini_32b", 2, 63, 130)])
+def test_forward_with_wide_query_groups(name, batch, nodes, ctx):
+    """132 and 130 rows (two items, the second with fewer rows), 256 (two whole items), 320 (three); one key range and
+    several, merged in the kernel and apart.  Bounds as above."""
+    base = W.get(name)
+    _check_rows(replace(base, batch=batch, ctx=ctx, parent=W.chain(nodes), shape=replace(base.shape, n_layers=2), n_routed=1))
 
 
 def test_forward_is_deterministic_and_slim_all_layers_equals_full():
