@@ -1138,6 +1138,34 @@ def test_kl_cost_matches_oracle(rows, vocab):
     assert lib.viasd_kl_cost(None, tp.data_ptr(), rows, vocab, 1.0, 0.0, 1.0, 0, 1.0, got.data_ptr(), None, None) == vb.VIASD_EINVAL
 
 
+@pytest.mark.parametrize("rows,vocab", [(301, 16387), (150, 65540), (149, 70001)])
+def test_scores_of_more_rows_than_clusters(rows, vocab):
+    """Two and four CTAs per row, more rows than the device holds clusters (each works through several), vocabularies of every
+    alignment, a value far above its row's others (a thread's reference moves).  Cost and masses against the oracle with the
+    bounds of the tests above; a row's bits do not depend on the rows around it."""
+    from oracle import cost
+    vb = _vb()
+    judge = synth.normal_f32(77, rows, (rows, vocab), 2.0)
+    prop = judge + synth.normal_f32(78, rows, (rows, vocab), 0.5)
+    judge[1, vocab - 2] += 60.0
+    prop[2, vocab // 2] += 45.0
+    tj, tp = torch.from_numpy(judge).cuda(), torch.from_numpy(prop).cuda()
+    got, total = vb.kl_cost(tj, tp)
+    want = cost.step_cost(judge, prop)
+    g = got.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(g - want) <= 2e-4 * np.maximum(1.0, np.abs(want)))
+    assert abs(float(total.item()) - want.sum()) <= 2e-4 * rows * max(1.0, np.abs(want).max())
+    lo, hi = float(np.log(0.02)), float(np.log(0.3))
+    mass, mean = vb.region_mass(tj, tp, hi, lo)
+    want = tiers.region_masses(judge, prop, lo, hi, 1.0)
+    assert np.abs(mass.cpu().numpy() - want).max() <= 2e-5
+    assert np.abs(mean.cpu().numpy() - want.mean(axis=0)).max() <= 2e-5
+    if vocab % 4 == 0:
+        r = rows - 1
+        assert torch.equal(vb.kl_cost(tj[r:].contiguous(), tp[r:].contiguous())[0][0], got[r])
+        assert torch.equal(vb.region_mass(tj[r:].contiguous(), tp[r:].contiguous(), hi, lo)[0][0], mass[r])
+
+
 # ---------------------------------------------------------------------------------------------
 # Algorithm 2 as printed: the slim verifier's own confidence gates the tiers, a tier-1 acceptance ends the block
 # ---------------------------------------------------------------------------------------------
