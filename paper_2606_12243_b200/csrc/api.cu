@@ -56,8 +56,7 @@ size_t carve(const viasd_config &c, char *base, Workspace *ws) {
     w.row_tok = cv.take<int>(R * 4);
     w.tree = cv.take<TreeInfo>(sizeof(TreeInfo) * (size_t)c.max_batch);
     w.stats = cv.take<DeviceStats>(sizeof(DeviceStats));
-    w.accept_scratch = cv.take<float>(((size_t)c.max_batch * (VIASD_MAX_JUDGES + 1) * c.vocab +
-                                       (size_t)c.max_batch * 3 * (VIASD_MAX_JUDGES + 1) * VIASD_MAX_ROWS_PER_SEQ) * 4);
+    w.accept_scratch = cv.take<float>((size_t)c.max_batch * 3 * (VIASD_MAX_JUDGES + 1) * VIASD_MAX_ROWS_PER_SEQ * 4);
     {
         const int nt = tc_pick_nt(R < 128 ? (int)R : 128, true);
         w.gemm_scratch = cv.take<float>(tc_scratch_floats(MAX_GEMM_CTAS, nt, true) * 4);
@@ -496,12 +495,12 @@ static int tier_accept_set(viasd_model *m, const viasd_draft *draft, const viasd
     if (draft->n_nodes < 1 || !draft->prow || !draft->drafter_logits || draft->n_prows < 1) return VIASD_EINVAL;
     for (int k = 1; k < js.n; ++k) if (!(js.log_tau[k] <= js.log_tau[k - 1])) return VIASD_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    if (phase & 1) {
+    if (phase == 1) {
         if ((rc = timed(m, VIASD_T_TIER_ACCEPT, st, [&] { return launch_tier(m, draft, params, js, result, st); }))) return rc;
     }
     if (phase & 2) {
         for (int k = 0; k < js.n; ++k) if (!js.logits[k]) return VIASD_EINVAL;
-        if ((rc = timed(m, VIASD_T_TIER_ACCEPT, st, [&] { return launch_accept(m, draft, params, js, result, tree_ready, st); })))
+        if ((rc = timed(m, VIASD_T_TIER_ACCEPT, st, [&] { return launch_accept(m, draft, params, js, result, tree_ready, (phase & 1) != 0, st); })))
             return rc;
     }
     return VIASD_OK;
@@ -580,8 +579,8 @@ static int verify_step_routed(viasd_model *m, viasd_cache *cache, const viasd_dr
     CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(int), st));
     AcceptProbe probe{G, flag, cache->len, cache->len_full};
     JudgeSet probe_set{2, {slim_logits, nullptr}, {params->log_tau_hi, params->log_tau_lo}};
-    if ((rc = timed(m, VIASD_T_TIER_ACCEPT, st, [&] { return launch_accept(m, draft, params, probe_set, result, true, st,
-                                                                      &probe); }))) return rc;
+    if ((rc = timed(m, VIASD_T_TIER_ACCEPT, st, [&] { return launch_accept(m, draft, params, probe_set, result, true,
+                                                                      false, st, &probe); }))) return rc;
     m->run_flag = flag;
     rc = forward_sweep(m, cache, draft, 0, full_logits, nullptr, st, G);
     m->run_flag = nullptr;
@@ -607,15 +606,10 @@ int viasd_verify_step(viasd_model *m, viasd_cache *cache, const viasd_draft *dra
         if ((rc = tier_accept_impl(m, draft, params, slim_logits, full_logits, 3, result, true, stream))) return rc;
         return viasd_kv_commit(m, cache, draft, result, stream);
     }
-    if (params->conf_source == 0) {
-        if ((rc = viasd_tier_accept(m, draft, params, nullptr, nullptr, 1, result, stream))) return rc;
-        if ((rc = viasd_slim_forward(m, cache, draft, slim_logits, stream))) return rc;
-    } else {
-        if ((rc = viasd_slim_forward(m, cache, draft, slim_logits, stream))) return rc;
-        if ((rc = viasd_tier_accept(m, draft, params, slim_logits, nullptr, 1, result, stream))) return rc;
-    }
+    if ((rc = viasd_slim_forward(m, cache, draft, slim_logits, stream))) return rc;
     if ((rc = viasd_full_forward(m, cache, draft, full_logits, stream))) return rc;
-    if ((rc = tier_accept_impl(m, draft, params, slim_logits, full_logits, 2, result, true, stream))) return rc;
+    // (no pass depends on the tiers: they come with the walk, from the statistics it reads)
+    if ((rc = tier_accept_impl(m, draft, params, slim_logits, full_logits, 3, result, true, stream))) return rc;
     return viasd_kv_commit(m, cache, draft, result, stream);
 }
 

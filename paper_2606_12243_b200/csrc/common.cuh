@@ -55,7 +55,7 @@ struct Workspace {                      // pointers into the caller's workspace 
     int *row_tok;                       // [R] token id per row
     TreeInfo *tree;                     // [max_batch]: every sequence has its own draft tree (copies when the call shares one)
     DeviceStats *stats;
-    float *accept_scratch;              // [B, 3, V] sampling-mode distributions, then [3][B, 3, 64] row statistics
+    float *accept_scratch;              // [3][B, judges + 1, 64] row statistics
     float *gemm_scratch;                // partial tiles of split GEMM work (tcgen05 kernel)
     int *gemm_counters;                 // per-tile arrival counters, zero between launches
     size_t n_counters;
@@ -121,26 +121,39 @@ struct viasd_model {
 #ifdef __CUDACC__
 // Lays out one sequence's draft tree: ancestor sets, depths, child lists.  parent[n] = -1: child of the pending token;
 // -2: the node is unused (a sequence with fewer nodes than the call's N): it is nobody's child and nothing attends to it.
-__device__ inline void build_tree(TreeInfo *tree, const int *parent, int N, DeviceStats *stats) {
-    const int M = N + 1;
-    int last_child[VIASD_MAX_ROWS_PER_SEQ];
-    for (int i = 0; i < M; ++i) { tree->first_child[i] = -1; tree->next_sibling[i] = -1; last_child[i] = -1; }
-    tree->anc[0] = 1ull;
-    tree->depth[0] = 0;
-    int chain = 1;
-    for (int n = 0; n < N; ++n) {
+// By one warp, a row per lane and turn; par_sh: [VIASD_MAX_ROWS_PER_SEQ] shared, the warp's own.  (One thread going through
+// the nodes in order, each a round trip through memory, took 7 us for a tree of 26 and 13 us for a chain of 63.)
+__device__ inline void build_tree(TreeInfo *tree, const int *parent, int N, DeviceStats *stats, int *par_sh) {
+    const int lane = threadIdx.x & 31, M = N + 1;
+    bool chain = true;
+    for (int n = lane; n < N; n += 32) {
         int p = parent[n];
-        const int i = n + 1;
-        if (p == -2) { tree->anc[i] = 1ull << i; tree->depth[i] = 0; chain = 0; continue; }
-        if (p < -1 || p >= n) { stats->device_status = VIASD_EDEVICE; p = -1; }
-        if (p != n - 1) chain = 0;
-        const int pr = p + 1;
-        tree->anc[i] = tree->anc[pr] | (1ull << i);
-        tree->depth[i] = tree->depth[pr] + 1;
-        if (last_child[pr] < 0) tree->first_child[pr] = n; else tree->next_sibling[last_child[pr]] = n;
-        last_child[pr] = n;
+        if (p != -2 && (p < -1 || p >= n)) { stats->device_status = VIASD_EDEVICE; p = -1; }
+        chain = chain && p == n - 1;
+        par_sh[n] = p;
     }
-    tree->is_chain = chain;
+    chain = __all_sync(0xffffffffu, chain);
+    __syncwarp();
+    for (int i = lane; i < M; i += 32) {                     // row i is node i - 1 (row 0: the pending token)
+        unsigned long long anc = 1ull << i;
+        int depth = 0, first = -1, next = -1;
+        if (i > 0 && par_sh[i - 1] != -2) {
+            int n = i - 1;                                   // a parent comes before its children, so this ends
+            for (; n >= 0 && par_sh[n] != -2; n = par_sh[n]) { anc |= 1ull << (n + 1); ++depth; }
+            anc |= 1ull << (n + 1);                          // the pending token's row
+        }
+        for (int n = N - 1; n >= 0; --n) {
+            const int p = par_sh[n];
+            if (p == i - 1) first = n;                       // lowest child of this row
+            if (i > 0 && n >= i && p != -2 && p == par_sh[i - 1]) next = n;      // lowest later sibling of node i - 1
+        }
+        tree->anc[i] = anc;
+        tree->depth[i] = depth;
+        tree->first_child[i] = first;
+        if (i > 0) tree->next_sibling[i - 1] = next;
+    }
+    if (lane == 0) { tree->is_chain = chain; tree->next_sibling[N] = -1; }
+    __syncwarp();                                            // par_sh may be used again
 }
 
 #endif
@@ -241,7 +254,7 @@ int launch_tier(const viasd_model *m, const viasd_draft *d, const viasd_params *
 // probe != null: the walk on the slim verifier's logits alone, deciding whether the full verifier's pass is needed
 struct AcceptProbe { int replay_rows; int *need_full; const int *len, *len_full; };
 int launch_accept(const viasd_model *m, const viasd_draft *d, const viasd_params *p, const JudgeSet &js, viasd_result *r,
-                  bool tree_ready, cudaStream_t st, const AcceptProbe *probe = nullptr);
+                  bool tree_ready, bool do_tier, cudaStream_t st, const AcceptProbe *probe = nullptr);   // do_tier: assign the tiers too
 
 // ---------------------------------------------------------------------------------------------
 // small device helpers

@@ -28,15 +28,17 @@ int launch_rope_table(const viasd_model *m, cudaStream_t st) {
 // ---------------------------------------------------------------------------------------------
 // per-pass preparation
 // ---------------------------------------------------------------------------------------------
+constexpr int PREP_WARPS = 16;
 // parent: [N] shared by the batch, or [B, N] when per_seq
 __global__ void prep_kernel(TreeInfo *tree, int *len_eff, int *row_tok, DeviceStats *stats, const int *len,
                             const int *pending, const int *draft_tok, const int *parent, int per_seq, int B, int N,
                             int max_ctx, int vocab, int full_pass) {
     const int M = N + 1;
     PDL_TRIGGER();
+    __shared__ int par_sh[PREP_WARPS][VIASD_MAX_ROWS_PER_SEQ];
     if (threadIdx.x == 0 && full_pass) stats->full_ran = 1;     // the full verifier's cache receives this block's rows
+    for (int b = threadIdx.x >> 5; b < B; b += PREP_WARPS) build_tree(tree + b, parent + (per_seq ? (size_t)b * N : 0), N, stats, par_sh[threadIdx.x >> 5]);
     for (int b = threadIdx.x; b < B; b += blockDim.x) {
-        build_tree(tree + b, parent + (per_seq ? (size_t)b * N : 0), N, stats);
         int l = len[b];
         int c = min(max(l, 0), max_ctx - M);
         if (c != l) stats->device_status = VIASD_ECAPACITY;
@@ -51,7 +53,7 @@ __global__ void prep_kernel(TreeInfo *tree, int *len_eff, int *row_tok, DeviceSt
 }
 
 int launch_prep(const viasd_model *m, const viasd_cache *c, const viasd_draft *d, bool full_pass, cudaStream_t st) {
-    prep_kernel<<<1, 128, 0, st>>>(m->ws.tree, m->ws.len_eff, m->ws.row_tok, m->ws.stats, c->len, c->pending,
+    prep_kernel<<<1, 32 * PREP_WARPS, 0, st>>>(m->ws.tree, m->ws.len_eff, m->ws.row_tok, m->ws.stats, c->len, c->pending,
                                    d->draft_tok, d->parent, d->per_sequence, d->batch, d->n_nodes, m->cfg.max_ctx,
                                    m->cfg.vocab, full_pass ? 1 : 0);
     LAUNCH_CHECK();

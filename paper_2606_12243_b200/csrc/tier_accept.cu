@@ -1,26 +1,29 @@
-// Fused confidence-tier kernel and accept / resolve kernel.
+// Confidence tiers and accept / resolve.
 //
-// Tier kernel (App. B, Eq. B.1-B.3): per drafted token v, d = l[v] - max_u l[u] on the gating logits;
-// tier 0 if d >= log_tau_hi, 1 if d >= log_tau_lo, else 2.  One CTA per gating row scans the
-// vocabulary once and serves every node gated by that row.
+// Tiers (App. B, Eq. B.1-B.3): per drafted token v, d = l[v] - max_u l[u] on the gating logits;
+// tier 0 if d >= log_tau_hi, 1 if d >= log_tau_lo, else 2.  Asked for alone (phase 1) a kernel with one CTA per gating
+// row scans the vocabulary; asked for together with the walk, the tiers come from the row statistics the walk needs anyway.
 //
 // Accept kernel (Algorithm 2, per-position loop; Algorithm 1, what is appended; App. A, Eq. A.2-A.3):
-// one CTA per sequence (a cluster of eight when it samples over a large vocabulary) walks the draft from the pending token: children of the current row are tried in
-// index order; tier-0 children are taken at once, tier-1 children are judged by q', tier-2 children by
-// q.  The first row where no child passes ends the walk and the strongest judge that rejected there
-// emits the replacement token.  The walk is sequential over depth, so everything that can be known before
-// it is: a row-statistics kernel (one CTA per logits row, all rows at once) leaves each row's maximum,
-// argmax and softmax denominator, which makes every first test at a position O(1).  Only a rejection in
-// sampling mode (residual, Eq. A.3: two sweeps) and the final draw still sweep the vocabulary inside the walk;
-// the CTAs of a cluster share each sweep and combine their block results through distributed shared memory in rank
-// order, so all of them hold the same values and walk the same way.
+// one CTA per sequence (a cluster of 8 or 16 when it samples over a large vocabulary) walks the draft from the pending
+// token: children of the current row are tried in index order; tier-0 children are taken at once, tier-1 children are
+// judged by q', tier-2 children by q.  The first row where no child passes ends the walk and the strongest judge that
+// rejected there emits the replacement token.  The walk is sequential over depth, so everything that can be known before
+// it is: a row-statistics kernel (one CTA per logits row, all rows at once, one sweep) leaves each row's maximum, argmax
+// and softmax denominator, and the walk starts by fetching the tree and every node's two logits at once, so that a test is
+// arithmetic on shared memory.  Only a rejection in sampling mode (residual, Eq. A.3) and the final draw sweep the
+// vocabulary: one sweep and one exchange among the cluster's CTAs each.  The residuals are not written out: an element is
+// worked out from the logits by replaying the rejections so far (a handful of scalars), in the arithmetic of Eq. A.3 round
+// by round.  CTAs exchange their sums by storing them into each other's shared memory before one cluster barrier; every
+// CTA adds them in the same order, so all of them walk the same way.
 #include "common.cuh"
 #include <string.h>
 #include <stdlib.h>
 
 namespace {
 
-constexpr int ACC_THREADS = 512;
+constexpr int ACC_THREADS = 512, ACC_WARPS = ACC_THREADS / 32;
+constexpr int MAX_TEAM = 16;
 constexpr int MAXJ = VIASD_MAX_JUDGES;    // verifiers that may judge a drafted token (the last one is q); 2 for three tiers
 constexpr int KINDS = MAXJ + 1;           // distributions kept per position: the proposal and the judges
 constexpr int ACC_TEAM = 8;               // CTAs per sequence in sampling mode (a portable cluster size)
@@ -44,13 +47,13 @@ __device__ __forceinline__ float unit_f32(unsigned long long key, unsigned long 
     return ((float)(w >> 41) + 0.5f) * 1.1920928955078125e-7f;
 }
 
-// ---- block reductions ---------------------------------------------------------------------------
+// ---- block reductions: in every thread; sh: a buffer nobody reads any more ----------------------
 struct MaxIdx { float v; int i; };
 __device__ __forceinline__ MaxIdx better(MaxIdx a, MaxIdx b) {   // larger value, lowest index on ties
     if (b.v > a.v || (b.v == a.v && b.i < a.i)) return b;
     return a;
 }
-__device__ MaxIdx block_argmax(MaxIdx x, MaxIdx *sh) {
+__device__ __forceinline__ MaxIdx warp_argmax(MaxIdx x) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         MaxIdx y;
@@ -58,30 +61,29 @@ __device__ MaxIdx block_argmax(MaxIdx x, MaxIdx *sh) {
         y.i = __shfl_xor_sync(0xffffffffu, x.i, o);
         x = better(x, y);
     }
-    __syncthreads();
+    return x;
+}
+__device__ __forceinline__ MaxIdx no_idx() { MaxIdx r; r.v = -INFINITY; r.i = 0x7fffffff; return r; }
+__device__ MaxIdx block_argmax(MaxIdx x, MaxIdx *sh) {
+    x = warp_argmax(x);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
     __syncthreads();
-    MaxIdx r = sh[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = better(r, sh[w]);
-    return r;
+    const int lane = threadIdx.x & 31;
+    return warp_argmax(lane < (int)(blockDim.x >> 5) ? sh[lane] : no_idx());
 }
 __device__ float block_sum(float x, float *sh) {
     x = warp_sum(x);
-    __syncthreads();
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
     __syncthreads();
-    float r = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += sh[w];
-    return r;
+    const int lane = threadIdx.x & 31;
+    return warp_sum(lane < (int)(blockDim.x >> 5) ? sh[lane] : 0.f);
 }
 __device__ float block_max(float x, float *sh) {
     x = warp_max(x);
-    __syncthreads();
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
     __syncthreads();
-    float r = sh[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = fmaxf(r, sh[w]);
-    return r;
+    const int lane = threadIdx.x & 31;
+    return warp_max(lane < (int)(blockDim.x >> 5) ? sh[lane] : -INFINITY);
 }
 
 // ---- tier kernel ------------------------------------------------------------------------------
@@ -132,51 +134,95 @@ tier_kernel(unsigned char *__restrict__ tier, float *__restrict__ conf, DeviceSt
 
 // ---- row statistics ---------------------------------------------------------------------------
 // grid (rows, B, 1 + judges): kind 0 = drafter rows [B, R, V], kind k = judge k's rows [B, M, V] (the last judge is q).
-// Per row: max, argmax (lowest index on ties) and, when want_z, sum exp((l - max) / T).
-constexpr int RS_STRIDE = VIASD_MAX_ROWS_PER_SEQ;
+// Per row: max, argmax (lowest index on ties) and, when wanted, sum exp((l - max) / T).
+// HBM-bound: every row once.  Maximum and denominator come from one sweep (a running reference per thread, moved when it is
+// exceeded by e^20); two sweeps read a batch's rows twice from HBM, 16 sequences' 1040 rows of 0.5 MB being far more than L2
+// holds.  Eight 16-byte loads per thread in flight: few rows are bound by what a CTA has under way.
+constexpr int RS_STRIDE = VIASD_MAX_ROWS_PER_SEQ, RS_THREADS = 512, RS_BATCH = 8;
+constexpr float RS_GAP = 20.f, LOG2E = 1.4426950408889634f;
 struct RowStats { float *mx; int *arg; float *z; };       // each [B, KINDS, RS_STRIDE]
 struct RowPtrs { const float *p[KINDS]; };                // drafter logits, then each judge's
 
-__global__ void __launch_bounds__(1024)
-row_stats_kernel(RowStats rs, RowPtrs src, int R, int M, int V, float inv_temp, int want_z) {
-    __shared__ float sh[32];
-    __shared__ MaxIdx shm[32];
+__device__ __forceinline__ float ex2(float x) {            // 2^x, hardware approximation (2 ulp)
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+template <bool WANT_Z>
+struct RowAcc {
+    float ref, lim, s;
+    MaxIdx best;
+    __device__ __forceinline__ void init() { ref = lim = -INFINITY; s = 0.f; best = no_idx(); }
+    // N values from index i on, in pieces of four `step` apart
+    template <int N>
+    __device__ __forceinline__ void add(const float (&x)[N], int i, int step, float scale2, float gap) {
+        float bm = x[0];
+#pragma unroll
+        for (int e = 1; e < N; ++e) bm = fmaxf(bm, x[e]);
+        if (bm > best.v) {                                 // rare after the first batches
+            best.v = bm;
+#pragma unroll
+            for (int e = N - 1; e >= 0; --e) if (x[e] == bm) best.i = i + (e >> 2) * step + (e & 3);
+        }
+        if (!WANT_Z) return;
+        if (bm > lim) {
+            s *= ex2((ref - bm) * scale2);
+            ref = bm;
+            lim = bm + gap;
+        }
+        const float r = ref == -INFINITY ? 0.f : ref;
+#pragma unroll
+        for (int e = 0; e < N; ++e) s += ex2((x[e] - r) * scale2);
+    }
+};
+
+template <bool WANT_Z>
+__global__ void __launch_bounds__(RS_THREADS, 2)
+row_stats_kernel(RowStats rs, RowPtrs src, int R, int M, int V, float inv_temp, DeviceStats *stats, int clear_needs,
+                 TreeInfo *tree, const int *parent, int per_seq) {
+    // tree != null: no forward pass of the same call has laid the trees out, so the first CTA of each sequence does
+    __shared__ float sh[RS_THREADS / 32];
+    __shared__ MaxIdx shm[RS_THREADS / 32];
     const int kind = blockIdx.z, b = blockIdx.y, r = blockIdx.x;
+    __shared__ int par_sh[VIASD_MAX_ROWS_PER_SEQ];
+    if (kind == 0 && r == 0) {
+        if (clear_needs && b == 0 && threadIdx.x == 0) stats->need_slim = stats->need_full = 0;
+        if (tree && threadIdx.x < 32) build_tree(tree + b, parent + (per_seq ? (size_t)b * (M - 1) : 0), M - 1, stats, par_sh);
+    }
     const float *base = src.p[kind];
     const int rows = kind == 0 ? R : M;
     if (!base || r >= rows) return;
     const float *row = base + ((size_t)b * rows + r) * V;
-    const bool vec = (V & 3) == 0 && ((uintptr_t)row & 15) == 0;
-    MaxIdx best; best.v = -INFINITY; best.i = 0x7fffffff;
-    if (vec) {
-        const float4 *r4 = reinterpret_cast<const float4 *>(row);
-        for (int i = threadIdx.x; i < V / 4; i += blockDim.x) {
-            const float4 v = r4[i];
-            MaxIdx c;
-            c.v = v.x; c.i = 4 * i; best = better(best, c);
-            c.v = v.y; c.i = 4 * i + 1; best = better(best, c);
-            c.v = v.z; c.i = 4 * i + 2; best = better(best, c);
-            c.v = v.w; c.i = 4 * i + 3; best = better(best, c);
+    const float scale2 = inv_temp * LOG2E, gap = RS_GAP / inv_temp;
+    RowAcc<WANT_Z> acc;
+    acc.init();
+    // up to three values in front of the first 16-byte boundary (an odd vocabulary), then 16-byte pieces, then the rest
+    const int head = min(V, (int)((4 - ((reinterpret_cast<uintptr_t>(row) >> 2) & 3)) & 3)), n4 = (V - head) >> 2, tail = V - head - 4 * n4;
+    const float4 *r4 = reinterpret_cast<const float4 *>(row + head);
+    if ((int)threadIdx.x < head) { const float x[1] = {row[threadIdx.x]}; acc.add(x, threadIdx.x, 0, scale2, gap); }
+    int i0 = threadIdx.x;
+#pragma unroll 1
+    for (; i0 + (RS_BATCH - 1) * RS_THREADS < n4; i0 += RS_BATCH * RS_THREADS) {
+        float x[4 * RS_BATCH];
+#pragma unroll
+        for (int j = 0; j < RS_BATCH; ++j) {
+            const float4 v = r4[i0 + j * RS_THREADS];
+            x[4 * j] = v.x; x[4 * j + 1] = v.y; x[4 * j + 2] = v.z; x[4 * j + 3] = v.w;
         }
-    } else {
-        for (int i = threadIdx.x; i < V; i += blockDim.x) { MaxIdx c; c.v = row[i]; c.i = i; best = better(best, c); }
+        acc.add(x, head + 4 * i0, 4 * RS_THREADS, scale2, gap);
     }
-    best = block_argmax(best, shm);
+#pragma unroll 1
+    for (; i0 < n4; i0 += 2 * RS_THREADS) {
+        const bool two = i0 + RS_THREADS < n4;
+        const float4 v = r4[i0], w = two ? r4[i0 + RS_THREADS] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        const float x[8] = {v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w};
+        acc.add(x, head + 4 * i0, 4 * RS_THREADS, scale2, gap);
+    }
+    if ((int)threadIdx.x < tail) { const float x[1] = {row[V - tail + threadIdx.x]}; acc.add(x, V - tail + threadIdx.x, 0, scale2, gap); }
+    const MaxIdx best = block_argmax(acc.best, shm);
     float z = 0.f;
-    if (want_z) {
-        const float mx = best.v;
-        if (vec) {
-            const float4 *r4 = reinterpret_cast<const float4 *>(row);
-            for (int i = threadIdx.x; i < V / 4; i += blockDim.x) {
-                const float4 v = r4[i];
-                z += expf((v.x - mx) * inv_temp) + expf((v.y - mx) * inv_temp) + expf((v.z - mx) * inv_temp) +
-                     expf((v.w - mx) * inv_temp);
-            }
-        } else {
-            for (int i = threadIdx.x; i < V; i += blockDim.x) z += expf((row[i] - mx) * inv_temp);
-        }
-        z = block_sum(z, sh);
-    }
+    if (WANT_Z) z = block_sum(acc.ref == -INFINITY ? 0.f : acc.s * ex2((acc.ref - best.v) * scale2), sh);
     if (threadIdx.x == 0) {
         const size_t o = ((size_t)b * KINDS + kind) * RS_STRIDE + r;
         rs.mx[o] = best.v;
@@ -191,10 +237,10 @@ struct AcceptArgs {
     const float *judges[KINDS];              // [1..n_judges]: each judge's logits [B, M, V], weakest first, q last
     const float *drafter;                    // [B, R, V]
     int n_judges;
-    const int *draft_tok, *prow;             // [B, N], [N]
-    const unsigned char *tier;               // [B, N]
+    const int *draft_tok, *prow, *parent;    // [B, N], [N], [N]
+    unsigned char *tier;                     // [B, N]
+    float *conf;                             // [B, N]: written with the tiers
     const TreeInfo *tree;
-    float *scratch;                          // [B, KINDS, V]
     int *n_acc, *path, *out_tok, *n_emit, *corr_src;
     unsigned char *judge;
     DeviceStats *stats;
@@ -203,6 +249,8 @@ struct AcceptArgs {
     float inv_temp, log1m_alpha, inv_beta;
     float log_acc_rel[KINDS];                // greedy gate per judging tier
     unsigned long long seed, step;
+    int do_tier, conf_source;                // do_tier: this launch also assigns the tiers, from the row statistics
+    TierCuts cuts;
     // Probe (routed execution policy): the same walk on the slim verifier's logits alone.  It stops where the full
     // verifier's judgment (a tier-2 node, or the bonus token at a leaf) would be needed and raises *need_full; it also
     // raises it when a sequence's backlog (len - len_full) plus this step's tokens would outgrow the replay window.
@@ -213,196 +261,256 @@ struct AcceptArgs {
     const int *len, *len_full;
 };
 
-// ---- the CTAs of a sequence (a thread-block cluster in sampling mode, else one CTA) ---------------------
-// Each CTA sweeps its share of the vocabulary (indices strided by CTAs x threads); block results are combined through
-// distributed shared memory in rank order, so every CTA holds the same value and takes the same branches.
+struct Rejection { int t, v; float sj, sp; };  // judging tier, token, 1 / (beta Z_judge) (negative: the residual vanished), 1 / Z_proposal
+
+struct Walk {                                  // per CTA: everything the walk reads
+    int first_child[RS_STRIDE], next_sibling[RS_STRIDE], tok[RS_STRIDE], prow[RS_STRIDE], tier[RS_STRIDE];
+    int judged[RS_STRIDE], path[RS_STRIDE];
+    float xj[RS_STRIDE], x0[RS_STRIDE];        // logit of the node's token in its judge's row and in its drafter row
+    float mx[KINDS][RS_STRIDE], z[KINDS][RS_STRIDE];
+    int arg[KINDS][RS_STRIDE];
+    Rejection rej[RS_STRIDE];
+    int tier_count[3];
+};
+
+// The CTAs of a sequence (a thread-block cluster in sampling mode, else one CTA).  Each sweeps its share of the vocabulary.
 struct Team {
     unsigned rank, size;
-    float *slot_f;              // [2] own slots, double-buffered by phase
-    MaxIdx *slot_m;             // [2]
+    float2 (*slots)[MAX_TEAM];     // [2]: what every CTA of the team has sent, by exchange parity
     int phase;
 };
 __device__ __forceinline__ void team_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ uint32_t remote_addr(const void *own, unsigned rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(own)), "r"(rank));
-    return r;
-}
-__device__ float team_sum(float x, float *sh, Team &tm) {
-    x = block_sum(x, sh);
-    if (tm.size == 1) return x;
-    float *slot = tm.slot_f + (tm.phase & 1);
-    if (threadIdx.x == 0) *slot = x;
-    team_barrier();
-    float r = 0.f;
-    for (unsigned k = 0; k < tm.size; ++k) {
-        float v;
-        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote_addr(slot, k)));
-        r += v;
-    }
+// Every CTA's two values in lanes 0 .. size - 1 of every warp (others: `none`).  A CTA stores its own into all others'
+// shared memory and one barrier follows: reading sixteen CTAs' slots one after the other took longer than the sweep.
+// (Slots alternate: a CTA sends again into a parity only after the barrier that its readers of it have passed.)
+__device__ __forceinline__ float2 team_exchange(float2 v, float2 none, Team &tm) {
+    float2 (&slot)[MAX_TEAM] = tm.slots[tm.phase & 1];
     ++tm.phase;
-    return r;
-}
-__device__ MaxIdx team_argmax(MaxIdx x, MaxIdx *shm, Team &tm) {
-    x = block_argmax(x, shm);
-    if (tm.size == 1) return x;
-    MaxIdx *slot = tm.slot_m + (tm.phase & 1);
-    if (threadIdx.x == 0) *slot = x;
-    team_barrier();
-    MaxIdx r; r.v = -INFINITY; r.i = 0x7fffffff;
-    for (unsigned k = 0; k < tm.size; ++k) {
-        MaxIdx y;
-        const uint32_t ra = remote_addr(slot, k);
-        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(y.v) : "r"(ra));
-        asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(y.i) : "r"(ra + 4));
-        r = better(r, y);
+    if (threadIdx.x < tm.size) {
+        uint32_t a;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(&slot[tm.rank])), "r"(threadIdx.x));
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
     }
-    ++tm.phase;
-    return r;
+    team_barrier();
+    const int lane = threadIdx.x & 31;
+    return lane < (int)tm.size ? slot[lane] : none;
 }
 
-// numerators of softmax(l / T) into dst (the row maximum comes from the row statistics); this CTA's share
-__device__ void softmax_numerators(float *dst, const float *row, int V, float inv_temp, float mx, const Team &tm) {
-    for (int i = tm.rank * blockDim.x + threadIdx.x; i < V; i += tm.size * blockDim.x) dst[i] = expf((row[i] - mx) * inv_temp);
-    __syncthreads();
-}
-
-// argmax_v (log w[v] - log(-log u_v)): a draw from w / sum(w)
-__device__ int gumbel_argmax(const float *w, int V, unsigned long long key, int row, MaxIdx *shm, Team &tm) {
-    MaxIdx best; best.v = -INFINITY; best.i = 0x7fffffff;
-    for (int i = tm.rank * blockDim.x + threadIdx.x; i < V; i += tm.size * blockDim.x) {
-        float wi = w[i];
-        if (wi > 0.f) {
-            float u = unit_f32(key, ((unsigned long long)row << 32) + (unsigned long long)i);
-            MaxIdx c; c.v = logf(wi) - logf(-logf(u)); c.i = i;
-            best = better(best, c);
+// f(i, x, y) for this CTA's share of a row's indices i; x, y: the values of two rows there (y: 0 when b is null)
+template <typename F>
+__device__ __forceinline__ void sweep_rows(const float *a, const float *b, int V, const Team &tm, F f) {
+    if ((V & 3) == 0 && ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0) {
+        const float4 *a4 = reinterpret_cast<const float4 *>(a), *b4 = reinterpret_cast<const float4 *>(b);
+        const int n4 = V >> 2, per = (n4 + (int)tm.size - 1) / (int)tm.size, lo = (int)tm.rank * per, hi = min(n4, lo + per);
+        // eight loads in flight, then a rolled loop over pieces of four values (indexed, so they pass through local memory): a
+        // CTA has 16 values per thread and sweep; unrolled, their code came from a cold instruction cache (8 us a sweep), one
+        // at a time they are a chain of latencies
+#pragma unroll 1
+        for (int i0 = lo + threadIdx.x; i0 < hi; i0 += 4 * ACC_THREADS) {
+            float4 x[4], y[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int i = min(i0 + j * ACC_THREADS, hi - 1);
+                x[j] = a4[i];
+                y[j] = b ? b4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            const int n = min(4, (hi - i0 + ACC_THREADS - 1) / ACC_THREADS);
+#pragma unroll 1
+            for (int j = 0; j < n; ++j) {
+                const int i = 4 * (i0 + j * ACC_THREADS);
+                const float4 u = x[j], v = y[j];
+                f(i, u.x, v.x); f(i + 1, u.y, v.y); f(i + 2, u.z, v.z); f(i + 3, u.w, v.w);
+            }
         }
+    } else {
+        for (int i = tm.rank * ACC_THREADS + threadIdx.x; i < V; i += tm.size * ACC_THREADS) f(i, a[i], b ? b[i] : 0.f);
     }
-    best = team_argmax(best, shm, tm);
-    return best.i == 0x7fffffff ? 0 : best.i;
 }
 
-__global__ void __launch_bounds__(ACC_THREADS)
+// Numerators at token i after the rejections so far: the judge of tier t (starting from jt) and the proposal (from pr).
+// Eq. A.3 round by round: the rejecting judge becomes its residual against the proposal (kept as it is if the residual
+// vanishes); the rejected token leaves the proposal.
+__device__ __forceinline__ void replay(const Rejection *rej, int n, int i, int t, float &jt, float &pr) {
+    for (int k = 0; k < n; ++k) {
+        const Rejection r = rej[k];
+        if (r.t == t && r.sj >= 0.f) jt = fmaxf(0.f, jt * r.sj - pr * r.sp);
+        if (i == r.v) pr = 0.f;
+    }
+}
+
+__global__ void __launch_bounds__(ACC_THREADS, 2)
 accept_kernel(AcceptArgs a) {
-    __shared__ MaxIdx shm[32];
-    __shared__ float sh[32];
-    __shared__ float slot_f[2];
-    __shared__ MaxIdx slot_m[2];
+    __shared__ Walk w;
+    __shared__ MaxIdx shm[ACC_WARPS];
+    __shared__ float sh[4][ACC_WARPS];
+    __shared__ float2 slots[2][MAX_TEAM];
     Team tm;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(tm.rank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(tm.size));
-    tm.slot_f = slot_f; tm.slot_m = slot_m; tm.phase = 0;
-    const bool lead = tm.rank == 0 && threadIdx.x == 0;       // the one thread that writes the results
+    tm.slots = slots; tm.phase = 0;
+    const int tid = threadIdx.x;
     const int b = blockIdx.x / tm.size, N = a.N, M = N + 1, V = a.V;
-    const TreeInfo *tree = a.tree + b;
-    const int *prow = a.prow + (a.per_seq ? (size_t)b * N : 0);
-    const bool sampling = a.mode == 1;
+    const bool sampling = a.mode == 1, writes = tm.rank == 0 && !a.probe;     // writes: this CTA stores the results
     const int J = a.n_judges;                                 // tier J is the full verifier's
-    float *P[KINDS];
-#pragma unroll
-    for (int k = 0; k < KINDS; ++k) P[k] = a.scratch + ((size_t)b * KINDS + k) * V;
-    const float *st_mx = a.rs.mx + (size_t)b * KINDS * RS_STRIDE, *st_z = a.rs.z + (size_t)b * KINDS * RS_STRIDE;
-    const int *st_arg = a.rs.arg + (size_t)b * KINDS * RS_STRIDE;
     const unsigned long long k_acc = stream_key(a.seed, a.step, b, 0), k_gum = stream_key(a.seed, a.step, b, 1);
-    if (tm.rank == 0 && !a.probe) for (int n = threadIdx.x; n < N; n += blockDim.x) a.judge[b * N + n] = 0;
-    __syncthreads();
 
-    int cur = 0, n_acc = 0, corr = -1, corr_src = 0;
+    // ---- everything the walk reads, at once
+    if (tid < 3) w.tier_count[tid] = 0;
+    const size_t st0 = (size_t)b * KINDS * RS_STRIDE;
+    for (int e = tid; e < (J + 1) * RS_STRIDE; e += ACC_THREADS) {
+        const int k = e / RS_STRIDE, r = e - k * RS_STRIDE;
+        if (r < (k == 0 ? a.R : M)) { w.mx[k][r] = a.rs.mx[st0 + e]; w.z[k][r] = a.rs.z[st0 + e]; w.arg[k][r] = a.rs.arg[st0 + e]; }
+    }
+    for (int r = tid; r < M; r += ACC_THREADS) w.first_child[r] = a.tree[b].first_child[r];
+    __syncthreads();
+    for (int n = tid; n < N; n += ACC_THREADS) {
+        const int par = a.parent[(a.per_seq ? (size_t)b * N : 0) + n], pr = a.prow[(a.per_seq ? (size_t)b * N : 0) + n];
+        const int v = min(max(a.draft_tok[b * N + n], 0), V - 1);
+        w.next_sibling[n] = a.tree[b].next_sibling[n];
+        w.tok[n] = v;
+        w.prow[n] = pr;
+        w.judged[n] = 0;
+        const bool pr_ok = pr >= 0 && pr < a.R;
+        const float x0 = a.drafter && pr_ok && par != -2 ? a.drafter[((size_t)b * a.R + pr) * V + v] : 0.f;
+        w.x0[n] = x0;
+        int t;
+        if (a.do_tier) {
+            t = 0;
+            float d = 0.f;
+            const int g = a.conf_source == 0 ? pr : par + 1;
+            if (par != -2 && (a.conf_source ? g >= 0 && g < M : pr_ok)) {                // -2: unused node of this sequence's tree
+                d = a.conf_source == 0 ? x0 - w.mx[0][g] : a.judges[1][((size_t)b * M + g) * V + v] - w.mx[1][g];
+                while (t < a.cuts.n && d < a.cuts.log_tau[t]) ++t;      // thresholds descend: the first one d reaches names the tier
+                atomicAdd(&w.tier_count[t == 0 ? 0 : (t == a.cuts.n ? 2 : 1)], 1);       // accepted / some slim verifier / q
+            }
+            if (writes) { a.tier[b * N + n] = (unsigned char)t; a.conf[b * N + n] = d; }
+        } else {
+            t = a.tier[b * N + n];
+        }
+        t = min(t, J);
+        w.tier[n] = t;
+        w.xj[n] = t > 0 && par >= -1 && par < N && a.judges[t] ? a.judges[t][((size_t)b * M + par + 1) * V + v] : 0.f;
+    }
+    if (tm.size > 1) team_barrier(); else __syncthreads();    // (every CTA of the cluster runs: its slots may be written)
+    if (a.do_tier && writes && tid < 3) {
+        if (w.tier_count[tid]) {
+            atomicAdd(&a.stats->tier_count[tid], (unsigned long long)w.tier_count[tid]);
+            if (tid == 1) a.stats->need_slim = 1;
+            if (tid == 2) a.stats->need_full = 1;
+        }
+        if (b == 0 && tid == 0) atomicAdd(&a.stats->steps, 1ull);
+    }
+
+    // argmax_v (log weight(v) - log(-log u_v)): a draw from the judge of tier t at block row `cur` after n_rej rejections
+    auto draw = [&](int t, int cur, const float *r0, float mx0, int n_rej) -> int {
+        const float *rt = a.judges[t] + ((size_t)b * M + cur) * V;
+        const float mxt = w.mx[t][cur];
+        MaxIdx best = no_idx();
+        sweep_rows(rt, n_rej ? r0 : nullptr, V, tm, [&](int i, float xt, float x0) {
+            float jt = 1.f, lw = (xt - mxt) * a.inv_temp;         // log weight; through the residuals once there are any
+            if (n_rej) {
+                jt = expf(lw);
+                float pr = expf((x0 - mx0) * a.inv_temp);
+                replay(w.rej, n_rej, i, t, jt, pr);
+                lw = logf(jt);
+            }
+            const float u = unit_f32(k_gum, ((unsigned long long)cur << 32) + (unsigned long long)i);
+            MaxIdx c; c.v = jt > 0.f ? lw - logf(-logf(u)) : -INFINITY; c.i = i;
+            best = better(best, c);
+        });
+        best = block_argmax(best, shm);
+        if (tm.size > 1) {
+            const float2 got = team_exchange(make_float2(best.v, __int_as_float(best.i)), make_float2(-INFINITY, __int_as_float(0x7fffffff)), tm);
+            MaxIdx c; c.v = got.x; c.i = __float_as_int(got.y);
+            best = warp_argmax(c);
+        }
+        return best.i == 0x7fffffff ? 0 : best.i;
+    };
+
+    int cur = 0, n_acc = 0, corr = -1, corr_src = 0, parity = 0, draw_t = 0, n_rej = 0;
+    const float *r0 = nullptr;                                   // the drafter row of this position and its maximum
+    float mx0 = 0.f;
+    const float scale2 = a.inv_temp * LOG2E;
     bool needs_q = false;
     while (true) {
-        int c = tree->first_child[cur];
+        int c = w.first_child[cur];
+        n_rej = 0;
+        r0 = nullptr;
         if (c < 0) {                                             // leaf: whole path accepted
             if (a.emit_bonus && a.probe) { needs_q = true; break; }
             if (a.emit_bonus) {
-                if (sampling) {
-                    softmax_numerators(P[J], a.judges[J] + ((size_t)b * M + cur) * V, V, a.inv_temp, st_mx[J * RS_STRIDE + cur], tm);
-                    corr = gumbel_argmax(P[J], V, k_gum, cur, shm, tm);
-                } else {
-                    corr = st_arg[J * RS_STRIDE + cur];
-                }
-                corr_src = J;
+                corr_src = draw_t = J;
             }
             break;
         }
-        // the distributions of this position: 0 = proposal (drafter row), k = judge k (the slim verifiers, then q).  Each
-        // starts as "row + statistics" and is written out as numerators (mat) only once a residual has to be formed.
-        const float *row[KINDS];
-        float mx[KINDS], Z[KINDS];
-        bool mat[KINDS];
-        row[0] = nullptr; mx[0] = 0.f; Z[0] = 0.f; mat[0] = false;
+        // the distributions of this position: the proposal (drafter row) and the judges; Z: denominators after n_rej rejections
+        float Z[KINDS];
 #pragma unroll
-        for (int k = 1; k < KINDS; ++k) {
-            const bool on = k <= J && a.judges[k] != nullptr;
-            row[k] = on ? a.judges[k] + ((size_t)b * M + cur) * V : nullptr;
-            mx[k] = on ? st_mx[k * RS_STRIDE + cur] : 0.f;
-            Z[k] = on ? st_z[k * RS_STRIDE + cur] : 0.f;
-            mat[k] = false;
-        }
-        int failed = 0, taken = -1, taken_tier = 0;
-        for (; c >= 0; c = tree->next_sibling[c]) {
-            const int t = min((int)a.tier[b * N + c], J);
-            int v = a.draft_tok[b * N + c];
-            v = min(max(v, 0), V - 1);
+        for (int k = 0; k < KINDS; ++k) Z[k] = k >= 1 && k <= J && a.judges[k] ? w.z[k][cur] : 0.f;
+        int failed = 0, taken = -1, taken_tier = 0, row0 = -1;
+        for (; c >= 0; c = w.next_sibling[c]) {
+            const int t = w.tier[c], v = w.tok[c];
             if (t == 0) {
                 taken = c; taken_tier = 0;
-                if (lead && !a.probe) a.judge[b * N + c] = 1;
+                if (tid == 0) w.judged[c] = 1;
                 break;
             }
             if (t == J && a.probe) { needs_q = true; break; }     // from here on the walk depends on q
+            const float mxt = w.mx[t][cur];
             bool pass;
+            float Zt = 0.f;
             if (!sampling) {
-                pass = (row[t][v] - mx[t]) >= a.log_acc_rel[t];
+                pass = (w.xj[c] - mxt) >= a.log_acc_rel[t];
             } else {
-                if (!row[0]) {
-                    const int pr = prow[c];
-                    row[0] = a.drafter + ((size_t)b * a.R + pr) * V;
-                    mx[0] = st_mx[pr];
-                    Z[0] = st_z[pr];
+                if (!r0) {
+                    row0 = w.prow[c];
+                    r0 = a.drafter + ((size_t)b * a.R + row0) * V;
+                    mx0 = w.mx[0][row0];
+                    Z[0] = w.z[0][row0];
                 }
+#pragma unroll
+                for (int k = 1; k < KINDS; ++k) if (k == t) Zt = Z[k];
                 const float u = unit_f32(k_acc, (unsigned long long)c);
-                const float pv = mat[0] ? __ldcg(&P[0][v]) : expf((row[0][v] - mx[0]) * a.inv_temp);
-                const float jv = mat[t] ? __ldcg(&P[t][v]) : expf((row[t][v] - mx[t]) * a.inv_temp);
+                // (a child that names another drafter row than its elder sibling is still tested against that sibling's)
+                const float x0 = w.prow[c] == row0 ? w.x0[c] : r0[v];
+                float pv = expf((x0 - mx0) * a.inv_temp), jv = expf((w.xj[c] - mxt) * a.inv_temp);
+                replay(w.rej, n_rej, v, t, jv, pv);
                 const float lp = logf(pv / Z[0]);
-                const float lj = logf(jv / Z[t]);
+                const float lj = logf(jv / Zt);
                 pass = (logf(u) + a.log1m_alpha + lp) < lj;       // u < j(v) / ((1 - alpha) p(v)), Eq. A.2
             }
             if (pass) {
                 taken = c; taken_tier = t;
-                if (lead && !a.probe) a.judge[b * N + c] = (unsigned char)(1 | (t << 4));
+                if (tid == 0) w.judged[c] = 1 | (t << 4);
                 break;
             }
-            if (lead && !a.probe) a.judge[b * N + c] = (unsigned char)(2 | (t << 4));
+            if (tid == 0) w.judged[c] = 2 | (t << 4);
             failed = max(failed, t);
             if (sampling) {
-                // Eq. A.3 round by round: the rejecting judge becomes its residual against the proposal (kept as is if
-                // the residual vanishes); the rejected token leaves the proposal.  Two sweeps of the vocabulary: the
-                // residual's mass, then both distributions written out (from the logits the first time at a position).
-                __syncthreads();                                  // every thread has read P[.][v] above
-                const float sj = a.inv_beta / Z[t], sp = 1.f / Z[0];
-                const bool mt = mat[t], m0 = mat[0];
-                const float *rt = row[t], *r0 = row[0];
-                const float mxt = mx[t], mx0 = mx[0];
-                float s = 0.f;
-                for (int i = tm.rank * blockDim.x + threadIdx.x; i < V; i += tm.size * blockDim.x) {
-                    const float jt = mt ? P[t][i] : expf((rt[i] - mxt) * a.inv_temp);
-                    const float pr = m0 ? P[0][i] : expf((r0[i] - mx0) * a.inv_temp);
+                // the masses of the judge's residual and of the proposal without the rejected token
+                const float sj = a.inv_beta / Zt, sp = 1.f / Z[0];
+                const float *rt = a.judges[t] + ((size_t)b * M + cur) * V;
+                float s = 0.f, z = 0.f;
+                sweep_rows(rt, r0, V, tm, [&](int i, float xt, float x0) {
+                    float jt = ex2((xt - mxt) * scale2), pr = ex2((x0 - mx0) * scale2);
+                    replay(w.rej, n_rej, i, t, jt, pr);
                     s += fmaxf(0.f, jt * sj - pr * sp);
+                    z += i == v ? 0.f : pr;
+                });
+                s = block_sum(s, sh[2 * parity]);
+                z = block_sum(z, sh[2 * parity + 1]);
+                parity ^= 1;
+                if (tm.size > 1) {
+                    const float2 got = team_exchange(make_float2(s, z), make_float2(0.f, 0.f), tm);
+                    s = warp_sum(got.x);
+                    z = warp_sum(got.y);
                 }
-                s = team_sum(s, sh, tm);
-                float z = 0.f;
-                for (int i = tm.rank * blockDim.x + threadIdx.x; i < V; i += tm.size * blockDim.x) {
-                    const float jt = mt ? P[t][i] : expf((rt[i] - mxt) * a.inv_temp);
-                    const float pr = m0 ? P[0][i] : expf((r0[i] - mx0) * a.inv_temp);
-                    P[t][i] = s > 0.f ? fmaxf(0.f, jt * sj - pr * sp) : jt;
-                    const float keep = i == v ? 0.f : pr;
-                    P[0][i] = keep;
-                    z += keep;
-                }
-                z = team_sum(z, sh, tm);                          // (its barrier also publishes the arrays to the other CTAs)
-                mat[t] = true; mat[0] = true;
-                if (s > 0.f) Z[t] = s;
+                if (tid == 0) w.rej[n_rej] = Rejection{t, v, s > 0.f ? sj : -1.f, sp};
+                ++n_rej;
+#pragma unroll
+                for (int k = 1; k < KINDS; ++k) if (k == t && s > 0.f) Z[k] = s;
                 if (z > 0.f) Z[0] = z;
                 __syncthreads();
             }
@@ -410,54 +518,51 @@ accept_kernel(AcceptArgs a) {
         if (needs_q) break;
         if (taken >= 0) {
             if (a.strict_break && taken_tier >= 1 && taken_tier < J) {
-                corr = min(max(a.draft_tok[b * N + taken], 0), V - 1);
+                corr = w.tok[taken];
                 corr_src = taken_tier;
                 break;
             }
-            if (lead && !a.probe) a.path[b * N + n_acc] = taken;
+            if (tid == 0) w.path[n_acc] = taken;
             ++n_acc;
             cur = taken + 1;
-            continue;
+            continue;                                             // (rej is written again only behind a barrier of the next sweep)
         }
-        corr_src = failed;
-        if (sampling) {
-            __syncthreads();
-            corr = gumbel_argmax(P[failed], V, k_gum, cur, shm, tm);
-        } else {
-            corr = st_arg[failed * RS_STRIDE + cur];
-        }
+        corr_src = draw_t = failed;
         break;
     }
+    if (draw_t > 0) corr = sampling ? draw(draw_t, cur, r0, mx0, n_rej) : w.arg[draw_t][cur];
     __syncthreads();
+    if (tm.rank != 0) return;                                     // (nothing is sent to this CTA any more)
     if (a.probe) {
-        if (lead) {
+        if (tid == 0) {
             // tokens this step emits if q is not asked: the accepted nodes and the replacement (or nothing at a leaf)
             const int ne = n_acc + (corr >= 0 ? 1 : 0);
             const bool room = a.len[b] - a.len_full[b] + ne <= a.replay_rows && a.len[b] >= a.replay_rows;
             if (needs_q || !room) atomicExch(a.need_full, 1);
         }
-        if (tm.size > 1) team_barrier();
         return;
     }
-    if (lead) {
-        int ne = 0;
-        for (int j = 0; j < n_acc; ++j) {
-            int node = a.path[b * N + j];
-            a.out_tok[b * (N + 1) + ne++] = min(max(a.draft_tok[b * N + node], 0), V - 1);
-        }
-        if (corr >= 0) a.out_tok[b * (N + 1) + ne++] = corr;
+    const int ne = n_acc + (corr >= 0 ? 1 : 0);
+    for (int n = tid; n < N; n += ACC_THREADS) a.judge[b * N + n] = (unsigned char)w.judged[n];
+    for (int j = tid; j < n_acc; j += ACC_THREADS) {
+        a.path[b * N + j] = w.path[j];
+        a.out_tok[b * (N + 1) + j] = w.tok[w.path[j]];
+    }
+    if (tid == 0) {
+        if (corr >= 0) a.out_tok[b * (N + 1) + n_acc] = corr;
         a.n_acc[b] = n_acc;
         a.n_emit[b] = ne;
         a.corr_src[b] = corr_src;
         atomicAdd(&a.stats->emitted, (unsigned long long)ne);
         atomicAdd(&a.stats->accepted, (unsigned long long)n_acc);
     }
-    if (tm.size > 1) team_barrier();          // no CTA leaves while another may still read its slots
 }
 
-// the accept kernel needs the tree layout but no cache: build it here when called on its own
-__global__ void tree_only_kernel(TreeInfo *tree, DeviceStats *stats, const int *parent, int per_seq, int B, int N) {
-    for (int b = threadIdx.x; b < B; b += blockDim.x) build_tree(tree + b, parent + (per_seq ? (size_t)b * N : 0), N, stats);
+TierCuts tier_cuts(const JudgeSet &js) {
+    TierCuts c;
+    c.n = js.n;
+    for (int k = 0; k < MAXJ; ++k) c.log_tau[k] = k < js.n ? js.log_tau[k] : 0.f;
+    return c;
 }
 
 }  // namespace
@@ -470,9 +575,7 @@ int launch_tier(const viasd_model *m, const viasd_draft *d, const viasd_params *
     const float *gate = p->conf_source == 0 ? d->drafter_logits : js.logits[0];   // Alg. 2 gates with the slim(mest) verifier
     const int rows = p->conf_source == 0 ? d->n_prows : M;
     if (!gate) return VIASD_EINVAL;
-    TierCuts cuts;
-    cuts.n = js.n;
-    for (int k = 0; k < MAXJ; ++k) cuts.log_tau[k] = k < js.n ? js.log_tau[k] : 0.f;
+    const TierCuts cuts = tier_cuts(js);
     // (a CTA per gate row: with few rows the launch is bound by the loads each CTA has in flight, hence 1024 threads)
     tier_kernel<<<dim3(rows, d->batch), 1024, 0, st>>>(r->tier, r->conf, m->ws.stats, gate, d->draft_tok, d->prow,
         d->parent, d->per_sequence, p->conf_source, rows, d->n_nodes, m->cfg.vocab, cuts);
@@ -504,33 +607,30 @@ static bool accept_team16_ok() {
 }
 
 int launch_accept(const viasd_model *m, const viasd_draft *d, const viasd_params *p, const JudgeSet &js, viasd_result *r,
-                  bool tree_ready, cudaStream_t st, const AcceptProbe *probe) {
+                  bool tree_ready, bool do_tier, cudaStream_t st, const AcceptProbe *probe) {
     if (js.n < 1 || js.n > MAXJ) return VIASD_EINVAL;
-    if (!tree_ready) {                       // a forward pass of the same call has laid the tree out already
-        tree_only_kernel<<<1, 64, 0, st>>>(m->ws.tree, m->ws.stats, d->parent, d->per_sequence, d->batch, d->n_nodes);
-        LAUNCH_CHECK();
-    }
     if (d->n_prows > RS_STRIDE) return VIASD_EINVAL;
     AcceptArgs a;
     {
-        // row statistics live behind the distribution buffers
-        float *base = m->ws.accept_scratch + (size_t)m->cfg.max_batch * KINDS * m->cfg.vocab;
+        float *base = m->ws.accept_scratch;
         const size_t n = (size_t)m->cfg.max_batch * KINDS * RS_STRIDE;
         a.rs.mx = base; a.rs.arg = reinterpret_cast<int *>(base + n); a.rs.z = base + 2 * n;
         const int M = d->n_nodes + 1, rows = M > d->n_prows ? M : d->n_prows;
         RowPtrs src;
-        src.p[0] = p->mode == 1 ? d->drafter_logits : nullptr;
+        src.p[0] = p->mode == 1 || (do_tier && p->conf_source == 0) ? d->drafter_logits : nullptr;
         for (int k = 1; k < KINDS; ++k) src.p[k] = k <= js.n ? js.logits[k - 1] : nullptr;
-        row_stats_kernel<<<dim3(rows, d->batch, js.n + 1), 1024, 0, st>>>(a.rs, src, d->n_prows, M, m->cfg.vocab,
-                                                                         1.0f / p->temperature, p->mode == 1);
+        auto kernel = p->mode == 1 ? row_stats_kernel<true> : row_stats_kernel<false>;
+        kernel<<<dim3(rows, d->batch, js.n + 1), RS_THREADS, 0, st>>>(a.rs, src, d->n_prows, M, m->cfg.vocab,
+            p->mode == 1 ? 1.0f / p->temperature : 1.0f, m->ws.stats, do_tier ? 1 : 0, tree_ready ? nullptr : m->ws.tree, d->parent, d->per_sequence);
         LAUNCH_CHECK();
     }
     a.judges[0] = nullptr;
     for (int k = 1; k < KINDS; ++k) a.judges[k] = k <= js.n ? js.logits[k - 1] : nullptr;
     a.n_judges = js.n;
     a.drafter = d->drafter_logits;
-    a.draft_tok = d->draft_tok; a.prow = d->prow; a.tier = r->tier; a.tree = m->ws.tree;
-    a.scratch = m->ws.accept_scratch;
+    a.draft_tok = d->draft_tok; a.prow = d->prow; a.parent = d->parent; a.tier = r->tier; a.conf = r->conf; a.tree = m->ws.tree;
+    a.do_tier = do_tier ? 1 : 0; a.conf_source = p->conf_source;
+    a.cuts = tier_cuts(js);
     a.n_acc = r->n_acc; a.path = r->path; a.out_tok = r->out_tok; a.n_emit = r->n_emit; a.corr_src = r->corr_src;
     a.judge = r->judge; a.stats = m->ws.stats;
     a.N = d->n_nodes; a.R = d->n_prows; a.V = m->cfg.vocab;

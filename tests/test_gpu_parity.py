@@ -295,6 +295,44 @@ def test_accept_sampling_full_vocabulary_tree():
     assert full >= 0.75 * nseq, (full, nseq)
 
 
+# the walk with everything that a rejection replays: many siblings, several judges rejecting in turn, residuals that vanish
+@pytest.mark.parametrize("vocab,team,alpha,beta", [(4099, 1, 0.0, 1.0), (33000, 8, 0.3, 0.7), (70004, 0, 0.0, 1.0), (50257, 4, 0.1, 1.5)])
+def test_accept_with_many_rejections(vocab, team, alpha, beta):
+    """A star of twelve children, each unlikely under its judges, sampling, half of them judged by either verifier: several
+    rejections per sequence, replayed in every later sweep, over vocabularies of every alignment and 1 to 16 CTAs per
+    sequence.  Tiers come from the same call (phase 3).  Decisions under the margin rule of the accept tests."""
+    base = replace(W.get("mini_8b_tree"), batch=6, parent=tuple([-1] * 12), shape=replace(W.get("mini_8b_tree").shape, vocab=vocab))
+    vb = _vb()
+    eng = _engine(replace(base, ctx=8), fill_context=False)
+    vb.set_option(eng.model, "accept_team", team)
+    si = W.step_inputs(base)
+    rng = np.random.default_rng(vocab)
+    B, M, V = base.batch, base.rows, vocab
+    near = np.repeat(si.drafter_logits[:, :1], M, axis=1)
+    slim = (near + rng.standard_normal((B, M, V))).astype(np.float32)
+    full = (near + rng.standard_normal((B, M, V))).astype(np.float32)
+    for b in range(B):
+        for n in range(12):                                   # the judges think little of the drafted tokens
+            slim[b, 0, si.draft_tok[b, n]] -= 2.5 + 0.2 * n
+            full[b, 0, si.draft_tok[b, n]] -= 2.5 + 0.1 * n
+    eng.set_inputs(si)
+    d = tiers.tier_rule(si.drafter_logits, si.draft_tok, si.prow, 0.0, 0.0)[1].ravel()
+    lo, hi = float(np.median(d)), 1.0                          # nothing is accepted outright
+    res = vb.alloc_result(B, base.n_nodes)
+    p = eng.params(log_tau_lo=lo, log_tau_hi=hi, mode=1, alpha=alpha, beta=beta)
+    vb.tier_accept(eng.model, eng.draft, p, torch.from_numpy(slim).cuda(), torch.from_numpy(full).cuda(), 3, res)
+    torch.cuda.synchronize()
+    tier, _ = tiers.tier_rule(si.drafter_logits, si.draft_tok, si.prow, lo, hi)
+    assert np.array_equal(res.tier.cpu().numpy(), tier)
+    P = tiers.Params(mode="sampling", temperature=base.temperature, seed=base.seed, alpha=alpha, beta=beta)
+    seqs = tiers.resolve(si.draft_tok, base.parent, si.prow, tier, si.drafter_logits, slim, full, P)
+    assert sum(int(((res.judge[b] & 3) == 2).sum()) for b in range(B)) >= 2 * B
+    pinned, total, whole = PU.compare_resolution(seqs, res.n_acc.cpu().numpy(), res.path.cpu().numpy(), res.out_tok.cpu().numpy(),
+                                                 res.n_emit.cpu().numpy(), res.corr_src.cpu().numpy(), eps_row=2.5e-5)
+    PU.assert_pinned(f"star of 12, vocabulary {vocab}", pinned, total, whole, B, FLOOR_FRAC, _floor_full(B))
+    assert vb.get_stats(eng.model).device_status == 0
+
+
 def test_accept_options_on_oracle_logits():
     wl = replace(W.get("mini_8b_tree"), mode="greedy")
     for pk in (dict(emit_bonus=True), dict(strict_break=True), dict(log_acc_rel=(0.0, -0.7, -0.3))):
