@@ -222,14 +222,9 @@ int forward_sweep(viasd_model *m, const viasd_cache *cache, const viasd_draft *d
     auto wseg = [&](TcLaunch &L, int i, const WMap &w, int n) { L.map_w[i] = &w.map; L.seg_n[i] = n; L.w_box_rows[i] = w.box_rows; };
     const int ssq_n = (c.d_model / 128) * 4;
 
-    if ((rc = timed(m, VIASD_T_EMBED, st, [&] { return replay ? launch_prep_replay(m, cache, d, replay, st)
-                                                              : launch_prep(m, cache, d, mode != 1, st); }))) return rc;
-    if (dual) {
-        if ((rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_embed_norm2(m, m->norm1[0], m->norm1[m->routed[0]], rows, st); })))
-            return rc;
-    } else {
-        if ((rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_embed_norm(m, m->norm1[layer_id(0)], rows, st); }))) return rc;
-    }
+    if (replay && (rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_prep_replay(m, cache, d, replay, st); }))) return rc;
+    if ((rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_embed_norm(m, cache, d, mode != 1, replay > 0, m->norm1[layer_id(0)],
+                                                                         dual ? m->norm1[m->routed[0]] : nullptr, rows, st); }))) return rc;
     for (int it = 0; it < n_run; ++it) {
         const int l = layer_id(it);
         const int so = routed_ord(l);                          // slim ordinal of this layer, -1 if unrouted
@@ -249,6 +244,7 @@ int forward_sweep(viasd_model *m, const viasd_cache *cache, const viasd_draft *d
             L.max_batch = c.max_batch; L.max_ctx = c.max_ctx; L.layer_ord = ord;
             L.kc2 = cache->k_slim; L.vc2 = cache->v_slim; L.layer_ord2 = so;
             L.kv_keep = replay ? cache->len_full : nullptr;
+            L.ordered = it == 0;                               // (attention reads what the embedding launch prepared ahead of its wait)
             if ((rc = gemm(L, m->maps_a, nrows))) return rc;
         }
         if (both) {
@@ -311,8 +307,7 @@ int forward(viasd_model *m, const viasd_cache *cache, const viasd_draft *d, bool
     const size_t R = m->ws.rows_alloc;
     const size_t pa = c.dtype ? R * c.d_model : 0, pq = c.dtype ? R * qd : 0, pf = c.dtype ? R * c.d_ff : 0;
 
-    if ((rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_prep(m, cache, d, !slim, st); }))) return rc;
-    if ((rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_embed(m, rows, st); }))) return rc;
+    if ((rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_embed(m, cache, d, !slim, rows, st); }))) return rc;
     for (int ord = 0; ord < n_run; ++ord) {
         const int l = slim ? m->routed[ord] : ord;
         const LayerMaps *lm = m->use_tc ? &m->lmaps[l] : nullptr;

@@ -35,6 +35,7 @@ struct DeviceStats {
     int need_slim, need_full;
     int full_ran;                       // the full verifier's pass of the current step ran (its cache holds the block's rows)
     unsigned long long full_skipped;    // steps whose full pass the routed execution policy skipped
+    int commit_ctas;                    // arrivals of the commit kernel's CTAs, zero between launches
 };
 
 struct Workspace {                      // pointers into the caller's workspace block
@@ -183,13 +184,13 @@ inline bool first_use_on_device(bool (&flags)[64]) {
 // before it touches anything that kernel reads or writes.  VIASD_PDL=0 turns the overlap off.
 extern int g_use_pdl;
 inline void pdl_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, dim3 grid, dim3 block, size_t smem,
-                       cudaStream_t st) {
+                       cudaStream_t st, bool overlap = true) {
     cfg = cudaLaunchConfig_t{};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = g_use_pdl ? 1 : 0;
+    cfg.numAttrs = g_use_pdl && overlap ? 1 : 0;
 }
 // A pass that runs only when a device flag says so (the full verifier's pass under the routed execution policy): every
 // kernel of it takes the flag's address and leaves at once when the flag is zero.  The flag is written by a kernel that
@@ -204,11 +205,12 @@ inline void pdl_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, dim3 
 // ---------------------------------------------------------------------------------------------
 // misc.cu
 int launch_rope_table(const viasd_model *m, cudaStream_t st);
-int launch_prep(const viasd_model *m, const viasd_cache *c, const viasd_draft *d, bool full_pass, cudaStream_t st);
 int launch_prep_replay(const viasd_model *m, const viasd_cache *c, const viasd_draft *d, int G, cudaStream_t st);
 int launch_compact_head_rows(const viasd_model *m, int batch, int M, int G, cudaStream_t st);
-int launch_embed(const viasd_model *m, int rows, cudaStream_t st);
-int launch_embed_norm(const viasd_model *m, const float *gain, int rows, cudaStream_t st);
+// these two also prepare the pass (tree, lengths, tokens); gain_slim: null, or the second row stream's first gain
+int launch_embed(const viasd_model *m, const viasd_cache *c, const viasd_draft *d, bool full_pass, int rows, cudaStream_t st);
+int launch_embed_norm(const viasd_model *m, const viasd_cache *c, const viasd_draft *d, bool full_pass, bool replay, const float *gain,
+                      const float *gain_slim, int rows, cudaStream_t st);
 int launch_rmsnorm(const viasd_model *m, const float *gain, int rows, cudaStream_t st);
 int launch_rope_append(const viasd_model *m, void *kc, void *vc, int layer_ord, int batch, int M,
                        cudaStream_t st);
@@ -243,7 +245,6 @@ int launch_attention_tk(viasd_model *m, const void *kc, const void *vc, bool sli
                          cudaStream_t st);
 int launch_attention_dual(viasd_model *m, const void *kf, const void *vf, int layer_full, const void *ks, const void *vs,
                           int ord_slim, int batch, int M, cudaStream_t st);
-int launch_embed_norm2(const viasd_model *m, const float *gain_full, const float *gain_slim, int rows, cudaStream_t st);
 
 // tier_accept.cu
 // The verifiers that may judge a drafted token, weakest first, q last (two for the three-tier method), with the

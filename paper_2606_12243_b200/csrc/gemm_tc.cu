@@ -610,7 +610,7 @@ int launch_gemm_tc(const TcLaunch &L, cudaStream_t st) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     const int groups = tc_groups(L);
-    pdl_config(cfg, attr, dim3(grid), dim3(64 + 128 * groups), smem, st);
+    pdl_config(cfg, attr, dim3(grid), dim3(64 + 128 * groups), smem, st, !L.ordered);
     static bool attr_done[64][16];           // the attribute belongs to a (kernel, device) pair
     const int boxes = tc_boxes(L);
     int dev = 0;

@@ -62,6 +62,7 @@ struct TcLaunch {                       // host-side description of one GEMM
     int rope_M, rope_H, rope_Hkv, max_batch, max_ctx, layer_ord, tree_stride;
     int split_row, layer_ord2; float *out_f32_2; const float *next_gain2; void *kc2, *vc2;
     const int *run_flag, *kv_keep;
+    int ordered;                        // 1: an ordinary launch (no overlap with the kernel before it)
     int ring_kb, epi_groups;            // stream-K kernel: ring size and epilogue groups; 0 = defaults (200 KB; by token tile)
 };
 

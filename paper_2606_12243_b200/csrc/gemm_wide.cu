@@ -573,7 +573,7 @@ int launch_gemm_wide(const TcLaunch &L, cudaStream_t st) {
     }
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    pdl_config(cfg, attr, dim3(2 * pairs), dim3(WTHREADS), smem, st);
+    pdl_config(cfg, attr, dim3(2 * pairs), dim3(WTHREADS), smem, st, !L.ordered);
     switch (L.epi) {
     case EPI_SWIGLU: CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_wide_kernel<EPI_SWIGLU>, w0, w1, w2, *L.map_x, p)); break;
     case EPI_ADD_NORM: CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_wide_kernel<EPI_ADD_NORM>, w0, w1, w2, *L.map_x, p)); break;

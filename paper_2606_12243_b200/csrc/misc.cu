@@ -1,5 +1,5 @@
 // Small memory-bound kernels of the decoder block and the cache bookkeeping:
-// rotary table, per-pass preparation (tree layout, row tokens, clamped lengths), embedding gather,
+// rotary table, embedding gather with the per-pass preparation (tree layout, row tokens, clamped lengths),
 // RMSNorm, rotary embedding + KV append, KV commit.
 #include "common.cuh"
 
@@ -26,38 +26,41 @@ int launch_rope_table(const viasd_model *m, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// per-pass preparation
+// per-pass preparation: part of the embedding kernels
 // ---------------------------------------------------------------------------------------------
-constexpr int PREP_WARPS = 16;
-// parent: [N] shared by the batch, or [B, N] when per_seq
-__global__ void prep_kernel(TreeInfo *tree, int *len_eff, int *row_tok, DeviceStats *stats, const int *len,
-                            const int *pending, const int *draft_tok, const int *parent, int per_seq, int B, int N,
-                            int max_ctx, int vocab, int full_pass) {
-    const int M = N + 1;
-    PDL_TRIGGER();
-    __shared__ int par_sh[PREP_WARPS][VIASD_MAX_ROWS_PER_SEQ];
-    if (threadIdx.x == 0 && full_pass) stats->full_ran = 1;     // the full verifier's cache receives this block's rows
-    for (int b = threadIdx.x >> 5; b < B; b += PREP_WARPS) build_tree(tree + b, parent + (per_seq ? (size_t)b * N : 0), N, stats, par_sh[threadIdx.x >> 5]);
-    for (int b = threadIdx.x; b < B; b += blockDim.x) {
-        int l = len[b];
-        int c = min(max(l, 0), max_ctx - M);
-        if (c != l) stats->device_status = VIASD_ECAPACITY;
-        len_eff[b] = c;
-    }
-    for (int r = threadIdx.x; r < B * M; r += blockDim.x) {
-        int b = r / M, i = r % M;
-        int t = (i == 0) ? pending[b] : draft_tok[b * N + i - 1];
-        if (t < 0 || t >= vocab) { stats->device_status = VIASD_EDEVICE; t = 0; }
-        row_tok[r] = t;
+// The first CTAs of an embedding launch, one per sequence, lay out the sequence's tree and clamp its length; a row's CTA
+// finds its own token.  (As a kernel of its own in front of the embedding, and again in front of the commit, this was 7 us
+// each time, most of it the launch.)  What attention reads of it before its dependency wait - tree and length - is complete
+// because the pass's first QKV launch is an ordinary one: nothing after it starts before the embedding has ended.
+struct PrepArgs {
+    TreeInfo *tree; int *len_eff; DeviceStats *stats;
+    const int *len, *pending, *draft_tok, *parent;       // parent: [N] shared by the batch, or [B, N] when per_seq
+    const int *row_tok;                                  // not null: a replay pass, whose preparation has run (no sequence CTAs)
+    int per_seq, B, N, max_ctx, vocab, full_pass;
+};
+__device__ __forceinline__ int prep_ctas(const PrepArgs &p) { return p.row_tok ? 0 : p.B; }
+__device__ __forceinline__ int clamped_len(const int *len, int b, int max_ctx, int M, DeviceStats *stats) {
+    const int l = len[b], c = min(max(l, 0), max_ctx - M);
+    if (c != l) stats->device_status = VIASD_ECAPACITY;
+    return c;
+}
+__device__ __forceinline__ void prep_sequence(const PrepArgs &p, int b, int *par_sh) {       // by the CTA's first warp
+    build_tree(p.tree + b, p.parent + (p.per_seq ? (size_t)b * p.N : 0), p.N, p.stats, par_sh);
+    if (threadIdx.x == 0) {
+        if (b == 0 && p.full_pass) p.stats->full_ran = 1;      // the full verifier's cache receives this block's rows
+        p.len_eff[b] = clamped_len(p.len, b, p.max_ctx, p.N + 1, p.stats);
     }
 }
-
-int launch_prep(const viasd_model *m, const viasd_cache *c, const viasd_draft *d, bool full_pass, cudaStream_t st) {
-    prep_kernel<<<1, 32 * PREP_WARPS, 0, st>>>(m->ws.tree, m->ws.len_eff, m->ws.row_tok, m->ws.stats, c->len, c->pending,
-                                   d->draft_tok, d->parent, d->per_sequence, d->batch, d->n_nodes, m->cfg.max_ctx,
-                                   m->cfg.vocab, full_pass ? 1 : 0);
-    LAUNCH_CHECK();
-    return VIASD_OK;
+__device__ __forceinline__ int prep_token(const PrepArgs &p, int r) {
+    if (p.row_tok) return p.row_tok[r];
+    const int M = p.N + 1, b = r / M, i = r - b * M;
+    int t = i == 0 ? p.pending[b] : p.draft_tok[b * p.N + i - 1];
+    if (t < 0 || t >= p.vocab) { p.stats->device_status = VIASD_EDEVICE; t = 0; }
+    return t;
+}
+static PrepArgs prep_args(const viasd_model *m, const viasd_cache *c, const viasd_draft *d, bool full_pass, bool replay) {
+    return PrepArgs{m->ws.tree, m->ws.len_eff, m->ws.stats, c->len, c->pending, d->draft_tok, d->parent,
+                    replay ? m->ws.row_tok : nullptr, d->per_sequence, d->batch, d->n_nodes, m->cfg.max_ctx, m->cfg.vocab, full_pass ? 1 : 0};
 }
 
 // Preparation of a replay pass (routed execution policy): the block of every sequence is extended, in front, by its
@@ -138,13 +141,15 @@ int launch_compact_head_rows(const viasd_model *m, int batch, int M, int G, cuda
 }
 
 // ---------------------------------------------------------------------------------------------
-// embedding gather: h[r] = E[row_tok[r]]
+// embedding gather: h[r] = E[token of row r]
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void embed_kernel(float *h, const T *E, const int *row_tok, int d) {
-    int r = blockIdx.x;
+__global__ void embed_kernel(float *h, const T *E, const PrepArgs p, int d) {
+    __shared__ int par_sh[VIASD_MAX_ROWS_PER_SEQ];
     PDL_TRIGGER();
-    const T *src = E + (size_t)row_tok[r] * d;
+    const int r = (int)blockIdx.x - prep_ctas(p);
+    if (r < 0) { if (threadIdx.x < 32) prep_sequence(p, blockIdx.x, par_sh); return; }
+    const T *src = E + (size_t)prep_token(p, r) * d;
     for (int i = threadIdx.x; i < d; i += blockDim.x) h[(size_t)r * d + i] = to_f32<T>(src[i]);
 }
 
@@ -177,50 +182,36 @@ __device__ __forceinline__ void embed_row(float *h, __nv_bfloat16 *a, size_t pla
 
 // Embedding gather fused with the preparation of the first RMSNorm of the pass (tensor-core path):
 // h = E[tok]; a = hi/lo(h * gain); partial sums of h^2 per 32 features in the layout the GEMM epilogue reads.
+// Rows from `rows` on are the second stream's (both verifiers in one sweep): the same tokens, prepared for the slim
+// verifier's first routed layer.
 __global__ void __launch_bounds__(256)
 embed_norm_kernel(float *h, __nv_bfloat16 *a, size_t plane, float *ssq, int ssq_stride, const __nv_bfloat16 *E,
-                  const float *gain, const int *row_tok, int d, const int *run_flag) {
+                  const float *gain_full, const float *gain_slim, const PrepArgs p, int d, int rows, const int *run_flag) {
     RUN_FLAG_EXIT(run_flag);
-    const int r = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ int par_sh[VIASD_MAX_ROWS_PER_SEQ];
+    const int r = (int)blockIdx.x - prep_ctas(p), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     PDL_TRIGGER();
-    const __nv_bfloat16 *src = E + (size_t)row_tok[r] * d;
-    embed_row(h, a, plane, ssq, ssq_stride, src, gain, r, d, warp, lane);
+    if (r < 0) { if (warp == 0) prep_sequence(p, blockIdx.x, par_sh); return; }
+    const __nv_bfloat16 *src = E + (size_t)prep_token(p, r < rows ? r : r - rows) * d;
+    embed_row(h, a, plane, ssq, ssq_stride, src, r < rows ? gain_full : gain_slim, r, d, warp, lane);
 }
 
-int launch_embed_norm(const viasd_model *m, const float *gain, int rows, cudaStream_t st) {
-    embed_norm_kernel<<<rows, 256, 0, st>>>(m->ws.h, (__nv_bfloat16 *)m->ws.a, m->ws.rows_alloc * m->cfg.d_model, m->ws.ssq,
-                                            (int)m->ws.rows_alloc, (const __nv_bfloat16 *)m->embed, gain, m->ws.row_tok,
-                                            m->cfg.d_model, m->run_flag);
+int launch_embed_norm(const viasd_model *m, const viasd_cache *c, const viasd_draft *d, bool full_pass, bool replay, const float *gain,
+                      const float *gain_slim, int rows, cudaStream_t st) {
+    const PrepArgs p = prep_args(m, c, d, full_pass, replay);
+    embed_norm_kernel<<<(replay ? 0 : d->batch) + (gain_slim ? 2 : 1) * rows, 256, 0, st>>>(
+        m->ws.h, (__nv_bfloat16 *)m->ws.a, m->ws.rows_alloc * m->cfg.d_model, m->ws.ssq, (int)m->ws.rows_alloc,
+        (const __nv_bfloat16 *)m->embed, gain, gain_slim, p, m->cfg.d_model, rows, m->run_flag);
     LAUNCH_CHECK();
     return VIASD_OK;
 }
 
-// Two row streams from the same block rows: rows [0, rows) prepared for the full verifier's first layer,
-// rows [rows, 2*rows) for the slim verifier's first routed layer (their first norms differ).
-__global__ void __launch_bounds__(256)
-embed_norm2_kernel(float *h, __nv_bfloat16 *a, size_t plane, float *ssq, int ssq_stride, const __nv_bfloat16 *E,
-                   const float *gain_full, const float *gain_slim, const int *row_tok, int d, int rows) {
-    const int r = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    PDL_TRIGGER();
-    const float *gain = r < rows ? gain_full : gain_slim;
-    const __nv_bfloat16 *src = E + (size_t)row_tok[r < rows ? r : r - rows] * d;
-    embed_row(h, a, plane, ssq, ssq_stride, src, gain, r, d, warp, lane);
-}
-
-int launch_embed_norm2(const viasd_model *m, const float *gain_full, const float *gain_slim, int rows, cudaStream_t st) {
-    embed_norm2_kernel<<<2 * rows, 256, 0, st>>>(m->ws.h, (__nv_bfloat16 *)m->ws.a, m->ws.rows_alloc * m->cfg.d_model,
-                                                 m->ws.ssq, (int)m->ws.rows_alloc, (const __nv_bfloat16 *)m->embed, gain_full,
-                                                 gain_slim, m->ws.row_tok, m->cfg.d_model, rows);
-    LAUNCH_CHECK();
-    return VIASD_OK;
-}
-
-int launch_embed(const viasd_model *m, int rows, cudaStream_t st) {
+int launch_embed(const viasd_model *m, const viasd_cache *c, const viasd_draft *d, bool full_pass, int rows, cudaStream_t st) {
+    const PrepArgs p = prep_args(m, c, d, full_pass, false);
     if (m->cfg.dtype == 0)
-        embed_kernel<float><<<rows, 256, 0, st>>>(m->ws.h, (const float *)m->embed, m->ws.row_tok, m->cfg.d_model);
+        embed_kernel<float><<<d->batch + rows, 256, 0, st>>>(m->ws.h, (const float *)m->embed, p, m->cfg.d_model);
     else
-        embed_kernel<__nv_bfloat16><<<rows, 256, 0, st>>>(m->ws.h, (const __nv_bfloat16 *)m->embed,
-                                                          m->ws.row_tok, m->cfg.d_model);
+        embed_kernel<__nv_bfloat16><<<d->batch + rows, 256, 0, st>>>(m->ws.h, (const __nv_bfloat16 *)m->embed, p, m->cfg.d_model);
     LAUNCH_CHECK();
     return VIASD_OK;
 }
@@ -334,50 +325,77 @@ int launch_rope_append(const viasd_model *m, void *kc, void *vc, int layer_ord, 
 }
 
 // ---------------------------------------------------------------------------------------------
-// KV commit: compact the accepted path, then advance len / pending / tokens
+// KV commit: compact the accepted path, advance len / pending / tokens
 // ---------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void commit_move_kernel(T *kf, T *vf, T *ks, T *vs, const int *len_eff, const int *n_acc,
-                                   const int *path, int N, int L, int Ls, int Hkv, int hd, int max_batch,
-                                   int max_ctx, const DeviceStats *stats, int layer0) {
-    int layer = layer0 + blockIdx.x, b = blockIdx.y, g = blockIdx.z;
-    if (layer < L && !stats->full_ran) return;                  // the full verifier's cache did not receive this block
-    T *kc = layer < L ? kf : ks;
-    T *vc = layer < L ? vf : vs;
-    int lo = layer < L ? layer : layer - L;
-    size_t base = (((size_t)lo * max_batch + b) * Hkv + g) * (size_t)max_ctx * hd;
-    int n = len_eff[b];
-    int na = min(n_acc[b], N);
-    // each thread owns fixed columns, so walking j in order is enough to keep sources intact
-    for (int j = 0; j < na; ++j) {
-        int node = path[b * N + j];
-        if (node < j || node >= N) break;           // not a valid path entry: stop (never moves rows up)
-        int src = n + node + 1, dst = n + 1 + j;
-        if (src == dst) continue;
-        for (int c = threadIdx.x; c < hd; c += blockDim.x) {
-            kc[base + (size_t)dst * hd + c] = kc[base + (size_t)src * hd + c];
-            vc[base + (size_t)dst * hd + c] = vc[base + (size_t)src * hd + c];
+// A warp moves the path's rows of one (layer, sequence, kv head), K by its first half and V by its second, eight rows of
+// 16-byte loads in flight; the last CTA to finish advances the lengths (nobody reads them before).  (Three launches -
+// lengths, rows one 2-byte column per thread and row after row, advance - were 15 to 27 us.)
+struct CommitArgs {
+    void *kf, *vf, *ks, *vs;
+    int *len, *len_full, *pending, *tokens;
+    const int *n_acc, *path, *n_emit, *out_tok;
+    DeviceStats *stats;
+    int B, N, L, Ls, layer0, Hkv, row_vecs, max_batch, max_ctx, slim_only;   // row_vecs: 16-byte pieces of a K (or V) row
+};
+constexpr int COMMIT_WARPS = 8;
+
+__global__ void __launch_bounds__(32 * COMMIT_WARPS) commit_kernel(const CommitArgs a) {
+    __shared__ int last_sh;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, M = a.N + 1;
+    const int item = blockIdx.x * COMMIT_WARPS + warp, n_items = (a.L + a.Ls - a.layer0) * a.B * a.Hkv;
+    const bool full_ran = a.stats->full_ran != 0;
+    if (item < n_items) {
+        const int g = item % a.Hkv, b = (item / a.Hkv) % a.B, layer = a.layer0 + item / (a.Hkv * a.B);
+        const bool is_full = layer < a.L;
+        if (full_ran || !is_full) {                            // else the full verifier's cache did not receive this block
+            const int half = lane >> 4, l16 = lane & 15;
+            uint4 *base = reinterpret_cast<uint4 *>(is_full ? (half ? a.vf : a.kf) : (half ? a.vs : a.ks)) +
+                          (((size_t)(is_full ? layer : layer - a.L) * a.max_batch + b) * a.Hkv + g) * (size_t)a.max_ctx * a.row_vecs;
+            const int n = clamped_len(a.len, b, a.max_ctx, M, a.stats), na = min(a.n_acc[b], a.N);
+            // a path's nodes never come before their position (node >= j), so rows only move down and no row that is still to
+            // be moved is overwritten; an invalid entry ends the path
+            bool more = true;
+            for (int j0 = 0; more && j0 < na; j0 += 8) {
+                int src[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int node = j0 + j < na ? a.path[b * a.N + j0 + j] : -1;
+                    more = more && node >= j0 + j && node < a.N;
+                    src[j] = more && node != j0 + j ? n + 1 + node : -1;
+                }
+                for (int c = l16; c < a.row_vecs; c += 16) {
+                    uint4 v[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) if (src[j] >= 0) v[j] = base[(size_t)src[j] * a.row_vecs + c];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) if (src[j] >= 0) base[(size_t)(n + 1 + j0 + j) * a.row_vecs + c] = v[j];
+                }
+            }
         }
     }
-}
-
-__global__ void commit_advance_kernel(int *len, int *len_full, int *pending, int *tokens, const int *len_eff,
-                                      const int *n_emit, const int *out_tok, int B, int N, int max_ctx,
-                                      DeviceStats *stats) {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    int n = len_eff[b];
-    int ne = min(max(n_emit[b], 0), N + 1);
-    // the full verifier's cache is complete up to the new length exactly when its pass ran in this step
-    if (len_full && stats->full_ran) len_full[b] = n + ne;
-    if (b == 0 && !stats->full_ran) ++stats->full_skipped;
-    if (ne == 0) return;
-    if (tokens) {
-        tokens[(size_t)b * max_ctx + n] = pending[b];
-        for (int j = 0; j + 1 < ne; ++j) tokens[(size_t)b * max_ctx + n + 1 + j] = out_tok[b * (N + 1) + j];
+    if (a.slim_only) return;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int old;
+        asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(&a.stats->commit_ctas) : "memory");
+        last_sh = old == (int)gridDim.x - 1;
+        if (last_sh) a.stats->commit_ctas = 0;
     }
-    len[b] = n + ne;
-    pending[b] = out_tok[b * (N + 1) + ne - 1];
+    __syncthreads();
+    if (!last_sh) return;
+    for (int b = threadIdx.x; b < a.B; b += blockDim.x) {
+        const int n = clamped_len(a.len, b, a.max_ctx, M, a.stats), ne = min(max(a.n_emit[b], 0), a.N + 1);
+        // the full verifier's cache is complete up to the new length exactly when its pass ran in this step
+        if (a.len_full && full_ran) a.len_full[b] = n + ne;
+        if (b == 0 && !full_ran) ++a.stats->full_skipped;
+        if (ne == 0) continue;
+        if (a.tokens) {
+            a.tokens[(size_t)b * a.max_ctx + n] = a.pending[b];
+            for (int j = 0; j + 1 < ne; ++j) a.tokens[(size_t)b * a.max_ctx + n + 1 + j] = a.out_tok[b * (a.N + 1) + j];
+        }
+        a.len[b] = n + ne;
+        a.pending[b] = a.out_tok[b * (a.N + 1) + ne - 1];
+    }
 }
 
 // slim_only: move the accepted rows in this handle's slim cache and nothing else (lengths, pending token and token
@@ -385,24 +403,16 @@ __global__ void commit_advance_kernel(int *len, int *len_full, int *pending, int
 int launch_commit(const viasd_model *m, viasd_cache *c, const viasd_draft *d, const viasd_result *r, bool slim_only,
                   cudaStream_t st) {
     const viasd_config &cf = m->cfg;
-    int rc = launch_prep(m, c, d, false, st);
-    if (rc) return rc;
-    const int layer0 = slim_only ? cf.n_layers : 0;
-    dim3 grid(cf.n_layers + m->n_routed - layer0, d->batch, cf.n_kv_heads);
-    int threads = cf.head_dim < 32 ? 32 : (cf.head_dim > 256 ? 256 : cf.head_dim);
-    if (cf.dtype == 0)
-        commit_move_kernel<float><<<grid, threads, 0, st>>>((float *)c->k_full, (float *)c->v_full, (float *)c->k_slim,
-            (float *)c->v_slim, m->ws.len_eff, r->n_acc, r->path, d->n_nodes, cf.n_layers, m->n_routed, cf.n_kv_heads,
-            cf.head_dim, cf.max_batch, cf.max_ctx, m->ws.stats, layer0);
-    else
-        commit_move_kernel<__nv_bfloat16><<<grid, threads, 0, st>>>((__nv_bfloat16 *)c->k_full,
-            (__nv_bfloat16 *)c->v_full, (__nv_bfloat16 *)c->k_slim, (__nv_bfloat16 *)c->v_slim, m->ws.len_eff, r->n_acc,
-            r->path, d->n_nodes, cf.n_layers, m->n_routed, cf.n_kv_heads, cf.head_dim, cf.max_batch, cf.max_ctx, m->ws.stats, layer0);
-    LAUNCH_CHECK();
-    if (slim_only) return VIASD_OK;
-    commit_advance_kernel<<<(d->batch + 63) / 64, 64, 0, st>>>(c->len, c->len_full, c->pending, c->tokens, m->ws.len_eff,
-                                                               r->n_emit, r->out_tok, d->batch, d->n_nodes, cf.max_ctx,
-                                                               m->ws.stats);
+    CommitArgs a;
+    a.kf = c->k_full; a.vf = c->v_full; a.ks = c->k_slim; a.vs = c->v_slim;
+    a.len = c->len; a.len_full = c->len_full; a.pending = c->pending; a.tokens = c->tokens;
+    a.n_acc = r->n_acc; a.path = r->path; a.n_emit = r->n_emit; a.out_tok = r->out_tok;
+    a.stats = m->ws.stats;
+    a.B = d->batch; a.N = d->n_nodes; a.L = cf.n_layers; a.Ls = m->n_routed; a.layer0 = slim_only ? cf.n_layers : 0;
+    a.Hkv = cf.n_kv_heads; a.row_vecs = cf.head_dim * (cf.dtype == 0 ? 4 : 2) / 16;
+    a.max_batch = cf.max_batch; a.max_ctx = cf.max_ctx; a.slim_only = slim_only ? 1 : 0;
+    const int items = (cf.n_layers + m->n_routed - a.layer0) * d->batch * cf.n_kv_heads;
+    commit_kernel<<<(items + COMMIT_WARPS - 1) / COMMIT_WARPS, 32 * COMMIT_WARPS, 0, st>>>(a);
     LAUNCH_CHECK();
     return VIASD_OK;
 }
