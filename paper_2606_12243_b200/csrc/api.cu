@@ -373,11 +373,11 @@ int viasd_init_model(const viasd_config *cfg, const viasd_weights *w, const unsi
     if (!w->embed || !w->lm_head || !w->final_norm || !w->wq || !w->wk || !w->wv || !w->wo || !w->wg || !w->wu ||
         !w->wd || !w->norm1 || !w->norm2) return VIASD_EINVAL;
     if (workspace_bytes < carve(*cfg, nullptr, nullptr)) return VIASD_ECAPACITY;
-    int dev = 0;
-    cudaDeviceProp prop;
+    int dev = 0, major = 0, sms = 0;                             // (two attributes: the whole property record takes milliseconds)
     CUDA_TRY(cudaGetDevice(&dev));
-    CUDA_TRY(cudaGetDeviceProperties(&prop, dev));
-    if (prop.major != 10) return VIASD_EUNSUPPORTED;
+    CUDA_TRY(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
+    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (major != 10) return VIASD_EUNSUPPORTED;
 
     if (g_use_pdl < 0) { const char *e = getenv("VIASD_PDL"); g_use_pdl = (e && e[0] == '0') ? 0 : 1; }
     viasd_model *m = new (std::nothrow) viasd_model();
@@ -385,7 +385,7 @@ int viasd_init_model(const viasd_config *cfg, const viasd_weights *w, const unsi
     memset(&m->timer, 0, sizeof(m->timer));
     default_options(m->opt);
     m->cfg = *cfg;
-    m->sm_count = prop.multiProcessorCount;
+    m->sm_count = sms;
     m->n_routed = 0;
     for (int l = 0; l < cfg->n_layers; ++l) if (route_mask[l]) m->routed[m->n_routed++] = l;
     if (m->n_routed == 0) { delete m; return VIASD_EINVAL; }

@@ -26,6 +26,7 @@ attention_split_kernel(float *__restrict__ part, const float *__restrict__ q, co
     __shared__ float Vs[TK][HD];
     constexpr int DPL = HD / 32;                     // output dims per lane
     PDL_TRIGGER();
+    PDL_WAIT();
     const int b = blockIdx.x / Hkv, g = blockIdx.x % Hkv, split = blockIdx.y, qg = blockIdx.z;
     const int grp = H / Hkv, QR = grp * M;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -62,15 +63,26 @@ attention_split_kernel(float *__restrict__ part, const float *__restrict__ q, co
 
     for (int k0 = k_begin; k0 < k_end; k0 += TK) {
         __syncthreads();
-        for (int idx = threadIdx.x; idx < TK * HD; idx += blockDim.x) {
-            int j = idx / HD, dd = idx % HD;
-            float kv = 0.f, vv = 0.f;
-            if (k0 + j < k_end) {
-                kv = to_f32<T>(kc[cbase + (size_t)(k0 + j) * HD + dd]);
-                vv = to_f32<T>(vc[cbase + (size_t)(k0 + j) * HD + dd]);
-            }
-            Ks[j][dd] = kv;
-            Vs[j][dd] = vv;
+        // 16-byte loads, all of a thread's in flight together
+        constexpr int VE = 16 / sizeof(T), NV = TK * HD / VE / (ATT_WARPS * 32);
+        static_assert(NV * VE * ATT_WARPS * 32 == TK * HD, "whole pieces per thread");
+        uint4 kraw[NV], vraw[NV];
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const int idx = (threadIdx.x + q * ATT_WARPS * 32) * VE, j = idx / HD;
+            const size_t o = cbase + (size_t)min(k0 + j, k_end - 1) * HD + idx % HD;
+            kraw[q] = *reinterpret_cast<const uint4 *>(kc + o);
+            vraw[q] = *reinterpret_cast<const uint4 *>(vc + o);
+        }
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const int idx = (threadIdx.x + q * ATT_WARPS * 32) * VE, j = idx / HD, dd = idx % HD;
+            const bool in = k0 + j < k_end;
+            T kv[VE], vv[VE];
+            *reinterpret_cast<uint4 *>(kv) = kraw[q];
+            *reinterpret_cast<uint4 *>(vv) = vraw[q];
+#pragma unroll
+            for (int e = 0; e < VE; ++e) { Ks[j][dd + e] = in ? to_f32<T>(kv[e]) : 0.f; Vs[j][dd + e] = in ? to_f32<T>(vv[e]) : 0.f; }
         }
         __syncthreads();
 #pragma unroll
@@ -116,6 +128,7 @@ __global__ void attention_combine_kernel(T *__restrict__ out, size_t plane, cons
     RUN_FLAG_EXIT(run_flag);
     const int r = blockIdx.x, h = blockIdx.y;        // r = b * M + i
     PDL_TRIGGER();
+    PDL_WAIT();
     const int b = r / M, i = r % M;
     const float *src = part + (((size_t)b * H + h) * M + i) * (size_t)nsplit * (HD + 2);
     float mmax = -INFINITY;
@@ -141,12 +154,12 @@ int run(const viasd_model *m, const void *kc, const void *vc, int layer_ord, int
     const int grp = c.n_heads / c.n_kv_heads;
     const int qgroups = (grp * M + QG - 1) / QG;
     dim3 grid(batch * c.n_kv_heads, nsplit, qgroups);
-    attention_split_kernel<T, HD><<<grid, ATT_WARPS * 32, 0, st>>>(m->ws.part, m->ws.q, (const T *)kc,
+    CUDA_TRY(launch_chained(attention_split_kernel<T, HD>, grid, ATT_WARPS * 32, st, m->ws.part, m->ws.q, (const T *)kc,
         (const T *)vc, m->ws.len_eff, m->ws.tree, M, c.n_heads, c.n_kv_heads, c.max_batch, c.max_ctx, layer_ord, nsplit,
-        1.0f / sqrtf((float)HD), m->run_flag);
+        1.0f / sqrtf((float)HD), m->run_flag));
     LAUNCH_CHECK();
-    attention_combine_kernel<T, HD><<<dim3(batch * M, c.n_heads), HD < 128 ? HD : 128, 0, st>>>((T *)m->ws.attn,
-        sizeof(T) == 2 ? m->ws.rows_alloc * (size_t)c.n_heads * HD : 0, m->ws.part, M, c.n_heads, nsplit, m->run_flag);
+    CUDA_TRY(launch_chained(attention_combine_kernel<T, HD>, dim3(batch * M, c.n_heads), HD < 128 ? HD : 128, st, (T *)m->ws.attn,
+        sizeof(T) == 2 ? m->ws.rows_alloc * (size_t)c.n_heads * HD : 0, m->ws.part, M, c.n_heads, nsplit, m->run_flag));
     LAUNCH_CHECK();
     return VIASD_OK;
 }
@@ -159,7 +172,7 @@ int attention_nsplit(const viasd_model *m, int batch, int M) {
     const int qgroups = (grp * M + QG - 1) / QG;
     int ctas = batch * c.n_kv_heads * qgroups;
     int nsplit = (2 * m->sm_count + ctas - 1) / ctas;
-    int by_len = (c.max_ctx + 127) / 128;            // at least 128 keys per split
+    int by_len = (c.max_ctx + TK - 1) / TK;          // at least one tile per split: with few CTAs a tile is a chain of latencies
     if (nsplit > by_len) nsplit = by_len;
     if (nsplit > 16) nsplit = 16;
     if (nsplit < 1) nsplit = 1;
@@ -247,8 +260,8 @@ static int mma_attention(viasd_model *m, const void *kc, const void *vc, bool sl
     else if (use == 1) rc = launch_attention_tc(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, nsplit, fuse ? 1 : 0, st);
     else rc = launch_attention_mma(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, nsplit, fuse ? 1 : 0, st);
     if (rc || n_part == 1 || fuse) return rc;
-    attention_combine_kernel<__nv_bfloat16, 128><<<dim3(streams * batch * M, c.n_heads), 128, 0, st>>>(
-        (__nv_bfloat16 *)m->ws.attn, m->ws.rows_alloc * (size_t)c.n_heads * 128, m->ws.part, M, c.n_heads, n_part, m->run_flag);
+    CUDA_TRY(launch_chained(attention_combine_kernel<__nv_bfloat16, 128>, dim3(streams * batch * M, c.n_heads), 128, st,
+        (__nv_bfloat16 *)m->ws.attn, m->ws.rows_alloc * (size_t)c.n_heads * 128, m->ws.part, M, c.n_heads, n_part, m->run_flag));
     LAUNCH_CHECK();
     return VIASD_OK;
 }

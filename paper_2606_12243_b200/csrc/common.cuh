@@ -192,6 +192,16 @@ inline void pdl_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, dim3 
     cfg.attrs = attr;
     cfg.numAttrs = g_use_pdl && overlap ? 1 : 0;
 }
+// Launches a kernel that opens with PDL_TRIGGER(); PDL_WAIT(): nothing of it overlaps the kernel before it but its launch,
+// which is most of a small kernel's time.  As every kernel of such a chain waits for the one before it, each sees the
+// results of all before it.
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    pdl_config(cfg, attr, grid, block, 0, st);
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 // A pass that runs only when a device flag says so (the full verifier's pass under the routed execution policy): every
 // kernel of it takes the flag's address and leaves at once when the flag is zero.  The flag is written by a kernel that
 // has completed before the pass's first kernel starts (the pass opens with ordinary, fully ordered launches), so

@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(256)
 rmsnorm_kernel(T *a, size_t plane, const float *h, const float *gain, int d, float eps) {
     __shared__ float red[8];
     PDL_TRIGGER();
+    PDL_WAIT();
     const int r = blockIdx.x;
     const float4 *x4 = reinterpret_cast<const float4 *>(h + (size_t)r * d);
     const float4 *g4 = reinterpret_cast<const float4 *>(gain);
@@ -262,10 +263,10 @@ rmsnorm_kernel(T *a, size_t plane, const float *h, const float *gain, int d, flo
 
 int launch_rmsnorm(const viasd_model *m, const float *gain, int rows, cudaStream_t st) {
     if (m->cfg.dtype == 0)
-        rmsnorm_kernel<float><<<rows, 256, 0, st>>>((float *)m->ws.a, 0, m->ws.h, gain, m->cfg.d_model, m->cfg.rms_eps);
+        CUDA_TRY(launch_chained(rmsnorm_kernel<float>, rows, 256, st, (float *)m->ws.a, 0, m->ws.h, gain, m->cfg.d_model, m->cfg.rms_eps));
     else
-        rmsnorm_kernel<__nv_bfloat16><<<rows, 256, 0, st>>>((__nv_bfloat16 *)m->ws.a, m->ws.rows_alloc * m->cfg.d_model,
-                                                            m->ws.h, gain, m->cfg.d_model, m->cfg.rms_eps);
+        CUDA_TRY(launch_chained(rmsnorm_kernel<__nv_bfloat16>, rows, 256, st, (__nv_bfloat16 *)m->ws.a, m->ws.rows_alloc * m->cfg.d_model,
+                                m->ws.h, gain, m->cfg.d_model, m->cfg.rms_eps));
     LAUNCH_CHECK();
     return VIASD_OK;
 }
@@ -279,6 +280,7 @@ __global__ void rope_append_kernel(float *q_out, T *kc, T *vc, const float *qkv,
                                    int max_batch, int max_ctx, int layer_ord) {
     int r = blockIdx.x, head = blockIdx.y;
     PDL_TRIGGER();
+    PDL_WAIT();
     int b = r / M, i = r % M;
     int half = hd >> 1;
     int n = len_eff[b];
@@ -313,10 +315,11 @@ int launch_rope_append(const viasd_model *m, void *kc, void *vc, int layer_ord, 
     dim3 grid(batch * M, c.n_heads + 2 * c.n_kv_heads);
     int threads = c.head_dim / 2 < 32 ? 32 : c.head_dim / 2;
     if (c.dtype == 0)
-        rope_append_kernel<float><<<grid, threads, 0, st>>>(m->ws.q, (float *)kc, (float *)vc, m->ws.qkv,
+        CUDA_TRY(launch_chained(rope_append_kernel<float>, grid, threads, st, m->ws.q, (float *)kc, (float *)vc, m->ws.qkv,
             m->ws.rope_cos, m->ws.rope_sin, m->ws.len_eff, m->ws.tree, M, c.n_heads, c.n_kv_heads, c.head_dim,
-            c.max_batch, c.max_ctx, layer_ord);
+            c.max_batch, c.max_ctx, layer_ord));
     else
+        // (an ordinary launch: the attention kernel behind it reads lengths and tree ahead of its wait)
         rope_append_kernel<__nv_bfloat16><<<grid, threads, 0, st>>>(m->ws.q, (__nv_bfloat16 *)kc,
             (__nv_bfloat16 *)vc, m->ws.qkv, m->ws.rope_cos, m->ws.rope_sin, m->ws.len_eff, m->ws.tree, M, c.n_heads,
             c.n_kv_heads, c.head_dim, c.max_batch, c.max_ctx, layer_ord);

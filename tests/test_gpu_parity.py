@@ -75,6 +75,25 @@ def test_gemm_matches_matmul(dtype, rows, n, k):
     assert np.abs(got - want).max() <= tol, (np.abs(got - want).max(), tol)
 
 
+# the fp32 kernels where their choices change: one warp per feature and four, row counts between the register tiles
+@pytest.mark.parametrize("rows,n,k", [(1, 40, 8), (4, 9472, 136), (5, 9470, 64), (8, 300, 1024), (13, 9480, 40), (25, 257, 520)])
+def test_fp32_gemm_edges(rows, n, k):
+    vb = _vb()
+    xw, ww = synth.normal_f32(3, 1, (rows, k), 1.0), synth.normal_f32(3, 2, (n, k), 0.05)
+    y = torch.full((rows, n), float("nan"), dtype=torch.float32, device="cuda")
+    scratch = torch.empty(max(256, vb.gemm_scratch_bytes(rows, n, k)), dtype=torch.uint8, device="cuda")
+    vb.gemm(torch.from_numpy(xw).cuda(), torch.from_numpy(ww).cuda(), y, scratch)
+    want = xw.astype(np.float64) @ ww.astype(np.float64).T
+    # exact products, fp32 accumulation of k terms
+    assert np.abs(y.cpu().numpy() - want).max() <= 2e-6 * np.sqrt(k) * np.abs(want).max() + 1e-6
+
+
+# bf16 products around the k from which a tile is split among CTAs (12 boxes of 64)
+@pytest.mark.parametrize("rows,n,k", [(9, 512, 704), (9, 512, 768), (9, 512, 776), (17, 18944, 768), (17, 19072, 640)])
+def test_gemm_around_the_split(rows, n, k):
+    test_gemm_matches_matmul("bf16", rows, n, k)
+
+
 # ---------------------------------------------------------------------------------------------
 # forward passes
 # ---------------------------------------------------------------------------------------------
