@@ -147,7 +147,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(WTHREADS, 1)
 gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CUtensorMap map_w1,
                  const __grid_constant__ CUtensorMap map_w2, const __grid_constant__ CUtensorMap map_x, const TcParams p) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) unsigned long long bars[2 * WSTAGES + 5];
+    __shared__ __align__(8) unsigned long long bars[2 * WSTAGES + 4];
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh, tfull_ok[2];
     __shared__ __align__(16) float xch[WGROUPS][CH * TILE_F];     // a chunk on its way from TMEM lanes to rows, per group
@@ -164,19 +164,17 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
     // boxes come from L2 and need only a few slots.  A box's two loads still share one full barrier and one commit: box i's
     // weights and box i - (SW - SX)'s activations are requested when box i - SW has been read.
     const int SW = p.stages, SX = p.x_stages;
-    const uint32_t x_bytes = (uint32_t)TH * 128u, xbox = TT * x_bytes, ring_bytes = SW * WBOX + SX * xbox;
+    const uint32_t x_bytes = (uint32_t)TH * 128u, xbox = TT * x_bytes;
     const uint32_t xring = smem_base + SW * WBOX;
     auto full_bar = [&](int s) { return smem_u32(&bars[s]); };
     auto empty_bar = [&](int s) { return smem_u32(&bars[WSTAGES + s]); };
     auto tfull_bar = [&](int b) { return smem_u32(&bars[2 * WSTAGES + b]); };
     auto tempty_bar = [&](int b) { return smem_u32(&bars[2 * WSTAGES + 2 + b]); };
-    const uint32_t gather_bar = smem_u32(&bars[2 * WSTAGES + 4]);
     const uint32_t acc_cols = (uint32_t)TT * 2u * TH;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < SW; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 2 * WGROUPS * 4); }
-        mbar_init(gather_bar, 4 * WGROUPS);
         abort_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -334,7 +332,6 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
         epi_sync();
 
         int acc_it = 0, u = u_begin, seg_i = 0;
-        uint32_t gather_ph = 0;
         Seg sg;
         bool ok = true;
         while (ok && next_seg(u, u_end, p.k_tiles, sg)) {
@@ -425,79 +422,49 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
                 gain_a = __ldg(reinterpret_cast<const float4 *>(p.next_gain + tile * TILE_F + 4 * lane));
                 gain_b = p.next_gain2 ? __ldg(reinterpret_cast<const float4 *>(p.next_gain2 + tile * TILE_F + 4 * lane)) : gain_a;
             }
-            // The other contributors' rows of the slice come into the idle ring by bulk copies, as many rows per round as
-            // fit (a range's last piece of work: nothing is in flight there any more); if not even a chunk of every
-            // contributor fits they are read where they are.
-            const int others = n_c - 1, my_rows = row_end - row_begin;
-            const int fit = others ? (int)(ring_bytes / ((uint32_t)others * TILE_F * 4u)) / CH * CH : WROWS;
-            const bool staged = others > 0 && my_rows > 0 && fit >= CH;
-            const int blk_rows = staged && fit < my_rows ? (fit >= WGROUPS * CH ? fit / (WGROUPS * CH) * (WGROUPS * CH) : fit) : max(my_rows, 1);
-            const bool in_step = blk_rows % (WGROUPS * CH) == 0 || blk_rows >= my_rows;    // else a round's first chunk is not the prefetched one
+            // The other contributors' rows are read where they are, a row per warp: 16-byte loads, up to four contributors of
+            // two rows in flight, asked for before the chunk's trip through shared memory.
+            const int others = n_c - 1;
             auto slot_of = [&](int c) {                            // contributor c's partial of this tile
                 const int cp = first + c, c_first = (cp * p.units_per_cta) / p.k_tiles;
-                return p.scratch + ((size_t)(2 * cp + (int)rank) * 2 + (c_first == sg.tile ? 0 : 1)) * slot_floats;
+                return p.scratch + ((size_t)(2 * cp + (int)rank) * 2 + (c_first == sg.tile ? 0 : 1)) * slot_floats + 4 * lane;
             };
-            for (int blk0 = row_begin; blk0 < row_end; blk0 += blk_rows) {
-                const int blk_end = min(row_end, blk0 + blk_rows), nr = min(p.rows, blk_end) - blk0;
-                if (staged) {
-                    if (blk0 > row_begin) epi_sync();              // everyone is done with the previous round's rows
-                    // One copy of a hundred rows runs at a tenth of the rate of several at once, and a thread takes 100 ns to
-                    // issue one: every warp asks for about a sixteenth of the rows.
-                    if (lane == 0) {
-                        asm volatile("fence.proxy.async.global;" ::: "memory");
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                        const int ew = warp - 2, per_c = max(1, 4 * WGROUPS / others);               // warps per contributor
-                        const int piece = ((nr + per_c - 1) / per_c + CH - 1) / CH * CH, pieces = (nr + piece - 1) / piece;
-                        uint32_t bytes = 0;
-                        for (int i = ew; i < others * pieces; i += 4 * WGROUPS) bytes += (uint32_t)min(piece, nr - (i % pieces) * piece) * TILE_F * 4u;
-                        if (bytes) mbar_expect_tx(gather_bar, bytes); else mbar_arrive(gather_bar);
-                        for (int i = ew; i < others * pieces; i += 4 * WGROUPS) {
-                            const int c = i / pieces, r = (i - c * pieces) * piece;
-                            bulk_load(smem_base + (uint32_t)(c * blk_rows + r) * TILE_F * 4u, slot_of(c < mine ? c : c + 1) + (size_t)(blk0 + r) * TILE_F,
-                                      (uint32_t)min(piece, nr - r) * TILE_F * 4u, gather_bar);
-                        }
-                    }
-                }
-                if (!in_step && blk0 > row_begin) load_aux(blk0 + group * CH, row_end);
-                bool gathered = !staged;
 #pragma unroll 1
-                for (int r0 = blk0 + group * CH; r0 < blk_end; r0 += WGROUPS * CH) {
-                    const int ra = r0 + 2 * gw;                    // this warp's two rows of the chunk
-                    float g[CH];
-                    load_chunk(r0, g);
-                    group_sync();                                  // the group has read its previous chunk
+            for (int r0 = row_begin + group * CH; r0 < row_end; r0 += WGROUPS * CH) {
+                const int ra = r0 + 2 * gw;                        // this warp's two rows of the chunk
+                float4 part[4][2];
 #pragma unroll
-                    for (int j = 0; j < CH; ++j) xg[j * TILE_F + f] = g[j];
-                    group_sync();
-                    if (!gathered) { gathered = true; if (!mbar_wait(gather_bar, gather_ph, &abort_sh, p.status)) ok = false; }
+                for (int c = 0; c < 4; ++c) {
+                    if (c < n_c && c != mine) {
+                        const float *from = slot_of(c);
 #pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        const int r = ra + i;
-                        if (r >= p.rows || r >= blk_end) continue;
-                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                        const float4 own = *reinterpret_cast<const float4 *>(xg + (2 * gw + i) * TILE_F + 4 * lane);
-                        if (others == 0) {
-                            v = own;
-                        } else if (staged) {
-                            const float *part = reinterpret_cast<const float *>(smem_raw + (smem_base - smem_u32(smem_raw))) + (size_t)(r - blk0) * TILE_F + 4 * lane;
-                            for (int c = 0; c < n_c; ++c) {        // in pair order, whoever adds them
-                                if (c == mine) { v = add4(v, own); continue; }
-                                v = add4(v, *reinterpret_cast<const float4 *>(part));
-                                part += (size_t)blk_rows * TILE_F;
-                            }
-                        } else {
-                            for (int c = 0; c < n_c; ++c)
-                                v = add4(v, c == mine ? own : __ldcg(reinterpret_cast<const float4 *>(slot_of(c) + (size_t)r * TILE_F + 4 * lane)));
-                        }
-                        finish_row<EPI>(p, tile, r, v, aux[i][0], aux[i][1], gain_a, gain_b, inv_sh, rowmeta, lane);
+                        for (int i = 0; i < 2; ++i)
+                            part[c][i] = __ldcg(reinterpret_cast<const float4 *>(from + (size_t)min(ra + i, p.rows - 1) * TILE_F));
                     }
-                    // (chunks go on into the next round of rows: blocks are whole rounds of the groups except the last)
-                    load_aux(r0 + WGROUPS * CH, row_end);
                 }
-                if (staged) {
-                    if (!gathered && !mbar_wait(gather_bar, gather_ph, &abort_sh, p.status)) ok = false;
-                    gather_ph ^= 1;
+                float g[CH];
+                load_chunk(r0, g);
+                group_sync();                                      // the group has read its previous chunk
+#pragma unroll
+                for (int j = 0; j < CH; ++j) xg[j * TILE_F + f] = g[j];
+                group_sync();
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int r = ra + i;
+                    if (r >= p.rows) continue;
+                    const float4 own = *reinterpret_cast<const float4 *>(xg + (2 * gw + i) * TILE_F + 4 * lane);
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (others == 0) {
+                        v = own;
+                    } else {                                       // in pair order, whoever adds them
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) if (c < n_c) v = add4(v, c == mine ? own : part[c][i]);
+                        for (int c = 4; c < n_c; ++c)
+                            v = add4(v, c == mine ? own : __ldcg(reinterpret_cast<const float4 *>(slot_of(c) + (size_t)r * TILE_F)));
+                    }
+                    finish_row<EPI>(p, tile, r, v, aux[i][0], aux[i][1], gain_a, gain_b, inv_sh, rowmeta, lane);
                 }
+                load_aux(r0 + WGROUPS * CH, row_end);
             }
             // this tile's accumulator may be overwritten
             tc_fence_before();
