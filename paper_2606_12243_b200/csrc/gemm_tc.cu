@@ -12,8 +12,8 @@
 // range per CTA, so every SM streams the same number of bytes whatever the shape.  A CTA that holds all
 // k-blocks of a tile finishes it from TMEM; otherwise it writes an fp32 partial and counts itself in.  The
 // contributors that end their range inside the tile then share its finishing: each waits (bounded) for the
-// count to be complete, pulls its slice of the token rows of every partial into the idle shared-memory ring
-// with bulk copies and sums them in CTA order - bit-reproducible whoever does it.  A contributor that
+// count to be complete, reads its slice of the token rows of every partial and sums them in CTA order -
+// bit-reproducible whoever does it.  A contributor that
 // continues into the next tile never waits, so waits cannot chain.
 //
 // Warp roles (320 threads): warp 0 issues TMA loads into a ring of stages, warp 1 allocates TMEM and
@@ -33,11 +33,11 @@ __global__ void __launch_bounds__(64 + 128 * GROUPS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CUtensorMap map_w1,
                const __grid_constant__ CUtensorMap map_w2, const __grid_constant__ CUtensorMap map_x, const TcParams p) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) unsigned long long bars[2 * MAX_STAGES + 5];
+    __shared__ __align__(8) unsigned long long bars[2 * MAX_STAGES + 4];
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh;
     __shared__ float inv_sh[128];                       // per-row 1/rms of the input (fused RMSNorm)
-    __shared__ float xch[GROUPS * CH * TILE_F];         // rotary partner exchange, one buffer per epilogue group
+    __shared__ __align__(16) float xch[GROUPS][EPI == EPI_SWIGLU ? 2 : 1][CH * TILE_F];   // a chunk on its way from TMEM lanes to rows, per group
     __shared__ int4 rowmeta[128];                       // per token row: rotary position, cache slot, offset in its cache
 
     constexpr bool DUAL = EPI == EPI_SWIGLU;
@@ -53,20 +53,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
     // longer than the stage's weights take to arrive: those launches streamed at 5.9 TB/s, not 6.5.
     constexpr int KB = DUAL ? 1 : KBT;                    // (the launch picks one box at wide token tiles: two would leave two stages)
     const uint32_t a_bytes = TILE_F * TILE_K * 2, b_bytes = (uint32_t)NT * TILE_K * 2;
-    const uint32_t box_bytes = NACC * a_bytes + 2 * b_bytes;          // one k-box of every operand
+    const int planes = p.has_lo ? 2 : 1;
+    const uint32_t box_bytes = NACC * a_bytes + planes * b_bytes;     // one k-box of every operand
     const uint32_t stage_bytes = KB * box_bytes;
     auto full_bar = [&](int s) { return smem_u32(&bars[s]); };
     auto empty_bar = [&](int s) { return smem_u32(&bars[MAX_STAGES + s]); };
     auto tfull_bar = [&](int b) { return smem_u32(&bars[2 * MAX_STAGES + b]); };
     auto tempty_bar = [&](int b) { return smem_u32(&bars[2 * MAX_STAGES + 2 + b]); };
-    const uint32_t gather_bar = smem_u32(&bars[2 * MAX_STAGES + 4]);
     const int NB = p.has_lo ? 2 * NT : NT;                  // MMA N: hi and lo token columns side by side
     const uint32_t acc_cols = NACC * NB;                    // TMEM columns per accumulator buffer
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), GROUPS * 4); }
-        mbar_init(gather_bar, GROUPS * 128);
         abort_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -112,7 +111,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
 #pragma unroll
                 for (int kb = 0; kb < KB; ++kb) {
                     tma_load_2d(base + kb * box_bytes, &map_x, full_bar(st), (kt + kb) * TILE_K, p.row0);
-                    tma_load_2d(base + kb * box_bytes + b_bytes, &map_x, full_bar(st), (kt + kb) * TILE_K, p.row0 + p.lo_row_offset);
+                    if (p.has_lo) tma_load_2d(base + kb * box_bytes + b_bytes, &map_x, full_bar(st), (kt + kb) * TILE_K, p.row0 + p.lo_row_offset);
                 }
             };
             const CUtensorMap *mw; int wrow, kt, sidx;
@@ -128,14 +127,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
             asm volatile("griddepcontrol.wait;" ::: "memory");
             for (int it = 0; it < pre; ++it) {
                 unit(it, mw, wrow, kt, sidx);
-                mbar_expect_tx(full_bar(it), KB * 2 * p.b_tx);
+                mbar_expect_tx(full_bar(it), KB * planes * p.b_tx);
                 load_x(it, kt);
             }
             for (int it = pre; it < n_it; ++it) {
                 const int st = it % S;
                 if (!mbar_wait(empty_bar(st), ((it / S) & 1) ^ 1, &abort_sh, p.status)) break;
                 unit(it, mw, wrow, kt, sidx);
-                mbar_expect_tx(full_bar(st), (DUAL ? 2 * p.a_tx[0] : KB * p.a_tx[sidx]) + KB * 2 * p.b_tx);
+                mbar_expect_tx(full_bar(st), (DUAL ? 2 * p.a_tx[0] : KB * p.a_tx[sidx]) + KB * planes * p.b_tx);
                 load_w(st, mw, wrow, kt);
                 load_x(st, kt);
             }
@@ -184,60 +183,85 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
         // One or two groups of 128 threads (the launch decides: the second group pays at wide token tiles, where the
         // finishing is many chunks long, and costs a little at narrow ones); wherever rows are handled chunk by
         // chunk, the groups take the chunks in turn.
-        const int quarter = warp & 3;
-        const int f = quarter * 32 + lane;                  // feature lane inside the tile, as TMEM lanes map to warps
-        const int et_all = threadIdx.x - 64;                // 0..255 among epilogue threads
-        const int group = GROUPS > 1 ? et_all >> 7 : 0, et = GROUPS > 1 ? (et_all & 127) : et_all;   // et: the thread's number in its group = its feature in staged tiles
-        constexpr int epi_threads = GROUPS * 128, n_groups = GROUPS;
+        const int quarter = warp & 3, f = quarter * 32 + lane;   // feature lane inside the tile, as TMEM lanes map to warps
+        const int et = threadIdx.x - 64, group = GROUPS > 1 ? et >> 7 : 0, gw = (et >> 5) & 3;
+        constexpr int epi_threads = GROUPS * 128;
         const size_t slot_floats = (size_t)NACC * NT * TILE_F;
-        // per-row tables (all 128 entries defined: chunks read a few rows past p.rows and discard them)
-        inv_sh[et] = 0.f;
-        rowmeta[et] = make_int4(0, 0, 0, 0);
-        asm volatile("bar.sync 1, %0;" ::"n"(epi_threads) : "memory");
+        float *xg = xch[group][0];
+        auto group_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(2 + group) : "memory"); };
+        auto epi_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(epi_threads) : "memory"); };
+        if (et < 128) { inv_sh[et] = 0.f; rowmeta[et] = make_int4(0, -1, 0, 0); }
+        epi_sync();
         // The tile this CTA's range ends in is the one it will help to finish: what that epilogue reads from
         // weights (not from the kernel before) is fetched now, off the critical path.
         const int last_tile = (u_end - 1) / p.k_tiles;
-        float2 last_gain = make_float2(0.f, 0.f);
-        if (EPI == EPI_ADD_NORM) {
-            const int n = last_tile * TILE_F + et;
-            if (n < p.seg_n[0]) {
-                last_gain.x = __ldg(p.next_gain + n);
-                last_gain.y = p.next_gain2 ? __ldg(p.next_gain2 + n) : last_gain.x;
-            }
-        }
+        float4 gain_a = make_float4(0.f, 0.f, 0.f, 0.f), gain_b = gain_a;
+        auto load_gain = [&](int tile) {
+            if (EPI != EPI_ADD_NORM) return;
+            gain_a = __ldg(reinterpret_cast<const float4 *>(p.next_gain + tile * TILE_F + 4 * lane));
+            gain_b = p.next_gain2 ? __ldg(reinterpret_cast<const float4 *>(p.next_gain2 + tile * TILE_F + 4 * lane)) : gain_a;
+        };
+        load_gain(last_tile);
 
-        // A tile is finished from one of three sources: the accumulator in TMEM (this CTA held all of K), the
-        // partials staged in shared memory, or the partials read straight from global memory.  All three feed ONE
-        // copy of the epilogue code, and that copy runs once "dry" (no row is live, nothing is stored) before
-        // the kernel waits for its predecessor: the epilogue otherwise runs exactly once per CTA, at the very end,
-        // from a cold instruction cache while HBM is saturated, and those instruction misses were the tail.
-        enum { SRC_DRY, SRC_TMEM, SRC_SMEM, SRC_GLOBAL };
+        // A tile is finished a row per warp, from the accumulator in TMEM (this CTA held all of K: chunks of 8 rows pass through
+        // shared memory) or from the contributors' partial rows in global memory, 16 bytes a lane and six contributors (three of
+        // the gate/up pair) in flight.  Finishing a feature per thread, from rows that bulk copies staged in the idle ring, took
+        // a further trip and wrote 2 bytes a lane (7B batch 1 step 3.48 -> 3.43 ms, 25 launches of the shrunken 7B 218 -> 201 us).
+        // One copy of the code serves both, and runs once "dry" (nothing is stored) before the kernel waits for its
+        // predecessor: otherwise it runs once per CTA, at the very end, from a cold instruction cache.
         int acc_it = 0, u = u_begin, seg_i = 0;
         Seg sg;
         sg.tile = last_tile; sg.ka = 0; sg.kb = 0;                 // dry pass: the tile this CTA is most likely to finish
         bool ok = true, dry = true;
         while (ok) {
-            int src = SRC_DRY, buf = 0, first_cta = 0, last_cta = 0;
+            int buf = 0, first_cta = blockIdx.x, n_c = 1;
             uint32_t t0 = 0;
-            const float *parts = nullptr, *aux = nullptr;
-            int stage_rows = 0, aux_kind = 0;                // staged gather: rows per round; 1: residual rows, 2: rotary tables
-            int row_begin = 0, row_end = p.rows;             // the rows this CTA finishes
-            if (dry) {
-                // the dry pass sums one "contributor" out of whatever the ring holds, so that the staged path's code is warm too
-                src = SRC_SMEM;
-                parts = reinterpret_cast<const float *>(smem_raw + (smem_base - smem_u32(smem_raw)));
-            } else {
+            int row_begin = 0, row_end = dry ? 1 : p.rows;         // the rows this CTA finishes
+            bool whole = false;
+            float4 aux[2][2];
+            // what finishing a row reads besides the sums, asked for ahead of the waits (rows r0 + gw and 4 further)
+            auto load_aux = [&](int r0, int r_end) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int r = r0 + gw + 4 * i;
+                    if (r >= r_end) continue;
+                    if (EPI == EPI_ADD_NORM) {
+                        aux[i][0] = __ldcg(reinterpret_cast<const float4 *>(p.out_f32 + (size_t)(p.row0 + r) * p.ld_out + sg.tile * TILE_F + 4 * lane));
+                    } else if (EPI == EPI_QKV_ROPE) {
+                        const size_t o = (size_t)rowmeta[r].x * 64 + (lane & 15) * 4;
+                        aux[i][0] = *reinterpret_cast<const float4 *>(p.cosv + o);
+                        aux[i][1] = *reinterpret_cast<const float4 *>(p.sinv + o);
+                    }
+                }
+            };
+#pragma unroll
+            for (int i = 0; i < 4; ++i) aux[i >> 1][i & 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (!dry) {
                 if (!next_seg(u, u_end, p.k_tiles, sg)) break;
                 buf = acc_it % p.acc_bufs;
+                whole = sg.ka == 0 && sg.kb == p.k_tiles;
+                const bool finisher = u >= u_end;                 // this range ends here; one that goes on only contributes
+                int last_cta = blockIdx.x, n_fin = 1;
+                if (!whole) {
+                    first_cta = (sg.tile * p.k_tiles) / p.units_per_cta;
+                    last_cta = ((sg.tile + 1) * p.k_tiles - 1) / p.units_per_cta;
+                    n_c = last_cta - first_cta + 1;
+                    const int last_range_end = min(total_units, (last_cta + 1) * p.units_per_cta);
+                    n_fin = n_c - (last_range_end > (sg.tile + 1) * p.k_tiles ? 1 : 0);
+                    // this finisher's rows, dealt one by one in order of CTA number
+                    const int per = (p.rows + n_fin - 1) / n_fin, mine = blockIdx.x - first_cta;
+                    row_begin = finisher ? min(p.rows, mine * per) : p.rows;
+                    row_end = finisher ? min(p.rows, (mine + 1) * per) : p.rows;
+                }
+                if (sg.tile != last_tile && row_begin < row_end) load_gain(sg.tile);
+                load_aux(row_begin + group * CH, row_end);
                 if (!(ok = mbar_wait(tfull_bar(buf), (acc_it / p.acc_bufs) & 1, &abort_sh, p.status))) break;
                 tc_fence_after();
                 t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * acc_cols;
-                if (sg.ka == 0 && sg.kb == p.k_tiles) {
-                    src = SRC_TMEM;
-                } else {
+                if (!whole) {
                     // partial of a split tile: slot 0 if the tile is the first one this CTA touches, else slot 1
                     float *slot = p.scratch + ((size_t)blockIdx.x * 2 + (seg_i == 0 ? 0 : 1)) * slot_floats;
-                    for (int c = group * CH; c < p.rows; c += n_groups * CH) {   // padding rows beyond p.rows are never read
+                    for (int c = group * CH; c < p.rows; c += GROUPS * CH) {   // padding rows beyond p.rows are never read
                         float g[CH], uu[CH];
                         if (p.has_lo) {                          // add the product with the lo plane
                             float lo[CH];
@@ -268,139 +292,96 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
                     // next tile only arrives and never waits, so no wait depends on another wait.
                     // (release / acquire: the barrier orders the group's stores before its first thread's release, which
                     // is cumulative; a fence per thread on both sides was a microsecond of the launch's tail)
-                    asm volatile("bar.sync 1, %0;" ::"n"(epi_threads) : "memory");
-                    first_cta = (sg.tile * p.k_tiles) / p.units_per_cta;
-                    last_cta = ((sg.tile + 1) * p.k_tiles - 1) / p.units_per_cta;
-                    if (et_all == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.counters + sg.tile) : "memory");   // low half: arrivals
-                    if (u < u_end) { ++acc_it; ++seg_i; continue; }
-                    const int n_c = last_cta - first_cta + 1;
-                    const int last_range_end = min(total_units, (last_cta + 1) * p.units_per_cta);
-                    const int n_fin = n_c - (last_range_end > (sg.tile + 1) * p.k_tiles ? 1 : 0);
-                    if (et_all == 0) {
+                    epi_sync();
+                    if (et == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.counters + sg.tile) : "memory");   // low half: arrivals
+                    if (!finisher) { ++acc_it; ++seg_i; continue; }
+                    if (et == 0) {
                         const int *ctr = p.counters + sg.tile;
                         auto arrived = [&]() { int v; asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory"); return v & 0xffff; };
                         const long long w0 = clock64();
                         while (arrived() < n_c) {
-                            if (abort_sh || clock64() - w0 > WAIT_LIMIT_CYCLES) { abort_sh = 1; atomicExch(p.status, VIASD_EDEVICE); break; }
-                            __nanosleep(64);
+                            if (*(volatile int *)&abort_sh || clock64() - w0 > WAIT_LIMIT_CYCLES) { abort_sh = 1; atomicExch(p.status, VIASD_EDEVICE); break; }
+                            __nanosleep(32);
                         }
                         // high half: finishers that have seen all arrivals; the last of them leaves the counter at zero
                         if (!abort_sh && (atomicAdd(&p.counters[sg.tile], 1 << 16) >> 16) == n_fin - 1) atomicExch(&p.counters[sg.tile], 0);
                     }
-                    asm volatile("bar.sync 1, %0;" ::"n"(epi_threads) : "memory");
+                    epi_sync();
                     if (abort_sh) { ok = false; break; }
-                    {
-                        // this finisher's rows: whole chunks, dealt in order of CTA number
-                        const int n_chunks = (p.rows + CH - 1) / CH, per = (n_chunks + n_fin - 1) / n_fin;
-                        const int mine = blockIdx.x - first_cta;
-                        row_begin = min(p.rows, mine * per * CH);
-                        row_end = min(p.rows, (mine + 1) * per * CH);
-                    }
-                    src = SRC_GLOBAL;
-                    // Staged gather: when this is the CTA's last piece of work the shared-memory ring is idle, so the
-                    // partials (and the rows the epilogue would otherwise fetch chunk by chunk) come in by bulk copies,
-                    // as many rows per round as the ring holds.  Same sums in the same order as the direct path.
-                    const int fit = (int)(((uint32_t)S * stage_bytes) / ((uint32_t)(n_c * NACC + 1) * TILE_F * 4u)) / CH * CH;
-                    if (fit >= CH && row_end > row_begin) {
-                        const int my_rows = (row_end - row_begin + CH - 1) / CH * CH;
-                        stage_rows = fit < my_rows ? fit : my_rows;
-                        if (EPI == EPI_ADD_NORM && (sg.tile + 1) * TILE_F <= p.seg_n[0]) aux_kind = 1;
-                        if (EPI == EPI_QKV_ROPE && sg.tile < p.seg_tile_end[1]) aux_kind = 2;
-                        src = SRC_SMEM;
-                    }
                 }
             }
-
-            // ---- the one finishing loop, over blocks of rows (one block unless the gather is staged in rounds)
-            const int fe = src == SRC_TMEM ? f : et;
-            const int rows_live = dry ? 0 : p.rows, rows_loop = dry ? CH : row_end;
-            const int blk_rows = stage_rows ? stage_rows : (rows_loop > 0 ? rows_loop : 1);
-            const int plane = stage_rows ? stage_rows * TILE_F : p.rows * TILE_F;     // floats between contributors in shared memory
-            int round = 0;
+            auto slot_of = [&](int c) {                            // contributor c's partial of this tile
+                const int cta = first_cta + c, c_first = (cta * p.units_per_cta) / p.k_tiles;
+                return p.scratch + ((size_t)cta * 2 + (c_first == sg.tile ? 0 : 1)) * slot_floats + 4 * lane;
+            };
+            constexpr int INFL = DUAL ? 3 : 6;                     // contributors whose rows are in flight together
 #pragma unroll 1
-            for (int blk0 = dry ? 0 : row_begin; blk0 < rows_loop && ok; blk0 += blk_rows, ++round) {
-            const int blk_end = min(rows_loop, blk0 + blk_rows);
-            if (stage_rows) {
-                // rows blk0 .. blk_end-1 of every contributor (and of the epilogue's own inputs) into the ring
-                const int nr = min(p.rows, blk_end) - blk0, n_c = last_cta - first_cta + 1;
-                const uint32_t row_bytes = TILE_F * 4u, aux_sh = smem_base, part_sh = smem_base + (uint32_t)stage_rows * row_bytes;
-                if (round > 0) asm volatile("bar.sync 1, %0;" ::"n"(epi_threads) : "memory");    // everyone is done with the previous round's rows
-                const bool has_part = et_all < n_c * NACC, has_aux = aux_kind && et_all < nr;   // nr <= 128: first group
-                asm volatile("fence.proxy.async.global;" ::: "memory");
-                if (has_part || has_aux) {
-                    mbar_expect_tx(gather_bar, (has_part ? (uint32_t)nr * row_bytes : 0u) + (has_aux ? row_bytes : 0u));
-                    if (has_part) {
-                        const int c = first_cta + et_all / NACC, half = et_all - (et_all / NACC) * NACC;
-                        const int c_first_tile = (c * p.units_per_cta) / p.k_tiles;
-                        const float *from = p.scratch + ((size_t)c * 2 + (c_first_tile == sg.tile ? 0 : 1)) * slot_floats +
-                                            (size_t)half * NT * TILE_F + (size_t)blk0 * TILE_F;
-                        bulk_load(part_sh + (uint32_t)et_all * (uint32_t)stage_rows * row_bytes, from, (uint32_t)nr * row_bytes, gather_bar);
-                    }
-                    if (has_aux) {
-                        const uint32_t dst = aux_sh + (uint32_t)et * row_bytes;
-                        if (aux_kind == 1) {
-                            bulk_load(dst, p.out_f32 + (size_t)(p.row0 + blk0 + et) * p.ld_out + sg.tile * TILE_F, row_bytes, gather_bar);
-                        } else {
-                            const int pos = rowmeta[blk0 + et].x;
-                            bulk_load(dst, p.cosv + (size_t)pos * 64, 256, gather_bar);
-                            bulk_load(dst + 256, p.sinv + (size_t)pos * 64, 256, gather_bar);
-                        }
-                    }
-                } else {
-                    mbar_arrive(gather_bar);
-                }
-                if (!(ok = mbar_wait(gather_bar, round & 1, &abort_sh, p.status))) break;
-                parts = reinterpret_cast<const float *>(smem_raw + (part_sh - smem_u32(smem_raw)));
-                // finish_chunk indexes the epilogue's rows by their number in the launch: shift the base by the block start
-                if (aux_kind) aux = reinterpret_cast<const float *>(smem_raw + (aux_sh - smem_u32(smem_raw))) - (size_t)blk0 * TILE_F;
-            }
-#pragma unroll 1
-            for (int r0 = blk0 + group * CH; r0 < blk_end; r0 += n_groups * CH) {
-                float g[CH], uu[CH];
+            for (int r0 = row_begin + group * CH; r0 < row_end; r0 += GROUPS * CH) {
+                float4 v[2], uu[2];
 #pragma unroll
-                for (int j = 0; j < CH; ++j) { g[j] = 0.f; uu[j] = 0.f; }
-                if (src == SRC_TMEM) {
-                    tc_ld8(t0 + r0, g);
-                    if (DUAL) tc_ld8(t0 + NB + r0, uu);
+                for (int i = 0; i < 2; ++i) v[i] = uu[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (whole) {
+                    float g[CH], lo[CH];
                     if (p.has_lo) {
-                        float lo[CH];
-                        tc_ld8(t0 + NT + r0, lo);
+                        tc_ld8x2(t0 + r0, t0 + NT + r0, g, lo);
 #pragma unroll
                         for (int j = 0; j < CH; ++j) g[j] += lo[j];
-                        if (DUAL) {
-                            tc_ld8(t0 + NB + NT + r0, lo);
-#pragma unroll
-                            for (int j = 0; j < CH; ++j) uu[j] += lo[j];
-                        }
+                    } else {
+                        tc_ld8(t0 + r0, g);
                     }
-                } else if (src == SRC_SMEM) {
-                    for (int c = 0; c <= last_cta - first_cta; ++c) {
+                    group_sync();                                  // the group has read its previous chunk
 #pragma unroll
-                        for (int j = 0; j < CH; ++j) {
-                            const int r = min(r0 + j, p.rows - 1) - blk0;  // row inside the staged block; rows past the end are discarded
-                            g[j] += parts[(c * NACC) * plane + r * TILE_F + et];
-                            if (DUAL) uu[j] += parts[(c * NACC + 1) * plane + r * TILE_F + et];
+                    for (int j = 0; j < CH; ++j) xg[j * TILE_F + f] = g[j];
+                    if (DUAL) {
+                        if (p.has_lo) {
+                            tc_ld8x2(t0 + NB + r0, t0 + NB + NT + r0, g, lo);
+#pragma unroll
+                            for (int j = 0; j < CH; ++j) g[j] += lo[j];
+                        } else {
+                            tc_ld8(t0 + NB + r0, g);
                         }
+#pragma unroll
+                        for (int j = 0; j < CH; ++j) xg[CH * TILE_F + j * TILE_F + f] = g[j];
                     }
-                } else if (src == SRC_GLOBAL) {
-                    // rare (a tile shared by more CTAs than the ring can stage a chunk of): plain loads, contributor by
-                    // contributor, kept small on purpose - the size of this loop's code is part of every launch's tail
+                    group_sync();
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        v[i] = *reinterpret_cast<const float4 *>(xg + (gw + 4 * i) * TILE_F + 4 * lane);
+                        if (DUAL) uu[i] = *reinterpret_cast<const float4 *>(xg + CH * TILE_F + (gw + 4 * i) * TILE_F + 4 * lane);
+                    }
+                } else if (r0 + gw < row_end) {
+                    // rows of every contributor, in CTA order, 16-byte loads of up to INFL contributors in flight
+                    const size_t ra = (size_t)(r0 + gw) * TILE_F, rb = (size_t)min(r0 + gw + 4, row_end - 1) * TILE_F;
 #pragma unroll 1
-                    for (int c = first_cta; c <= last_cta; ++c) {
-                        const int c_first_tile = (c * p.units_per_cta) / p.k_tiles;
-                        const float *from = p.scratch + ((size_t)c * 2 + (c_first_tile == sg.tile ? 0 : 1)) * slot_floats +
-                                            (size_t)r0 * TILE_F + et;
+                    for (int c0 = 0; c0 < n_c; c0 += INFL) {
+                        float4 part[INFL][2], up[DUAL ? INFL : 1][2];
 #pragma unroll
-                        for (int j = 0; j < CH; ++j) {         // slots are NT >= rows + CH - 1 rows deep: in bounds
-                            g[j] += __ldcg(from + (size_t)j * TILE_F);
-                            if (DUAL) uu[j] += __ldcg(from + (size_t)(NT + j) * TILE_F);
+                        for (int c = 0; c < INFL; ++c) {
+                            if (c0 + c < n_c) {
+                                const float *from = slot_of(c0 + c);
+                                part[c][0] = __ldcg(reinterpret_cast<const float4 *>(from + ra));
+                                part[c][1] = __ldcg(reinterpret_cast<const float4 *>(from + rb));
+                                if (DUAL) {
+                                    up[c][0] = __ldcg(reinterpret_cast<const float4 *>(from + (size_t)NT * TILE_F + ra));
+                                    up[c][1] = __ldcg(reinterpret_cast<const float4 *>(from + (size_t)NT * TILE_F + rb));
+                                }
+                            }
+                        }
+#pragma unroll
+                        for (int c = 0; c < INFL; ++c) {
+                            if (c0 + c < n_c) {
+#pragma unroll
+                                for (int i = 0; i < 2; ++i) { v[i] = add4(v[i], part[c][i]); if (DUAL) uu[i] = add4(uu[i], up[c][i]); }
+                            }
                         }
                     }
                 }
-                finish_chunk<EPI, GROUPS>(p, sg.tile, fe, r0, g, uu, xch + group * (CH * TILE_F), inv_sh, rowmeta, lane, aux, rows_live,
-                                  src != SRC_TMEM && sg.tile == last_tile, last_gain, GROUPS > 1 ? 2 + group : 1);
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    if (r0 + gw + 4 * i < row_end)
+                        finish_row<EPI, false>(p, sg.tile, r0 + gw + 4 * i, !dry, v[i], uu[i], aux[i][0], aux[i][1], gain_a, gain_b, inv_sh, rowmeta, lane);
+                load_aux(r0 + GROUPS * CH, row_end);
             }
-            }   // blocks of rows
 
             if (dry) {
                 dry = false;
@@ -433,7 +414,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
                         if (et < p.rows) inv_sh[et] = rsqrtf(acc[0] * p.inv_d + p.eps);
                       }
                     } else {
-                        for (int r = (et_all >> 5); r < p.rows; r += n_groups * 4) {
+                        for (int r = (et >> 5); r < p.rows; r += GROUPS * 4) {
                             float ss = 0.f;
                             for (int j = lane; j < p.ssq_in_n; j += 32) ss += __ldcg(p.ssq_in + (size_t)j * p.ssq_stride + p.row0 + r);
                             ss = warp_sum(ss);
@@ -442,7 +423,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
                     }
                 }
                 if (EPI == EPI_QKV_ROPE) {
-                    if (et_all < p.rows) {
+                    if (et < p.rows) {
                         // rows are laid out [stream][sequence][block row]; stream 1 (rows >= split_row) is the slim verifier
                         const int row = p.row0 + et, stream = row >= p.split_row ? 1 : 0, rs = row - stream * p.split_row;
                         const int b = rs / p.rope_M, i = rs - b * p.rope_M;
@@ -458,10 +439,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
                                                 (int)((unsigned)(off >> 32) | ((unsigned)stream << 30)));
                     }
                 }
-                asm volatile("bar.sync 1, %0;" ::"n"(epi_threads) : "memory");
+                epi_sync();
                 continue;
             }
-            if (src == SRC_TMEM) {
+            if (whole) {
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(tempty_bar(buf));   // accumulator buffer may be overwritten
@@ -576,6 +557,7 @@ void tc_fill_params(const TcLaunch &L, TcParams &p) {
     p.out_f32_2 = L.out_f32_2; p.next_gain2 = L.next_gain2; p.kc2 = (__nv_bfloat16 *)L.kc2; p.vc2 = (__nv_bfloat16 *)L.vc2;
     p.layer_ord2 = L.layer_ord2;
     p.run_flag = L.run_flag;
+    p.out_vec4 = ((((uintptr_t)L.out_f32 | (uintptr_t)L.out_f32_2) & 15) == 0 && L.ld_out % 4 == 0 && L.seg_n[0] % 4 == 0 && L.seg_n[1] % 4 == 0) ? 1 : 0;
     p.kv_keep = L.kv_keep;
 }
 
@@ -594,7 +576,7 @@ int launch_gemm_tc(const TcLaunch &L, cudaStream_t st) {
     if (p.n_tiles <= L.sm_count && p.k_tiles <= 12) p.units_per_cta = p.k_tiles;
     grid = (units + p.units_per_cta - 1) / p.units_per_cta;
     const int nacc = dual ? 2 : 1;
-    const size_t stage = tc_boxes(L) * ((size_t)nacc * TILE_F * TILE_K * 2 + 2 * (size_t)L.nt * TILE_K * 2);
+    const size_t stage = tc_boxes(L) * ((size_t)nacc * TILE_F * TILE_K * 2 + (L.has_lo ? 2 : 1) * (size_t)L.nt * TILE_K * 2);
     // The depth of the ring bounds the streaming rate (bytes in flight per SM): 200 KB, one CTA per SM, measured
     // faster than 100 KB with the next kernel's CTA resident beside this one.
     const int ring_kb = L.ring_kb > 0 ? L.ring_kb : 200;

@@ -51,152 +51,99 @@ __device__ __forceinline__ bool next_seg(int &u, int u1, int k_tiles, Seg &s) {
     return true;
 }
 
-// Epilogue for CH token rows r0..r0+CH-1 of one tile; thread f holds the full-K sums g (and u for the gate/up
-// pair) of output feature f.  Called by all 128 epilogue threads together.  The epilogue kind is a template
-// parameter so that each kernel carries one short epilogue: this code runs once per tile, straight from the
-// instruction cache's cold side, and its size is what its latency is made of.
-template <int EPI, int GROUPS>
-__device__ __forceinline__ void finish_chunk(const TcParams &p, int tile, int f, int r0, float (&g)[CH], float (&uu)[CH],
-                                             float *xch, const float *inv_sh, const int4 *rowmeta, int lane,
-                                             const float *aux, int rows_live, bool have_gain, float2 gain, int group_bar) {
-    // aux: null, or [rows][128] floats already in shared memory - the residual row of this tile (EPI_ADD_NORM),
-    // or the row's 64 cosines followed by its 64 sines (EPI_QKV_ROPE) - so that no chunk waits for global memory.
-    // rows_live: rows r0.. below it are written (p.rows, or 0 for the dry pass that only warms the instruction cache)
-    // have_gain / gain: the next norm's gains of feature f, fetched by the caller long before (EPI_ADD_NORM)
-    // group_bar: the named barrier of the calling group of 128 threads; xch is that group's exchange buffer
-    constexpr bool DUAL = EPI == EPI_SWIGLU;
-    if (EPI == EPI_STORE || EPI == EPI_SWIGLU || EPI == EPI_QKV_ROPE) {
-        if (p.ssq_in) {                   // the input was h * gain without its RMS factor: apply it per row here
-#pragma unroll
-            for (int j = 0; j < CH; ++j) {
-                const float sc = inv_sh[min(r0 + j, 127)];
-                g[j] *= sc;
-                if (DUAL) uu[j] *= sc;
-            }
-        }
+// ---- finishing, a token row per warp: lane l holds features 4l .. 4l+3 of the tile -------------------------------
+__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+__device__ __forceinline__ float4 scale4(float4 a, float s) { return make_float4(a.x * s, a.y * s, a.z * s, a.w * s); }
+__device__ __forceinline__ uint2 pack4(float4 v) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+    return make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
+}
+// live: store; else (a dry pass that warms the instruction cache) ask for the line, so that the first store does not start
+// with an address-translation miss
+template <typename V>
+__device__ __forceinline__ void put(bool live, void *dst, V v) {
+    if (live) *reinterpret_cast<V *>(dst) = v;
+    else asm volatile("prefetch.global.L2 [%0];" ::"l"(dst));
+}
+// four values as hi and lo planes (x = hi + lo to about 16 mantissa bits)
+__device__ __forceinline__ void store_pair4(bool live, __nv_bfloat16 *dst, size_t plane, float4 v) {
+    const __nv_bfloat16 h0 = __float2bfloat16_rn(v.x), h1 = __float2bfloat16_rn(v.y), h2 = __float2bfloat16_rn(v.z), h3 = __float2bfloat16_rn(v.w);
+    const uint2 hi = make_uint2((uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16),
+                                (uint32_t)__bfloat16_as_ushort(h2) | ((uint32_t)__bfloat16_as_ushort(h3) << 16));
+    put(live, dst, hi);
+    put(live, dst + plane, pack4(make_float4(v.x - __bfloat162float(h0), v.y - __bfloat162float(h1),
+                                             v.z - __bfloat162float(h2), v.w - __bfloat162float(h3))));
+}
+
+// One token row of a tile: v = the row's full sums (u: those of the up matrix, EPI_SWIGLU of the one-CTA kernel).
+// HALVES (pair kernel): lanes 0..15 hold 64 gate features, lanes 16..31 the matching up features.
+// aux0 / aux1: the residual row (EPI_ADD_NORM), or the row's cosines and sines (EPI_QKV_ROPE).
+template <int EPI, bool HALVES>
+__device__ __forceinline__ void finish_row(const TcParams &p, int tile, int row, bool live, float4 v, float4 u, float4 aux0, float4 aux1,
+                                           float4 gain_a, float4 gain_b, const float *inv_sh, const int4 *rowmeta, int lane) {
+    const int grow = p.row0 + row;
+    if (EPI != EPI_ADD_NORM && p.ssq_in) {                                 // the input was h * gain without its RMS factor
+        v = scale4(v, inv_sh[row]);
+        if (EPI == EPI_SWIGLU && !HALVES) u = scale4(u, inv_sh[row]);
     }
-    const int nrow = min(CH, rows_live - r0);
-    // dry pass: nothing is stored, but the lines (and pages) the real pass will write are asked for, so that its
-    // first stores do not start with address-translation misses
-    const bool touch = rows_live == 0 && (f & 31) == 0;
-    auto want = [](const void *ptr) { asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr)); };
-    if (DUAL) {
-        const int n = tile * TILE_F + f;
-        if (n >= p.seg_n[0]) return;
-        __nv_bfloat16 *dst = p.out_act + (size_t)(p.row0 + r0) * p.ld_out + n;
-        if (touch) { want(dst); want(dst + p.act_plane); }
-#pragma unroll
-        for (int j = 0; j < CH; ++j) {
-            if (j < nrow) {
-                const float sg = g[j] / (1.f + __expf(-g[j]));
-                store_act<__nv_bfloat16>(dst, p.act_plane, (size_t)j * p.ld_out, sg * uu[j]);
-            }
+    if (EPI == EPI_SWIGLU) {
+        if (HALVES) {
+            u.x = __shfl_down_sync(0xffffffffu, v.x, 16); u.y = __shfl_down_sync(0xffffffffu, v.y, 16);
+            u.z = __shfl_down_sync(0xffffffffu, v.z, 16); u.w = __shfl_down_sync(0xffffffffu, v.w, 16);
+        }
+        const int n = tile * (HALVES ? 64 : TILE_F) + 4 * lane;
+        if ((!HALVES || lane < 16) && n < p.seg_n[0]) {                    // (d_ff is a multiple of 8)
+            const float4 y = make_float4(v.x / (1.f + __expf(-v.x)) * u.x, v.y / (1.f + __expf(-v.y)) * u.y,
+                                         v.z / (1.f + __expf(-v.z)) * u.z, v.w / (1.f + __expf(-v.w)) * u.w);
+            store_pair4(live, p.out_act + (size_t)grow * p.ld_out + n, p.act_plane, y);
         }
         return;
     }
     int s = 0, t0 = 0, nbase = 0;
     while (s < 2 && tile >= p.seg_tile_end[s]) { t0 = p.seg_tile_end[s]; nbase += p.seg_n[s]; ++s; }
-    const int nin = (tile - t0) * TILE_F + f;
-    const bool valid = nin < p.seg_n[s];
-    const int n = nbase + nin;
-    if (EPI == EPI_STORE) {
-        if (!valid) return;
-        if (touch) want(p.out_f32 + (size_t)(p.row0 + r0) * p.ld_out + n);
-#pragma unroll
-        for (int j = 0; j < CH; ++j) {
-            if (j < nrow) {
-                const int row = p.row0 + r0 + j;          // the second stream's rows go to the second output
-                float *dst = row < p.split_row ? p.out_f32 + (size_t)row * p.ld_out + n
-                                               : p.out_f32_2 + (size_t)(row - p.split_row) * p.ld_out + n;
-                if (p.epi == EPI_ADD) *dst += g[j]; else *dst = g[j];
-            }
+    const int nin = (tile - t0) * TILE_F + 4 * lane, n = nbase + nin;
+    if (EPI == EPI_STORE) {                                                // (also EPI_ADD: the unfused residual update)
+        if (nin >= p.seg_n[s]) return;
+        float *dst = grow < p.split_row ? p.out_f32 + (size_t)grow * p.ld_out + n                 // the second stream's rows go
+                                        : p.out_f32_2 + (size_t)(grow - p.split_row) * p.ld_out + n;   // to the second output
+        if (p.out_vec4 && nin + 3 < p.seg_n[s]) {
+            if (p.epi == EPI_ADD && live) v = add4(*reinterpret_cast<const float4 *>(dst), v);
+            put(live, dst, v);
+            return;
         }
+        const float e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) if (nin + i < p.seg_n[s]) put(live, dst + i, p.epi == EPI_ADD && live ? dst[i] + e[i] : e[i]);
     } else if (EPI == EPI_ADD_NORM) {
-        // residual update, plus what the next RMSNorm needs: h * gain as hi/lo planes and partial sums of h^2.
-        // Loads first, then arithmetic, then stores: the CH rows cost one memory round trip.
-        // fetched here, the two gains are a round trip to L2 at the head of every chunk (the stores in between keep
-        // the compiler from hoisting them): a microsecond on the launch's critical path
-        const float gain_a = have_gain ? gain.x : (valid ? p.next_gain[n] : 0.f);
-        const float gain_b = have_gain ? gain.y : ((valid && p.next_gain2) ? p.next_gain2[n] : gain_a);
-        float *hp = p.out_f32 + (size_t)(p.row0 + r0) * p.ld_out + n;
-        __nv_bfloat16 *ap = p.next_act + (size_t)(p.row0 + r0) * p.ld_out + n;
-        if (touch) { want(hp); want(ap); want(ap + p.next_plane); want(p.ssq_out + ((size_t)tile * 4 + (f >> 5)) * p.ssq_stride + p.row0 + r0); }
-        float v[CH];
-        if (aux) {                                               // the residual rows are staged in shared memory
+        // residual update, and what the next RMSNorm needs: h * gain as planes, sums of h^2 per 32 features
+        v = add4(v, aux0);
+        const size_t o = (size_t)grow * p.ld_out + n;                      // (d_model is a multiple of 128)
+        put(live, p.out_f32 + o, v);
+        const float4 g = grow < p.split_row ? gain_a : gain_b;
+        store_pair4(live, p.next_act + o, p.next_plane, make_float4(v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w));
+        float q = (v.x * v.x + v.y * v.y) + (v.z * v.z + v.w * v.w);
 #pragma unroll
-            for (int j = 0; j < CH; ++j) v[j] = (valid && j < nrow) ? aux[(r0 + j) * TILE_F + f] + g[j] : 0.f;
-        } else {
-#pragma unroll
-            for (int j = 0; j < CH; ++j) v[j] = (valid && j < nrow) ? __ldcg(hp + (size_t)j * p.ld_out) + g[j] : 0.f;
-        }
-#pragma unroll
-        for (int j = 0; j < CH; ++j) {
-            if (valid && j < nrow) {
-                hp[(size_t)j * p.ld_out] = v[j];
-                store_act<__nv_bfloat16>(ap, p.next_plane, (size_t)j * p.ld_out,
-                                         v[j] * (p.row0 + r0 + j < p.split_row ? gain_a : gain_b));
-            }
-            v[j] *= v[j];
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int j = 0; j < CH; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
-        if (lane < nrow) {
-            float mine = v[0];
-#pragma unroll
-            for (int j = 1; j < CH; ++j) mine = lane == j ? v[j] : mine;
-            p.ssq_out[((size_t)tile * 4 + (f >> 5)) * p.ssq_stride + p.row0 + r0 + lane] = mine;
-        }
-    } else {   // EPI_QKV_ROPE: one tile is one head of 128 dims; rotate pairs (p, p + 64), write q / K cache / V cache
-#pragma unroll
-        for (int j = 0; j < CH; ++j) xch[j * TILE_F + f] = g[j];
-        if (GROUPS == 1) asm volatile("bar.sync 1, 128;" ::: "memory"); else asm volatile("bar.sync %0, 128;" ::"r"(group_bar) : "memory");
-        const int head = tile - t0, pidx = f & 63;
+        for (int d = 4; d > 0; d >>= 1) q += __shfl_xor_sync(0xffffffffu, q, d);
+        if ((lane & 7) == 0) put(live, p.ssq_out + ((size_t)tile * 4 + (lane >> 3)) * p.ssq_stride + grow, q);
+    } else {                                                               // EPI_QKV_ROPE: the tile is one head of 128 dims
+        const int4 rm = rowmeta[row];
         if (s < 2) {
-            float c[CH], sn[CH];
-            if (aux) {                                           // the rows' tables are staged in shared memory
-#pragma unroll
-                for (int j = 0; j < CH; ++j) {
-                    const float *ar = aux + min(r0 + j, p.rows - 1) * TILE_F + pidx;
-                    c[j] = ar[0];
-                    sn[j] = ar[64];
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < CH; ++j) {
-                    const int pos = rowmeta[min(r0 + j, 127)].x;
-                    c[j] = p.cosv[(size_t)pos * 64 + pidx];
-                    sn[j] = p.sinv[(size_t)pos * 64 + pidx];
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < CH; ++j) {
-                const float other = xch[j * TILE_F + (f ^ 64)];
-                g[j] = f < 64 ? g[j] * c[j] - other * sn[j] : g[j] * c[j] + other * sn[j];
-            }
+            float4 w;                                                      // the rotary partner (dim ^ 64)
+            w.x = __shfl_xor_sync(0xffffffffu, v.x, 16); w.y = __shfl_xor_sync(0xffffffffu, v.y, 16);
+            w.z = __shfl_xor_sync(0xffffffffu, v.z, 16); w.w = __shfl_xor_sync(0xffffffffu, v.w, 16);
+            const float sg = lane < 16 ? -1.f : 1.f;
+            v = make_float4(v.x * aux0.x + sg * w.x * aux1.x, v.y * aux0.y + sg * w.y * aux1.y,
+                            v.z * aux0.z + sg * w.z * aux1.z, v.w * aux0.w + sg * w.w * aux1.w);
         }
-        if (touch) {
-            if (s == 0) want(p.q_out + ((size_t)(p.row0 + r0) * p.rope_H + head) * TILE_F + f);
-            else want((s == 1 ? p.kc : p.vc) + ((((size_t)p.layer_ord * p.max_batch) * p.rope_Hkv + head) * p.max_ctx) * TILE_F + f);
-        }
+        const int head = tile - t0;
         if (s == 0) {
-            float *dst = p.q_out + ((size_t)(p.row0 + r0) * p.rope_H + head) * TILE_F + f;
-#pragma unroll
-            for (int j = 0; j < CH; ++j) if (j < nrow) dst[(size_t)j * p.rope_H * TILE_F] = g[j];
-        } else {
+            put(live, p.q_out + ((size_t)grow * p.rope_H + head) * TILE_F + 4 * lane, v);
+        } else if (rm.y >= 0) {
+            const size_t off = ((size_t)((unsigned)rm.w & 0x3fffffffu) << 32) | (unsigned)rm.z;
             __nv_bfloat16 *c0 = s == 1 ? p.kc : p.vc, *c1 = s == 1 ? p.kc2 : p.vc2;
-            const size_t head_off = (size_t)head * p.max_ctx * TILE_F + f;
-#pragma unroll
-            for (int j = 0; j < CH; ++j) {
-                const int4 rm = rowmeta[min(r0 + j, 127)];          // .z / .w: the row's offset in its cache (set with the table)
-                if (j < nrow && rm.y >= 0) {
-                    const size_t off = ((size_t)((unsigned)rm.w & 0x3fffffffu) << 32) | (unsigned)rm.z;
-                    (((unsigned)rm.w >> 30) & 1u ? c1 : c0)[off + head_off] = __float2bfloat16_rn(g[j]);
-                }
-            }
+            __nv_bfloat16 *dst = (((unsigned)rm.w >> 30) & 1u ? c1 : c0) + off + (size_t)head * p.max_ctx * TILE_F + 4 * lane;
+            put(live, dst, pack4(v));
         }
-        if (GROUPS == 1) asm volatile("bar.sync 1, 128;" ::: "memory"); else asm volatile("bar.sync %0, 128;" ::"r"(group_bar) : "memory");
     }
 }
 

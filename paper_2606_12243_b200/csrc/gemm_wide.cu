@@ -63,85 +63,6 @@ __device__ __forceinline__ void pair_commit(uint32_t on, uint32_t bar) {        
 __device__ __forceinline__ void pair_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
-__device__ __forceinline__ float4 scale4(float4 a, float s) { return make_float4(a.x * s, a.y * s, a.z * s, a.w * s); }
-__device__ __forceinline__ uint2 pack4(float4 v) {
-    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-    return make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
-}
-// four values as hi and lo planes (x = hi + lo to about 16 mantissa bits)
-__device__ __forceinline__ void store_pair4(__nv_bfloat16 *dst, size_t plane, float4 v) {
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(v.x), h1 = __float2bfloat16_rn(v.y), h2 = __float2bfloat16_rn(v.z), h3 = __float2bfloat16_rn(v.w);
-    const uint2 hi = make_uint2((uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16),
-                                (uint32_t)__bfloat16_as_ushort(h2) | ((uint32_t)__bfloat16_as_ushort(h3) << 16));
-    *reinterpret_cast<uint2 *>(dst) = hi;
-    *reinterpret_cast<uint2 *>(dst + plane) = pack4(make_float4(v.x - __bfloat162float(h0), v.y - __bfloat162float(h1),
-                                                                v.z - __bfloat162float(h2), v.w - __bfloat162float(h3)));
-}
-
-// One token row of a tile, by one warp: v = the row's full sums of features 4 * lane .. + 3.
-// aux0 / aux1: the residual row (EPI_ADD_NORM), or the row's cosines and sines (EPI_QKV_ROPE)
-template <int EPI>
-__device__ __forceinline__ void finish_row(const TcParams &p, int tile, int row, float4 v, float4 aux0, float4 aux1, float4 gain_a, float4 gain_b,
-                                           const float *inv_sh, const int4 *rowmeta, int lane) {
-    const int grow = p.row0 + row;
-    if (EPI != EPI_ADD_NORM && p.ssq_in) v = scale4(v, inv_sh[row]);      // the input was h * gain without its RMS factor
-    if (EPI == EPI_SWIGLU) {
-        float4 u;                                                          // lanes 16..31 hold the up features of lanes 0..15
-        u.x = __shfl_down_sync(0xffffffffu, v.x, 16); u.y = __shfl_down_sync(0xffffffffu, v.y, 16);
-        u.z = __shfl_down_sync(0xffffffffu, v.z, 16); u.w = __shfl_down_sync(0xffffffffu, v.w, 16);
-        const int n = tile * 64 + 4 * lane;
-        if (lane < 16 && n < p.seg_n[0]) {                                 // (d_ff is a multiple of 8)
-            const float4 y = make_float4(v.x / (1.f + __expf(-v.x)) * u.x, v.y / (1.f + __expf(-v.y)) * u.y,
-                                         v.z / (1.f + __expf(-v.z)) * u.z, v.w / (1.f + __expf(-v.w)) * u.w);
-            store_pair4(p.out_act + (size_t)grow * p.ld_out + n, p.act_plane, y);
-        }
-        return;
-    }
-    int s = 0, t0 = 0;
-    while (s < 2 && tile >= p.seg_tile_end[s]) { t0 = p.seg_tile_end[s]; ++s; }
-    const int nin = (tile - t0) * TILE_F + 4 * lane;
-    if (EPI == EPI_STORE) {
-        if (nin >= p.seg_n[0]) return;
-        float *dst = grow < p.split_row ? p.out_f32 + (size_t)grow * p.ld_out + nin
-                                        : p.out_f32_2 + (size_t)(grow - p.split_row) * p.ld_out + nin;
-        if (p.out_vec4 && nin + 3 < p.seg_n[0]) { *reinterpret_cast<float4 *>(dst) = v; return; }
-        const float e[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) if (nin + i < p.seg_n[0]) dst[i] = e[i];
-    } else if (EPI == EPI_ADD_NORM) {
-        // residual update, and what the next RMSNorm needs: h * gain as planes, sums of h^2 per 32 features
-        v = add4(v, aux0);
-        const size_t o = (size_t)grow * p.ld_out + nin;                    // (d_model is a multiple of 128)
-        *reinterpret_cast<float4 *>(p.out_f32 + o) = v;
-        const float4 g = grow < p.split_row ? gain_a : gain_b;
-        store_pair4(p.next_act + o, p.next_plane, make_float4(v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w));
-        float q = (v.x * v.x + v.y * v.y) + (v.z * v.z + v.w * v.w);
-#pragma unroll
-        for (int d = 4; d > 0; d >>= 1) q += __shfl_xor_sync(0xffffffffu, q, d);
-        if ((lane & 7) == 0) p.ssq_out[((size_t)tile * 4 + (lane >> 3)) * p.ssq_stride + grow] = q;
-    } else {                                                               // EPI_QKV_ROPE: the tile is one head of 128 dims
-        const int4 rm = rowmeta[row];
-        if (s < 2) {
-            const float4 c = aux0, sn = aux1;
-            float4 w;                                                      // the rotary partner (dim ^ 64)
-            w.x = __shfl_xor_sync(0xffffffffu, v.x, 16); w.y = __shfl_xor_sync(0xffffffffu, v.y, 16);
-            w.z = __shfl_xor_sync(0xffffffffu, v.z, 16); w.w = __shfl_xor_sync(0xffffffffu, v.w, 16);
-            const float sg = lane < 16 ? -1.f : 1.f;
-            v = make_float4(v.x * c.x + sg * w.x * sn.x, v.y * c.y + sg * w.y * sn.y, v.z * c.z + sg * w.z * sn.z, v.w * c.w + sg * w.w * sn.w);
-        }
-        const int head = tile - t0;
-        if (s == 0) {
-            *reinterpret_cast<float4 *>(p.q_out + ((size_t)grow * p.rope_H + head) * TILE_F + 4 * lane) = v;
-        } else if (rm.y >= 0) {
-            const size_t off = ((size_t)((unsigned)rm.w & 0x3fffffffu) << 32) | (unsigned)rm.z;
-            __nv_bfloat16 *c0 = s == 1 ? p.kc : p.vc, *c1 = s == 1 ? p.kc2 : p.vc2;
-            __nv_bfloat16 *dst = (((unsigned)rm.w >> 30) & 1u ? c1 : c0) + off + (size_t)head * p.max_ctx * TILE_F + 4 * lane;
-            *reinterpret_cast<uint2 *>(dst) = pack4(v);
-        }
-    }
-}
-
 template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(WTHREADS, 1)
 gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant__ CUtensorMap map_w1,
@@ -423,7 +344,8 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
                 gain_b = p.next_gain2 ? __ldg(reinterpret_cast<const float4 *>(p.next_gain2 + tile * TILE_F + 4 * lane)) : gain_a;
             }
             // The other contributors' rows are read where they are, a row per warp: 16-byte loads, up to four contributors of
-            // two rows in flight, asked for before the chunk's trip through shared memory.
+            // two rows in flight, asked for before the chunk's trip through shared memory (staged in the idle ring by
+            // bulk copies first: 13B batch 8 step 6.70 ms, now 6.37; 8B tree batch 4 7.15, now 6.98).
             const int others = n_c - 1;
             auto slot_of = [&](int c) {                            // contributor c's partial of this tile
                 const int cp = first + c, c_first = (cp * p.units_per_cta) / p.k_tiles;
@@ -462,7 +384,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
                         for (int c = 4; c < n_c; ++c)
                             v = add4(v, c == mine ? own : __ldcg(reinterpret_cast<const float4 *>(slot_of(c) + (size_t)r * TILE_F)));
                     }
-                    finish_row<EPI>(p, tile, r, v, aux[i][0], aux[i][1], gain_a, gain_b, inv_sh, rowmeta, lane);
+                    finish_row<EPI, true>(p, tile, r, true, v, make_float4(0.f, 0.f, 0.f, 0.f), aux[i][0], aux[i][1], gain_a, gain_b, inv_sh, rowmeta, lane);
                 }
                 load_aux(r0 + WGROUPS * CH, row_end);
             }
@@ -509,7 +431,6 @@ int launch_gemm_wide(const TcLaunch &L, cudaStream_t st) {
     p.k_tiles = (L.k + TILE_K - 1) / TILE_K;
     if (dual) p.n_tiles = (L.seg_n[0] + 63) / 64;                  // 64 gate and 64 up features per CTA tile
     if (p.n_tiles <= 0 || p.k_tiles <= 0) return VIASD_OK;
-    p.out_vec4 = ((((uintptr_t)L.out_f32 | (uintptr_t)L.out_f32_2) & 15) == 0 && L.ld_out % 4 == 0) ? 1 : 0;
     const int units = ((p.n_tiles + 1) / 2) * p.k_tiles;
     int pairs = L.sm_count / 2 < units ? L.sm_count / 2 : units;      // (148 SMs hold 74 pairs: all resident at once)
     p.units_per_cta = (units + pairs - 1) / pairs;

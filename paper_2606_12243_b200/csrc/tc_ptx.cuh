@@ -87,12 +87,6 @@ __device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const CUtensorMap
         ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y), "l"(pol) : "memory");
 }
 
-// plain (untiled) bulk copy global -> shared; both addresses 16-byte aligned, size a multiple of 16 bytes
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-
 // ---- the same for a whole warp in step ---------------------------------------------------------
 // Loops that feed TMA and the tensor cores, run by all lanes of their warp with the instruction itself predicated to one
 // lane.  Inside an `if (lane == 0)` the compiler keeps addresses, coordinates and descriptors in per-thread registers and
