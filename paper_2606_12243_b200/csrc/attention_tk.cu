@@ -198,7 +198,7 @@ attention_tk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     constexpr uint32_t QCH = (uint32_t)NC * 128u;           // one 64-wide chunk of an [NC rows] operand
     RUN_FLAG_EXIT(a.run_flag);
     PDL_TRIGGER();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int NK = a.nk, NV = a.nv;
     const int HkvV = a.Hkv * a.subs, grp = a.H / HkvV, QR = grp * a.M;   // query heads and rows per item group
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -244,8 +244,8 @@ attention_tk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_base_sh;
-    const int per = per_sh;
+    const uint32_t tmem = uniform(tmem_base_sh);
+    const int per = uniform(per_sh);
 
     if (warp == 0) {
         // ---------------- TMA producer: the CTA's (item, tile) list, flattened ----------------
@@ -328,57 +328,64 @@ attention_tk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NC >> 3) << 17) | ((128u >> 4) << 24);
-            const uint32_t idesc_pv = idesc | (1u << 15);                 // A (the V tile) is MN-major
-            int c_tile = 0, n_q = 0, o_uses = 0, q_be = -1, q_g = -1;   // c_tile: tiles of earlier items (ring and buffer phase)
-            bool ok = true;
-            // tile g (counted over the whole CTA) uses K slot g % NK, V slot g % NV, S^T buffer g & 1 and P^T buffer g & 1
-            auto issue_qk = [&](int g) -> bool {
-                const int st = g % NK, sb = g & 1;
-                if (!mbar_wait(fullk_bar(st), (g / NK) & 1, &abort_sh, a.status)) return false;
-                tc_fence_after();
-                const uint32_t kst = ring + st * (SPLIT ? 1 : 2) * SLOT_BYTES, d = tmem + TM_S + sb * 64;
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NC >> 3) << 17) | ((128u >> 4) << 24);
+        const uint32_t idesc_pv = idesc | (1u << 15);                 // A (the V tile) is MN-major
+        int c_tile = 0, n_q = 0, o_uses = 0, q_be = -1, q_g = -1;   // c_tile: tiles of earlier items (ring and buffer phase)
+        bool ok = true;
+        // tile g (counted over the whole CTA) uses K slot g % NK, V slot g % NV, S^T buffer g & 1 and P^T buffer g & 1
+        int kslot = 0, kphase = 0, vslot = 0, vphase = 0;
+        auto issue_qk = [&](int g) -> bool {
+            const int sb = g & 1;
+            if (!warp_wait(fullk_bar(kslot), kphase, &abort_sh, a.status)) return false;
+            tc_fence_after();
+            if (elect_one()) {
+                const uint64_t kd = smem_desc(ring + kslot * (SPLIT ? 1 : 2) * SLOT_BYTES), qd = smem_desc(qsm);
+                const uint32_t d = tmem + TM_S + sb * 64;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)
-                    tc_mma(d, smem_desc(kst + (ks >> 2) * HALF_BYTES + (ks & 3) * 32), smem_desc(qsm + (ks >> 2) * QCH + (ks & 3) * 32),
-                           idesc, ks > 0 ? 1u : 0u);
-                if (SPLIT) tc_commit(emptyk_bar(st));                     // the K slot is free once these MMAs have read it
+                    tc_mma(d, kd + (ks >> 2) * (HALF_BYTES >> 4) + (ks & 3) * 2, qd + (ks >> 2) * (QCH >> 4) + (ks & 3) * 2, idesc, ks > 0 ? 1u : 0u);
+                if (SPLIT) tc_commit(emptyk_bar(kslot));              // the K slot is free once these MMAs have read it
                 tc_commit(sfull_bar(sb));
-                return true;
-            };
-            ItemSrc src;
-            src_init(a, src);
-            Item it;
-            while (ok && next_item(a, per, src, it)) {
-                if (it.be != q_be || it.g != q_g) {
-                    if (!(ok = mbar_wait(qfull_bar, n_q & 1, &abort_sh, a.status))) break;
-                    ++n_q; q_be = it.be; q_g = it.g;
-                }
-                if (it.n_tiles == 0) continue;
-                // issue order S(0), S(1), O(0), S(2), O(1), ...: S(t + 2) is only issued once the softmax of tile t has
-                // read its buffer (it arrived on p_full(t)), and its completion implies that O(t) has read P^T(t)
-                if (!(ok = issue_qk(c_tile))) break;
-                if (it.n_tiles > 1 && !(ok = issue_qk(c_tile + 1))) break;
-                for (int t = 0; t < it.n_tiles; ++t) {
-                    const int g = c_tile + t, sb = g & 1, st = g % NV;
-                    if (t == 0 && o_uses > 0 && !(ok = mbar_wait(ofree_bar, (o_uses - 1) & 1, &abort_sh, a.status))) break;
-                    if (SPLIT && !(ok = mbar_wait(fullv_bar(st), (g / NV) & 1, &abort_sh, a.status))) break;
-                    if (!(ok = mbar_wait(pfull_bar(sb), (g >> 1) & 1, &abort_sh, a.status))) break;
-                    tc_fence_after();
-                    const uint32_t vst = SPLIT ? ring + (uint32_t)(NK + st) * SLOT_BYTES : ring + (uint32_t)(2 * st + 1) * SLOT_BYTES;
-                    const uint32_t pb = psm + sb * 2 * QCH;
-#pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)                        // 16 keys per step: two 8-key groups of 1024 bytes
-                        tc_mma(tmem + TM_O, smem_desc_mn(vst + kk * 2048, HALF_BYTES, 1024),
-                               smem_desc(pb + (kk >> 2) * QCH + (kk & 3) * 32), idesc_pv, (t > 0 || kk > 0) ? 1u : 0u);
-                    tc_commit(SPLIT ? emptyv_bar(st) : emptyk_bar(st));   // the slot is free once these MMAs have read it
-                    tc_commit(pvdone_bar(sb));
-                    if (t + 2 < it.n_tiles && !(ok = issue_qk(g + 2))) break;
-                }
-                c_tile += it.n_tiles;
-                ++o_uses;
             }
+            __syncwarp();
+            if (++kslot == NK) { kslot = 0; kphase ^= 1; }
+            return true;
+        };
+        ItemSrc src;
+        src_init(a, src);
+        Item it;
+        while (ok && next_item(a, per, src, it)) {
+            const int n = uniform(it.n_tiles);
+            if (it.be != q_be || it.g != q_g) {
+                if (!(ok = warp_wait(qfull_bar, n_q & 1, &abort_sh, a.status))) break;
+                ++n_q; q_be = it.be; q_g = it.g;
+            }
+            if (n == 0) continue;
+            // issue order S(0), S(1), O(0), S(2), O(1), ...: S(t + 2) is only issued once the softmax of tile t has
+            // read its buffer (it arrived on p_full(t)), and its completion implies that O(t) has read P^T(t)
+            if (!(ok = issue_qk(c_tile))) break;
+            if (n > 1 && !(ok = issue_qk(c_tile + 1))) break;
+            for (int t = 0; t < n; ++t) {
+                const int g = c_tile + t, sb = g & 1;
+                if (t == 0 && o_uses > 0 && !(ok = warp_wait(ofree_bar, (o_uses - 1) & 1, &abort_sh, a.status))) break;
+                if (SPLIT && !(ok = warp_wait(fullv_bar(vslot), vphase, &abort_sh, a.status))) break;
+                if (!(ok = warp_wait(pfull_bar(sb), (g >> 1) & 1, &abort_sh, a.status))) break;
+                tc_fence_after();
+                if (elect_one()) {
+                    const uint64_t vd = smem_desc_mn(SPLIT ? ring + (uint32_t)(NK + vslot) * SLOT_BYTES : ring + (uint32_t)(2 * vslot + 1) * SLOT_BYTES, HALF_BYTES, 1024);
+                    const uint64_t pd = smem_desc(psm + sb * 2 * QCH);
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk)                    // 16 keys per step: two 8-key groups of 1024 bytes
+                        tc_mma(tmem + TM_O, vd + kk * (2048 >> 4), pd + (kk >> 2) * (QCH >> 4) + (kk & 3) * 2, idesc_pv, (t > 0 || kk > 0) ? 1u : 0u);
+                    tc_commit(SPLIT ? emptyv_bar(vslot) : emptyk_bar(vslot));   // the slot is free once these MMAs have read it
+                    tc_commit(pvdone_bar(sb));
+                }
+                __syncwarp();
+                if (++vslot == NV) { vslot = 0; vphase ^= 1; }
+                if (t + 2 < n && !(ok = issue_qk(g + 2))) break;
+            }
+            c_tile += n;
+            ++o_uses;
         }
     } else {
         // ---------------- softmax / epilogue (warps 2..5 <-> TMEM lane quarters 2,3,0,1): one thread, one key (later one dim) ----------------

@@ -87,6 +87,21 @@ __device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const CUtensorMap
         ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y), "l"(pol) : "memory");
 }
 
+// ---- single-thread instructions of a warp in step -----------------------------------------------
+// tcgen05.mma and the TMA instructions take their operands from uniform registers.  The compiler only keeps descriptors and
+// addresses there when it can see that the warp is in step and one thread executes them: the branch to the role on a warp
+// number that went through a shuffle, the instructions under elect.sync.  Then an MMA issues every 10 cycles; under
+// `if (lane == 0)` the operands are moved over each time, 48 - 63 cycles per MMA (N = 16: 49 -> 40 cycles per MMA with A in
+// shared memory, 49 -> 11 with A in TMEM; N = 64: 48 -> 47 and 48 -> 33; N = 128: 65 either way, as long as nothing else
+// sits between the MMAs).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
+}
+template <typename T>
+__device__ __forceinline__ T uniform(T x) { return (T)__shfl_sync(0xffffffffu, x, 0); }
+
 // ---- the same for a whole warp in step ---------------------------------------------------------
 // Loops that feed TMA and the tensor cores, run by all lanes of their warp with the instruction itself predicated to one
 // lane.  Inside an `if (lane == 0)` the compiler keeps addresses, coordinates and descriptors in per-thread registers and
