@@ -186,18 +186,17 @@ int attention_nsplit(const viasd_model *m, int batch, int M) {
 // CTAs in equal contiguous shares, each item costs a fixed part (query staging, merge, partial) plus its tiles,
 // and every extra range adds merge work.  Depends on batch, heads and M only, so the one-stream and the two-stream
 // launch cut the keys at the same places and produce the same bits.
-static int mma_nsplit(const viasd_model *m, int batch, int M, int streams, bool tc, int reps, int subs, int tk_rows) {
+static int mma_nsplit(const viasd_model *m, int batch, int M, int streams, int subs, int tk_rows) {
     const viasd_config &c = m->cfg;
     const int base = batch * c.n_kv_heads * subs, sms = m->sm_count;      // subs: items per kv head (keys-on-lanes kernel)
     const int mt = ((c.n_heads / c.n_kv_heads) * M + 15) / 16;
     const int tiles = (c.max_ctx + 127) / 128;
-    int max_s = tiles < 16 / reps ? tiles : 16 / reps;          // the partial buffer holds 16 ranges per (row, head)
-    if (max_s < 1) max_s = 1;
-    // microseconds, roughly: the tcgen05 kernel's tile does not depend on the number of query tiles
+    const int max_s = tiles < 16 ? tiles : 16;                  // the partial buffer holds 16 ranges per (row, head)
+    // microseconds, roughly
     // (keys-on-lanes kernel, measured: a tile costs its softmax chain, 1.1 - 1.8 us with 8 - 32 rows per item, an item
     // 5 - 10 us of query staging, result rows and merge)
-    const double t_tile = tk_rows > 16 ? 1.8 : tk_rows > 8 ? 1.3 : tk_rows > 0 ? 1.1 : tc ? 0.7 : 0.5 + 0.8 * mt;
-    const double t_item = tk_rows > 16 ? 8.0 : tk_rows > 0 ? 5.0 : tc ? 4.0 : 3.0;
+    const double t_tile = tk_rows > 16 ? 1.8 : tk_rows > 8 ? 1.3 : tk_rows > 0 ? 1.1 : 0.5 + 0.8 * mt;
+    const double t_item = tk_rows > 16 ? 8.0 : tk_rows > 0 ? 5.0 : 3.0;
     // One choice for the whole model, whichever call runs (the cuts must not depend on it): the routed layers are
     // charged as two-stream launches, as the verify step runs them, the others as one-stream launches.
     const int n_dual = m->n_routed, n_single = c.n_layers - m->n_routed;
@@ -205,7 +204,7 @@ static int mma_nsplit(const viasd_model *m, int batch, int M, int streams, bool 
     double best_cost = 1e30;
     for (int s = 1; s <= max_s; ++s) {
         const int tpi = ((tiles + s - 1) / s);
-        double cost = 0.15 * s * reps * (n_dual + n_single);
+        double cost = 0.15 * s * (n_dual + n_single);
         for (int st2 = 1; st2 <= 2; ++st2) {
             const int n = base * s * st2, ipc = (n + sms - 1) / sms;
             cost += (st2 == 2 ? n_dual : n_single) * ipc * (tpi * t_tile + t_item);
@@ -213,7 +212,7 @@ static int mma_nsplit(const viasd_model *m, int batch, int M, int streams, bool 
         if (cost < best_cost - 1e-9) { best_cost = cost; best = s; }
     }
     if (m->opt.attn_splits >= 1 && m->opt.attn_splits <= max_s) best = m->opt.attn_splits;
-    size_t per_split = (size_t)streams * batch * c.n_heads * M * (c.head_dim + 2) * sizeof(float) * reps;
+    size_t per_split = (size_t)streams * batch * c.n_heads * M * (c.head_dim + 2) * sizeof(float);
     while (best > 1 && per_split * best > m->ws.part_bytes) --best;
     return best;
 }
@@ -226,25 +225,23 @@ static int mma_attention(viasd_model *m, const void *kc, const void *vc, bool sl
     // tcgen05 with the keys on the lanes (few query rows only).  Default: keys-on-lanes where it applies, else mma.sync.
     const int kind = m->opt.attn_kernel == 1 ? 0 : m->opt.attn_kernel == 2 ? 1 : m->opt.attn_kernel == 3 ? 2 : 3;   // 0 mma, 1 tc, 2 tk, 3 default
     const int QR = (c.n_heads / c.n_kv_heads) * M;
-    // keys-on-lanes pays off when a CTA streams many tiles; with a handful per CTA (one short sequence) the
-    // mma.sync kernel's shorter latency chain wins
-    const long long tiles_total = (long long)streams * batch * c.n_kv_heads * ((c.max_ctx + 127) / 128);
+    // More than 32 query rows per kv head: the rows-on-lanes kernel, whose tile costs the same whatever the rows (per layer,
+    // 32 / 8 heads, against the better of the two others: 36 rows, 1 sequence of 2048 -1.7 us, 16 sequences of 1000 -16 us;
+    // 108 rows, 1 sequence of 100 -2.7 us, of 2048 -5, 4 sequences of 2048 -12, 16 of 1000 -66; at 32 rows and 2048 keys or
+    // more it is 0.6 - 1.5 us behind).  17 - 32 rows: keys-on-lanes, whose MMAs are that much narrower, from one tile per SM
+    // on (24 rows, 1 sequence of 8000 -3.2 us), rows-on-lanes for less (1 sequence of 100: -4.8 us, of 600 -2.2).  Up to 16
+    // rows: mma.sync, whose chain is the shortest for a few tiles, until keys-on-lanes streams 24 tiles per SM (32 kv heads,
+    // 9 rows: 2 sequences of 2048 +6.2 us, 4 of 2048 -3.5, 8 of 1500 -14; 8 kv heads, 16 rows, 8 sequences of 4000: even).
+    // Tiles of both row streams, whichever the launch has: the choice must not depend on it.
+    const long long tiles_two = 2LL * batch * c.n_kv_heads * ((c.max_ctx + 127) / 128);
     const int grp = c.n_heads / c.n_kv_heads, hpi = attention_tk_heads_per_item(grp, M);
     const int subs = hpi ? grp / hpi : 1, QRi = hpi * M;       // keys-on-lanes: items per kv head, query rows per item
-    // (with more than 32 query rows per kv head the mma.sync kernel has one key group per query tile and is bound by
-    // its MMA issue: there the keys-on-lanes kernel wins from two tiles per SM on)
-    // (and with 17 - 32 query rows per kv head, two query tiles for the mma.sync kernel, from one tile per SM on: 32B
-    // shape at batch 1, 264 tiles, attention 1.78 -> 1.61 ms per step)
-    int use = kind == 3 ? (hpi && tiles_total * subs >= (subs > 1 ? 2LL : QRi > 16 ? 1LL : 8LL) * m->sm_count ? 2 : 0) : kind;
+    int use = kind != 3 ? kind : QR > 32 ? 1 : QR > 16 ? (tiles_two >= m->sm_count ? 2 : 1) : tiles_two >= 24LL * m->sm_count ? 2 : 0;
     if (use == 2 && !hpi) use = 0;
-    // more than 128 query rows per kv head are more than the mma.sync kernel's eight query tiles: the rows-on-lanes kernel
-    // takes them in items of at most 128, whose MMAs are then full (8 sequences x 8 kv heads x 256 rows against 1000 keys:
-    // 816 us on the CUDA cores, 55 us)
-    if (use == 0 && QR > 128) use = 1;
-    const int reps = use == 1 ? attention_tc_replicas(QR) : 1;
-    const int nsplit = mma_nsplit(m, batch, M, streams, use != 0, reps, use == 2 ? subs : use == 1 ? attention_tc_items(QR) : 1, use == 2 ? QRi : 0);
-    const int n_part = nsplit * reps;        // key ranges per (row, head) that have to be merged
-    const bool fuse = n_part > 1 && n_part <= 32 && (use == 2 ? QRi : QR) * n_part <= 160 && attention_tc_items(QR) <= VIASD_ATTN_ITEMS_PER_KV_HEAD;
+    if (use == 0 && QR > 128) use = 1;                         // more than the mma.sync kernel's eight query tiles
+    if (use == 1) return launch_attention_tc(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, st);
+    const int nsplit = mma_nsplit(m, batch, M, streams, use == 2 ? subs : 1, use == 2 ? QRi : 0);
+    const bool fuse = nsplit > 1 && (use == 2 ? QRi : QR) * nsplit <= 160;
     int rc;
     if (use == 2) {
         // The keys-on-lanes kernel deals tiles, not key ranges, evenly to the CTAs (nsplit 0) when the partial buffer
@@ -257,11 +254,10 @@ static int mma_attention(viasd_model *m, const void *kc, const void *vc, bool sl
             return launch_attention_tk(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, 0, 1, st);
         rc = launch_attention_tk(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, nsplit, fuse ? 1 : 0, st);
     }
-    else if (use == 1) rc = launch_attention_tc(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, nsplit, fuse ? 1 : 0, st);
     else rc = launch_attention_mma(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, nsplit, fuse ? 1 : 0, st);
-    if (rc || n_part == 1 || fuse) return rc;
+    if (rc || nsplit == 1 || fuse) return rc;
     CUDA_TRY(launch_chained(attention_combine_kernel<__nv_bfloat16, 128>, dim3(streams * batch * M, c.n_heads), 128, st,
-        (__nv_bfloat16 *)m->ws.attn, m->ws.rows_alloc * (size_t)c.n_heads * 128, m->ws.part, M, c.n_heads, n_part, m->run_flag));
+        (__nv_bfloat16 *)m->ws.attn, m->ws.rows_alloc * (size_t)c.n_heads * 128, m->ws.part, M, c.n_heads, nsplit, m->run_flag));
     LAUNCH_CHECK();
     return VIASD_OK;
 }

@@ -1,27 +1,33 @@
-// Block attention on the 5th-generation tensor cores (tcgen05 + TMEM), bf16 caches, head_dim 128.
+// Block attention on the 5th-generation tensor cores (tcgen05 + TMEM), bf16 caches, head_dim 128: query rows on the lanes.
 //
-// Same work as attention_mma.cu - the M block rows of a sequence (all query heads of one kv head, dealt to items of at
-// most 128 rows: a prompt chunk of 64 rows under 4 query heads per kv head is two) against the committed context plus the block's own rows under the ancestor
-// mask, split over key ranges - but with both contractions on tcgen05:
+// The M block rows of a sequence under all query heads of one kv head (dealt to items of at most 128 rows) against the
+// committed context plus the block's own rows under the ancestor mask:
 //
 //   S[rows, 128 keys] = Q K^T      A = Q (shared memory, K-major, hi and lo planes: two MMAs into one S)
 //                                  B = K tile exactly as its TMA box lands (K-major, 128-byte swizzle)
 //   O[rows, 128 dims] += P V       A = P in TMEM (bf16 pairs, hi and lo planes: two MMAs into one O)
 //                                  B = V tile as it lands, read MN-major (keys are the contraction)
 //
-// One TMEM lane is one query row, so a softmax thread owns a row: row maximum and row sum need no exchange
-// between threads.  With few query rows (<= 32, or <= 64) the rows are staged 4 (or 2) times, once per block of
-// 32 (64) lanes, and replica r looks only at keys [r * 128/R, (r + 1) * 128/R) of every tile: the four softmax
-// warps then share a tile's exponentials instead of one warp doing them all, and each replica ends as a key
-// range of its own (own maximum, sum and O rows) that the range merge adds to the others.  The running maximum is only raised when a tile exceeds it by more than 2^8 (the weights
-// stay below 2^8 otherwise, harmless in fp32), which makes the rescaling of O in TMEM rare.
+// What bounds it: 32 MMAs of 128 x 128 x 16 per tile, about 2300 cycles whatever the rows (so it is for 33 rows and more;
+// fewer go to the kernels that put the keys on the lanes or use mma.sync), and with a few tiles per CTA the chain around
+// them: queries, first S, softmax, last P V, result, merge.
 //
-// Warp roles (192 threads): warp 0 requests K/V tiles by TMA into a ring that runs across the CTA's items,
-// warp 1 owns TMEM and issues the MMAs, warps 2-5 stage Q, run the softmax and write the result.
-// TMEM: two S buffers of 128 columns and O (128).  The softmax overwrites a tile's scores with its weights in
-// place (per 16 keys: 8 columns of bf16 pairs hi, 8 columns lo), so P is double-buffered with S and a tile's
-// softmax does not wait for the previous tile's P V.  MMAs run in issue order, which is what lets Q K^T of tile
-// t + 2 reuse the buffer P V of tile t reads.
+// One TMEM lane is one query row; two warps share a lane quarter and take 64 of a tile's 128 keys each, exchanging row
+// maxima once per tile.  The running maximum only moves when a tile exceeds it by 2^8 (the weights stay below 2^8
+// otherwise, harmless in fp32), which makes the rescaling of O in TMEM rare.  P overwrites S in place (per 16 keys 8
+// columns of bf16 pairs hi, 8 lo), two buffers; MMAs run in issue order, which is what lets Q K^T of tile t + 2 reuse the
+// buffer that P V of tile t reads.  The last tile of a range multiplies only the 16-key groups that it has.
+//
+// Split of the work (chosen by the kernel from the lengths, see the cost below): either every (sequence, kv head, item) pair is
+// cut into k ranges of tiles and the ranges are dealt to the CTAs in equal shares, or the tiles of all pairs laid end to
+// end are cut into one range per CTA and row stream.  The cuts depend on the lengths, the heads and the grid only, so a
+// one-stream and a two-stream launch cut alike and produce the same bits.  A pair that lies in several ranges is finished
+// by all of their CTAs: each publishes its partial rows, goes on with its other items, and at its very end waits (bounded)
+// for the other ranges of each such pair and merges its own slice of the rows, in range order.  All CTAs of a launch are
+// resident together and publish before they wait, so no wait depends on another.
+//
+// Warp roles (320 threads): warp 0 requests K and V tiles by TMA into a ring that runs across the CTA's items, in the
+// order the MMAs use them, warp 1 owns TMEM and issues the MMAs, warps 2-9 stage Q, run the softmax and write the result.
 // Every wait is bounded: on expiry the CTA records VIASD_EDEVICE, lets its copies land and leaves.
 #include "common.cuh"
 #include "tc_ptx.cuh"
@@ -32,56 +38,110 @@ namespace {
 constexpr int HD = 128;                        // head dimension
 constexpr int TKEYS = 128;                     // keys per tile
 constexpr int HALF_BYTES = TKEYS * 128;        // 128 keys x 64 dims of bf16, as one TMA box lands
-constexpr int STAGE_BYTES = 4 * HALF_BYTES;    // K dims 0..63, K dims 64..127, V dims 0..63, V dims 64..127
-constexpr int AT_THREADS = 192;
-constexpr int AT_MAX_STAGE = 3;
-constexpr int ROWF = HD + 2;                   // partial row: 128 numerators, max (natural-log units), sum
+constexpr int SLOT_BYTES = 2 * HALF_BYTES;     // one tile of K or of V: dims 0..63, dims 64..127
+constexpr int SW = 8;                          // softmax warps
+constexpr int AT_THREADS = 64 + SW * 32;
+constexpr int AT_MAX_SLOTS = 6;
+constexpr int PART_ROW = HD + 2;               // floats per partial row: numerators, max (log2 units), sum
+constexpr int QROWS = 128 / SW;                // query rows a warp stages at most
+// costs in tiles (2300 cycles): what an item costs besides its tiles (queries, first and last MMA, result), and a merge
+constexpr int COST_ITEM = 4, COST_MERGE = 3;
+constexpr int MAX_SPLITS = 16, MAX_SLOTS = 32; // ranges of a pair: cut evenly, in any case (a lane each when merged)
 constexpr float RESCALE_GAP = 8.f;             // log2 units
 
 constexpr uint32_t TM_S = 0, TM_O = 256;       // TMEM column offsets: S / P buffers (2 x 128), O (128)
 
 struct AttnTcArgs {
     const float *q;             // [rows, H * HD] rotated queries
-    float *part;                // [b][h][i][split][HD + 2]
+    float *part;                // [pair][slot]: [32 groups of 4 dims][rows8] float4, then [rows8] (max, sum)
     __nv_bfloat16 *out;         // attention output planes (hi, lo)
     size_t out_plane;
     const int *len_eff;
     const TreeInfo *tree;
     int *status;
     const int *run_flag;        // null, or a device flag: the kernel leaves at once when it is zero
-    int M, H, Hkv, max_batch, max_ctx, layer_ord, nsplit;
+    int M, H, Hkv, max_batch, max_ctx, layer_ord;
     int batch, layer_ord2;      // second row stream: rows batch*M.., its own cache and layer ordinal
-    int streams, n_items, items_per_cta, fuse_merge, nstage;
-    int subs, rows_sub;         // items per kv head and the query rows of each (whole rows of 8 but for the last)
-    int qrows8;                 // query rows of an item rounded up to 8
-    int reps, rows_per_rep;     // R replicas of the query rows, 128 / R lanes each
-    uint32_t qoff[4];           // byte offsets of the staged query regions: hi dims 0..63, hi 64..127, lo 0..63, lo 64..127
-    uint32_t q_bytes;           // staged queries in all; the ring follows
-    int *counters;              // arrivals per (stream, sequence, kv head), zero between launches
+    int streams, ring_slots;
+    int subs, rows_sub, rows8;  // items per kv head, query rows of each (but the last), the same rounded up to 8
+    int slots;                  // ranges a pair may be cut into (the partial buffer's slots)
+    int splits;                 // 0, or ranges per pair as asked for by the caller
+    int w_one, w_two;           // the model's layers that run one row stream in a verify step, and those that run both
+    unsigned long long m_recip; // 2^32 / M, rounded up: r / M for the few hundred query rows there are
+    unsigned *counters;         // per pair: arrivals, then finishers; zero between launches
     float scale;                // log2(e) / sqrt(hd)
 };
 
-struct Item { int be, b, g, row0, rows, stream, split, n_ctx, k_begin, k_end, n_tiles, row_base; };   // rows row0 .. of kv head g / subs
+struct Item { int pair, be, b, kvh, row0, rows, stream, split, n_split, n_ctx, k_begin, k_end, n_tiles, row_base; };
 
-__device__ __forceinline__ Item decode_item(const AttnTcArgs &a, int item) {
-    Item it;
-    it.split = item % a.nsplit;
-    const int bg = item / a.nsplit;
-    it.g = bg % (a.Hkv * a.subs);
-    it.be = bg / (a.Hkv * a.subs);
-    it.row0 = (it.g % a.subs) * a.rows_sub;
+// The CTA's work list.  k > 0: its share of the k ranges of every pair; k == 0: its range of `per` tiles of one row stream, or
+// of both in turn.
+struct Cut { int k, per; };
+struct ItemSrc { int s, s_end, range, b, g, off; };             // k > 0: the next item is `off`, the share ends at `range`
+__device__ __forceinline__ void src_init(const AttnTcArgs &a, const Cut &cut, int ranges, ItemSrc &c) {
+    const int x = blockIdx.x;
+    c.b = c.g = c.s = c.s_end = 0;
+    if (cut.k > 0) {
+        c.off = x * cut.per;
+        c.range = min(a.streams * a.batch * a.Hkv * a.subs * cut.k, c.off + cut.per);
+        return;
+    }
+    c.off = 0;
+    if (a.streams * ranges <= (int)gridDim.x) {                // a CTA per range and stream
+        c.s = x / ranges;
+        c.s_end = c.s < a.streams ? c.s + 1 : c.s;
+        c.range = x - c.s * ranges;
+    } else {
+        c.s_end = x < ranges ? a.streams : 0;
+        c.range = x;
+    }
+}
+// range `split` of n_split: tiles t0 .. t1 - 1 of pair (stream s, sequence b, item g of its kv heads)
+__device__ __forceinline__ void set_item(const AttnTcArgs &a, int s, int b, int g, int n_ctx, int t0, int t1, int split, int n_split, Item &it) {
+    it.b = b; it.stream = s; it.be = s * a.batch + b;
+    it.pair = it.be * a.Hkv * a.subs + g; it.kvh = g / a.subs;
+    it.row0 = (g - it.kvh * a.subs) * a.rows_sub;
     it.rows = min(a.rows_sub, a.H / a.Hkv * a.M - it.row0);
-    it.stream = it.be / a.batch;
-    it.b = it.be - it.stream * a.batch;
-    it.n_ctx = a.len_eff[it.b];
-    const int Tk = it.n_ctx + a.M;
-    int chunk = (Tk + a.nsplit - 1) / a.nsplit;
-    chunk = (chunk + TKEYS - 1) / TKEYS * TKEYS;
-    it.k_begin = it.split * chunk;
-    it.k_end = min(Tk, it.k_begin + chunk);
-    it.n_tiles = it.k_end > it.k_begin ? (it.k_end - it.k_begin + TKEYS - 1) / TKEYS : 0;
-    it.row_base = (((it.stream ? a.layer_ord2 : a.layer_ord) * a.max_batch + it.b) * a.Hkv + it.g / a.subs) * a.max_ctx;
-    return it;
+    it.split = split; it.n_split = n_split;
+    it.n_ctx = n_ctx; it.k_begin = t0 * TKEYS; it.k_end = min(n_ctx + a.M, t1 * TKEYS); it.n_tiles = t1 - t0;
+    it.row_base = (((s ? a.layer_ord2 : a.layer_ord) * a.max_batch + b) * a.Hkv + it.kvh) * a.max_ctx;
+}
+__device__ __forceinline__ bool next_item(const AttnTcArgs &a, const Cut &cut, ItemSrc &c, Item &it) {
+    const int Hs = a.Hkv * a.subs;
+    if (cut.k > 0) {
+        while (c.off < c.range) {
+            const int id = c.off++, bg = id / cut.k, split = id - bg * cut.k, be = bg / Hs, s = be / a.batch, b = be - s * a.batch;
+            const int n_ctx = a.len_eff[b], tb = (n_ctx + a.M + TKEYS - 1) / TKEYS, n_split = min(cut.k, tb);
+            if (split >= n_split) continue;                                                   // a short sequence has fewer ranges
+            set_item(a, s, b, bg - be * Hs, n_ctx, split * tb / n_split, (split + 1) * tb / n_split, split, n_split, it);
+            return true;
+        }
+        return false;
+    }
+    const int per = cut.per, lo = c.range * per, hi = lo + per;
+    while (c.s < c.s_end) {
+        if (c.b >= a.batch || c.off >= hi) { ++c.s; c.b = c.g = c.off = 0; continue; }      // done with this stream
+        const int n_ctx = a.len_eff[c.b], tb = (n_ctx + a.M + TKEYS - 1) / TKEYS;
+        if (c.off + Hs * tb <= lo) { c.off += Hs * tb; ++c.b; c.g = 0; continue; }            // this sequence ends before the range
+        if (c.g == 0 && c.off < lo) c.g = (lo - c.off) / tb;                                  // its first pair that reaches into the range
+        const int p_lo = c.off + c.g * tb, p_hi = p_lo + tb;
+        if (c.g >= Hs) { c.off += Hs * tb; ++c.b; c.g = 0; continue; }
+        if (p_lo >= hi) { ++c.s; c.b = c.g = c.off = 0; continue; }
+        const int first = p_lo / per, last = (p_hi - 1) / per;
+        set_item(a, c.s, c.b, c.g, n_ctx, max(lo, p_lo) - p_lo, min(hi, p_hi) - p_lo, c.range - first, last - first + 1, it);
+        ++c.g;
+        return true;
+    }
+    return false;
+}
+// The j-th of an item's 2 n requests, in the order the MMAs take them: K0 K1 V0 K2 V1 ... K(n-1) V(n-2) V(n-1)
+__device__ __forceinline__ int request_tile(int j, int n, bool &is_v) {
+    is_v = false;
+    if (j == 0) return 0;
+    if (j == 1) { is_v = n == 1; return n == 1 ? 0 : 1; }
+    if ((j & 1) && (j + 1) / 2 < n) return (j + 1) / 2;
+    is_v = true;
+    return (j & 1) ? n - 1 : (j - 2) / 2;
 }
 
 __device__ __forceinline__ float ex2(float x) {            // 2^x, hardware approximation (2 ulp)
@@ -118,21 +178,13 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
           "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
           "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
           "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-          "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
     asm volatile(
@@ -144,13 +196,6 @@ __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32])
           "r"(r[30]), "r"(r[31])
         : "memory");
 }
-__device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
-        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-          "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-        : "memory");
-}
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 
@@ -158,37 +203,68 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
 attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ CUtensorMap map_k2, const __grid_constant__ CUtensorMap map_v2, const AttnTcArgs a) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) unsigned long long bars[2 * AT_MAX_STAGE + 9];
+    __shared__ __align__(8) unsigned long long bars[2 * AT_MAX_SLOTS + 12];
     __shared__ uint32_t tmem_base_sh;
-    __shared__ int abort_sh, last_sh;
+    __shared__ int abort_sh, k_sh, per_sh, ranges_sh;
+    __shared__ float xch_sh[2][2][128];                 // exchange between the two warps of a lane quarter: [parity][half][row]
 
     RUN_FLAG_EXIT(a.run_flag);
     PDL_TRIGGER();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int NSTAGE = a.nstage;
-    const int grp = a.H / a.Hkv;
-    // staged queries first (the MMA reads 128 rows from each chunk: what lies behind the live rows is the ring)
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t qsm = base, ring = base + a.q_bytes;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int NS = a.ring_slots, grp = a.H / a.Hkv;
+    // staged queries first (the MMA reads 128 rows from each 64-dim chunk: what lies behind the live rows is the ring)
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, qchunk = (uint32_t)a.rows8 * 128u;
+    const uint32_t qsm = base, ring = base + 4 * qchunk;
     uint8_t *q_gen = smem_raw + (base - smem_u32(smem_raw));
     auto full_bar = [&](int s) { return smem_u32(&bars[s]); };
-    auto empty_bar = [&](int s) { return smem_u32(&bars[AT_MAX_STAGE + s]); };
-    auto sfull_bar = [&](int b) { return smem_u32(&bars[2 * AT_MAX_STAGE + b]); };
-    auto pfull_bar = [&](int b) { return smem_u32(&bars[2 * AT_MAX_STAGE + 2 + b]); };
-    auto pvdone_bar = [&](int b) { return smem_u32(&bars[2 * AT_MAX_STAGE + 4 + b]); };
-    const uint32_t ofree_bar = smem_u32(&bars[2 * AT_MAX_STAGE + 6]), qfull_bar = smem_u32(&bars[2 * AT_MAX_STAGE + 7]);
-    const uint32_t wg_bar = smem_u32(&bars[2 * AT_MAX_STAGE + 8]);      // the softmax warps among themselves (bounded, unlike bar.sync)
+    auto empty_bar = [&](int s) { return smem_u32(&bars[AT_MAX_SLOTS + s]); };
+    auto sfull_bar = [&](int b) { return smem_u32(&bars[2 * AT_MAX_SLOTS + b]); };
+    auto pfull_bar = [&](int b) { return smem_u32(&bars[2 * AT_MAX_SLOTS + 2 + b]); };
+    auto pvdone_bar = [&](int b) { return smem_u32(&bars[2 * AT_MAX_SLOTS + 4 + b]); };
+    auto pair_bar = [&](int qt) { return smem_u32(&bars[2 * AT_MAX_SLOTS + 6 + qt]); };
+    const uint32_t qfull_bar = smem_u32(&bars[2 * AT_MAX_SLOTS + 10]);
+    const uint32_t wg_bar = smem_u32(&bars[2 * AT_MAX_SLOTS + 11]);      // the softmax warps among themselves (bounded, unlike bar.sync)
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < NSTAGE; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(sfull_bar(b), 1); mbar_init(pfull_bar(b), 4); mbar_init(pvdone_bar(b), 1); }
-        mbar_init(ofree_bar, 4);
-        mbar_init(qfull_bar, 4);
-        mbar_init(wg_bar, 128);
+        for (int s = 0; s < NS; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(sfull_bar(b), 1); mbar_init(pfull_bar(b), SW); mbar_init(pvdone_bar(b), 1); }
+        for (int qt = 0; qt < 4; ++qt) mbar_init(pair_bar(qt), 2);
+        mbar_init(qfull_bar, SW);
+        mbar_init(wg_bar, SW);
         abort_sh = 0;
-        last_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 2) {
+        // The cut: a lane per candidate k, and the even cut on the last lane.  Costs are summed over one-stream and two-stream
+        // layers, as the model has them, so that both kinds of launch choose alike.  (Per pair: 8 kv heads of one sequence, 17
+        // tiles each: 9 ranges; 32 pairs: 4; 128 pairs on 148 CTAs: whole pairs, where an even cut would have two items and a
+        // merge per CTA.  Even: 160 pairs of 65 tiles.)
+        int T = 0, tmax = 1;
+        for (int b = lane; b < a.batch; b += 32) {
+            const int tb = (a.len_eff[b] + a.M + TKEYS - 1) / TKEYS;
+            T += tb;
+            tmax = max(tmax, tb);
+        }
+        T = __reduce_add_sync(0xffffffffu, T) * a.Hkv * a.subs;
+        tmax = __reduce_max_sync(0xffffffffu, tmax);
+        const int G = gridDim.x, P = a.batch * a.Hkv * a.subs, kmax = max(1, min(MAX_SPLITS, a.slots)), k = lane + 1;
+        // even cut: no pair in more ranges than it has slots
+        const int per = a.slots < 2 ? T : max((T + G - 1) / G, (tmax + a.slots - 2) / (a.slots - 1)), ranges = (T + per - 1) / per;
+        int cost = 1 << 26;
+        if (k <= kmax && (a.splits == 0 || k == min(a.splits, kmax))) {
+            const int item = (tmax + k - 1) / k + COST_ITEM, merge = k > 1 ? COST_MERGE : 0;
+            cost = a.w_one * ((P * k + G - 1) / G * item + merge) + a.w_two * ((2 * P * k + G - 1) / G * item + merge);
+        } else if (lane == 31 && a.splits == 0 && a.slots >= 2) {
+            const int share = per + 2 * COST_ITEM;
+            cost = a.w_one * (share + COST_MERGE) + a.w_two * ((2 * ranges <= G ? share : 2 * share) + COST_MERGE);
+        }
+        const unsigned best = __reduce_min_sync(0xffffffffu, ((unsigned)min(cost, 1 << 26) << 5) + lane) & 31u;
+        if (lane == 0) {
+            k_sh = best == 31 ? 0 : best + 1;
+            per_sh = best == 31 ? per : (a.streams * P * ((int)best + 1) + G - 1) / G;
+            ranges_sh = ranges;
+        }
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_sh)), "r"(512) : "memory");
@@ -197,253 +273,256 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_base_sh;
-    const int i0 = blockIdx.x * a.items_per_cta, i1 = min(a.n_items, i0 + a.items_per_cta);
+    const uint32_t tmem = uniform(tmem_base_sh);
+    const Cut cut{uniform(k_sh), uniform(per_sh)};
+    const int ranges = uniform(ranges_sh);
+    ItemSrc src;
+    src_init(a, cut, ranges, src);
+    Item it;
 
     if (warp == 0) {
-        // ---------------- TMA producer: the CTA's (item, tile) list, flattened ----------------
+        // ---------------- TMA producer: the CTA's requests, item after item ----------------
         if (lane == 0) {
             const uint64_t kvpol = l2_evict_first_policy();    // the cache passes through once per layer
-            int p_item = i0, p_tile = 0, p_count = 0;
-            bool ok = true;
-            Item pit = i0 < i1 ? decode_item(a, i0) : Item{};
+            int j = 0, count = 0;
+            bool ok = true, more = next_item(a, cut, src, it);
             auto issue_next = [&](bool context_only) -> bool {  // false: nothing (more) to request under this condition
-                while (p_item < i1 && p_tile >= pit.n_tiles) { ++p_item; p_tile = 0; if (p_item < i1) pit = decode_item(a, p_item); }
-                if (p_item >= i1) return false;
-                const int k0 = pit.k_begin + p_tile * TKEYS;
-                if (context_only && k0 + TKEYS > pit.n_ctx) return false;   // this tile holds rows the previous kernel writes
-                const int st = p_count % NSTAGE;
-                if (p_count >= NSTAGE && !(ok = mbar_wait(empty_bar(st), ((p_count / NSTAGE) & 1) ^ 1, &abort_sh, a.status))) return false;
-                const uint32_t bar = full_bar(st), dst = ring + st * STAGE_BYTES;
-                const CUtensorMap *mk = pit.stream ? &map_k2 : &map_k, *mv = pit.stream ? &map_v2 : &map_v;
-                const int y = pit.row_base + k0;
-                mbar_expect_tx(bar, STAGE_BYTES);
-                tma_load_2d_hint(dst, mk, bar, 0, y, kvpol);
-                tma_load_2d_hint(dst + HALF_BYTES, mk, bar, 64, y, kvpol);
-                tma_load_2d_hint(dst + 2 * HALF_BYTES, mv, bar, 0, y, kvpol);
-                tma_load_2d_hint(dst + 3 * HALF_BYTES, mv, bar, 64, y, kvpol);
-                ++p_tile; ++p_count;
+                if (more && j >= 2 * it.n_tiles) { j = 0; more = next_item(a, cut, src, it); }
+                if (!more) return false;
+                bool is_v;
+                const int k0 = it.k_begin + request_tile(j, it.n_tiles, is_v) * TKEYS;
+                if (context_only && k0 + TKEYS > it.n_ctx) return false;   // this tile holds rows the previous kernel writes
+                const int st = count % NS;
+                if (count >= NS && !(ok = mbar_wait(empty_bar(st), ((count / NS) & 1) ^ 1, &abort_sh, a.status))) return false;
+                const uint32_t dst = ring + st * SLOT_BYTES;
+                const CUtensorMap *mp = is_v ? (it.stream ? &map_v2 : &map_v) : (it.stream ? &map_k2 : &map_k);
+                mbar_expect_tx(full_bar(st), SLOT_BYTES);
+                tma_load_2d_hint(dst, mp, full_bar(st), 0, it.row_base + k0, kvpol);
+                tma_load_2d_hint(dst + HALF_BYTES, mp, full_bar(st), 64, it.row_base + k0, kvpol);
+                ++j; ++count;
                 return true;
             };
             // committed context does not change during the pass: ask for it before waiting for the previous kernel
-            while (p_count < NSTAGE && issue_next(true)) { }
+            while (count < NS && issue_next(true)) { }
             PDL_WAIT();
             while (ok && issue_next(false)) { }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TKEYS >> 3) << 17) | ((128u >> 4) << 24);
-            const uint32_t idesc_pv = idesc | (1u << 16);                 // B (the V tile) is MN-major
-            int c_tile = 0, n_q = 0, o_uses = 0, q_be = -1, q_g = -1;   // c_tile: tiles of earlier items (ring and buffer phase)
-            bool ok = true;
-            // tile g (counted over the whole CTA) uses stage g % NSTAGE and S / P buffer g & 1
-            auto issue_qk = [&](int g) -> bool {
-                const int st = g % NSTAGE, sb = g & 1;
-                if (!mbar_wait(full_bar(st), (g / NSTAGE) & 1, &abort_sh, a.status)) return false;
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);          // without N
+        const uint32_t idesc_pv = idesc | ((uint32_t)(HD >> 3) << 17) | (1u << 16);               // B (the V tile) is MN-major
+        int st = 0, st_ph = 0, s_cnt = 0, n_q = 0;               // ring slot and its phase, tiles of the whole CTA, staged query sets
+        bool ok = true;
+        auto next_slot = [&]() { if (++st == NS) { st = 0; st_ph ^= 1; } };
+        while (ok && next_item(a, cut, src, it)) {
+            const int n = uniform(it.n_tiles), keys = uniform(it.k_end - it.k_begin);
+            auto groups16 = [&](int t) { return (min(TKEYS, keys - t * TKEYS) + 15) >> 4; };   // 16-key groups of tile t
+            auto issue_qk = [&](int t) -> bool {                 // tile t of the item, s_cnt + t of the CTA
+                if (!warp_wait(full_bar(st), st_ph, &abort_sh, a.status)) return false;
                 tc_fence_after();
-                const uint32_t kst = ring + st * STAGE_BYTES, d = tmem + TM_S + sb * 128;
+                if (elect_one()) {
+                    const uint64_t kd = smem_desc(ring + st * SLOT_BYTES), q0 = smem_desc(qsm), q_step = qchunk >> 4;
+                    const uint32_t sb = (s_cnt + t) & 1, d = tmem + TM_S + sb * 128, id = idesc | ((uint32_t)(2 * groups16(t)) << 17);
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint64_t kb = smem_desc(kst + (ks >> 2) * HALF_BYTES + (ks & 3) * 32);
-                    tc_mma(d, smem_desc(qsm + a.qoff[ks >> 2] + (ks & 3) * 32), kb, idesc, ks > 0 ? 1u : 0u);
-                    tc_mma(d, smem_desc(qsm + a.qoff[2 + (ks >> 2)] + (ks & 3) * 32), kb, idesc, 1u);   // lo plane of the queries
+                    for (int ks = 0; ks < 8; ++ks) {
+                        const uint64_t kb = kd + (ks >> 2) * (HALF_BYTES >> 4) + (ks & 3) * 2, qa = q0 + (ks >> 2) * q_step + (ks & 3) * 2;
+                        tc_mma(d, qa, kb, id, ks > 0 ? 1u : 0u);
+                        tc_mma(d, qa + 2 * q_step, kb, id, 1u);          // lo plane of the queries
+                    }
+                    tc_commit(empty_bar(st));
+                    tc_commit(sfull_bar(sb));
                 }
-                tc_commit(sfull_bar(sb));
+                __syncwarp();
+                next_slot();
                 return true;
             };
-            for (int item = i0; item < i1 && ok; ++item) {
-                const Item it = decode_item(a, item);
-                if (it.be != q_be || it.g != q_g) {
-                    if (!(ok = mbar_wait(qfull_bar, n_q & 1, &abort_sh, a.status))) break;
-                    ++n_q; q_be = it.be; q_g = it.g;
-                }
-                if (it.n_tiles == 0) continue;
-                // issue order Q K^T(0), Q K^T(1), P V(0), Q K^T(2), P V(1), ...: Q K^T(t + 2) overwrites the buffer P V(t) reads
-                if (!(ok = issue_qk(c_tile))) break;
-                if (it.n_tiles > 1 && !(ok = issue_qk(c_tile + 1))) break;
-                for (int t = 0; t < it.n_tiles; ++t) {
-                    const int g = c_tile + t, sb = g & 1, st = g % NSTAGE;
-                    if (t == 0 && o_uses > 0 && !(ok = mbar_wait(ofree_bar, (o_uses - 1) & 1, &abort_sh, a.status))) break;
-                    if (!(ok = mbar_wait(pfull_bar(sb), (g >> 1) & 1, &abort_sh, a.status))) break;
-                    tc_fence_after();
-                    const uint32_t vst = ring + st * STAGE_BYTES + 2 * HALF_BYTES, pb = tmem + TM_S + sb * 128;
+            // (staged queries also mean that the previous item's O has been read)
+            if (!(ok = warp_wait(qfull_bar, n_q & 1, &abort_sh, a.status))) break;
+            ++n_q;
+            // issue order Q K^T(0), Q K^T(1), P V(0), Q K^T(2), P V(1), ...: Q K^T(t + 2) overwrites the buffer P V(t) reads
+            if (!(ok = issue_qk(0))) break;
+            if (n > 1 && !(ok = issue_qk(1))) break;
+            for (int t = 0; t < n; ++t) {
+                const int g = s_cnt + t, sb = g & 1;
+                if (!(ok = warp_wait(full_bar(st), st_ph, &abort_sh, a.status))) break;
+                if (!(ok = warp_wait(pfull_bar(sb), (g >> 1) & 1, &abort_sh, a.status))) break;
+                tc_fence_after();
+                if (elect_one()) {
+                    const uint64_t vd = smem_desc_mn(ring + st * SLOT_BYTES, HALF_BYTES, 1024);
+                    const uint32_t pb = tmem + TM_S + sb * 128;
+                    const int nk = groups16(t);
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) {                      // 16 keys per step: two 8-key groups of 1024 bytes
-                        const uint64_t vb = smem_desc_mn(vst + kk * 2048, HALF_BYTES, 1024);
-                        const uint32_t pa = pb + kk * 16;                        // 16 keys: 8 columns hi, 8 columns lo
-                        tc_mma_ts(tmem + TM_O, pa, vb, idesc_pv, (t > 0 || kk > 0) ? 1u : 0u);
-                        tc_mma_ts(tmem + TM_O, pa + 8, vb, idesc_pv, 1u);         // lo plane of the weights
+                    for (int kk = 0; kk < 8; ++kk) {                  // 16 keys per step: two 8-key groups of 1024 bytes
+                        if (kk >= nk) break;
+                        tc_mma_ts(tmem + TM_O, pb + kk * 16, vd + kk * (2048 >> 4), idesc_pv, (t > 0 || kk > 0) ? 1u : 0u);
+                        tc_mma_ts(tmem + TM_O, pb + kk * 16 + 8, vd + kk * (2048 >> 4), idesc_pv, 1u);   // lo plane of the weights
                     }
-                    tc_commit(empty_bar(st));                             // the stage is free once these MMAs have read it
+                    tc_commit(empty_bar(st));                         // the slot is free once these MMAs have read it
                     tc_commit(pvdone_bar(sb));
-                    if (t + 2 < it.n_tiles && !(ok = issue_qk(g + 2))) break;
                 }
-                c_tile += it.n_tiles;
-                ++o_uses;
+                __syncwarp();
+                next_slot();
+                if (t + 2 < n && !(ok = issue_qk(t + 2))) break;
             }
+            s_cnt += n;
         }
     } else {
-        // ---------------- softmax / epilogue (warps 2..5 <-> TMEM lane quarters 2,3,0,1): one thread, one query row ----------------
-        const int quarter = warp & 3, trow = quarter * 32 + lane, et = threadIdx.x - 64;
-        const int rep = trow / a.rows_per_rep, row = trow - rep * a.rows_per_rep;     // replica, query row
-        const int KR = TKEYS / a.reps, key0 = rep * KR;                                // this replica's keys of a tile
+        // ---------------- softmax / result (warps 2..5 and 6..9 <-> TMEM lane quarters 2,3,0,1): one query row, half of the keys ----------------
+        const int quarter = warp & 3, sw = warp - 2, half = sw >> 2, trow = quarter * 32 + lane, et = threadIdx.x - 64;
         const uint32_t tlane = tmem + ((uint32_t)(quarter * 32) << 16);
-        PDL_WAIT();
-        int s_cnt = 0, q_be = -1, q_g = -1, wg_phase = 0;        // s_cnt: tiles this CTA has finished (buffer phase)
-        bool ok = true;
+        const size_t part_floats = (size_t)a.rows8 * PART_ROW;
+        int s_cnt = 0, x_cnt = 0, wg_phase = 0;                  // tiles (buffer phase), exchanges, group barriers
+        bool ok = true, first = true;
         auto wg_sync = [&]() -> bool {
-            mbar_arrive(wg_bar);
-            const bool done = mbar_wait(wg_bar, wg_phase & 1, &abort_sh, a.status);
-            ++wg_phase;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(wg_bar);
+            return warp_wait(wg_bar, wg_phase++ & 1, &abort_sh, a.status);
+        };
+        // the other half's value for this row (both warps of the lane quarter call it together)
+        auto exchange = [&](float mine, float &other) -> bool {
+            const int p = x_cnt & 1;
+            xch_sh[p][half][trow] = mine;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(pair_bar(quarter));
+            const bool done = warp_wait(pair_bar(quarter), p, &abort_sh, a.status);
+            other = xch_sh[p][half ^ 1][trow];
+            ++x_cnt;
             return done;
         };
-        for (int item = i0; item < i1 && ok; ++item) {
-            const Item it = decode_item(a, item);
-            if (it.be != q_be || it.g != q_g) {
-                // stage the item's query rows as bf16 hi / lo planes, pre-scaled, in the K-major 128-byte-swizzled layout
-                // the MMA reads; a warp takes whole rows, eight 16-byte loads per thread in flight
-                for (int rb = warp - 2; rb < a.qrows8; rb += 8 * 4) {
-                    float4 v[8];
+        // a query row's place in q and in the output
+        auto row_off = [&](const Item &i, int r) -> size_t {
+            const int g2 = i.row0 + r, hq = (int)((g2 * a.m_recip) >> 32);
+            return ((size_t)(i.be * a.M + g2 - hq * a.M) * a.H + i.kvh * grp + hq) * HD;
+        };
+        while (ok && next_item(a, cut, src, it)) {
+            const bool live = trow < it.rows, warp_live = quarter * 32 < it.rows;
+            const size_t o0 = row_off(it, live ? trow : 0);
+            const int g0 = it.row0 + (live ? trow : 0);
+            const unsigned long long anc = a.tree[it.b].anc[g0 - (int)((g0 * a.m_recip) >> 32) * a.M];
+            // stage the item's query rows as bf16 hi / lo planes, pre-scaled, in the K-major 128-byte-swizzled layout the MMA
+            // reads; a warp takes whole rows, all its loads in flight (addresses first: they do not wait for anything)
+            uint32_t qrow[QROWS];
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const int r = rb + q * 4;
-                        v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (r < it.rows) {
-                            const int gr = it.row0 + r, h = (it.g / a.subs) * grp + gr / a.M, i = gr % a.M;
-                            v[q] = __ldcg(reinterpret_cast<const float4 *>(a.q + ((size_t)(it.be * a.M + i) * a.H + h) * HD + 4 * lane));
-                        }
-                    }
+            for (int q = 0; q < QROWS; ++q) qrow[q] = (uint32_t)(row_off(it, min(sw + q * SW, it.rows - 1)) >> 2) + lane;
+            if (first) PDL_WAIT();
+            else if (!(ok = wg_sync())) break;                   // the rows staged in the query region have been written out
+            first = false;
+            float4 v[QROWS];
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const int r = rb + q * 4, d4 = 4 * lane;
-                        if (r >= a.qrows8) continue;
-                        uint2 hi, lo;
-                        split_pair(v[q].x * a.scale, v[q].y * a.scale, hi.x, lo.x);
-                        split_pair(v[q].z * a.scale, v[q].w * a.scale, hi.y, lo.y);
-                        const int dc = d4 & 63;                                    // dim inside its 64-dim chunk
-                        for (int rp = 0; rp < a.reps; ++rp) {                      // one copy per replica's block of lanes
-                            const uint32_t rr = (uint32_t)(rp * a.rows_per_rep + r);
-                            const uint32_t off = rr * 128u + ((((uint32_t)dc >> 3) ^ (rr & 7u)) << 4) + ((uint32_t)dc & 7u) * 2u;
-                            *reinterpret_cast<uint2 *>(q_gen + a.qoff[d4 >> 6] + off) = hi;
-                            *reinterpret_cast<uint2 *>(q_gen + a.qoff[2 + (d4 >> 6)] + off) = lo;
-                        }
-                    }
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> the MMA's reads
-                __syncwarp();
-                if (lane == 0) mbar_arrive(qfull_bar);
-                q_be = it.be; q_g = it.g;
+            for (int q = 0; q < QROWS; ++q) {
+                v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (sw + q * SW < it.rows) v[q] = __ldcg(reinterpret_cast<const float4 *>(a.q) + qrow[q]);
             }
-            const bool live = row < it.rows, warp_live = (quarter * 32) % a.rows_per_rep < it.rows;
-            const int h = (it.g / a.subs) * grp + (it.row0 + row) / a.M, node = (it.row0 + row) % a.M;
-            const unsigned long long anc = live ? a.tree[it.b].anc[node] : 0ull;
-            float m_run = -INFINITY, l_run = 0.f;
+#pragma unroll
+            for (int q = 0; q < QROWS; ++q) {
+                const uint32_t r = sw + q * SW, d4 = 4 * lane, dc = d4 & 63;       // dc: dim inside its 64-dim chunk
+                if (r >= (uint32_t)a.rows8) break;
+                uint2 hi, lo;
+                split_pair(v[q].x * a.scale, v[q].y * a.scale, hi.x, lo.x);
+                split_pair(v[q].z * a.scale, v[q].w * a.scale, hi.y, lo.y);
+                uint8_t *dst = q_gen + (d4 >> 6) * qchunk + r * 128u + (((dc >> 3) ^ (r & 7u)) << 4) + (dc & 7u) * 2u;
+                *reinterpret_cast<uint2 *>(dst) = hi;
+                *reinterpret_cast<uint2 *>(dst + 2 * qchunk) = lo;
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> the MMA's reads
+            __syncwarp();
+            if (lane == 0) mbar_arrive(qfull_bar);
 
+            float m_run = -INFINITY, l_run = 0.f;                // m_run: the whole row's, l_run: of this half's keys
             for (int t = 0; t < it.n_tiles; ++t, ++s_cnt) {
                 const int sb = s_cnt & 1;
-                if (!(ok = mbar_wait(sfull_bar(sb), (s_cnt >> 1) & 1, &abort_sh, a.status))) break;
+                if (!(ok = warp_wait(sfull_bar(sb), (s_cnt >> 1) & 1, &abort_sh, a.status))) break;
                 tc_fence_after();
-                const int j0 = it.k_begin + t * TKEYS;
-                const bool masked = j0 + TKEYS > it.n_ctx || j0 + TKEYS > it.k_end;
-                const uint32_t tb = tlane + TM_S + sb * 128;               // this tile's S / P buffer, this warp's lanes
-                const int jr = j0 + key0;                                  // first key of this replica's share
-                // which of 16 keys from `base` on this row may see: inside the range, and committed context or an ancestor
-                auto visible16 = [&](int base) -> uint32_t {
-                    if (!masked) return 0xffffu;
-                    const int nr = it.k_end - base, nc = it.n_ctx - base;
-                    const uint32_t in_range = nr >= 16 ? 0xffffu : nr <= 0 ? 0u : (1u << nr) - 1u;
-                    const uint32_t in_ctx = nc >= 16 ? 0xffffu : nc <= 0 ? 0u : (1u << nc) - 1u;
-                    const uint32_t tree_bits = nc >= 16 ? 0u : nc > 0 ? (uint32_t)(anc << nc) : (nc > -64 ? (uint32_t)(anc >> -nc) : 0u);
-                    return in_range & (in_ctx | tree_bits) & 0xffffu;
+                const int j0 = it.k_begin + t * TKEYS + half * 64;           // first key of this half
+                const bool masked = j0 + 64 > it.n_ctx || j0 + 64 > it.k_end;
+                const int cols = warp_live ? min(64, it.k_end - j0) : 0;     // columns of this half that hold scores (may be negative)
+                const uint32_t tb = tlane + TM_S + sb * 128 + half * 64;
+                // which of 32 keys from `key` on this row may see: inside the range, and committed context or an ancestor
+                auto visible32 = [&](int key) -> uint32_t {
+                    const int nr = it.k_end - key, nc = it.n_ctx - key;
+                    const uint32_t in_range = nr >= 32 ? 0xffffffffu : nr <= 0 ? 0u : (1u << nr) - 1u;
+                    const uint32_t in_ctx = nc >= 32 ? 0xffffffffu : nc <= 0 ? 0u : (1u << nc) - 1u;
+                    const uint32_t tree_bits = nc >= 32 ? 0u : nc > 0 ? (uint32_t)(anc << nc) : (nc > -64 ? (uint32_t)(anc >> -nc) : 0u);
+                    return in_range & (in_ctx | tree_bits);
                 };
-                // pass 1: the row maximum over this replica's keys of the tile (16 keys at a time: the loop body stays
-                // small enough to live in the instruction cache)
-                float m_tile = -INFINITY;
-                if (warp_live) {
-#pragma unroll 1
-                    for (int c = 0; c < KR / 16; ++c) {
-                        uint32_t r[16];
-                        tc_ld16(tb + key0 + c * 16, r);
-                        const uint32_t vis = visible16(jr + c * 16);
+                auto load = [&](int c, uint32_t (&r)[32]) {                   // 32 scores, those out of sight -inf
+                    tc_ld32(tb + c * 32, r);
+                    if (masked) {
+                        const uint32_t vis = visible32(j0 + c * 32);
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) m_tile = fmaxf(m_tile, ((vis >> e) & 1u) ? __uint_as_float(r[e]) : -INFINITY);
+                        for (int e = 0; e < 32; ++e) r[e] = (vis >> e) & 1u ? r[e] : 0xff800000u;
                     }
+                };
+                // pass 1: the row maximum (rolled: the loop bodies stay small enough to live in the instruction cache)
+                float m_half = -INFINITY;
+#pragma unroll 1
+                for (int c = 0; c * 32 < cols; ++c) {
+                    uint32_t r[32];
+                    load(c, r);
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) m_half = fmaxf(m_half, __uint_as_float(r[e]));
                 }
-                float m_new = m_run, corr = 1.f;
+                float m_tile;
+                if (!(ok = exchange(m_half, m_tile))) break;
+                m_tile = fmaxf(m_tile, m_half);
+                float corr = 1.f;
                 if (live && m_tile > m_run + RESCALE_GAP) {            // also the first tile with a visible key (m_run = -inf)
-                    m_new = m_tile;
-                    corr = (m_run == -INFINITY) ? 1.f : ex2(m_run - m_new);
+                    corr = (m_run == -INFINITY) ? 1.f : ex2(m_run - m_tile);
+                    m_run = m_tile;
                 }
-                if (warp_live && __any_sync(0xffffffffu, corr != 1.f)) {
-                    // rare: the running maximum moved.  O is rescaled once the previous tile's P V has written it
-                    // (the one before that finished earlier: MMAs complete in order).
-                    if (s_cnt > 0 && !(ok = mbar_wait(pvdone_bar(sb ^ 1), ((s_cnt - 1) >> 1) & 1, &abort_sh, a.status))) break;
+                if (__any_sync(0xffffffffu, corr != 1.f)) {
+                    // rare: the running maximum moved (both warps of the quarter see it).  Each rescales its half of O once
+                    // the previous tile's P V has written it (the one before that finished earlier: MMAs complete in order).
+                    if (!(ok = warp_wait(pvdone_bar(sb ^ 1), ((s_cnt - 1) >> 1) & 1, &abort_sh, a.status))) break;
                     tc_fence_after();
 #pragma unroll 1
-                    for (int c = 0; c < 4; ++c) {
+                    for (int c = 0; c < 2; ++c) {
                         uint32_t r[32];
-                        tc_ld32(tlane + TM_O + c * 32, r);
+                        tc_ld32(tlane + TM_O + half * 64 + c * 32, r);
 #pragma unroll
                         for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * corr);
-                        tc_st32(tlane + TM_O + c * 32, r);
+                        tc_st32(tlane + TM_O + half * 64 + c * 32, r);
                     }
+                    l_run *= corr;
                 }
-                // pass 2: weights and their row sum; P replaces S in place, per 16 keys 8 columns of bf16 pairs hi and
-                // 8 columns lo; the key columns of the other replicas are zeroed (their scores are not this row's business)
-                float l_tile = 0.f;
-                if (warp_live) {
-                    const float m_use = m_new == -INFINITY ? 0.f : m_new;   // no visible key yet: every weight is masked to 0
+                // pass 2: weights and their row sum; P replaces S in place
+                const float m_use = m_run == -INFINITY ? 0.f : m_run;   // no visible key yet: every weight is 2^-inf
 #pragma unroll 1
-                    for (int c = 0; c < TKEYS / 16; ++c) {
-                        uint32_t w[16];
-                        if (c * 16 < key0 || c * 16 >= key0 + KR) {
+                for (int c = 0; c * 32 < cols; ++c) {
+                    uint32_t r[32], w[32];
+                    load(c, r);
+                    float l4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) w[e] = 0u;
-                        } else {
-                            uint32_t r[16];
-                            tc_ld16(tb + c * 16, r);
-                            const uint32_t vis = visible16(j0 + c * 16);
-#pragma unroll
-                            for (int e = 0; e < 16; e += 2) {
-                                const float p0 = ((vis >> e) & 1u) ? ex2(__uint_as_float(r[e]) - m_use) : 0.f;
-                                const float p1 = ((vis >> (e + 1)) & 1u) ? ex2(__uint_as_float(r[e + 1]) - m_use) : 0.f;
-                                l_tile += p0 + p1;
-                                split_pair(p0, p1, w[e >> 1], w[8 + (e >> 1)]);
-                            }
-                        }
-                        tc_st16(tb + c * 16, w);
+                    for (int e = 0; e < 32; e += 2) {
+                        const float p0 = ex2(__uint_as_float(r[e]) - m_use), p1 = ex2(__uint_as_float(r[e + 1]) - m_use);
+                        l4[(e >> 1) & 3] += p0 + p1;
+                        split_pair(p0, p1, w[(e >> 4) * 16 + ((e & 15) >> 1)], w[(e >> 4) * 16 + 8 + ((e & 15) >> 1)]);
                     }
+                    l_run += (l4[0] + l4[1]) + (l4[2] + l4[3]);
+                    tc_st32(tb + c * 32, w);
                 }
                 tc_wait_st();
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(pfull_bar(sb));             // P (and the rescaled O) are in place
-                l_run = l_run * corr + l_tile;
-                m_run = m_new;
             }
             if (!ok) break;
-            // the last P V of the item (and with it all earlier ones) has written O
-            if (it.n_tiles > 0 && !(ok = mbar_wait(pvdone_bar((s_cnt - 1) & 1), ((s_cnt - 1) >> 1) & 1, &abort_sh, a.status))) break;
+            // ---- the item's result, once the last P V (and with it all earlier ones) has written O ----
+            float l_other;
+            if (!(ok = exchange(l_run, l_other))) break;
+            const float l = half ? l_other + l_run : l_run + l_other;
+            if (!(ok = warp_wait(pvdone_bar((s_cnt - 1) & 1), ((s_cnt - 1) >> 1) & 1, &abort_sh, a.status))) break;
             tc_fence_after();
-            // ---- the item's result: O row from TMEM (zeros for an empty key range) ----
-            const int n_part = a.nsplit * a.reps;                      // key ranges to merge: CTAs x replicas
-            const bool single = n_part == 1;
-            const size_t o0 = ((size_t)(it.be * a.M + node) * a.H + h) * HD;
-            float *pdst = a.part + ((((size_t)it.be * a.H + h) * a.M + node) * n_part + it.split * a.reps + rep) * ROWF;
-            const float inv = single ? 1.f / l_run : 1.f;
+            const bool single = it.n_split == 1;
+            float *pdst = a.part + ((size_t)it.pair * a.slots + it.split) * part_floats;
             if (warp_live) {
+                const float inv = 1.f / l;
 #pragma unroll 1
-                for (int c = 0; c < 4; ++c) {
+                for (int c = 0; c < 2; ++c) {
                     uint32_t r[32];
-                    if (it.n_tiles > 0) {
-                        tc_ld32(tlane + TM_O + c * 32, r);
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) r[e] = 0u;
-                    }
-                    if (!live) continue;
+                    tc_ld32(tlane + TM_O + half * 64 + c * 32, r);
                     if (single) {
+                        // through the query region (every MMA that read it is done), so that whole rows go out together
 #pragma unroll
                         for (int e = 0; e < 32; e += 8) {
                             uint4 hi, lo;
@@ -451,69 +530,113 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                             split_pair(__uint_as_float(r[e + 2]) * inv, __uint_as_float(r[e + 3]) * inv, hi.y, lo.y);
                             split_pair(__uint_as_float(r[e + 4]) * inv, __uint_as_float(r[e + 5]) * inv, hi.z, lo.z);
                             split_pair(__uint_as_float(r[e + 6]) * inv, __uint_as_float(r[e + 7]) * inv, hi.w, lo.w);
-                            *reinterpret_cast<uint4 *>(a.out + o0 + c * 32 + e) = hi;
-                            *reinterpret_cast<uint4 *>(a.out + a.out_plane + o0 + c * 32 + e) = lo;
-                        }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 32; e += 2)
-                            *reinterpret_cast<float2 *>(pdst + c * 32 + e) = make_float2(__uint_as_float(r[e]), __uint_as_float(r[e + 1]));
-                    }
-                }
-                if (live && !single) { pdst[HD] = m_run * 0.6931471805599453f; pdst[HD + 1] = l_run; }   // natural-log units
-            }
-            if (it.n_tiles > 0) {
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(ofree_bar);                 // the next item may overwrite O
-            }
-            if (!single && a.fuse_merge) {
-                // last key range of this (sequence, kv head) to finish merges all of them, in range order
-                __threadfence();
-                if (!(ok = wg_sync())) break;
-                if (et == 0) {
-                    int *ctr = a.counters + it.be * a.Hkv * a.subs + it.g;
-                    const int old = atomicAdd(ctr, 1);
-                    last_sh = old == a.nsplit - 1;
-                    if (last_sh) *ctr = 0;
-                }
-                if (!(ok = wg_sync())) break;
-                if (last_sh) {
-                    __threadfence();
-                    for (int r = warp - 2; r < it.rows; r += 4) {
-                        const int hh = (it.g / a.subs) * grp + (it.row0 + r) / a.M, i = (it.row0 + r) % a.M;
-                        const float *src = a.part + (((size_t)it.be * a.H + hh) * a.M + i) * (size_t)n_part * ROWF;
-                        // lane s holds range s's (max, sum); the weights go round by shuffle (at most 32 ranges when fused)
-                        float ms = -INFINITY, ls = 0.f;
-                        if (lane < n_part) { ms = __ldcg(src + (size_t)lane * ROWF + HD); ls = __ldcg(src + (size_t)lane * ROWF + HD + 1); }
-                        float num[HD / 32];
-#pragma unroll
-                        for (int e = 0; e < HD / 32; ++e) num[e] = 0.f;
-                        const float mmax = warp_max(ms);
-                        const float w = (ms == -INFINITY) ? 0.f : expf(ms - mmax);
-                        const float den = warp_sum(ls * w);
-                        for (int s0 = 0; s0 < n_part; s0 += 4) {
-                            float v[4][HD / 32];
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                                for (int e = 0; e < HD / 32; ++e)
-                                    v[q][e] = s0 + q < n_part ? __ldcg(src + (size_t)(s0 + q) * ROWF + lane + 32 * e) : 0.f;
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const float wq = __shfl_sync(0xffffffffu, w, (s0 + q) & 31);
-#pragma unroll
-                                for (int e = 0; e < HD / 32; ++e) num[e] = fmaf(v[q][e], s0 + q < n_part ? wq : 0.f, num[e]);
+                            if (live) {
+                                uint8_t *dst = q_gen + trow * 256 + (((half * 8 + c * 4 + (e >> 3)) ^ (trow & 15)) << 4);
+                                *reinterpret_cast<uint4 *>(dst) = hi;
+                                *reinterpret_cast<uint4 *>(dst + 2 * qchunk) = lo;
                             }
                         }
-                        const float invd = 1.f / den;
+                    } else if (live) {
+                        // lanes are rows: 512 contiguous bytes per store
 #pragma unroll
-                        for (int e = 0; e < HD / 32; ++e)
-                            store_act<__nv_bfloat16>(a.out, a.out_plane, ((size_t)(it.be * a.M + i) * a.H + hh) * HD + lane + 32 * e,
-                                                     num[e] * invd);
+                        for (int e = 0; e < 32; e += 4)
+                            *reinterpret_cast<uint4 *>(pdst + ((size_t)(half * 16 + c * 8 + (e >> 2)) * a.rows8 + trow) * 4) = make_uint4(r[e], r[e + 1], r[e + 2], r[e + 3]);
                     }
                 }
-                if (!(ok = wg_sync())) break;                          // last_sh is reused by the next item
+            }
+            tc_fence_before();
+            if (single) {
+                float unused;
+                if (!(ok = exchange(0.f, unused))) break;              // both halves of the rows are in place
+                if (warp_live) {
+#pragma unroll 1
+                    for (int i = 0; i < 8; ++i) {
+                        const int r = half * 16 + i * 2 + (lane >> 4), rr = quarter * 32 + r, ch = lane & 15;   // half a warp per row
+                        const size_t ro = __shfl_sync(0xffffffffu, (unsigned long long)o0, r) + ch * 8;
+                        if (rr >= it.rows) continue;
+                        const uint8_t *from = q_gen + rr * 256 + ((ch ^ (rr & 15)) << 4);
+                        *reinterpret_cast<uint4 *>(a.out + ro) = *reinterpret_cast<const uint4 *>(from);
+                        *reinterpret_cast<uint4 *>(a.out + a.out_plane + ro) = *reinterpret_cast<const uint4 *>(from + 2 * qchunk);
+                    }
+                }
+            } else {
+                if (live && half == 0) *reinterpret_cast<float2 *>(pdst + (size_t)HD * a.rows8 + 2 * trow) = make_float2(m_run, l);
+                if (!(ok = wg_sync())) break;
+                // (the barrier orders the group's stores before this thread's release, which is cumulative)
+                if (et == 0) asm volatile("red.release.gpu.global.inc.u32 [%0], %1;" ::"l"(a.counters + it.pair), "r"(2 * it.n_split - 1) : "memory");
+            }
+        }
+        // ---- the split pairs of this CTA's list: its slice of each one's rows ----
+        src_init(a, cut, ranges, src);
+        while (ok && next_item(a, cut, src, it)) {
+            if (it.n_split == 1) continue;
+            if (et == 0) {
+                // n_split arrivals, then as many finishers that have seen them: the last of those wraps the counter to zero
+                unsigned *ctr = a.counters + it.pair;
+                auto arrived = [&]() { unsigned v; asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory"); return v; };
+                const long long w0 = clock64();
+                while (arrived() < (unsigned)it.n_split) {
+                    if (*(volatile int *)&abort_sh || clock64() - w0 > WAIT_LIMIT_CYCLES) { abort_sh = 1; atomicExch(a.status, VIASD_EDEVICE); break; }
+                }
+                asm volatile("red.relaxed.gpu.global.inc.u32 [%0], %1;" ::"l"(ctr), "r"(2 * it.n_split - 1) : "memory");
+            }
+            if (!(ok = wg_sync()) || *(volatile int *)&abort_sh) break;
+            const int rper = (it.rows + it.n_split - 1) / it.n_split, r0 = min(it.rows, it.split * rper), nr = min(it.rows, r0 + rper) - r0;
+            const float *psrc = a.part + (size_t)it.pair * a.slots * part_floats;
+            // A lane takes a row, a warp every eighth group of dims.  All its pieces (16 bytes of a range's row) come into the idle
+            // ring by asynchronous copies: one trip to L2 however many ranges there are, and no thread reads what another
+            // copied, so there is no barrier.  (Loads into registers, 8 ranges at a time, were a trip of 1000 cycles per 8 ranges;
+            // copies with a barrier and a warp per row for the weights 6800 cycles in all for 12 rows of 9 ranges.)
+#pragma unroll 1
+            for (int row = lane; row < nr; row += 32) {
+                const float *from = psrc + ((size_t)sw * a.rows8 + r0 + row) * 4, *from_ml = psrc + (size_t)HD * a.rows8 + 2 * (r0 + row);
+                const uint32_t at = qsm + (uint32_t)(sw * nr + row) * 16u, step = (uint32_t)(SW * nr) * 16u;
+                const uint32_t at_ml = qsm + (uint32_t)(it.n_split * 4) * step + (uint32_t)(sw * nr + row) * 8u;
+#pragma unroll 1
+                for (int s = 0; s < it.n_split; ++s) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at + (uint32_t)(4 * s + i) * step), "l"(from + (size_t)(i * SW * 4) * a.rows8) : "memory");
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(at_ml + (uint32_t)s * (step >> 1)), "l"(from_ml) : "memory");
+                    from += part_floats; from_ml += part_floats;
+                }
+                __nv_bfloat16 *dst = a.out + row_off(it, r0 + row) + 4 * sw;
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                const uint8_t *pieces = q_gen + (at - qsm);
+                float2 *ml = reinterpret_cast<float2 *>(q_gen + (at_ml - qsm));
+                const int ml_step = (int)(step >> 4);
+                float m = -INFINITY, den = 0.f;
+#pragma unroll 4
+                for (int s = 0; s < it.n_split; ++s) m = fmaxf(m, ml[s * ml_step].x);   // (every row sees at least itself: finite)
+#pragma unroll 4
+                for (int s = 0; s < it.n_split; ++s) {
+                    const float2 x = ml[s * ml_step];
+                    const float w = ex2(x.x - m);
+                    den = fmaf(x.y, w, den);
+                    ml[s * ml_step].x = w;
+                }
+                const float inv = 1.f / den;
+                float4 num[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) num[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+                for (int s = 0; s < it.n_split; ++s) {
+                    const float w = ml[s * ml_step].x;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 v = *reinterpret_cast<const float4 *>(pieces + (uint32_t)(4 * s + i) * step);
+                        num[i].x = fmaf(v.x, w, num[i].x); num[i].y = fmaf(v.y, w, num[i].y);
+                        num[i].z = fmaf(v.z, w, num[i].z); num[i].w = fmaf(v.w, w, num[i].w);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    uint2 hi, lo;
+                    split_pair(num[i].x * inv, num[i].y * inv, hi.x, lo.x);
+                    split_pair(num[i].z * inv, num[i].w * inv, hi.y, lo.y);
+                    *reinterpret_cast<uint2 *>(dst + i * SW * 4) = hi;
+                    *reinterpret_cast<uint2 *>(dst + a.out_plane + i * SW * 4) = lo;
+                }
             }
         }
     }
@@ -535,14 +658,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 
 }  // namespace
 
-// Items per kv head (at most 128 query rows each)
-int attention_tc_items(int query_rows) { return (query_rows + 127) / 128; }
-// Replicas of an item's query rows across the 128 TMEM lanes (each takes a share of every tile's keys)
-int attention_tc_replicas(int query_rows) {
-    query_rows = (query_rows + attention_tc_items(query_rows) - 1) / attention_tc_items(query_rows);
-    return query_rows <= 32 ? 4 : query_rows <= 64 ? 2 : 1;
-}
-
 // tensor maps over the caches are rebuilt only when the caller's pointers change
 static int cache_maps_tc(viasd_model *m, CacheMaps &cm, const void *kc, const void *vc, int n_layers) {
     if (cm.k_ptr == kc && cm.v_ptr == vc) return VIASD_OK;
@@ -558,8 +673,7 @@ static int cache_maps_tc(viasd_model *m, CacheMaps &cm, const void *kc, const vo
 // streams = 1: one cache (full or slim).  streams = 2: rows [0, batch*M) against the full cache at layer_ord and
 // rows [batch*M, 2*batch*M) against the slim cache at layer_ord2, in one launch.
 int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, const void *kc2,
-                        const void *vc2, int layer_ord2, int streams, int batch, int M, int nsplit, int fuse_merge,
-                        cudaStream_t st) {
+                        const void *vc2, int layer_ord2, int streams, int batch, int M, cudaStream_t st) {
     const viasd_config &c = m->cfg;
     CacheMaps &cm = slim ? m->cmaps_slim : m->cmaps_full;
     int rc;
@@ -571,40 +685,33 @@ int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool sli
     }
     const int QR = c.n_heads / c.n_kv_heads * M;
     AttnTcArgs a;
-    a.subs = attention_tc_items(QR);
+    a.subs = (QR + 127) / 128;
     a.rows_sub = a.subs == 1 ? QR : ((QR + a.subs - 1) / a.subs + 7) / 8 * 8;
     a.subs = (QR + a.rows_sub - 1) / a.rows_sub;
-    if (fuse_merge && a.subs > VIASD_ATTN_ITEMS_PER_KV_HEAD) return VIASD_EINVAL;
+    a.rows8 = (a.rows_sub + 7) / 8 * 8;
     a.q = m->ws.q; a.part = m->ws.part; a.out = (__nv_bfloat16 *)m->ws.attn;
     a.out_plane = m->ws.rows_alloc * (size_t)c.n_heads * HD;
     a.len_eff = m->ws.len_eff; a.tree = m->ws.tree; a.status = &m->ws.stats->device_status; a.run_flag = m->run_flag;
     a.M = M; a.H = c.n_heads; a.Hkv = c.n_kv_heads; a.max_batch = c.max_batch; a.max_ctx = c.max_ctx;
-    a.layer_ord = layer_ord; a.nsplit = nsplit; a.scale = 1.4426950408889634f / sqrtf((float)HD);   // log2(e) / sqrt(hd)
+    a.layer_ord = layer_ord; a.scale = 1.4426950408889634f / sqrtf((float)HD);   // log2(e) / sqrt(hd)
     a.batch = batch; a.layer_ord2 = layer_ord2; a.streams = streams;
-    a.counters = m->ws.attn_counters;
-    a.fuse_merge = fuse_merge;
-    a.qrows8 = (a.rows_sub + 7) / 8 * 8;
-    a.reps = attention_tc_replicas(QR);
-    a.rows_per_rep = 128 / a.reps;
-    {
-        // staged query regions (hi / lo x two 64-dim chunks).  A region nominally spans 128 rows of 128 bytes, but
-        // only qrows8 rows per replica block are live, so regions are interleaved in the dead rows where they fit.
-        const uint32_t slot = (uint32_t)a.qrows8 * 128u, period = (uint32_t)a.rows_per_rep * 128u;
-        const uint32_t per_period = a.reps == 1 ? 1u : period / slot;
-        for (uint32_t k = 0; k < 4; ++k)
-            a.qoff[k] = a.reps == 1 ? k * slot : (k / per_period) * 16384u + (k % per_period) * slot;
-        a.q_bytes = a.qoff[3] + (uint32_t)(a.reps - 1) * period + slot;
-    }
-    a.n_items = streams * batch * c.n_kv_heads * a.subs * nsplit;
-    int grid = a.n_items < m->sm_count ? a.n_items : m->sm_count;
-    a.items_per_cta = (a.n_items + grid - 1) / grid;
-    grid = (a.n_items + a.items_per_cta - 1) / a.items_per_cta;
-    const size_t q_bytes = a.q_bytes;
-    a.nstage = 1024 + q_bytes + 3 * (size_t)STAGE_BYTES <= 220 * 1024 ? 3 : 2;
-    const size_t smem = 1024 + q_bytes + a.nstage * (size_t)STAGE_BYTES;
+    a.counters = (unsigned *)m->ws.attn_counters;
+    // (always counted for two streams: the cuts must not depend on how many a launch has)
+    const size_t slot_bytes = (size_t)2 * batch * c.n_kv_heads * a.subs * a.rows8 * PART_ROW * sizeof(float);
+    const size_t fit = m->ws.part_bytes / slot_bytes;
+    a.slots = fit > MAX_SLOTS ? MAX_SLOTS : (int)fit;
+    a.splits = m->opt.attn_splits;
+    a.w_one = c.n_layers - m->n_routed; a.w_two = m->n_routed;
+    a.m_recip = ((1ull << 32) + M - 1) / M;
+    int grid = m->sm_count;
+    if (m->opt.tk_grid >= 1 && m->opt.tk_grid < grid) grid = m->opt.tk_grid;     // tests: long ranges per CTA on small cases
+    const size_t q_bytes = (size_t)a.rows8 * 512, smem_max = 229000;
+    a.ring_slots = (int)((smem_max - 1024 - q_bytes) / SLOT_BYTES);
+    if (a.ring_slots > AT_MAX_SLOTS) a.ring_slots = AT_MAX_SLOTS;
+    const size_t smem = 1024 + q_bytes + (size_t)a.ring_slots * SLOT_BYTES;
     static bool attr_done[64];
     if (first_use_on_device(attr_done)) {
-        CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+        CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
     }
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
@@ -613,4 +720,3 @@ int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool sli
     LAUNCH_CHECK();
     return VIASD_OK;
 }
-

@@ -11,8 +11,9 @@
 // Arrival counters of the attention kernels: one per (stream, sequence, kv head, item of that kv head).  The
 // keys-on-lanes kernel deals the query heads of a kv head to at most this many items.
 #define VIASD_ATTN_ITEMS_PER_KV_HEAD 4
-inline size_t attn_counter_count(int max_batch, int n_kv_heads) {
-    return (size_t)2 * max_batch * n_kv_heads * VIASD_ATTN_ITEMS_PER_KV_HEAD;
+inline size_t attn_counter_count(int max_batch, int n_heads, int n_kv_heads) {
+    const int tc = (n_heads / n_kv_heads * VIASD_MAX_ROWS_PER_SEQ + 127) / 128;      // rows-on-lanes kernel: items of up to 128 rows
+    return (size_t)2 * max_batch * n_kv_heads * (tc > VIASD_ATTN_ITEMS_PER_KV_HEAD ? tc : VIASD_ATTN_ITEMS_PER_KV_HEAD);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -242,12 +243,9 @@ int attention_mma_supported(const viasd_model *m, int M);
 int launch_attention_mma(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, const void *kc2,
                          const void *vc2, int layer_ord2, int streams, int batch, int M, int nsplit, int fuse_merge,
                          cudaStream_t st);
-int attention_tc_replicas(int query_rows);
-int attention_tc_items(int query_rows);
 int attention_tensor_supported(const viasd_model *m);
 int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, const void *kc2,
-                         const void *vc2, int layer_ord2, int streams, int batch, int M, int nsplit, int fuse_merge,
-                         cudaStream_t st);
+                         const void *vc2, int layer_ord2, int streams, int batch, int M, cudaStream_t st);
 int attention_tk_heads_per_item(int group_heads, int M);
 int attention_tk_supported(int group_heads, int M);
 int launch_attention_tk(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, const void *kc2,

@@ -191,6 +191,18 @@ def test_forward_with_wide_query_groups(name, batch, nodes, ctx):
     _check_rows(replace(base, batch=batch, ctx=ctx, parent=W.chain(nodes), shape=replace(base.shape, n_layers=2), n_routed=1))
 
 
+# The rows-on-lanes kernel at its edges: 33+ and exactly 128 rows, a context that ends on a tile and one past it, no context,
+# each way of cutting the keys (whole pairs, k ranges per pair, tiles dealt evenly over a small grid).  Bounds as above.
+@pytest.mark.parametrize("nodes,batch,ctx,env", [(8, 1, 0, {}), (15, 1, 112, {}), (15, 2, 113, {}), (31, 2, 500, {"VIASD_ATTN_NSPLIT": "1"}),
+                                                 (31, 3, 700, {"VIASD_ATTN_NSPLIT": "3"}), (8, 1, 2300, {}),
+                                                 (26, 8, 700, {"VIASD_TK_GRID": "3"}), (3, 2, 300, {"VIASD_ATTN": "tc"})])
+def test_rows_on_lanes_attention_edges(nodes, batch, ctx, env, monkeypatch):
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
+    base = W.get("mini_8b_tree")
+    _check_rows(replace(base, batch=batch, ctx=ctx, parent=W.chain(nodes), shape=replace(base.shape, n_layers=2), n_routed=1))
+
+
 def test_forward_is_deterministic_and_slim_all_layers_equals_full():
     wl = replace(W.get("mini_8b_tree"), n_routed=W.get("mini_8b_tree").shape.n_layers, name="mini_8b_tree")
     vb = _vb()
