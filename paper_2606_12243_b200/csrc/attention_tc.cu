@@ -68,7 +68,7 @@ struct AttnTcArgs {
     int splits;                 // 0, or ranges per pair as asked for by the caller
     int w_one, w_two;           // the model's layers that run one row stream in a verify step, and those that run both
     unsigned long long m_recip; // 2^32 / M, rounded up: r / M for the few hundred query rows there are
-    unsigned *counters;         // per pair: arrivals, then finishers; zero between launches
+    int *counters;              // per pair: arrivals, then finishers; zero between launches
     float scale;                // log2(e) / sqrt(hd)
 };
 
@@ -563,23 +563,14 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 if (live && half == 0) *reinterpret_cast<float2 *>(pdst + (size_t)HD * a.rows8 + 2 * trow) = make_float2(m_run, l);
                 if (!(ok = wg_sync())) break;
                 // (the barrier orders the group's stores before this thread's release, which is cumulative)
-                if (et == 0) asm volatile("red.release.gpu.global.inc.u32 [%0], %1;" ::"l"(a.counters + it.pair), "r"(2 * it.n_split - 1) : "memory");
+                if (et == 0) counter_arrive(a.counters + it.pair, it.n_split, it.n_split);
             }
         }
         // ---- the split pairs of this CTA's list: its slice of each one's rows ----
         src_init(a, cut, ranges, src);
         while (ok && next_item(a, cut, src, it)) {
             if (it.n_split == 1) continue;
-            if (et == 0) {
-                // n_split arrivals, then as many finishers that have seen them: the last of those wraps the counter to zero
-                unsigned *ctr = a.counters + it.pair;
-                auto arrived = [&]() { unsigned v; asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory"); return v; };
-                const long long w0 = clock64();
-                while (arrived() < (unsigned)it.n_split) {
-                    if (*(volatile int *)&abort_sh || clock64() - w0 > WAIT_LIMIT_CYCLES) { abort_sh = 1; atomicExch(a.status, VIASD_EDEVICE); break; }
-                }
-                asm volatile("red.relaxed.gpu.global.inc.u32 [%0], %1;" ::"l"(ctr), "r"(2 * it.n_split - 1) : "memory");
-            }
+            if (et == 0) counter_wait(a.counters + it.pair, it.n_split, it.n_split, &abort_sh, a.status);
             if (!(ok = wg_sync()) || *(volatile int *)&abort_sh) break;
             const int rper = (it.rows + it.n_split - 1) / it.n_split, r0 = min(it.rows, it.split * rper), nr = min(it.rows, r0 + rper) - r0;
             const float *psrc = a.part + (size_t)it.pair * a.slots * part_floats;
@@ -695,7 +686,7 @@ int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool sli
     a.M = M; a.H = c.n_heads; a.Hkv = c.n_kv_heads; a.max_batch = c.max_batch; a.max_ctx = c.max_ctx;
     a.layer_ord = layer_ord; a.scale = 1.4426950408889634f / sqrtf((float)HD);   // log2(e) / sqrt(hd)
     a.batch = batch; a.layer_ord2 = layer_ord2; a.streams = streams;
-    a.counters = (unsigned *)m->ws.attn_counters;
+    a.counters = m->ws.attn_counters;
     // (always counted for two streams: the cuts must not depend on how many a launch has)
     const size_t slot_bytes = (size_t)2 * batch * c.n_kv_heads * a.subs * a.rows8 * PART_ROW * sizeof(float);
     const size_t fit = m->ws.part_bytes / slot_bytes;

@@ -42,7 +42,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
 
     constexpr bool DUAL = EPI == EPI_SWIGLU;
     RUN_FLAG_EXIT(p.run_flag);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next kernel may start its prologue
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const int NT = p.nt, S = p.stages;
@@ -78,7 +78,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = tmem_base_sh;
+    const uint32_t tmem_base = uniform(tmem_base_sh);
 
     const int total_units = p.n_tiles * p.k_tiles;
     const int u_begin = blockIdx.x * p.units_per_cta;
@@ -86,7 +86,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
-        if (lane == 0) {
+        if (elect_one()) {
             const int n_it = (u_end - u_begin) / KB;          // stages: ranges and tiles are whole numbers of KB boxes
             // unit -> weight matrix, its first row, k-block
             auto unit = [&](int it, const CUtensorMap *&mw, int &wrow, int &kt, int &sidx) {
@@ -141,26 +141,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NB >> 3) << 17) | ((TILE_F >> 4) << 24);
-            int it = 0, acc_it = 0, u = u_begin;
-            Seg sg;
-            bool ok = true;
-            while (ok && next_seg(u, u_end, p.k_tiles, sg)) {
-                const int buf = acc_it % p.acc_bufs;
-                if (!(ok = mbar_wait(tempty_bar(buf), ((acc_it / p.acc_bufs) & 1) ^ 1, &abort_sh, p.status))) break;
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NB >> 3) << 17) | ((TILE_F >> 4) << 24);
+        int st = 0, ph = 0, acc_it = 0, u = u_begin;
+        Seg sg;
+        bool ok = true;
+        while (ok && next_seg(u, u_end, p.k_tiles, sg)) {
+            const int buf = acc_it % p.acc_bufs;
+            if (!(ok = warp_wait(tempty_bar(buf), ((acc_it / p.acc_bufs) & 1) ^ 1, &abort_sh, p.status))) break;
+            tc_fence_after();
+            const uint32_t d0 = tmem_base + buf * acc_cols;
+            for (int kt = sg.ka; kt < sg.kb; kt += KB) {
+                if (!(ok = warp_wait(full_bar(st), ph, &abort_sh, p.status))) break;
                 tc_fence_after();
-                const uint32_t d0 = tmem_base + buf * acc_cols;
-                for (int kt = sg.ka; kt < sg.kb; kt += KB, ++it) {
-                    const int st = it % S;
-                    if (!(ok = mbar_wait(full_bar(st), (it / S) & 1, &abort_sh, p.status))) break;
-                    tc_fence_after();
+                if (elect_one()) {
                     const uint32_t base = smem_base + st * stage_bytes;
                     // the hi tile is followed by the lo tile: together one K-major operand of NB rows
                     const uint32_t bh = base + NACC * a_bytes;
-                    // one descriptor per operand and stage; a k-step of 16 columns is 32 bytes further on, 2 in the
-                    // descriptor's address field (the MMA-issuing thread is a single instruction stream that has about
-                    // the arrival time of a stage to get through all this: every instruction here counts)
+                    // one descriptor per operand and box; a k-step of 16 columns is 32 bytes further on, 2 in the
+                    // descriptor's address field
                     const uint64_t da2 = DUAL ? smem_desc(base + a_bytes) : 0ull;
 #pragma unroll
                     for (int kb = 0; kb < KB; ++kb) {
@@ -172,11 +170,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
                             if (DUAL) tc_mma(d0 + NB, da2 + 2 * k, db + 2 * k, idesc, acc);
                         }
                     }
-                    tc_commit(empty_bar(st));              // the stage is free once these MMAs have read it
+                    tc_commit(empty_bar(st));                  // the stage is free once these MMAs have read it
+                    if (kt + KB >= sg.kb) tc_commit(tfull_bar(buf));   // accumulator complete
                 }
-                if (ok) tc_commit(tfull_bar(buf));          // accumulator complete
-                ++acc_it;
+                __syncwarp();
+                if (++st == S) { st = 0; ph ^= 1; }
             }
+            ++acc_it;
         }
     } else {
         // ---------------- epilogue (warps 2..5 and 6..9 <-> TMEM lane quarters 2,3,0,1) ----------------
@@ -293,19 +293,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
                     // (release / acquire: the barrier orders the group's stores before its first thread's release, which
                     // is cumulative; a fence per thread on both sides was a microsecond of the launch's tail)
                     epi_sync();
-                    if (et == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.counters + sg.tile) : "memory");   // low half: arrivals
+                    if (et == 0) counter_arrive(p.counters + sg.tile, n_c, n_fin);
                     if (!finisher) { ++acc_it; ++seg_i; continue; }
-                    if (et == 0) {
-                        const int *ctr = p.counters + sg.tile;
-                        auto arrived = [&]() { int v; asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory"); return v & 0xffff; };
-                        const long long w0 = clock64();
-                        while (arrived() < n_c) {
-                            if (*(volatile int *)&abort_sh || clock64() - w0 > WAIT_LIMIT_CYCLES) { abort_sh = 1; atomicExch(p.status, VIASD_EDEVICE); break; }
-                            __nanosleep(32);
-                        }
-                        // high half: finishers that have seen all arrivals; the last of them leaves the counter at zero
-                        if (!abort_sh && (atomicAdd(&p.counters[sg.tile], 1 << 16) >> 16) == n_fin - 1) atomicExch(&p.counters[sg.tile], 0);
-                    }
+                    if (et == 0) counter_wait(p.counters + sg.tile, n_c, n_fin, &abort_sh, p.status);
                     epi_sync();
                     if (abort_sh) { ok = false; break; }
                 }

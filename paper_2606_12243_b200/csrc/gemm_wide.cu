@@ -76,7 +76,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
     __shared__ int4 rowmeta[EPI == EPI_QKV_ROPE ? WROWS : 1];
 
     RUN_FLAG_EXIT(p.run_flag);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t rank = blockIdx.x & 1;                         // this CTA's place in its pair
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -116,7 +116,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
 
     if (warp == 0) {
         // ---------------- TMA producer: this CTA's weight rows and its plane of the activations ----------------
-        const uint32_t on = lane == 0, lead = lane == 0 && rank == 0;
+        const uint32_t on = elect_one(), lead = on && rank == 0;
         const int n_it = u_end - u_begin;
         const CUtensorMap *mw = &map_w0;
         int wrow = 0, kt = 0, ptile = 0;
@@ -180,7 +180,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
     } else if (warp == 1) {
         // ---------------- MMA issuer (CTA 0, for both) ----------------
         if (rank == 0) {
-            const uint32_t on = lane == 0;
+            const uint32_t on = elect_one();
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(2 * TH >> 3) << 17) | ((256u >> 4) << 24);
             int st = 0, sx = 0, acc_it = 0, u = u_begin;
             uint32_t ph = 0;
@@ -320,19 +320,9 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
                     }
                     epi_sync();
                     // (the barrier orders the CTA's stores before this release, which is cumulative)
-                    if (et == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.counters + tile) : "memory");
+                    if (et == 0) counter_arrive(p.counters + tile, n_c, n_fin);
                     if (finisher) {
-                        if (et == 0) {
-                            const int *ctr = p.counters + tile;
-                            auto arrived = [&]() { int v; asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory"); return v & 0xffff; };
-                            const long long w0 = clock64();
-                            while (arrived() < n_c) {
-                                if (*(volatile int *)&abort_sh || clock64() - w0 > WAIT_LIMIT_CYCLES) { abort_sh = 1; atomicExch(p.status, VIASD_EDEVICE); break; }
-                                __nanosleep(32);
-                            }
-                            // high half: finishers that have seen all arrivals; the last of them leaves the counter at zero
-                            if (!abort_sh && (atomicAdd(&p.counters[tile], 1 << 16) >> 16) == n_fin - 1) atomicExch(&p.counters[tile], 0);
-                        }
+                        if (et == 0) counter_wait(p.counters + tile, n_c, n_fin, &abort_sh, p.status);
                         epi_sync();
                         if (abort_sh) { ok = false; break; }
                     }

@@ -87,6 +87,26 @@ __device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const CUtensorMap
         ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y), "l"(pol) : "memory");
 }
 
+// ---- arrival counters in global memory: `arrivals` releases, then `readers` acknowledgements, the last of which leaves the
+// counter at zero for the next launch (inc wraps).  None of it returns a value: an atomic that told the last reader to
+// clear the counter was a trip to L2 between the last arrival and the first sum of every split tile.
+__device__ __forceinline__ void counter_arrive(int *ctr, int arrivals, int readers) {
+    asm volatile("red.release.gpu.global.inc.u32 [%0], %1;" ::"l"(ctr), "r"(arrivals + readers - 1) : "memory");
+}
+__device__ __forceinline__ void counter_ack(int *ctr, int arrivals, int readers) {
+    asm volatile("red.relaxed.gpu.global.inc.u32 [%0], %1;" ::"l"(ctr), "r"(arrivals + readers - 1) : "memory");
+}
+// one thread waits, bounded, and acknowledges; false: gave up (the caller's other threads learn it from abort_flag)
+__device__ __forceinline__ bool counter_wait(int *ctr, int arrivals, int readers, volatile int *abort_flag, int *status) {
+    auto arrived = [&]() { int v; asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory"); return v; };
+    const long long t0 = clock64();
+    while (arrived() < arrivals) {
+        if (*abort_flag || clock64() - t0 > WAIT_LIMIT_CYCLES) { *abort_flag = 1; atomicExch(status, VIASD_EDEVICE); return false; }
+    }
+    counter_ack(ctr, arrivals, readers);
+    return true;
+}
+
 // ---- single-thread instructions of a warp in step -----------------------------------------------
 // tcgen05.mma and the TMA instructions take their operands from uniform registers.  The compiler only keeps descriptors and
 // addresses there when it can see that the warp is in step and one thread executes them: the branch to the role on a warp
