@@ -182,21 +182,18 @@ int attention_nsplit(const viasd_model *m, int batch, int M) {
     return nsplit;
 }
 
-// Key ranges per (sequence, kv head) for the tensor-core kernel, from a small cost model: items are dealt to
+// Key ranges per (sequence, kv head) for the keys-on-lanes kernel, from a small cost model: items are dealt to
 // CTAs in equal contiguous shares, each item costs a fixed part (query staging, merge, partial) plus its tiles,
 // and every extra range adds merge work.  Depends on batch, heads and M only, so the one-stream and the two-stream
 // launch cut the keys at the same places and produce the same bits.
-static int mma_nsplit(const viasd_model *m, int batch, int M, int streams, int subs, int tk_rows) {
+static int tk_nsplit(const viasd_model *m, int batch, int M, int streams, int subs, int rows) {
     const viasd_config &c = m->cfg;
-    const int base = batch * c.n_kv_heads * subs, sms = m->sm_count;      // subs: items per kv head (keys-on-lanes kernel)
-    const int mt = ((c.n_heads / c.n_kv_heads) * M + 15) / 16;
+    const int base = batch * c.n_kv_heads * subs, sms = m->sm_count;      // subs: items per kv head
     const int tiles = (c.max_ctx + 127) / 128;
     const int max_s = tiles < 16 ? tiles : 16;                  // the partial buffer holds 16 ranges per (row, head)
-    // microseconds, roughly
-    // (keys-on-lanes kernel, measured: a tile costs its softmax chain, 1.1 - 1.8 us with 8 - 32 rows per item, an item
-    // 5 - 10 us of query staging, result rows and merge)
-    const double t_tile = tk_rows > 16 ? 1.8 : tk_rows > 8 ? 1.3 : tk_rows > 0 ? 1.1 : 0.5 + 0.8 * mt;
-    const double t_item = tk_rows > 16 ? 8.0 : tk_rows > 0 ? 5.0 : 3.0;
+    // microseconds, roughly: a tile costs its softmax chain, 1.1 - 1.8 us with 8 - 32 rows per item, an item 5 - 10 us of
+    // query staging, result rows and merge
+    const double t_tile = rows > 16 ? 1.8 : rows > 8 ? 1.3 : 1.1, t_item = rows > 16 ? 8.0 : 5.0;
     // One choice for the whole model, whichever call runs (the cuts must not depend on it): the routed layers are
     // charged as two-stream launches, as the verify step runs them, the others as one-stream launches.
     const int n_dual = m->n_routed, n_single = c.n_layers - m->n_routed;
@@ -230,31 +227,28 @@ static int mma_attention(viasd_model *m, const void *kc, const void *vc, bool sl
     // 108 rows, 1 sequence of 100 -2.7 us, of 2048 -5, 4 sequences of 2048 -12, 16 of 1000 -66; at 32 rows and 2048 keys or
     // more it is 0.6 - 1.5 us behind).  17 - 32 rows: keys-on-lanes, whose MMAs are that much narrower, from one tile per SM
     // on (24 rows, 1 sequence of 8000 -3.2 us), rows-on-lanes for less (1 sequence of 100: -4.8 us, of 600 -2.2).  Up to 16
-    // rows: mma.sync, whose chain is the shortest for a few tiles, until keys-on-lanes streams 24 tiles per SM (32 kv heads,
-    // 9 rows: 2 sequences of 2048 +6.2 us, 4 of 2048 -3.5, 8 of 1500 -14; 8 kv heads, 16 rows, 8 sequences of 4000: even).
+    // rows: mma.sync, whose chain is the shortest for a few tiles, until keys-on-lanes streams 36 tiles per SM (32 kv heads,
+    // 9 rows: 2 sequences of 2048 +11 us, 4 of 2048 (31 tiles) +5, 8 of 1500 (45) -9; 8 kv heads, 16 rows, 8 of 4000 +4.6).
     // Tiles of both row streams, whichever the launch has: the choice must not depend on it.
     const long long tiles_two = 2LL * batch * c.n_kv_heads * ((c.max_ctx + 127) / 128);
     const int grp = c.n_heads / c.n_kv_heads, hpi = attention_tk_heads_per_item(grp, M);
     const int subs = hpi ? grp / hpi : 1, QRi = hpi * M;       // keys-on-lanes: items per kv head, query rows per item
-    int use = kind != 3 ? kind : QR > 32 ? 1 : QR > 16 ? (tiles_two >= m->sm_count ? 2 : 1) : tiles_two >= 24LL * m->sm_count ? 2 : 0;
+    int use = kind != 3 ? kind : QR > 32 ? 1 : QR > 16 ? (tiles_two >= m->sm_count ? 2 : 1) : tiles_two >= 36LL * m->sm_count ? 2 : 0;
     if (use == 2 && !hpi) use = 0;
-    if (use == 0 && QR > 128) use = 1;                         // more than the mma.sync kernel's eight query tiles
+    if (use == 0 && !attention_mma_supported(m, M)) use = 1;   // (asked for by option, with more rows than its one query tile)
     if (use == 1) return launch_attention_tc(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, st);
-    const int nsplit = mma_nsplit(m, batch, M, streams, use == 2 ? subs : 1, use == 2 ? QRi : 0);
-    const bool fuse = nsplit > 1 && (use == 2 ? QRi : QR) * nsplit <= 160;
-    int rc;
-    if (use == 2) {
-        // The keys-on-lanes kernel deals tiles, not key ranges, evenly to the CTAs (nsplit 0) when the partial buffer
-        // has its 16 slots per (row, head): whole (sequence, head) items leave SMs idle (320 items on 148 SMs: a
-        // quarter of them).  Its merges are then always fused.  Not with more than 16 query rows per kv head: there an
-        // item's fixed cost (staging 32 rows of queries, 32 rows of results) is worth a dozen tiles, and the extra
-        // item per CTA cost more than the balance won (32B batch-16 step 36.5 -> 39.0 ms).  VIASD_OPT_TK_FLAT overrides.
-        const size_t need = (size_t)streams * batch * c.n_heads * M * 16 * (c.head_dim + 2) * sizeof(float);
-        if ((m->opt.tk_flat >= 0 ? m->opt.tk_flat != 0 : QR <= 16) && subs == 1 && need <= m->ws.part_bytes)
-            return launch_attention_tk(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, 0, 1, st);
-        rc = launch_attention_tk(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, nsplit, fuse ? 1 : 0, st);
-    }
-    else rc = launch_attention_mma(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, nsplit, fuse ? 1 : 0, st);
+    if (use == 0) return launch_attention_mma(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, st);
+    // The keys-on-lanes kernel deals tiles, not key ranges, evenly to the CTAs (nsplit 0) when the partial buffer has its 16
+    // slots per (row, head): whole (sequence, head) items leave SMs idle (320 items on 148 SMs: a quarter of them).  Its
+    // merges are then always fused.  Not with more than 16 query rows per kv head: there an item's fixed cost (staging 32
+    // rows of queries, 32 rows of results) is worth a dozen tiles, and the extra item per CTA cost more than the balance
+    // won (32B batch-16 step 36.5 -> 39.0 ms).  VIASD_OPT_TK_FLAT overrides.
+    const size_t need = (size_t)streams * batch * c.n_heads * M * 16 * (c.head_dim + 2) * sizeof(float);
+    if ((m->opt.tk_flat >= 0 ? m->opt.tk_flat != 0 : QR <= 16) && subs == 1 && need <= m->ws.part_bytes)
+        return launch_attention_tk(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, 0, 1, st);
+    const int nsplit = tk_nsplit(m, batch, M, streams, subs, QRi);
+    const bool fuse = nsplit > 1 && QRi * nsplit <= 160;
+    int rc = launch_attention_tk(m, kc, vc, slim, layer_ord, kc2, vc2, layer_ord2, streams, batch, M, nsplit, fuse ? 1 : 0, st);
     if (rc || nsplit == 1 || fuse) return rc;
     CUDA_TRY(launch_chained(attention_combine_kernel<__nv_bfloat16, 128>, dim3(streams * batch * M, c.n_heads), 128, st,
         (__nv_bfloat16 *)m->ws.attn, m->ws.rows_alloc * (size_t)c.n_heads * 128, m->ws.part, M, c.n_heads, nsplit, m->run_flag));

@@ -18,122 +18,26 @@
 // columns of bf16 pairs hi, 8 lo), two buffers; MMAs run in issue order, which is what lets Q K^T of tile t + 2 reuse the
 // buffer that P V of tile t reads.  The last tile of a range multiplies only the 16-key groups that it has.
 //
-// Split of the work (chosen by the kernel from the lengths, see the cost below): either every (sequence, kv head, item) pair is
-// cut into k ranges of tiles and the ranges are dealt to the CTAs in equal shares, or the tiles of all pairs laid end to
-// end are cut into one range per CTA and row stream.  The cuts depend on the lengths, the heads and the grid only, so a
-// one-stream and a two-stream launch cut alike and produce the same bits.  A pair that lies in several ranges is finished
-// by all of their CTAs: each publishes its partial rows, goes on with its other items, and at its very end waits (bounded)
-// for the other ranges of each such pair and merges its own slice of the rows, in range order.  All CTAs of a launch are
-// resident together and publish before they wait, so no wait depends on another.
+// Split of the work: attention_work.cuh.  Partial rows: [32 groups of 4 dims][rows8] float4, then [rows8] (max, sum).
 //
 // Warp roles (320 threads): warp 0 requests K and V tiles by TMA into a ring that runs across the CTA's items, in the
 // order the MMAs use them, warp 1 owns TMEM and issues the MMAs, warps 2-9 stage Q, run the softmax and write the result.
 // Every wait is bounded: on expiry the CTA records VIASD_EDEVICE, lets its copies land and leaves.
 #include "common.cuh"
+#include "attention_work.cuh"
 #include "tc_ptx.cuh"
 #include <stdlib.h>
 
 namespace {
 
-constexpr int HD = 128;                        // head dimension
-constexpr int TKEYS = 128;                     // keys per tile
-constexpr int HALF_BYTES = TKEYS * 128;        // 128 keys x 64 dims of bf16, as one TMA box lands
-constexpr int SLOT_BYTES = 2 * HALF_BYTES;     // one tile of K or of V: dims 0..63, dims 64..127
 constexpr int SW = 8;                          // softmax warps
 constexpr int AT_THREADS = 64 + SW * 32;
 constexpr int AT_MAX_SLOTS = 6;
-constexpr int PART_ROW = HD + 2;               // floats per partial row: numerators, max (log2 units), sum
 constexpr int QROWS = 128 / SW;                // query rows a warp stages at most
-// costs in tiles (2300 cycles): what an item costs besides its tiles (queries, first and last MMA, result), and a merge
-constexpr int COST_ITEM = 4, COST_MERGE = 3;
-constexpr int MAX_SPLITS = 16, MAX_SLOTS = 32; // ranges of a pair: cut evenly, in any case (a lane each when merged)
 constexpr float RESCALE_GAP = 8.f;             // log2 units
 
 constexpr uint32_t TM_S = 0, TM_O = 256;       // TMEM column offsets: S / P buffers (2 x 128), O (128)
 
-struct AttnTcArgs {
-    const float *q;             // [rows, H * HD] rotated queries
-    float *part;                // [pair][slot]: [32 groups of 4 dims][rows8] float4, then [rows8] (max, sum)
-    __nv_bfloat16 *out;         // attention output planes (hi, lo)
-    size_t out_plane;
-    const int *len_eff;
-    const TreeInfo *tree;
-    int *status;
-    const int *run_flag;        // null, or a device flag: the kernel leaves at once when it is zero
-    int M, H, Hkv, max_batch, max_ctx, layer_ord;
-    int batch, layer_ord2;      // second row stream: rows batch*M.., its own cache and layer ordinal
-    int streams, ring_slots;
-    int subs, rows_sub, rows8;  // items per kv head, query rows of each (but the last), the same rounded up to 8
-    int slots;                  // ranges a pair may be cut into (the partial buffer's slots)
-    int splits;                 // 0, or ranges per pair as asked for by the caller
-    int w_one, w_two;           // the model's layers that run one row stream in a verify step, and those that run both
-    unsigned long long m_recip; // 2^32 / M, rounded up: r / M for the few hundred query rows there are
-    int *counters;              // per pair: arrivals, then finishers; zero between launches
-    float scale;                // log2(e) / sqrt(hd)
-};
-
-struct Item { int pair, be, b, kvh, row0, rows, stream, split, n_split, n_ctx, k_begin, k_end, n_tiles, row_base; };
-
-// The CTA's work list.  k > 0: its share of the k ranges of every pair; k == 0: its range of `per` tiles of one row stream, or
-// of both in turn.
-struct Cut { int k, per; };
-struct ItemSrc { int s, s_end, range, b, g, off; };             // k > 0: the next item is `off`, the share ends at `range`
-__device__ __forceinline__ void src_init(const AttnTcArgs &a, const Cut &cut, int ranges, ItemSrc &c) {
-    const int x = blockIdx.x;
-    c.b = c.g = c.s = c.s_end = 0;
-    if (cut.k > 0) {
-        c.off = x * cut.per;
-        c.range = min(a.streams * a.batch * a.Hkv * a.subs * cut.k, c.off + cut.per);
-        return;
-    }
-    c.off = 0;
-    if (a.streams * ranges <= (int)gridDim.x) {                // a CTA per range and stream
-        c.s = x / ranges;
-        c.s_end = c.s < a.streams ? c.s + 1 : c.s;
-        c.range = x - c.s * ranges;
-    } else {
-        c.s_end = x < ranges ? a.streams : 0;
-        c.range = x;
-    }
-}
-// range `split` of n_split: tiles t0 .. t1 - 1 of pair (stream s, sequence b, item g of its kv heads)
-__device__ __forceinline__ void set_item(const AttnTcArgs &a, int s, int b, int g, int n_ctx, int t0, int t1, int split, int n_split, Item &it) {
-    it.b = b; it.stream = s; it.be = s * a.batch + b;
-    it.pair = it.be * a.Hkv * a.subs + g; it.kvh = g / a.subs;
-    it.row0 = (g - it.kvh * a.subs) * a.rows_sub;
-    it.rows = min(a.rows_sub, a.H / a.Hkv * a.M - it.row0);
-    it.split = split; it.n_split = n_split;
-    it.n_ctx = n_ctx; it.k_begin = t0 * TKEYS; it.k_end = min(n_ctx + a.M, t1 * TKEYS); it.n_tiles = t1 - t0;
-    it.row_base = (((s ? a.layer_ord2 : a.layer_ord) * a.max_batch + b) * a.Hkv + it.kvh) * a.max_ctx;
-}
-__device__ __forceinline__ bool next_item(const AttnTcArgs &a, const Cut &cut, ItemSrc &c, Item &it) {
-    const int Hs = a.Hkv * a.subs;
-    if (cut.k > 0) {
-        while (c.off < c.range) {
-            const int id = c.off++, bg = id / cut.k, split = id - bg * cut.k, be = bg / Hs, s = be / a.batch, b = be - s * a.batch;
-            const int n_ctx = a.len_eff[b], tb = (n_ctx + a.M + TKEYS - 1) / TKEYS, n_split = min(cut.k, tb);
-            if (split >= n_split) continue;                                                   // a short sequence has fewer ranges
-            set_item(a, s, b, bg - be * Hs, n_ctx, split * tb / n_split, (split + 1) * tb / n_split, split, n_split, it);
-            return true;
-        }
-        return false;
-    }
-    const int per = cut.per, lo = c.range * per, hi = lo + per;
-    while (c.s < c.s_end) {
-        if (c.b >= a.batch || c.off >= hi) { ++c.s; c.b = c.g = c.off = 0; continue; }      // done with this stream
-        const int n_ctx = a.len_eff[c.b], tb = (n_ctx + a.M + TKEYS - 1) / TKEYS;
-        if (c.off + Hs * tb <= lo) { c.off += Hs * tb; ++c.b; c.g = 0; continue; }            // this sequence ends before the range
-        if (c.g == 0 && c.off < lo) c.g = (lo - c.off) / tb;                                  // its first pair that reaches into the range
-        const int p_lo = c.off + c.g * tb, p_hi = p_lo + tb;
-        if (c.g >= Hs) { c.off += Hs * tb; ++c.b; c.g = 0; continue; }
-        if (p_lo >= hi) { ++c.s; c.b = c.g = c.off = 0; continue; }
-        const int first = p_lo / per, last = (p_hi - 1) / per;
-        set_item(a, c.s, c.b, c.g, n_ctx, max(lo, p_lo) - p_lo, min(hi, p_hi) - p_lo, c.range - first, last - first + 1, it);
-        ++c.g;
-        return true;
-    }
-    return false;
-}
 // The j-th of an item's 2 n requests, in the order the MMAs take them: K0 K1 V0 K2 V1 ... K(n-1) V(n-2) V(n-1)
 __device__ __forceinline__ int request_tile(int j, int n, bool &is_v) {
     is_v = false;
@@ -142,20 +46,6 @@ __device__ __forceinline__ int request_tile(int j, int n, bool &is_v) {
     if ((j & 1) && (j + 1) / 2 < n) return (j + 1) / 2;
     is_v = true;
     return (j & 1) ? n - 1 : (j - 2) / 2;
-}
-
-__device__ __forceinline__ float ex2(float x) {            // 2^x, hardware approximation (2 ulp)
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// x0, x1 -> packed bf16 pairs hi = bf16(x), lo = bf16(x - hi); the low half word is the even element
-__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t &hi, uint32_t &lo) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
-    hi = *reinterpret_cast<const uint32_t *>(&h);
-    const __nv_bfloat162 l = __floats2bfloat162_rn(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u));
-    lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 
 // MN-major operand tile with the 128-byte swizzle: 64 contiguous elements along MN per row of 128 bytes,
@@ -201,17 +91,18 @@ __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sy
 
 __global__ void __launch_bounds__(AT_THREADS, 1)
 attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                    const __grid_constant__ CUtensorMap map_k2, const __grid_constant__ CUtensorMap map_v2, const AttnTcArgs a) {
+                    const __grid_constant__ CUtensorMap map_k2, const __grid_constant__ CUtensorMap map_v2, const AttnWork a) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) unsigned long long bars[2 * AT_MAX_SLOTS + 12];
     __shared__ uint32_t tmem_base_sh;
-    __shared__ int abort_sh, k_sh, per_sh, ranges_sh;
+    __shared__ int abort_sh, ranges_sh;
+    __shared__ Cut cut_sh;
     __shared__ float xch_sh[2][2][128];                 // exchange between the two warps of a lane quarter: [parity][half][row]
 
     RUN_FLAG_EXIT(a.run_flag);
     PDL_TRIGGER();
     const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
-    const int NS = a.ring_slots, grp = a.H / a.Hkv;
+    const int NS = a.ring_slots;
     // staged queries first (the MMA reads 128 rows from each 64-dim chunk: what lies behind the live rows is the ring)
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, qchunk = (uint32_t)a.rows8 * 128u;
     const uint32_t qsm = base, ring = base + 4 * qchunk;
@@ -236,35 +127,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 2) {
-        // The cut: a lane per candidate k, and the even cut on the last lane.  Costs are summed over one-stream and two-stream
-        // layers, as the model has them, so that both kinds of launch choose alike.  (Per pair: 8 kv heads of one sequence, 17
-        // tiles each: 9 ranges; 32 pairs: 4; 128 pairs on 148 CTAs: whole pairs, where an even cut would have two items and a
-        // merge per CTA.  Even: 160 pairs of 65 tiles.)
-        int T = 0, tmax = 1;
-        for (int b = lane; b < a.batch; b += 32) {
-            const int tb = (a.len_eff[b] + a.M + TKEYS - 1) / TKEYS;
-            T += tb;
-            tmax = max(tmax, tb);
-        }
-        T = __reduce_add_sync(0xffffffffu, T) * a.Hkv * a.subs;
-        tmax = __reduce_max_sync(0xffffffffu, tmax);
-        const int G = gridDim.x, P = a.batch * a.Hkv * a.subs, kmax = max(1, min(MAX_SPLITS, a.slots)), k = lane + 1;
-        // even cut: no pair in more ranges than it has slots
-        const int per = a.slots < 2 ? T : max((T + G - 1) / G, (tmax + a.slots - 2) / (a.slots - 1)), ranges = (T + per - 1) / per;
-        int cost = 1 << 26;
-        if (k <= kmax && (a.splits == 0 || k == min(a.splits, kmax))) {
-            const int item = (tmax + k - 1) / k + COST_ITEM, merge = k > 1 ? COST_MERGE : 0;
-            cost = a.w_one * ((P * k + G - 1) / G * item + merge) + a.w_two * ((2 * P * k + G - 1) / G * item + merge);
-        } else if (lane == 31 && a.splits == 0 && a.slots >= 2) {
-            const int share = per + 2 * COST_ITEM;
-            cost = a.w_one * (share + COST_MERGE) + a.w_two * ((2 * ranges <= G ? share : 2 * share) + COST_MERGE);
-        }
-        const unsigned best = __reduce_min_sync(0xffffffffu, ((unsigned)min(cost, 1 << 26) << 5) + lane) & 31u;
-        if (lane == 0) {
-            k_sh = best == 31 ? 0 : best + 1;
-            per_sh = best == 31 ? per : (a.streams * P * ((int)best + 1) + G - 1) / G;
-            ranges_sh = ranges;
-        }
+        Cut c;
+        int n;
+        choose_cut(a, lane, c, n);
+        if (lane == 0) { cut_sh = c; ranges_sh = n; }
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_sh)), "r"(512) : "memory");
@@ -274,7 +140,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = uniform(tmem_base_sh);
-    const Cut cut{uniform(k_sh), uniform(per_sh)};
+    const Cut cut{uniform(cut_sh.k), uniform(cut_sh.per)};
     const int ranges = uniform(ranges_sh);
     ItemSrc src;
     src_init(a, cut, ranges, src);
@@ -389,21 +255,16 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             ++x_cnt;
             return done;
         };
-        // a query row's place in q and in the output
-        auto row_off = [&](const Item &i, int r) -> size_t {
-            const int g2 = i.row0 + r, hq = (int)((g2 * a.m_recip) >> 32);
-            return ((size_t)(i.be * a.M + g2 - hq * a.M) * a.H + i.kvh * grp + hq) * HD;
-        };
         while (ok && next_item(a, cut, src, it)) {
             const bool live = trow < it.rows, warp_live = quarter * 32 < it.rows;
-            const size_t o0 = row_off(it, live ? trow : 0);
+            const size_t o0 = row_off(a, it, live ? trow : 0);
             const int g0 = it.row0 + (live ? trow : 0);
             const unsigned long long anc = a.tree[it.b].anc[g0 - (int)((g0 * a.m_recip) >> 32) * a.M];
             // stage the item's query rows as bf16 hi / lo planes, pre-scaled, in the K-major 128-byte-swizzled layout the MMA
             // reads; a warp takes whole rows, all its loads in flight (addresses first: they do not wait for anything)
             uint32_t qrow[QROWS];
 #pragma unroll
-            for (int q = 0; q < QROWS; ++q) qrow[q] = (uint32_t)(row_off(it, min(sw + q * SW, it.rows - 1)) >> 2) + lane;
+            for (int q = 0; q < QROWS; ++q) qrow[q] = (uint32_t)(row_off(a, it, min(sw + q * SW, it.rows - 1)) >> 2) + lane;
             if (first) PDL_WAIT();
             else if (!(ok = wg_sync())) break;                   // the rows staged in the query region have been written out
             first = false;
@@ -591,7 +452,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(at_ml + (uint32_t)s * (step >> 1)), "l"(from_ml) : "memory");
                     from += part_floats; from_ml += part_floats;
                 }
-                __nv_bfloat16 *dst = a.out + row_off(it, r0 + row) + 4 * sw;
+                __nv_bfloat16 *dst = a.out + row_off(a, it, r0 + row) + 4 * sw;
                 asm volatile("cp.async.wait_all;" ::: "memory");
                 const uint8_t *pieces = q_gen + (at - qsm);
                 float2 *ml = reinterpret_cast<float2 *>(q_gen + (at_ml - qsm));
@@ -675,27 +536,12 @@ int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool sli
         if ((rc = cache_maps_tc(m, *cm2, kc2, vc2, m->n_routed))) return rc;
     }
     const int QR = c.n_heads / c.n_kv_heads * M;
-    AttnTcArgs a;
+    AttnWork a;
     a.subs = (QR + 127) / 128;
     a.rows_sub = a.subs == 1 ? QR : ((QR + a.subs - 1) / a.subs + 7) / 8 * 8;
     a.subs = (QR + a.rows_sub - 1) / a.rows_sub;
-    a.rows8 = (a.rows_sub + 7) / 8 * 8;
-    a.q = m->ws.q; a.part = m->ws.part; a.out = (__nv_bfloat16 *)m->ws.attn;
-    a.out_plane = m->ws.rows_alloc * (size_t)c.n_heads * HD;
-    a.len_eff = m->ws.len_eff; a.tree = m->ws.tree; a.status = &m->ws.stats->device_status; a.run_flag = m->run_flag;
-    a.M = M; a.H = c.n_heads; a.Hkv = c.n_kv_heads; a.max_batch = c.max_batch; a.max_ctx = c.max_ctx;
-    a.layer_ord = layer_ord; a.scale = 1.4426950408889634f / sqrtf((float)HD);   // log2(e) / sqrt(hd)
-    a.batch = batch; a.layer_ord2 = layer_ord2; a.streams = streams;
-    a.counters = m->ws.attn_counters;
-    // (always counted for two streams: the cuts must not depend on how many a launch has)
-    const size_t slot_bytes = (size_t)2 * batch * c.n_kv_heads * a.subs * a.rows8 * PART_ROW * sizeof(float);
-    const size_t fit = m->ws.part_bytes / slot_bytes;
-    a.slots = fit > MAX_SLOTS ? MAX_SLOTS : (int)fit;
-    a.splits = m->opt.attn_splits;
-    a.w_one = c.n_layers - m->n_routed; a.w_two = m->n_routed;
-    a.m_recip = ((1ull << 32) + M - 1) / M;
-    int grid = m->sm_count;
-    if (m->opt.tk_grid >= 1 && m->opt.tk_grid < grid) grid = m->opt.tk_grid;     // tests: long ranges per CTA on small cases
+    fill_work(m, a, layer_ord, layer_ord2, streams, batch, M);
+    const int grid = work_grid(m);
     const size_t q_bytes = (size_t)a.rows8 * 512, smem_max = 229000;
     a.ring_slots = (int)((smem_max - 1024 - q_bytes) / SLOT_BYTES);
     if (a.ring_slots > AT_MAX_SLOTS) a.ring_slots = AT_MAX_SLOTS;

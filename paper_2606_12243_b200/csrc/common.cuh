@@ -241,8 +241,7 @@ int launch_attention(viasd_model *m, const void *kc, const void *vc, bool slim, 
 // attention_mma.cu
 int attention_mma_supported(const viasd_model *m, int M);
 int launch_attention_mma(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, const void *kc2,
-                         const void *vc2, int layer_ord2, int streams, int batch, int M, int nsplit, int fuse_merge,
-                         cudaStream_t st);
+                         const void *vc2, int layer_ord2, int streams, int batch, int M, cudaStream_t st);
 int attention_tensor_supported(const viasd_model *m);
 int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, const void *kc2,
                          const void *vc2, int layer_ord2, int streams, int batch, int M, cudaStream_t st);

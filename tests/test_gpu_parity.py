@@ -203,6 +203,18 @@ def test_rows_on_lanes_attention_edges(nodes, batch, ctx, env, monkeypatch):
     _check_rows(replace(base, batch=batch, ctx=ctx, parent=W.chain(nodes), shape=replace(base.shape, n_layers=2), n_routed=1))
 
 
+# The mma.sync kernel likewise: 2 to 16 rows, contexts that end on a tile and one past it, no context, each way of cutting.
+@pytest.mark.parametrize("nodes,batch,ctx,env", [(8, 1, 0, {}), (15, 2, 112, {}), (15, 1, 113, {}), (1, 1, 1500, {}),
+                                                 (3, 3, 700, {"VIASD_ATTN_NSPLIT": "3"}), (8, 2, 500, {"VIASD_ATTN_NSPLIT": "1"}),
+                                                 (8, 6, 700, {"VIASD_TK_GRID": "3"})])
+def test_few_rows_attention_edges(nodes, batch, ctx, env, monkeypatch):
+    monkeypatch.setenv("VIASD_ATTN", "mma")
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
+    base = W.get("mini_7b")
+    _check_rows(replace(base, batch=batch, ctx=ctx, parent=W.chain(nodes), shape=replace(base.shape, n_layers=2), n_routed=1))
+
+
 def test_forward_is_deterministic_and_slim_all_layers_equals_full():
     wl = replace(W.get("mini_8b_tree"), n_routed=W.get("mini_8b_tree").shape.n_layers, name="mini_8b_tree")
     vb = _vb()
