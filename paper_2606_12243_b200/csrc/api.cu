@@ -723,7 +723,9 @@ int viasd_gemm(const void *x, const void *w, float *y, int rows, int n, int k, i
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if (sms > MAX_SMS) sms = MAX_SMS;
     const size_t counter_bytes = align_up((size_t)(tc_tiles(n) + 1) * 4, 256);
-    CUDA_TRY(cudaMemsetAsync(scratch, 0, counter_bytes, st));       // tile counters and the status word
+    // tile counters and the status word.  By a kernel that lets the product's launch overlap it: behind a memset the product
+    // waited for its end before it set up or asked for a weight (41 x 13824 x 5120: 35.0 -> 34.7 us).
+    if (int e = launch_clear_words((int *)scratch, tc_tiles(n) + 1, st)) return e;
     CUtensorMap mw, mx;
     int rc;
     const uint32_t wbox = tc_box_rows(n, 128);

@@ -49,7 +49,7 @@ extern "C" int viasd_gemm_static(const void *x, const void *w, float *y, int row
     if (sms > STATIC_CTAS) sms = STATIC_CTAS;
     char *base = (char *)g_scratch_ptr[dev];
     // the array keeps whatever the last call left: counters and the status word must start at zero
-    CUDA_TRY(cudaMemsetAsync(base, 0, STATIC_COUNTER_BYTES, st));
+    if (int e = launch_clear_words((int *)base, (int)(STATIC_COUNTER_BYTES / 4), st)) return e;
     CUtensorMap mw, mx;
     int rc;
     const uint32_t wbox = tc_box_rows(n, 128), xbox = tc_box_rows(rows, 16);

@@ -551,6 +551,18 @@ void tc_fill_params(const TcLaunch &L, TcParams &p) {
     p.kv_keep = L.kv_keep;
 }
 
+// Ordinary launch (everything before it is done), but it lets the product behind it start at once: that one asks for weights
+// and waits for this only before it touches the counters.
+static __global__ void clear_words_kernel(int *words, int n) {
+    PDL_TRIGGER();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) words[i] = 0;
+}
+int launch_clear_words(int *words, int n, cudaStream_t st) {
+    clear_words_kernel<<<1, 256, 0, st>>>(words, n);
+    LAUNCH_CHECK();
+    return VIASD_OK;
+}
+
 int launch_gemm_tc(const TcLaunch &L, cudaStream_t st) {
     TcParams p;
     tc_fill_params(L, p);

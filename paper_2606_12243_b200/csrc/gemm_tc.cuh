@@ -73,6 +73,7 @@ uint32_t tc_box_rows(uint64_t tensor_rows, uint32_t want);
 size_t tc_scratch_floats(int sm_count, int nt, bool dual);
 int tc_tiles(int n);
 int launch_gemm_tc(const TcLaunch &L, cudaStream_t st);
+int launch_clear_words(int *words, int n, cudaStream_t st);   // counters of a stand-alone product
 // gemm_wide.cu: pairs of CTAs, up to 256 token rows; L.nt = tc_wide_th(rows), gate/up maps with 64-row boxes
 constexpr int TC_WIDE_ROWS = 256;
 // Token rows of one verifier from which a pass runs on the pair kernel (the choice may not depend on whether the other
