@@ -455,7 +455,7 @@ def run_sweep(main: Bench, peak: float, tf_peak: float, n: int) -> dict:
         b = Bench(wl, weights_from=share, fill_context="device")
         sb = RL.step_bytes(wl)
         rec = {"config": config_of(wl)}
-        step_bytes = sb["total_shared"] if 2 * wl.batch * wl.rows <= 128 else sb["total"]
+        step_bytes = sb["total_shared"] if RL.runs_one_sweep(wl) else sb["total"]
         for cname, fn, nbytes, flops in (("verify_step", b.verify_step, step_bytes, sb["flops"]),
                                          ("full_forward", b.full_forward, sb["full"]["total"], sb["full"]["flops"]),
                                          ("slim_forward", b.slim_forward, sb["slim"]["total"], sb["slim"]["flops"])):
@@ -579,7 +579,7 @@ def run_ours(args, wl) -> None:
 
     peak, tf_peak, peak_kind = measured_peaks()
     sb = RL.step_bytes(wl)
-    one_sweep = 2 * wl.batch * wl.rows <= 128
+    one_sweep = RL.runs_one_sweep(wl)
     # When both verifiers' rows fit one launch, verify_step streams every layer's weights once and applies the routed
     # layers to both row streams: the bytes its GEMM launches move are the "shared" figure.
     gemm_bytes = sb["gemm_shared"] if one_sweep else sb["gemm"]

@@ -97,6 +97,13 @@ NCU_GEMM_TRAFFIC_MB = {
 }
 
 
+def runs_one_sweep(wl) -> bool:
+    """Whether a verify step runs both verifiers in one sweep over the layers: their rows fit one launch of the GEMM (128 rows, 256 for the
+    pair kernel, which takes over at 48 rows per verifier)."""
+    rows = wl.batch * wl.rows
+    return 2 * rows <= (256 if rows >= 48 else 128)
+
+
 def gemm_traffic(wl: Workload):
     """Measured DRAM bytes of the step's GEMM launches: per-launch ncu figures of the workload's layer shapes scaled
     by the launches of the step (traffic is per launch, and every layer launches the same shapes).  None when a
@@ -104,7 +111,7 @@ def gemm_traffic(wl: Workload):
     s = wl.shape
     qd, kvd = s.n_heads * s.head_dim, s.n_kv_heads * s.head_dim
     shapes = [(qd + 2 * kvd, s.d_model), (s.d_model, qd), (2 * s.d_ff, s.d_model), (s.d_model, s.d_ff)]
-    one_sweep = 2 * wl.batch * wl.rows <= 128
+    one_sweep = runs_one_sweep(wl)
     layer_launches = s.n_layers if one_sweep else s.n_layers + wl.n_routed
     head_launches = 1 if one_sweep else 2
     total = 0.0
