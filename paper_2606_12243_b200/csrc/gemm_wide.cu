@@ -333,49 +333,59 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
                 gain_a = __ldg(reinterpret_cast<const float4 *>(p.next_gain + tile * TILE_F + 4 * lane));
                 gain_b = p.next_gain2 ? __ldg(reinterpret_cast<const float4 *>(p.next_gain2 + tile * TILE_F + 4 * lane)) : gain_a;
             }
-            // The other contributors' rows are read where they are, a row per warp: 16-byte loads, up to four contributors of
-            // two rows in flight, asked for before the chunk's trip through shared memory (staged in the idle ring by
-            // bulk copies first: 13B batch 8 step 6.70 ms, now 6.37; 8B tree batch 4 7.15, now 6.98).
+            // The other contributors' rows are read where they are, a row per warp: 16-byte loads, four contributors of two rows
+            // in flight, a chunk ahead (staged in the idle ring by bulk copies first: 13B batch 8 step 6.70 ms, then 6.37; 8B
+            // tree batch 4 7.15, then 6.98; a chunk's loads only when its turn came and contributors past the fourth row by
+            // row, a trip to L2 each: 8B batch 4 6.72, now 6.57; prompt chunk 25.1, now 24.5).
             const int others = n_c - 1;
-            auto slot_of = [&](int c) {                            // contributor c's partial of this tile
-                const int cp = first + c, c_first = (cp * p.units_per_cta) / p.k_tiles;
-                return p.scratch + ((size_t)(2 * cp + (int)rank) * 2 + (c_first == sg.tile ? 0 : 1)) * slot_floats + 4 * lane;
+            // contributor c's partial of this tile: its first piece of work, but for a first contributor that came from the tile before
+            auto slot_of = [&](int c) {
+                const int second = c == 0 && first * p.units_per_cta < sg.tile * p.k_tiles;
+                return p.scratch + ((size_t)(2 * (first + c) + (int)rank) * 2 + second) * slot_floats + 4 * lane;
             };
-#pragma unroll 1
-            for (int r0 = row_begin + group * CH; r0 < row_end; r0 += WGROUPS * CH) {
-                const int ra = r0 + 2 * gw;                        // this warp's two rows of the chunk
-                float4 part[4][2];
+            float4 part[4][2];
+            auto load_part = [&](int c0, int ra) {
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
-                    if (c < n_c && c != mine) {
-                        const float *from = slot_of(c);
+                    if (c0 + c < n_c && c0 + c != mine && ra < row_end) {
+                        const float *from = slot_of(c0 + c);
 #pragma unroll
                         for (int i = 0; i < 2; ++i)
                             part[c][i] = __ldcg(reinterpret_cast<const float4 *>(from + (size_t)min(ra + i, p.rows - 1) * TILE_F));
                     }
                 }
+            };
+            load_part(0, row_begin + group * CH + 2 * gw);
+#pragma unroll 1
+            for (int r0 = row_begin + group * CH; r0 < row_end; r0 += WGROUPS * CH) {
+                const int ra = r0 + 2 * gw;                        // this warp's two rows of the chunk
                 float g[CH];
                 load_chunk(r0, g);
                 group_sync();                                      // the group has read its previous chunk
 #pragma unroll
                 for (int j = 0; j < CH; ++j) xg[j * TILE_F + f] = g[j];
                 group_sync();
+                float4 v[2];
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const int r = ra + i;
-                    if (r >= p.rows) continue;
-                    const float4 own = *reinterpret_cast<const float4 *>(xg + (2 * gw + i) * TILE_F + 4 * lane);
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (others == 0) {
-                        v = own;
-                    } else {                                       // in pair order, whoever adds them
+                for (int i = 0; i < 2; ++i) v[i] = *reinterpret_cast<const float4 *>(xg + (2 * gw + i) * TILE_F + 4 * lane);
+                if (others > 0) {                                  // in pair order, whoever adds them
+                    const float4 own[2] = {v[0], v[1]};
+                    v[0] = v[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+                    for (int c0 = 0; c0 < n_c; c0 += 4) {
+                        if (c0 > 0) load_part(c0, ra);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) if (c < n_c) v = add4(v, c == mine ? own : part[c][i]);
-                        for (int c = 4; c < n_c; ++c)
-                            v = add4(v, c == mine ? own : __ldcg(reinterpret_cast<const float4 *>(slot_of(c) + (size_t)r * TILE_F)));
+                        for (int c = 0; c < 4; ++c)
+#pragma unroll
+                            for (int i = 0; i < 2; ++i)
+                                if (c0 + c < n_c) v[i] = add4(v[i], c0 + c == mine ? own[i] : part[c][i]);
                     }
-                    finish_row<EPI, true>(p, tile, r, true, v, make_float4(0.f, 0.f, 0.f, 0.f), aux[i][0], aux[i][1], gain_a, gain_b, inv_sh, rowmeta, lane);
+                    load_part(0, ra + WGROUPS * CH);
                 }
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    if (ra + i < p.rows)
+                        finish_row<EPI, true>(p, tile, ra + i, true, v[i], make_float4(0.f, 0.f, 0.f, 0.f), aux[i][0], aux[i][1], gain_a, gain_b, inv_sh, rowmeta, lane);
                 load_aux(r0 + WGROUPS * CH, row_end);
             }
             // this tile's accumulator may be overwritten
