@@ -24,7 +24,12 @@
 namespace {
 
 constexpr int WARPS = 8;
-constexpr int RING = 5;                        // slots of one K or V tile; beside them the merge buffer's 64 KB
+// Slots of one K or V tile; beside them the merge buffer's 64 KB.  Even and odd tiles go to different groups of warps with
+// no step in common, and a parity wait is only good for a warp that has waited for the slot's use before: so every use of
+// a slot belongs to one group.  (With five slots tile 3's K had the slot of tile 0's V: had that V landed after tile 1, the odd
+// group would have taken it for its K.)
+constexpr int RING = 4;
+static_assert(RING % 4 == 0, "a slot's uses alternate between the groups of warps");
 
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
