@@ -26,6 +26,8 @@
  *   - A block has N draft nodes and M = N + 1 rows per sequence: row 0 is the pending token (the last
  *     emitted token, whose K/V is not cached yet), row n + 1 is draft node n.  The logits of a row are
  *     the next-token distribution for that row's children.  M <= 64.
+ *   - Weight matrices (lm_head among them), viasd_gemm's operands and, in bf16 models with head_dim 128, the KV caches are
+ *     16-byte aligned (EINVAL otherwise), the workspace 256; every other array only to its element.
  *   - Matrices are row-major [out, in].  dtype 0 = fp32, 1 = bf16 applies to weights and KV caches;
  *     norm gains, logits and the residual stream are fp32.
  */

@@ -372,6 +372,7 @@ int viasd_init_model(const viasd_config *cfg, const viasd_weights *w, const unsi
     if (((uintptr_t)workspace & 255) != 0) return VIASD_EINVAL;
     if (!w->embed || !w->lm_head || !w->final_norm || !w->wq || !w->wk || !w->wv || !w->wo || !w->wg || !w->wu ||
         !w->wd || !w->norm1 || !w->norm2) return VIASD_EINVAL;
+    if ((uintptr_t)w->lm_head & 15) return VIASD_EINVAL;
     if (workspace_bytes < carve(*cfg, nullptr, nullptr)) return VIASD_ECAPACITY;
     int dev = 0, major = 0, sms = 0;                             // (two attributes: the whole property record takes milliseconds)
     CUDA_TRY(cudaGetDevice(&dev));

@@ -7,6 +7,7 @@
 #include "common.cuh"
 #include <string.h>
 #include <stdlib.h>
+#include <type_traits>
 
 namespace {
 
@@ -14,7 +15,8 @@ constexpr int TK = 32;          // keys per shared-memory tile
 constexpr int QG = 16;          // query rows per CTA (2 per warp, 8 warps)
 constexpr int ATT_WARPS = 8;
 
-template <typename T, int HD>
+// VEC: K and V are aligned to 16 bytes (the caller's caches need not be)
+template <typename T, int HD, bool VEC>
 __global__ void __launch_bounds__(ATT_WARPS * 32)
 attention_split_kernel(float *__restrict__ part, const float *__restrict__ q, const T *__restrict__ kc,
                        const T *__restrict__ vc, const int *__restrict__ len_eff, const TreeInfo *__restrict__ tree,
@@ -63,26 +65,31 @@ attention_split_kernel(float *__restrict__ part, const float *__restrict__ q, co
 
     for (int k0 = k_begin; k0 < k_end; k0 += TK) {
         __syncthreads();
-        // 16-byte loads, all of a thread's in flight together
-        constexpr int VE = 16 / sizeof(T), NV = TK * HD / VE / (ATT_WARPS * 32);
-        static_assert(NV * VE * ATT_WARPS * 32 == TK * HD, "whole pieces per thread");
-        uint4 kraw[NV], vraw[NV];
+        // 16-byte loads, all of a thread's in flight together; an element at a time where the caches are not aligned to that
+        constexpr int VE = VEC ? 16 / (int)sizeof(T) : 1, NV = VEC ? TK * HD / VE / (ATT_WARPS * 32) : 4;
+        constexpr int STEP = NV * VE * ATT_WARPS * 32;
+        using Piece = typename std::conditional<VEC, uint4, T>::type;
+        static_assert(TK * HD % STEP == 0, "whole pieces per thread");
+#pragma unroll 1
+        for (int at = 0; at < TK * HD; at += STEP) {
+            Piece kraw[NV], vraw[NV];
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            const int idx = (threadIdx.x + q * ATT_WARPS * 32) * VE, j = idx / HD;
-            const size_t o = cbase + (size_t)min(k0 + j, k_end - 1) * HD + idx % HD;
-            kraw[q] = *reinterpret_cast<const uint4 *>(kc + o);
-            vraw[q] = *reinterpret_cast<const uint4 *>(vc + o);
-        }
+            for (int q = 0; q < NV; ++q) {
+                const int idx = at + (threadIdx.x + q * ATT_WARPS * 32) * VE, j = idx / HD;
+                const size_t o = cbase + (size_t)min(k0 + j, k_end - 1) * HD + idx % HD;
+                kraw[q] = *reinterpret_cast<const Piece *>(kc + o);
+                vraw[q] = *reinterpret_cast<const Piece *>(vc + o);
+            }
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            const int idx = (threadIdx.x + q * ATT_WARPS * 32) * VE, j = idx / HD, dd = idx % HD;
-            const bool in = k0 + j < k_end;
-            T kv[VE], vv[VE];
-            *reinterpret_cast<uint4 *>(kv) = kraw[q];
-            *reinterpret_cast<uint4 *>(vv) = vraw[q];
+            for (int q = 0; q < NV; ++q) {
+                const int idx = at + (threadIdx.x + q * ATT_WARPS * 32) * VE, j = idx / HD, dd = idx % HD;
+                const bool in = k0 + j < k_end;
+                alignas(16) T kv[VE], vv[VE];
+                *reinterpret_cast<Piece *>(kv) = kraw[q];
+                *reinterpret_cast<Piece *>(vv) = vraw[q];
 #pragma unroll
-            for (int e = 0; e < VE; ++e) { Ks[j][dd + e] = in ? to_f32<T>(kv[e]) : 0.f; Vs[j][dd + e] = in ? to_f32<T>(vv[e]) : 0.f; }
+                for (int e = 0; e < VE; ++e) { Ks[j][dd + e] = in ? to_f32<T>(kv[e]) : 0.f; Vs[j][dd + e] = in ? to_f32<T>(vv[e]) : 0.f; }
+            }
         }
         __syncthreads();
 #pragma unroll
@@ -154,7 +161,8 @@ int run(const viasd_model *m, const void *kc, const void *vc, int layer_ord, int
     const int grp = c.n_heads / c.n_kv_heads;
     const int qgroups = (grp * M + QG - 1) / QG;
     dim3 grid(batch * c.n_kv_heads, nsplit, qgroups);
-    CUDA_TRY(launch_chained(attention_split_kernel<T, HD>, grid, ATT_WARPS * 32, st, m->ws.part, m->ws.q, (const T *)kc,
+    const bool vec = (((uintptr_t)kc | (uintptr_t)vc) & 15) == 0;
+    CUDA_TRY(launch_chained(vec ? attention_split_kernel<T, HD, true> : attention_split_kernel<T, HD, false>, grid, ATT_WARPS * 32, st, m->ws.part, m->ws.q, (const T *)kc,
         (const T *)vc, m->ws.len_eff, m->ws.tree, M, c.n_heads, c.n_kv_heads, c.max_batch, c.max_ctx, layer_ord, nsplit,
         1.0f / sqrtf((float)HD), m->run_flag));
     LAUNCH_CHECK();

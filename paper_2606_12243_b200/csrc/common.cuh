@@ -283,6 +283,12 @@ template <> __device__ __forceinline__ void store_act<__nv_bfloat16>(__nv_bfloat
     if (plane) buf[plane + idx] = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
 
+// four floats of a caller's array (norm gains), which need only be aligned to a float
+__device__ __forceinline__ float4 load_floats4(const float *p) {
+    if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) return __ldg(reinterpret_cast<const float4 *>(p));
+    return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -198,8 +198,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
         float4 gain_a = make_float4(0.f, 0.f, 0.f, 0.f), gain_b = gain_a;
         auto load_gain = [&](int tile) {
             if (EPI != EPI_ADD_NORM) return;
-            gain_a = __ldg(reinterpret_cast<const float4 *>(p.next_gain + tile * TILE_F + 4 * lane));
-            gain_b = p.next_gain2 ? __ldg(reinterpret_cast<const float4 *>(p.next_gain2 + tile * TILE_F + 4 * lane)) : gain_a;
+            gain_a = load_floats4(p.next_gain + tile * TILE_F + 4 * lane);
+            gain_b = p.next_gain2 ? load_floats4(p.next_gain2 + tile * TILE_F + 4 * lane) : gain_a;
         };
         load_gain(last_tile);
 

@@ -330,8 +330,8 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
             }
             float4 gain_a = make_float4(0.f, 0.f, 0.f, 0.f), gain_b = gain_a;
             if (EPI == EPI_ADD_NORM && row_begin < row_end) {
-                gain_a = __ldg(reinterpret_cast<const float4 *>(p.next_gain + tile * TILE_F + 4 * lane));
-                gain_b = p.next_gain2 ? __ldg(reinterpret_cast<const float4 *>(p.next_gain2 + tile * TILE_F + 4 * lane)) : gain_a;
+                gain_a = load_floats4(p.next_gain + tile * TILE_F + 4 * lane);
+                gain_b = p.next_gain2 ? load_floats4(p.next_gain2 + tile * TILE_F + 4 * lane) : gain_a;
             }
             // The other contributors' rows are read where they are, a row per warp: 16-byte loads, four contributors of two rows
             // in flight, a chunk ahead (staged in the idle ring by bulk copies first: 13B batch 8 step 6.70 ms, then 6.37; 8B

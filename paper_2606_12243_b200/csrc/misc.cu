@@ -227,7 +227,6 @@ rmsnorm_kernel(T *a, size_t plane, const float *h, const float *gain, int d, flo
     PDL_WAIT();
     const int r = blockIdx.x;
     const float4 *x4 = reinterpret_cast<const float4 *>(h + (size_t)r * d);
-    const float4 *g4 = reinterpret_cast<const float4 *>(gain);
     constexpr int MAXV = 8;                           // up to 8 float4 per thread: d <= 8192 stays in registers
     const int nv = d >> 2;
     float4 v[MAXV];
@@ -246,7 +245,7 @@ rmsnorm_kernel(T *a, size_t plane, const float *h, const float *gain, int d, flo
     for (int w = 0; w < 8; ++w) tot += red[w];
     const float inv = rsqrtf(tot / (float)d + eps);
     auto emit = [&](int i, float4 t) {
-        const float4 g = g4[i];
+        const float4 g = load_floats4(gain + 4 * i);
         const size_t o = (size_t)r * d + (size_t)i * 4;
         store_act<T>(a, plane, o, t.x * inv * g.x);
         store_act<T>(a, plane, o + 1, t.y * inv * g.y);
@@ -330,18 +329,20 @@ int launch_rope_append(const viasd_model *m, void *kc, void *vc, int layer_ord, 
 // ---------------------------------------------------------------------------------------------
 // KV commit: compact the accepted path, advance len / pending / tokens
 // ---------------------------------------------------------------------------------------------
-// A warp moves the path's rows of one (layer, sequence, kv head), K by its first half and V by its second, eight rows of
-// 16-byte loads in flight; the last CTA to finish advances the lengths (nobody reads them before).  (Three launches -
+// A warp moves the path's rows of one (layer, sequence, kv head), K by its first half and V by its second, eight rows in
+// flight, in pieces of 16 bytes where the caches are aligned to that (an fp32 cache, or one of head_dim 64, need not be), else
+// of one element; the last CTA to finish advances the lengths (nobody reads them before).  (Three launches -
 // lengths, rows one 2-byte column per thread and row after row, advance - were 15 to 27 us.)
 struct CommitArgs {
     void *kf, *vf, *ks, *vs;
     int *len, *len_full, *pending, *tokens;
     const int *n_acc, *path, *n_emit, *out_tok;
     DeviceStats *stats;
-    int B, N, L, Ls, layer0, Hkv, row_vecs, max_batch, max_ctx, slim_only;   // row_vecs: 16-byte pieces of a K (or V) row
+    int B, N, L, Ls, layer0, Hkv, row_vecs, max_batch, max_ctx, slim_only;   // row_vecs: pieces of a K (or V) row
 };
 constexpr int COMMIT_WARPS = 8;
 
+template <typename Piece>
 __global__ void __launch_bounds__(32 * COMMIT_WARPS) commit_kernel(const CommitArgs a) {
     __shared__ int last_sh;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, M = a.N + 1;
@@ -352,7 +353,7 @@ __global__ void __launch_bounds__(32 * COMMIT_WARPS) commit_kernel(const CommitA
         const bool is_full = layer < a.L;
         if (full_ran || !is_full) {                            // else the full verifier's cache did not receive this block
             const int half = lane >> 4, l16 = lane & 15;
-            uint4 *base = reinterpret_cast<uint4 *>(is_full ? (half ? a.vf : a.kf) : (half ? a.vs : a.ks)) +
+            Piece *base = reinterpret_cast<Piece *>(is_full ? (half ? a.vf : a.kf) : (half ? a.vs : a.ks)) +
                           (((size_t)(is_full ? layer : layer - a.L) * a.max_batch + b) * a.Hkv + g) * (size_t)a.max_ctx * a.row_vecs;
             const int n = clamped_len(a.len, b, a.max_ctx, M, a.stats), na = min(a.n_acc[b], a.N);
             // a path's nodes never come before their position (node >= j), so rows only move down and no row that is still to
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(32 * COMMIT_WARPS) commit_kernel(const CommitA
                     src[j] = more && node != j0 + j ? n + 1 + node : -1;
                 }
                 for (int c = l16; c < a.row_vecs; c += 16) {
-                    uint4 v[8];
+                    Piece v[8];
 #pragma unroll
                     for (int j = 0; j < 8; ++j) if (src[j] >= 0) v[j] = base[(size_t)src[j] * a.row_vecs + c];
 #pragma unroll
@@ -412,10 +413,13 @@ int launch_commit(const viasd_model *m, viasd_cache *c, const viasd_draft *d, co
     a.n_acc = r->n_acc; a.path = r->path; a.n_emit = r->n_emit; a.out_tok = r->out_tok;
     a.stats = m->ws.stats;
     a.B = d->batch; a.N = d->n_nodes; a.L = cf.n_layers; a.Ls = m->n_routed; a.layer0 = slim_only ? cf.n_layers : 0;
-    a.Hkv = cf.n_kv_heads; a.row_vecs = cf.head_dim * (cf.dtype == 0 ? 4 : 2) / 16;
+    a.Hkv = cf.n_kv_heads; 
     a.max_batch = cf.max_batch; a.max_ctx = cf.max_ctx; a.slim_only = slim_only ? 1 : 0;
     const int items = (cf.n_layers + m->n_routed - a.layer0) * d->batch * cf.n_kv_heads;
-    commit_kernel<<<(items + COMMIT_WARPS - 1) / COMMIT_WARPS, 32 * COMMIT_WARPS, 0, st>>>(a);
+    const bool vec = (((uintptr_t)a.kf | (uintptr_t)a.vf | (uintptr_t)a.ks | (uintptr_t)a.vs) & 15) == 0;
+    auto kernel = vec ? commit_kernel<uint4> : cf.dtype == 0 ? commit_kernel<uint32_t> : commit_kernel<uint16_t>;
+    a.row_vecs = vec ? cf.head_dim * (cf.dtype == 0 ? 4 : 2) / 16 : cf.head_dim;
+    kernel<<<(items + COMMIT_WARPS - 1) / COMMIT_WARPS, 32 * COMMIT_WARPS, 0, st>>>(a);
     LAUNCH_CHECK();
     return VIASD_OK;
 }

@@ -1,0 +1,66 @@
+"""GPU tests of calls at the edges of what the entry points take, each compared with the ordinary form of the same call."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+
+from synth import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def _vb():
+    from paper_2606_12243_b200 import binding
+    return binding
+
+
+def _engine(wl, **kw):
+    from paper_2606_12243_b200.engine import Engine
+    eng = Engine(wl, fill_context="device", **kw)
+    eng.set_inputs(W.step_inputs(wl))
+    return eng
+
+
+def _shifted(t):
+    """The same values one element off a 16-byte boundary."""
+    s = torch.empty(t.numel() + 1, dtype=t.dtype, device=t.device)[1:].view(t.shape).copy_(t)
+    assert s.data_ptr() % 16 != 0
+    return s
+
+
+def _step(eng, model, cache, batch, nodes):
+    vb = _vb()
+    slim, full, res = eng.logits_buffer(), eng.logits_buffer(), vb.alloc_result(batch, nodes)
+    vb.verify_step(model, cache, eng.draft, eng.params(), slim, full, res)
+    torch.cuda.synchronize()
+    assert vb.get_stats(model).device_status == 0
+    return [slim, full, res.tier, res.n_acc, res.path, res.out_tok, res.n_emit, res.judge, res.corr_src]
+
+
+# ---------------------------------------------------------------------------------------------
+# arrays that need not be aligned beyond their element
+# ---------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("name,batch,head_dim", [("c1_tiny", None, None), ("mini_7b", None, None), ("mini_7b", 8, None), ("mini_7b", None, 64)])
+def test_gains_and_caches_need_no_alignment(name, batch, head_dim):
+    """Norm gains at an odd float offset (fp32 path, one-CTA GEMM, pair GEMM from 48 rows on, unfused bf16 path), and where
+    no tensor map is built over them (fp32, head_dim 64) caches at an odd element: same bits as aligned."""
+    vb = _vb()
+    base = W.get(name)
+    wl = replace(base, batch=batch or base.batch, shape=replace(base.shape, head_dim=head_dim or base.shape.head_dim))
+    eng = _engine(wl)
+    state = [t.clone() for t in (eng.k_full, eng.v_full, eng.k_slim, eng.v_slim, eng.len, eng.pending, eng.tokens, eng.len_full)]
+    want = _step(eng, eng.model, eng.cache, wl.batch, wl.n_nodes)
+    layers = [{k: _shifted(v) if k.startswith("norm") else v for k, v in l.items()} for l in eng.layers]
+    ws = torch.empty_like(eng.workspace)
+    assert ws.data_ptr() % 256 == 0
+    mask = [int(l in eng.routed) for l in range(wl.shape.n_layers)]
+    model = vb.init_model(eng.cfg, eng.embed, eng.lm_head, _shifted(eng.final_norm), layers, mask, ws)
+    if wl.shape.dtype == "f32" or wl.shape.head_dim == 64:
+        state[:4] = [_shifted(t) for t in state[:4]]
+    got = _step(eng, model, vb.make_cache(*state), wl.batch, wl.n_nodes)
+    for w, g in zip(want, got):
+        assert torch.equal(w, g)
+    for w, g in zip((eng.k_full, eng.v_full, eng.k_slim, eng.v_slim, eng.len, eng.pending, eng.tokens), state):
+        assert torch.equal(w, g)
