@@ -222,7 +222,7 @@ attention_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
     } else {
         const int g = lane >> 2, t2 = (lane & 3) * 2, r0 = (warp & 3) * 32;   // rows g, g + 8; first column; this warp's keys of its tiles
         const size_t part_floats = (size_t)a.rows8 * PART_ROW;
-        int c_tile = 0, wg_phase = 0, n_item = 0;                // tiles of earlier items
+        int c_tile = 0, wg_phase = 0, n_item = 0, arrived = 0, acked = 0;   // c_tile: tiles of earlier items
         bool ok = true;
         auto wg_sync = [&]() -> bool {
             __syncwarp();
@@ -338,6 +338,7 @@ attention_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
                 if (!(ok = wg_sync())) break;
                 // (the barrier orders the group's stores before this thread's release, which is cumulative)
                 if (threadIdx.x == 0) counter_arrive(a.counters + it.pair, it.n_split, it.n_split);
+                ++arrived;
             }
         }
         // ---- the split pairs of this CTA's list: its slice of each one's rows ----
@@ -345,7 +346,8 @@ attention_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
         while (ok && next_item(a, cut, src, it)) {
             if (it.n_split == 1) continue;
             if (threadIdx.x == 0) counter_wait(a.counters + it.pair, it.n_split, it.n_split, &abort_sh, a.status);
-            if (!(ok = wg_sync()) || *(volatile int *)&abort_sh) break;
+            ++acked;
+            if (!(ok = wg_sync())) break;
             const int rper = (it.rows + it.n_split - 1) / it.n_split, r_end = min(it.rows, (it.split + 1) * rper);
             const float *psrc = a.part + (size_t)it.pair * a.slots * part_floats;
 #pragma unroll 1
@@ -375,6 +377,7 @@ attention_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
                 store_row(a, row_off(a, it, row) + 4 * lane, v, inv);
             }
         }
+        if (!ok && threadIdx.x == 0) settle_counters(a, cut, ranges, arrived, acked);
     }
     __syncwarp();
     if (abort_sh && threadIdx.x == 0) {

@@ -238,6 +238,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         const uint32_t tlane = tmem + ((uint32_t)(quarter * 32) << 16);
         const size_t part_floats = (size_t)a.rows8 * PART_ROW;
         int s_cnt = 0, x_cnt = 0, wg_phase = 0;                  // tiles (buffer phase), exchanges, group barriers
+        int arrived = 0, acked = 0;                              // split pairs counted in and out
         bool ok = true, first = true;
         auto wg_sync = [&]() -> bool {
             __syncwarp();
@@ -425,6 +426,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 if (!(ok = wg_sync())) break;
                 // (the barrier orders the group's stores before this thread's release, which is cumulative)
                 if (et == 0) counter_arrive(a.counters + it.pair, it.n_split, it.n_split);
+                ++arrived;
             }
         }
         // ---- the split pairs of this CTA's list: its slice of each one's rows ----
@@ -432,7 +434,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         while (ok && next_item(a, cut, src, it)) {
             if (it.n_split == 1) continue;
             if (et == 0) counter_wait(a.counters + it.pair, it.n_split, it.n_split, &abort_sh, a.status);
-            if (!(ok = wg_sync()) || *(volatile int *)&abort_sh) break;
+            ++acked;
+            if (!(ok = wg_sync())) break;
             const int rper = (it.rows + it.n_split - 1) / it.n_split, r0 = min(it.rows, it.split * rper), nr = min(it.rows, r0 + rper) - r0;
             const float *psrc = a.part + (size_t)it.pair * a.slots * part_floats;
             // A lane takes a row, a warp every eighth group of dims.  All its pieces (16 bytes of a range's row) come into the idle
@@ -491,6 +494,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 }
             }
         }
+        if (!ok && et == 0) settle_counters(a, cut, ranges, arrived, acked);
     }
 
     // ---------------- teardown ----------------

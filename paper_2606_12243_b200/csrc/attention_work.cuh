@@ -9,6 +9,7 @@
 // and publish before they wait, so no wait depends on another.
 #pragma once
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace {
 
@@ -132,6 +133,19 @@ __device__ __forceinline__ void choose_cut(const AttnWork &a, int lane, Cut &cut
     cut.k = best == 31 ? 0 : (int)best + 1;
     cut.per = best == 31 ? per : (a.streams * P * ((int)best + 1) + G - 1) / G;
     n_ranges = ranges;
+}
+// A CTA that gave up (one thread): what it still owes the counters of its split pairs, `arrived` and `acked` of which it has
+// counted in and out, so that they are zero for the next launch and the other CTAs do not wait for this one.
+__device__ __forceinline__ void settle_counters(const AttnWork &a, const Cut &cut, int ranges, int arrived, int acked) {
+    ItemSrc src;
+    Item it;
+    src_init(a, cut, ranges, src);
+    for (int i = 0; next_item(a, cut, src, it); ) {
+        if (it.n_split == 1) continue;
+        if (i >= arrived) counter_arrive(a.counters + it.pair, it.n_split, it.n_split);
+        if (i >= acked) counter_ack(a.counters + it.pair, it.n_split, it.n_split);
+        ++i;
+    }
 }
 // a query row's place in q and in the output
 __device__ __forceinline__ size_t row_off(const AttnWork &a, const Item &i, int r) {

@@ -212,8 +212,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
         int acc_it = 0, u = u_begin, seg_i = 0;
         Seg sg;
         sg.tile = last_tile; sg.ka = 0; sg.kb = 0;                 // dry pass: the tile this CTA is most likely to finish
-        bool ok = true, dry = true;
-        while (ok) {
+        // A wait that expires does not end this loop: the epilogue's threads share barriers without a limit, so all of them go
+        // on through the same ones (no wait blocks any more, see counter_wait).
+        bool dry = true;
+        while (true) {
             int buf = 0, first_cta = blockIdx.x, n_c = 1;
             uint32_t t0 = 0;
             int row_begin = 0, row_end = dry ? 1 : p.rows;         // the rows this CTA finishes
@@ -255,7 +257,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
                 }
                 if (sg.tile != last_tile && row_begin < row_end) load_gain(sg.tile);
                 load_aux(row_begin + group * CH, row_end);
-                if (!(ok = mbar_wait(tfull_bar(buf), (acc_it / p.acc_bufs) & 1, &abort_sh, p.status))) break;
+                mbar_wait(tfull_bar(buf), (acc_it / p.acc_bufs) & 1, &abort_sh, p.status);
+                __syncwarp();
                 tc_fence_after();
                 t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * acc_cols;
                 if (!whole) {
@@ -297,7 +300,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_constant
                     if (!finisher) { ++acc_it; ++seg_i; continue; }
                     if (et == 0) counter_wait(p.counters + sg.tile, n_c, n_fin, &abort_sh, p.status);
                     epi_sync();
-                    if (abort_sh) { ok = false; break; }
                 }
             }
             // contributor c's partial of this tile: its first piece of work, but for a first contributor that came from the tile

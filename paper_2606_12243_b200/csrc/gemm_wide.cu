@@ -70,7 +70,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) unsigned long long bars[2 * WSTAGES + 4];
     __shared__ uint32_t tmem_base_sh;
-    __shared__ int abort_sh, tfull_ok[2];
+    __shared__ int abort_sh;
     __shared__ __align__(16) float xch[WGROUPS][CH * TILE_F];     // a chunk on its way from TMEM lanes to rows, per group
     __shared__ float inv_sh[WROWS];
     __shared__ int4 rowmeta[EPI == EPI_QKV_ROPE ? WROWS : 1];
@@ -254,16 +254,13 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
 
         int acc_it = 0, u = u_begin, seg_i = 0;
         Seg sg;
-        bool ok = true;
-        while (ok && next_seg(u, u_end, p.k_tiles, sg)) {
+        // (a wait that expires does not end this loop: all threads go on through the same barriers, none of which waits any
+        // more for another CTA, see counter_wait)
+        while (next_seg(u, u_end, p.k_tiles, sg)) {
             const int buf = acc_it % p.acc_bufs, tile = 2 * sg.tile + (int)rank;
             // one warp polls the barrier, the others sleep in a named barrier
-            if (warp == 2) {
-                const bool full = mbar_wait(tfull_bar(buf), (acc_it / p.acc_bufs) & 1, &abort_sh, p.status);
-                if (lane == 0) tfull_ok[acc_it & 1] = full;
-            }
+            if (warp == 2) mbar_wait(tfull_bar(buf), (acc_it / p.acc_bufs) & 1, &abort_sh, p.status);
             epi_sync();
-            if (!(ok = tfull_ok[acc_it & 1] != 0)) break;
             tc_fence_after();
             const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * acc_cols;
             // the sums of 8 token rows from r0 on, feature f: hi and lo products added
@@ -324,7 +321,6 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w0, const __grid_consta
                     if (finisher) {
                         if (et == 0) counter_wait(p.counters + tile, n_c, n_fin, &abort_sh, p.status);
                         epi_sync();
-                        if (abort_sh) { ok = false; break; }
                     }
                 }
             }

@@ -32,11 +32,25 @@ int launch_rope_table(const viasd_model *m, cudaStream_t st) {
 // finds its own token.  (As a kernel of its own in front of the embedding, and again in front of the commit, this was 7 us
 // each time, most of it the launch.)  What attention reads of it before its dependency wait - tree and length - is complete
 // because the pass's first QKV launch is an ordinary one: nothing after it starts before the embedding has ended.
+// Arrival counters of the GEMMs and of attention, zero between launches.  After a wait that expired they may not be: a pass
+// that finds the status word saying so starts from clean ones (nothing before it in the stream is still running).
+struct Counters { int *gemm, *attn; int n_gemm, n_attn; };
+__device__ __forceinline__ void clear_counters_if_failed(const Counters &c, const DeviceStats *stats, int thread, int threads) {
+    if (*reinterpret_cast<const volatile int *>(&stats->device_status) != VIASD_EDEVICE) return;
+    for (int i = thread; i < c.n_gemm; i += threads) c.gemm[i] = 0;
+    for (int i = thread; i < c.n_attn; i += threads) c.attn[i] = 0;
+}
+static Counters counters_of(const viasd_model *m) {
+    return Counters{m->ws.gemm_counters, m->ws.attn_counters, (int)m->ws.n_counters,
+                    (int)attn_counter_count(m->cfg.max_batch, m->cfg.n_heads, m->cfg.n_kv_heads)};
+}
+
 struct PrepArgs {
     TreeInfo *tree; int *len_eff; DeviceStats *stats;
     const int *len, *pending, *draft_tok, *parent;       // parent: [N] shared by the batch, or [B, N] when per_seq
     const int *row_tok;                                  // not null: a replay pass, whose preparation has run (no sequence CTAs)
     int per_seq, B, N, max_ctx, vocab, full_pass;
+    Counters counters;
 };
 __device__ __forceinline__ int prep_ctas(const PrepArgs &p) { return p.row_tok ? 0 : p.B; }
 __device__ __forceinline__ int clamped_len(const int *len, int b, int max_ctx, int M, DeviceStats *stats) {
@@ -45,6 +59,7 @@ __device__ __forceinline__ int clamped_len(const int *len, int b, int max_ctx, i
     return c;
 }
 __device__ __forceinline__ void prep_sequence(const PrepArgs &p, int b, int *par_sh) {       // by the CTA's first warp
+    if (b == 0) clear_counters_if_failed(p.counters, p.stats, threadIdx.x, 32);
     build_tree(p.tree + b, p.parent + (p.per_seq ? (size_t)b * p.N : 0), p.N, p.stats, par_sh);
     if (threadIdx.x == 0) {
         if (b == 0 && p.full_pass) p.stats->full_ran = 1;      // the full verifier's cache receives this block's rows
@@ -60,7 +75,8 @@ __device__ __forceinline__ int prep_token(const PrepArgs &p, int r) {
 }
 static PrepArgs prep_args(const viasd_model *m, const viasd_cache *c, const viasd_draft *d, bool full_pass, bool replay) {
     return PrepArgs{m->ws.tree, m->ws.len_eff, m->ws.stats, c->len, c->pending, d->draft_tok, d->parent,
-                    replay ? m->ws.row_tok : nullptr, d->per_sequence, d->batch, d->n_nodes, m->cfg.max_ctx, m->cfg.vocab, full_pass ? 1 : 0};
+                    replay ? m->ws.row_tok : nullptr, d->per_sequence, d->batch, d->n_nodes, m->cfg.max_ctx, m->cfg.vocab, full_pass ? 1 : 0,
+                    counters_of(m)};
 }
 
 // Preparation of a replay pass (routed execution policy): the block of every sequence is extended, in front, by its
@@ -72,8 +88,9 @@ static PrepArgs prep_args(const viasd_model *m, const viasd_cache *c, const vias
 // where its cache had them, the missing ones where a skipped pass left a gap) on its way to the block's own rows.
 __global__ void prep_replay_kernel(TreeInfo *tree, int *len_eff, int *row_tok, DeviceStats *stats, const int *len,
                                    const int *pending, const int *draft_tok, const int *parent, int per_seq,
-                                   const int *tokens, int B, int N, int G, int max_ctx, int vocab, const int *run_flag) {
+                                   const int *tokens, int B, int N, int G, int max_ctx, int vocab, const Counters counters, const int *run_flag) {
     RUN_FLAG_EXIT(run_flag);
+    clear_counters_if_failed(counters, stats, threadIdx.x, blockDim.x);
     const int Mx = G + N + 1;
     if (threadIdx.x == 0) stats->full_ran = 1;
     for (int b = threadIdx.x; b < B; b += blockDim.x) {
@@ -112,7 +129,7 @@ __global__ void prep_replay_kernel(TreeInfo *tree, int *len_eff, int *row_tok, D
 int launch_prep_replay(const viasd_model *m, const viasd_cache *c, const viasd_draft *d, int G, cudaStream_t st) {
     prep_replay_kernel<<<1, 128, 0, st>>>(m->ws.tree, m->ws.len_eff, m->ws.row_tok, m->ws.stats, c->len, c->pending,
                                           d->draft_tok, d->parent, d->per_sequence, c->tokens, d->batch, d->n_nodes, G,
-                                          m->cfg.max_ctx, m->cfg.vocab, m->run_flag);
+                                          m->cfg.max_ctx, m->cfg.vocab, counters_of(m), m->run_flag);
     LAUNCH_CHECK();
     return VIASD_OK;
 }

@@ -96,15 +96,16 @@ __device__ __forceinline__ void counter_arrive(int *ctr, int arrivals, int reade
 __device__ __forceinline__ void counter_ack(int *ctr, int arrivals, int readers) {
     asm volatile("red.relaxed.gpu.global.inc.u32 [%0], %1;" ::"l"(ctr), "r"(arrivals + readers - 1) : "memory");
 }
-// one thread waits, bounded, and acknowledges; false: gave up (the caller's other threads learn it from abort_flag)
-__device__ __forceinline__ bool counter_wait(int *ctr, int arrivals, int readers, volatile int *abort_flag, int *status) {
+// One thread waits, bounded, and acknowledges.  A wait that gave up acknowledges too, and its caller goes on as if it had
+// not: every CTA then takes the same barriers, arrivals and acknowledgements whatever expired, so nobody is left in a barrier
+// and the counter comes back to zero (what is computed meanwhile is void, as the status word says).
+__device__ __forceinline__ void counter_wait(int *ctr, int arrivals, int readers, volatile int *abort_flag, int *status) {
     auto arrived = [&]() { int v; asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory"); return v; };
     const long long t0 = clock64();
     while (arrived() < arrivals) {
-        if (*abort_flag || clock64() - t0 > WAIT_LIMIT_CYCLES) { *abort_flag = 1; atomicExch(status, VIASD_EDEVICE); return false; }
+        if (*abort_flag || clock64() - t0 > WAIT_LIMIT_CYCLES) { *abort_flag = 1; atomicExch(status, VIASD_EDEVICE); break; }
     }
     counter_ack(ctr, arrivals, readers);
-    return true;
 }
 
 // ---- single-thread instructions of a warp in step -----------------------------------------------

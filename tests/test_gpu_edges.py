@@ -64,3 +64,33 @@ def test_gains_and_caches_need_no_alignment(name, batch, head_dim):
         assert torch.equal(w, g)
     for w, g in zip((eng.k_full, eng.v_full, eng.k_slim, eng.v_slim, eng.len, eng.pending, eng.tokens), state):
         assert torch.equal(w, g)
+
+
+# ---------------------------------------------------------------------------------------------
+# a wait that expires
+# ---------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("name,batch", [("mini_7b", 1), ("mini_13b", 8)])
+def test_expired_wait_leaves_a_usable_handle(name, batch):
+    """One arrival counter is off (as after a failure): the tile it belongs to gives up its wait after its limit, the pass ends,
+    the status says so, and the next pass on the same handle computes what it did before.  One-CTA and pair GEMM."""
+    vb = _vb()
+    base = W.get(name)
+    # one layer, k = 2048: the first tile of the O and down projections is split among CTAs
+    wl = replace(base, batch=batch, shape=replace(base.shape, n_layers=1, d_model=2048, d_ff=2048), n_routed=1)
+    eng = _engine(wl)
+    want, got = eng.logits_buffer(), eng.logits_buffer()
+    vb.full_forward(eng.model, eng.cache, eng.draft, want)
+    torch.cuda.synchronize()
+    # the counters are the workspace's last piece
+    s = wl.shape
+    n = 4 * (max(s.vocab, s.n_heads * s.head_dim + 2 * s.n_kv_heads * s.head_dim, s.d_ff) // 64 + 8)
+    at = eng.workspace.numel() - (n + 255) // 256 * 256
+    counters = eng.workspace[at:at + n].view(torch.int32)
+    assert int(counters.abs().max()) == 0
+    counters[0] = 1 << 20                                      # the first arrival wraps it: one is missing
+    vb.full_forward(eng.model, eng.cache, eng.draft, got)
+    torch.cuda.synchronize()
+    assert vb.get_stats(eng.model).device_status == vb.VIASD_EDEVICE
+    vb.full_forward(eng.model, eng.cache, eng.draft, got)
+    torch.cuda.synchronize()
+    assert torch.equal(want, got) and int(counters.abs().max()) == 0
