@@ -89,7 +89,8 @@ typedef struct {
     int batch, n_nodes;                /* B, N */
     const int *draft_tok;              /* [B, N] */
     const int *parent;                 /* [N] parent node, -1 = child of the pending token; parents first */
-    const int *prow;                   /* [N] drafter-logit row the node was drafted from */
+    const int *prow;                   /* [N] drafter-logit row the node was drafted from (one outside [0, R) is recorded in the
+                                          device status; as a gate it puts the node in the strictest tier) */
     int n_prows;                       /* R, 1..64 (one drafter row per distinct parent at most) */
     const float *drafter_logits;       /* [B, R, vocab] */
     int per_sequence;                  /* 0: one tree for the whole batch (parent and prow are [N]).  1: every sequence

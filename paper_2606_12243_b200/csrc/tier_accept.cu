@@ -117,10 +117,12 @@ tier_kernel(unsigned char *__restrict__ tier, float *__restrict__ conf, DeviceSt
             continue;
         }
         int g = conf_source == 0 ? prow[n] : parent[n] + 1;
-        if (g != gr) continue;
+        const bool ok = g >= 0 && g < rows_per_seq;              // no such gate row: an error, and the strictest tier
+        if (g != gr && (ok || gr > 0)) continue;
+        if (!ok) stats->device_status = VIASD_EDEVICE;
         int t = draft_tok[b * N + n];
         t = min(max(t, 0), V - 1);
-        float d = row[t] - mx;
+        float d = ok ? row[t] - mx : -INFINITY;
         int tr = 0;                                              // thresholds descend: the first one d reaches names the tier
         while (tr < cuts.n && d < cuts.log_tau[tr]) ++tr;
         tier[b * N + n] = (unsigned char)tr;
@@ -370,18 +372,22 @@ accept_kernel(AcceptArgs a) {
         const int v = min(max(a.draft_tok[b * N + n], 0), V - 1);
         w.next_sibling[n] = a.tree[b].next_sibling[n];
         w.tok[n] = v;
-        w.prow[n] = pr;
         w.judged[n] = 0;
-        const bool pr_ok = pr >= 0 && pr < a.R;
-        const float x0 = a.drafter && pr_ok && par != -2 ? a.drafter[((size_t)b * a.R + pr) * V + v] : 0.f;
+        const bool pr_ok = pr >= 0 && pr < a.R, used = par != -2;      // -2: unused node of this sequence's tree
+        w.prow[n] = pr_ok ? pr : 0;
+        if (used && sampling && !pr_ok) a.stats->device_status = VIASD_EDEVICE;
+        const float x0 = a.drafter && used ? a.drafter[((size_t)b * a.R + w.prow[n]) * V + v] : 0.f;
         w.x0[n] = x0;
         int t;
         if (a.do_tier) {
             t = 0;
             float d = 0.f;
             const int g = a.conf_source == 0 ? pr : par + 1;
-            if (par != -2 && (a.conf_source ? g >= 0 && g < M : pr_ok)) {                // -2: unused node of this sequence's tree
-                d = a.conf_source == 0 ? x0 - w.mx[0][g] : a.judges[1][((size_t)b * M + g) * V + v] - w.mx[1][g];
+            if (used) {
+                // no such gate row: an error, and the strictest tier, as in the tier kernel
+                d = -INFINITY;
+                if (a.conf_source ? g < 0 || g >= M : !pr_ok) a.stats->device_status = VIASD_EDEVICE;
+                else d = a.conf_source == 0 ? x0 - w.mx[0][g] : a.judges[1][((size_t)b * M + g) * V + v] - w.mx[1][g];
                 while (t < a.cuts.n && d < a.cuts.log_tau[t]) ++t;      // thresholds descend: the first one d reaches names the tier
                 atomicAdd(&w.tier_count[t == 0 ? 0 : (t == a.cuts.n ? 2 : 1)], 1);       // accepted / some slim verifier / q
             }

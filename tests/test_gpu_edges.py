@@ -94,3 +94,32 @@ def test_expired_wait_leaves_a_usable_handle(name, batch):
     vb.full_forward(eng.model, eng.cache, eng.draft, got)
     torch.cuda.synchronize()
     assert torch.equal(want, got) and int(counters.abs().max()) == 0
+
+
+# ---------------------------------------------------------------------------------------------
+# a node whose gate row does not exist
+# ---------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("phases", [(3,), (1, 2)])
+@pytest.mark.parametrize("mode,bad", [("greedy", -1), ("greedy", 99), ("sampling", 8)])
+def test_node_without_a_gate_row_goes_to_the_full_verifier(phases, mode, bad):
+    """prow outside [0, R): recorded, and the node is judged by q, never accepted outright; alone or with the walk."""
+    vb = _vb()
+    wl = replace(W.get("mini_7b"), mode=mode)
+    eng = _engine(wl)
+    prow = eng.prow.clone()
+    prow[2] = bad
+    draft = vb.make_draft(eng.draft_tok, eng.parent, prow, eng.inputs.n_prows, eng.drafter_logits)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    slim, full = (torch.randn(eng.logits_buffer().shape, device="cuda", generator=g) for _ in range(2))
+    results = []
+    for d in (eng.draft, draft):
+        r = vb.alloc_result(wl.batch, wl.n_nodes)
+        for phase in phases:
+            # every token is accepted outright where its gate row exists
+            vb.tier_accept(eng.model, d, eng.params(log_tau_lo=-1e9, log_tau_hi=-1e9), slim, full, phase, r)
+        torch.cuda.synchronize()
+        results.append((r, vb.get_stats(eng.model).device_status))
+    (good, s0), (r, s1) = results
+    assert s0 == 0 and int(good.n_acc[0]) == wl.n_nodes and s1 == vb.VIASD_EDEVICE
+    assert r.tier[0].tolist() == [2 if n == 2 else 0 for n in range(wl.n_nodes)]
+    assert r.conf[0, 2].item() == -float("inf") and int(r.judge[0, 2]) >> 4 == 2
