@@ -220,8 +220,8 @@ enum {
                                           greedy; sampling: 8 from 16384 tokens on, 16 from 65536 on where the device
                                           takes clusters of 16) */
     VIASD_OPT_DUAL_MAX_ROWS,           /* most token rows (both verifiers together) that viasd_verify_step runs as one
-                                          sweep over the layers, 0..128 (default 128, which from 48 rows per verifier on
-                                          means 256: the GEMM for many rows takes that many); above it the passes run in turn */
+                                          sweep over the layers, 0..128; -1 (default): as many as one launch of the GEMM
+                                          takes, 128, or 256 from 48 rows per verifier on; above it the passes run in turn */
     VIASD_OPT_TK_GRID,                 /* keys-on-lanes attention with tiles dealt evenly: CTAs to use; 0 = one per SM */
     VIASD_OPT_TK_FLAT,                 /* keys-on-lanes attention: deal tiles 1, key ranges 0; -1 = by shape (default) */
     VIASD_OPT_GEMM_RING_KB,            /* stream-K GEMM: shared-memory ring in KB, 32..200; 0 = default (200) */

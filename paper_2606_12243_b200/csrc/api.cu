@@ -99,7 +99,7 @@ void default_options(ModelOptions &o) {
     o.attn_splits = env_int("VIASD_ATTN_NSPLIT", 0);
     o.attn_lo = env_int("VIASD_ATTN_LO", 2);
     o.accept_team = env_int("VIASD_ACCEPT_TEAM", 0);
-    o.dual_max_rows = env_int("VIASD_DUAL_MAX", 128);
+    o.dual_max_rows = env_int("VIASD_DUAL_MAX", -1);
     o.tk_grid = env_int("VIASD_TK_GRID", 0);
     o.tk_flat = env_int("VIASD_TK_FLAT", -1);
     o.ring_kb = env_int("VIASD_TC_RING_KB", 0);
@@ -595,7 +595,7 @@ int viasd_verify_step(viasd_model *m, viasd_cache *cache, const viasd_draft *dra
     // row streams together fit one launch (128 token rows, 256 where the pair kernel runs the pass); beyond
     // that a sweep would stream every routed layer twice anyway, and the passes run one after the other.
     const int block_rows = draft ? draft->batch * (draft->n_nodes + 1) : 0;
-    const int dual_max = !m ? 0 : m->opt.dual_max_rows == 128 && block_rows >= TC_WIDE_MIN_ROWS ? TC_WIDE_ROWS : m->opt.dual_max_rows;
+    const int dual_max = !m ? 0 : m->opt.dual_max_rows >= 0 ? m->opt.dual_max_rows : block_rows >= TC_WIDE_MIN_ROWS ? TC_WIDE_ROWS : 128;
     if (m && m->fused && draft && 2 * block_rows <= dual_max) {
         if ((rc = check_draft(m, draft)) || (rc = check_cache(cache))) return rc;
         if ((rc = forward_sweep(m, cache, draft, 2, full_logits, slim_logits, (cudaStream_t)stream))) return rc;
@@ -634,7 +634,7 @@ int viasd_set_option(viasd_model *m, int option, int value) {
     case VIASD_OPT_ATTENTION_SPLITS: if (value < 0 || value > 16) return VIASD_EINVAL; o.attn_splits = value; break;
     case VIASD_OPT_ATTENTION_LO: if (value < 0 || value > 2) return VIASD_EINVAL; o.attn_lo = value; break;
     case VIASD_OPT_ACCEPT_TEAM: if (value != 0 && value != 1 && value != 2 && value != 4 && value != 8) return VIASD_EINVAL; o.accept_team = value; break;
-    case VIASD_OPT_DUAL_MAX_ROWS: if (value < 0 || value > 128) return VIASD_EINVAL; o.dual_max_rows = value; break;
+    case VIASD_OPT_DUAL_MAX_ROWS: if (value < -1 || value > 128) return VIASD_EINVAL; o.dual_max_rows = value; break;
     case VIASD_OPT_TK_GRID: if (value < 0) return VIASD_EINVAL; o.tk_grid = value; break;
     case VIASD_OPT_TK_FLAT: if (value < -1 || value > 1) return VIASD_EINVAL; o.tk_flat = value; break;
     case VIASD_OPT_GEMM_RING_KB: if (value != 0 && (value < 32 || value > 200)) return VIASD_EINVAL; o.ring_kb = value; break;

@@ -90,7 +90,7 @@ struct ModelOptions {
     int attn_splits;        // VIASD_OPT_ATTENTION_SPLITS: key ranges per (sequence, kv head); 0 = cost model
     int attn_lo;            // VIASD_OPT_ATTENTION_LO: mma.sync kernel, hi/lo split of Q and P (2), of Q only (1), none (0)
     int accept_team;        // VIASD_OPT_ACCEPT_TEAM: CTAs per sequence in the accept walk; 0 = by mode and vocabulary
-    int dual_max_rows;      // VIASD_OPT_DUAL_MAX_ROWS: most rows (both verifiers) the one-sweep schedule takes
+    int dual_max_rows;      // VIASD_OPT_DUAL_MAX_ROWS: most rows (both verifiers) the one-sweep schedule takes; -1 = what one launch holds
     int tk_grid;            // VIASD_OPT_TK_GRID: CTAs of the keys-on-lanes kernel when tiles are dealt evenly; 0 = one per SM
     int tk_flat;            // VIASD_OPT_TK_FLAT: deal tiles (1) or key ranges (0); -1 = by shape
     int ring_kb;            // VIASD_OPT_GEMM_RING_KB: shared-memory ring of the stream-K GEMM

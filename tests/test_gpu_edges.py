@@ -123,3 +123,39 @@ def test_node_without_a_gate_row_goes_to_the_full_verifier(phases, mode, bad):
     assert s0 == 0 and int(good.n_acc[0]) == wl.n_nodes and s1 == vb.VIASD_EDEVICE
     assert r.tier[0].tolist() == [2 if n == 2 else 0 for n in range(wl.n_nodes)]
     assert r.conf[0, 2].item() == -float("inf") and int(r.judge[0, 2]) >> 4 == 2
+
+
+# ---------------------------------------------------------------------------------------------
+# one sweep for both verifiers on the GEMM for many rows
+# ---------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("batch,nodes", [(7, 6), (5, 12), (2, 63)])
+def test_one_sweep_of_many_rows_is_the_two_passes(batch, nodes):
+    """49, 65 and 128 rows per verifier, routed layers 98 (one sub-tile), 130 (the second stream begins inside a sub-tile) and
+    256 (a full launch): logits and caches bit for bit those of the separate passes; 128 as the option's value means 128."""
+    vb = _vb()
+    base = W.get("mini_13b")
+    wl = replace(base, batch=batch, ctx=70, parent=W.chain(nodes))
+    eng = _engine(wl)
+    slim, full, res = eng.logits_buffer(), eng.logits_buffer(), vb.alloc_result(batch, nodes)
+    caches = (eng.k_full, eng.v_full, eng.k_slim, eng.v_slim)
+    before, pending = [t.clone() for t in caches], eng.pending.clone()
+    vb.full_forward(eng.model, eng.cache, eng.draft, full)
+    vb.slim_forward(eng.model, eng.cache, eng.draft, slim)
+    torch.cuda.synchronize()
+    want = [t.clone() for t in (full, slim, *caches)]
+    launches = []
+    for option in (-1, 128):
+        for t, b in zip(caches, before):
+            t.copy_(b)
+        eng.len.fill_(wl.ctx)
+        eng.pending.copy_(pending)
+        vb.set_option(eng.model, "dual_max_rows", option)
+        n0 = vb.launch_count()
+        # nothing is accepted, so the commit moves no row
+        vb.verify_step(eng.model, eng.cache, eng.draft, eng.params(log_tau_lo=1e9, log_tau_hi=1e9, log_acc_rel=(1e9, 1e9, 1e9)), slim, full, res)
+        torch.cuda.synchronize()
+        launches.append(vb.launch_count() - n0)
+        for w, t in zip(want, (full, slim, *caches)):
+            assert torch.equal(w, t)
+    assert vb.get_stats(eng.model).device_status == 0 and int(res.n_acc.sum()) == 0
+    assert (launches[0] < launches[1]) == (2 * batch * (nodes + 1) > 128)
