@@ -3,20 +3,28 @@
 // The M block rows of a sequence under all query heads of one kv head (dealt to items of at most 128 rows) against the
 // committed context plus the block's own rows under the ancestor mask:
 //
-//   S[rows, 128 keys] = Q K^T      A = Q (shared memory, K-major, hi and lo planes: two MMAs into one S)
+//   S[rows, 128 keys] = Q K^T      A = Q (shared memory, K-major, 2 or 3 bf16 planes: an MMA each into one S)
 //                                  B = K tile exactly as its TMA box lands (K-major, 128-byte swizzle)
-//   O[rows, 128 dims] += P V       A = P in TMEM (bf16 pairs, hi and lo planes: two MMAs into one O)
+//   O[rows, 128 dims] += P V       A = P in TMEM (bf16 pairs, as many planes: an MMA each into one O)
 //                                  B = V tile as it lands, read MN-major (keys are the contraction)
 //
-// What bounds it: 32 MMAs of 128 x 128 x 16 per tile, about 2300 cycles whatever the rows (so it is for 33 rows and more;
-// fewer go to the kernels that put the keys on the lanes or use mma.sync), and with a few tiles per CTA the chain around
-// them: queries, first S, softmax, last P V, result, merge.
+// Precision.  Up to 128 query rows per kv head queries and weights are bf16 pairs, as in the other two kernels; more rows
+// belonged to an fp32 kernel, and three planes hold all of an fp32 value.  O is summed over the tiles in fp32 outside the MMAs
+// (GROUP).  Error of the output against 64 bits, before / now: fp32 kernel / three planes 2.56 - 2.84e-6 / 2.53 - 2.56e-6
+// (132 to 256 rows, 348 to 4033 keys), mma.sync / two planes 5.1 - 5.3e-6 / 5.0 - 5.1e-6 (36 to 108 rows); most of it is the
+// output itself, which is stored as a bf16 pair.
+//
+// What bounds it: 32 (48) MMAs of 128 x 128 x 16 per tile, about 2300 (3200) cycles whatever the rows (so it is for 33 rows
+// and more; fewer go to the kernels that put the keys on the lanes or use mma.sync), and with a few tiles per CTA the chain
+// around them: queries, first S, softmax, last P V, result, merge.  Keeping the precision costs 0 - 3 % of a layer with a small
+// feed-forward at two planes, 4 - 12 % at three (eight sequences, 33 rows each, 4000 keys: 206 us a layer, now 231; the fp32
+// kernel took 2230).
 //
 // One TMEM lane is one query row; two warps share a lane quarter and take 64 of a tile's 128 keys each, exchanging row
 // maxima once per tile.  The running maximum only moves when a tile exceeds it by 2^8 (the weights stay below 2^8
-// otherwise, harmless in fp32), which makes the rescaling of O in TMEM rare.  P overwrites S in place (per 16 keys 8
-// columns of bf16 pairs hi, 8 lo), two buffers; MMAs run in issue order, which is what lets Q K^T of tile t + 2 reuse the
-// buffer that P V of tile t reads.  The last tile of a range multiplies only the 16-key groups that it has.
+// otherwise, harmless in fp32), which makes rescaling O rare.  P overwrites S in place (per 16 keys 8
+// columns of bf16 pairs hi, 8 of the next plane), two buffers; MMAs run in issue order, which is what lets Q K^T of tile t + 2
+// reuse the buffer that P V of tile t reads.  The last tile of a range multiplies only the 16-key groups that it has.
 //
 // Split of the work: attention_work.cuh.  Partial rows: [32 groups of 4 dims][rows8] float4, then [rows8] (max, sum).
 //
@@ -34,9 +42,14 @@ constexpr int SW = 8;                          // softmax warps
 constexpr int AT_THREADS = 64 + SW * 32;
 constexpr int AT_MAX_SLOTS = 6;
 constexpr int QROWS = 128 / SW;                // query rows a warp stages at most
+// Tiles whose P V the tensor cores add up in one accumulator, before it is added to the item's sum in fp32 (rounded; what an
+// MMA adds is cut off, so a sum over all tiles drifts towards zero: 36 rows against 1000 keys, error of the attention output
+// 5.9e-6 over all tiles, 5.1e-6 with two, 5.0e-6 with one, where every added tile waits for the one before it to be read).
+template <int PLANES> constexpr int GROUP = PLANES == 3 ? 1 : 2;
 constexpr float RESCALE_GAP = 8.f;             // log2 units
 
-constexpr uint32_t TM_S = 0, TM_O = 256;       // TMEM column offsets: S / P buffers (2 x 128), O (128)
+constexpr uint32_t TM_S = 0, TM_O = 256, TM_X = 384;   // TMEM columns: S / P buffers (2 x 128), O of one tile (128), and the
+                                                             // sum of the tiles' O (128), or third planes of P (2 x 64)
 
 // The j-th of an item's 2 n requests, in the order the MMAs take them: K0 K1 V0 K2 V1 ... K(n-1) V(n-2) V(n-1)
 __device__ __forceinline__ int request_tile(int j, int n, bool &is_v) {
@@ -76,6 +89,35 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
           "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr) : "memory");
 }
+// 32 columns from each of two places under one wait
+__device__ __forceinline__ void tc_ld32x2(uint32_t ta, uint32_t tb, uint32_t (&r)[32], uint32_t (&s)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(r[0]),"=r"(r[1]),"=r"(r[2]),"=r"(r[3]),"=r"(r[4]),"=r"(r[5]),"=r"(r[6]),"=r"(r[7]),
+          "=r"(r[8]),"=r"(r[9]),"=r"(r[10]),"=r"(r[11]),"=r"(r[12]),"=r"(r[13]),"=r"(r[14]),"=r"(r[15]),
+          "=r"(r[16]),"=r"(r[17]),"=r"(r[18]),"=r"(r[19]),"=r"(r[20]),"=r"(r[21]),"=r"(r[22]),"=r"(r[23]),
+          "=r"(r[24]),"=r"(r[25]),"=r"(r[26]),"=r"(r[27]),"=r"(r[28]),"=r"(r[29]),"=r"(r[30]),"=r"(r[31])
+        : "r"(ta));
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(s[0]),"=r"(s[1]),"=r"(s[2]),"=r"(s[3]),"=r"(s[4]),"=r"(s[5]),"=r"(s[6]),"=r"(s[7]),
+          "=r"(s[8]),"=r"(s[9]),"=r"(s[10]),"=r"(s[11]),"=r"(s[12]),"=r"(s[13]),"=r"(s[14]),"=r"(s[15]),
+          "=r"(s[16]),"=r"(s[17]),"=r"(s[18]),"=r"(s[19]),"=r"(s[20]),"=r"(s[21]),"=r"(s[22]),"=r"(s[23]),
+          "=r"(s[24]),"=r"(s[25]),"=r"(s[26]),"=r"(s[27]),"=r"(s[28]),"=r"(s[29]),"=r"(s[30]),"=r"(s[31])
+        : "r"(tb));
+    // (an empty statement per half names the registers: no use of them is scheduled ahead of the wait)
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    asm volatile("" : "+r"(r[0]),"+r"(r[1]),"+r"(r[2]),"+r"(r[3]),"+r"(r[4]),"+r"(r[5]),"+r"(r[6]),"+r"(r[7]),
+          "+r"(r[8]),"+r"(r[9]),"+r"(r[10]),"+r"(r[11]),"+r"(r[12]),"+r"(r[13]),"+r"(r[14]),"+r"(r[15]),
+          "+r"(r[16]),"+r"(r[17]),"+r"(r[18]),"+r"(r[19]),"+r"(r[20]),"+r"(r[21]),"+r"(r[22]),"+r"(r[23]),
+          "+r"(r[24]),"+r"(r[25]),"+r"(r[26]),"+r"(r[27]),"+r"(r[28]),"+r"(r[29]),"+r"(r[30]),"+r"(r[31]));
+    asm volatile("" : "+r"(s[0]),"+r"(s[1]),"+r"(s[2]),"+r"(s[3]),"+r"(s[4]),"+r"(s[5]),"+r"(s[6]),"+r"(s[7]),
+          "+r"(s[8]),"+r"(s[9]),"+r"(s[10]),"+r"(s[11]),"+r"(s[12]),"+r"(s[13]),"+r"(s[14]),"+r"(s[15]),
+          "+r"(s[16]),"+r"(s[17]),"+r"(s[18]),"+r"(s[19]),"+r"(s[20]),"+r"(s[21]),"+r"(s[22]),"+r"(s[23]),
+          "+r"(s[24]),"+r"(s[25]),"+r"(s[26]),"+r"(s[27]),"+r"(s[28]),"+r"(s[29]),"+r"(s[30]),"+r"(s[31]));
+}
 __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
@@ -86,9 +128,22 @@ __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32])
           "r"(r[30]), "r"(r[31])
         : "memory");
 }
+// x0, x1 -> three packed bf16 pairs whose sums are x0 and x1 to the last bit of fp32
+__device__ __forceinline__ void split_triple(float x0, float x1, uint32_t &hi, uint32_t &mid, uint32_t &lo) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+    hi = *reinterpret_cast<const uint32_t *>(&h);
+    split_pair(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u), mid, lo);
+}
+__device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+          "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
+}
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-
+// PLANES: bf16 planes of the queries and of the weights
+template <int PLANES>
 __global__ void __launch_bounds__(AT_THREADS, 1)
 attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ CUtensorMap map_k2, const __grid_constant__ CUtensorMap map_v2, const AttnWork a) {
@@ -105,7 +160,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     const int NS = a.ring_slots;
     // staged queries first (the MMA reads 128 rows from each 64-dim chunk: what lies behind the live rows is the ring)
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, qchunk = (uint32_t)a.rows8 * 128u;
-    const uint32_t qsm = base, ring = base + 4 * qchunk;
+    const uint32_t qsm = base, ring = base + 2 * PLANES * qchunk;
     uint8_t *q_gen = smem_raw + (base - smem_u32(smem_raw));
     auto full_bar = [&](int s) { return smem_u32(&bars[s]); };
     auto empty_bar = [&](int s) { return smem_u32(&bars[AT_MAX_SLOTS + s]); };
@@ -189,11 +244,13 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 if (elect_one()) {
                     const uint64_t kd = smem_desc(ring + st * SLOT_BYTES), q0 = smem_desc(qsm), q_step = qchunk >> 4;
                     const uint32_t sb = (s_cnt + t) & 1, d = tmem + TM_S + sb * 128, id = idesc | ((uint32_t)(2 * groups16(t)) << 17);
+                    // small planes first: what an MMA adds is cut off, not rounded, at the size of what it is added to (error of the
+                    // output at 256 rows against 1000 keys 2.55e-6, the other way round 2.79e-6)
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks) {
+                    for (int i = 0; i < 8 * PLANES; ++i) {
+                        const int ks = i & 7, plane = PLANES - 1 - (i >> 3);
                         const uint64_t kb = kd + (ks >> 2) * (HALF_BYTES >> 4) + (ks & 3) * 2, qa = q0 + (ks >> 2) * q_step + (ks & 3) * 2;
-                        tc_mma(d, qa, kb, id, ks > 0 ? 1u : 0u);
-                        tc_mma(d, qa + 2 * q_step, kb, id, 1u);          // lo plane of the queries
+                        tc_mma(d, qa + 2 * plane * q_step, kb, id, i > 0 ? 1u : 0u);
                     }
                     tc_commit(empty_bar(st));
                     tc_commit(sfull_bar(sb));
@@ -215,13 +272,15 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 tc_fence_after();
                 if (elect_one()) {
                     const uint64_t vd = smem_desc_mn(ring + st * SLOT_BYTES, HALF_BYTES, 1024);
-                    const uint32_t pb = tmem + TM_S + sb * 128;
+                    const uint32_t pb = tmem + TM_S + sb * 128, p3 = tmem + TM_X + sb * 64;
                     const int nk = groups16(t);
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk) {                  // 16 keys per step: two 8-key groups of 1024 bytes
                         if (kk >= nk) break;
-                        tc_mma_ts(tmem + TM_O, pb + kk * 16, vd + kk * (2048 >> 4), idesc_pv, (t > 0 || kk > 0) ? 1u : 0u);
-                        tc_mma_ts(tmem + TM_O, pb + kk * 16 + 8, vd + kk * (2048 >> 4), idesc_pv, 1u);   // lo plane of the weights
+#pragma unroll
+                        for (int plane = PLANES - 1; plane >= 0; --plane)
+                            tc_mma_ts(tmem + TM_O, plane == 2 ? p3 + kk * 8 : pb + kk * 16 + plane * 8, vd + kk * (2048 >> 4), idesc_pv,
+                                      (plane < PLANES - 1 || kk > 0 || t % GROUP<PLANES> != 0) ? 1u : 0u);
                     }
                     tc_commit(empty_bar(st));                         // the slot is free once these MMAs have read it
                     tc_commit(pvdone_bar(sb));
@@ -261,7 +320,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             const size_t o0 = row_off(a, it, live ? trow : 0);
             const int g0 = it.row0 + (live ? trow : 0);
             const unsigned long long anc = a.tree[it.b].anc[g0 - (int)((g0 * a.m_recip) >> 32) * a.M];
-            // stage the item's query rows as bf16 hi / lo planes, pre-scaled, in the K-major 128-byte-swizzled layout the MMA
+            // stage the item's query rows as bf16 planes, pre-scaled, in the K-major 128-byte-swizzled layout the MMA
             // reads; a warp takes whole rows, all its loads in flight (addresses first: they do not wait for anything)
             uint32_t qrow[QROWS];
 #pragma unroll
@@ -279,18 +338,58 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             for (int q = 0; q < QROWS; ++q) {
                 const uint32_t r = sw + q * SW, d4 = 4 * lane, dc = d4 & 63;       // dc: dim inside its 64-dim chunk
                 if (r >= (uint32_t)a.rows8) break;
-                uint2 hi, lo;
-                split_pair(v[q].x * a.scale, v[q].y * a.scale, hi.x, lo.x);
-                split_pair(v[q].z * a.scale, v[q].w * a.scale, hi.y, lo.y);
+                uint2 hi, lo, lo2;
+                split_triple(v[q].x * a.scale, v[q].y * a.scale, hi.x, lo.x, lo2.x);
+                split_triple(v[q].z * a.scale, v[q].w * a.scale, hi.y, lo.y, lo2.y);
                 uint8_t *dst = q_gen + (d4 >> 6) * qchunk + r * 128u + (((dc >> 3) ^ (r & 7u)) << 4) + (dc & 7u) * 2u;
                 *reinterpret_cast<uint2 *>(dst) = hi;
                 *reinterpret_cast<uint2 *>(dst + 2 * qchunk) = lo;
+                if (PLANES == 3) *reinterpret_cast<uint2 *>(dst + 4 * qchunk) = lo2;
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> the MMA's reads
             __syncwarp();
             if (lane == 0) mbar_arrive(qfull_bar);
 
             float m_run = -INFINITY, l_run = 0.f;                // m_run: the whole row's, l_run: of this half's keys
+            // O of the tiles so far, this half's dims: in registers, or (two planes leave room) in TMEM, by rolled loops
+            float o[PLANES == 3 ? 64 : 1];
+#pragma unroll
+            for (int e = 0; e < (PLANES == 3 ? 64 : 1); ++e) o[e] = 0.f;
+            // Adds a group's O once its last P V (of tile g of the CTA) has written it, and moves the sum to the new maximum.  32
+            // columns at a time; `first`: the sum is empty, `last`: it is not kept, but handed to `use`.
+            auto add_group = [&](int g, float corr, bool first, bool last, auto use) -> bool {
+                if (!warp_wait(pvdone_bar(g & 1), (g >> 1) & 1, &abort_sh, a.status)) return false;
+                tc_fence_after();
+                if (!warp_live) return true;
+                if constexpr (PLANES == 3) {
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        uint32_t r[32];
+                        tc_ld32(tlane + TM_O + half * 64 + c * 32, r);
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(o[c * 32 + e] = (o[c * 32 + e] + __uint_as_float(r[e])) * corr);
+                        if (last) use(c, r);
+                    }
+                } else {
+#pragma unroll 1
+                    for (int c = 0; c < 2; ++c) {
+                        const uint32_t from = tlane + half * 64 + c * 32;
+                        uint32_t r[32], s[32];
+                        if (first) {
+                            tc_ld32(from + TM_O, r);
+                        } else {
+                            tc_ld32x2(from + TM_O, from + TM_X, r, s);
+#pragma unroll
+                            for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) + __uint_as_float(s[e]));
+                        }
+                        if (last) { use(c, r); continue; }
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * corr);
+                        tc_st32(from + TM_X, r);
+                    }
+                }
+                return true;
+            };
             for (int t = 0; t < it.n_tiles; ++t, ++s_cnt) {
                 const int sb = s_cnt & 1;
                 if (!(ok = warp_wait(sfull_bar(sb), (s_cnt >> 1) & 1, &abort_sh, a.status))) break;
@@ -332,80 +431,79 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     corr = (m_run == -INFINITY) ? 1.f : ex2(m_run - m_tile);
                     m_run = m_tile;
                 }
-                if (__any_sync(0xffffffffu, corr != 1.f)) {
-                    // rare: the running maximum moved (both warps of the quarter see it).  Each rescales its half of O once
-                    // the previous tile's P V has written it (the one before that finished earlier: MMAs complete in order).
-                    if (!(ok = warp_wait(pvdone_bar(sb ^ 1), ((s_cnt - 1) >> 1) & 1, &abort_sh, a.status))) break;
-                    tc_fence_after();
-#pragma unroll 1
-                    for (int c = 0; c < 2; ++c) {
-                        uint32_t r[32];
-                        tc_ld32(tlane + TM_O + half * 64 + c * 32, r);
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * corr);
-                        tc_st32(tlane + TM_O + half * 64 + c * 32, r);
-                    }
-                    l_run *= corr;
-                }
+                l_run *= corr;
                 // pass 2: weights and their row sum; P replaces S in place
                 const float m_use = m_run == -INFINITY ? 0.f : m_run;   // no visible key yet: every weight is 2^-inf
 #pragma unroll 1
                 for (int c = 0; c * 32 < cols; ++c) {
-                    uint32_t r[32], w[32];
+                    uint32_t r[32], w[32], w3[16];
                     load(c, r);
                     float l4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                     for (int e = 0; e < 32; e += 2) {
                         const float p0 = ex2(__uint_as_float(r[e]) - m_use), p1 = ex2(__uint_as_float(r[e + 1]) - m_use);
                         l4[(e >> 1) & 3] += p0 + p1;
-                        split_pair(p0, p1, w[(e >> 4) * 16 + ((e & 15) >> 1)], w[(e >> 4) * 16 + 8 + ((e & 15) >> 1)]);
+                        const int at = (e >> 4) * 16 + ((e & 15) >> 1);
+                        if (PLANES == 3) split_triple(p0, p1, w[at], w[at + 8], w3[e >> 1]);
+                        else split_pair(p0, p1, w[at], w[at + 8]);
                     }
                     l_run += (l4[0] + l4[1]) + (l4[2] + l4[3]);
                     tc_st32(tb + c * 32, w);
+                    if (PLANES == 3) tc_st16(tlane + TM_X + sb * 64 + half * 32 + c * 16, w3);
+                }
+                if (t > 0 && t % GROUP<PLANES> == 0) {
+                    if (!(ok = add_group(s_cnt - 1, corr, t == GROUP<PLANES>, false, [](int, const uint32_t (&)[32]) {}))) break;
+                } else if (t > 0 && __any_sync(0xffffffffu, corr != 1.f)) {
+                    // rare: the maximum moved inside a group.  Its O, and the sum before it, move along.
+                    if (!(ok = warp_wait(pvdone_bar(sb ^ 1), ((s_cnt - 1) >> 1) & 1, &abort_sh, a.status))) break;
+                    tc_fence_after();
+#pragma unroll 1
+                    for (int c = 0; c < (t > GROUP<PLANES> ? 4 : 2); ++c) {
+                        const uint32_t at = tlane + (c < 2 ? TM_O : TM_X) + half * 64 + (c & 1) * 32;
+                        uint32_t r[32];
+                        tc_ld32(at, r);
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * corr);
+                        tc_st32(at, r);
+                    }
                 }
                 tc_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(pfull_bar(sb));             // P (and the rescaled O) are in place
+                if (lane == 0) mbar_arrive(pfull_bar(sb));             // P is in place, O may be overwritten
             }
             if (!ok) break;
             // ---- the item's result, once the last P V (and with it all earlier ones) has written O ----
             float l_other;
             if (!(ok = exchange(l_run, l_other))) break;
             const float l = half ? l_other + l_run : l_run + l_other;
-            if (!(ok = warp_wait(pvdone_bar((s_cnt - 1) & 1), ((s_cnt - 1) >> 1) & 1, &abort_sh, a.status))) break;
-            tc_fence_after();
             const bool single = it.n_split == 1;
             float *pdst = a.part + ((size_t)it.pair * a.slots + it.split) * part_floats;
-            if (warp_live) {
-                const float inv = 1.f / l;
-#pragma unroll 1
-                for (int c = 0; c < 2; ++c) {
-                    uint32_t r[32];
-                    tc_ld32(tlane + TM_O + half * 64 + c * 32, r);
-                    if (single) {
-                        // through the query region (every MMA that read it is done), so that whole rows go out together
+            const float inv = 1.f / l;
+            auto put = [&](int c, const uint32_t (&r)[32]) {
+                if (single) {
+                    // through the query region (every MMA that read it is done), so that whole rows go out together
 #pragma unroll
-                        for (int e = 0; e < 32; e += 8) {
-                            uint4 hi, lo;
-                            split_pair(__uint_as_float(r[e]) * inv, __uint_as_float(r[e + 1]) * inv, hi.x, lo.x);
-                            split_pair(__uint_as_float(r[e + 2]) * inv, __uint_as_float(r[e + 3]) * inv, hi.y, lo.y);
-                            split_pair(__uint_as_float(r[e + 4]) * inv, __uint_as_float(r[e + 5]) * inv, hi.z, lo.z);
-                            split_pair(__uint_as_float(r[e + 6]) * inv, __uint_as_float(r[e + 7]) * inv, hi.w, lo.w);
-                            if (live) {
-                                uint8_t *dst = q_gen + trow * 256 + (((half * 8 + c * 4 + (e >> 3)) ^ (trow & 15)) << 4);
-                                *reinterpret_cast<uint4 *>(dst) = hi;
-                                *reinterpret_cast<uint4 *>(dst + 2 * qchunk) = lo;
-                            }
+                    for (int e = 0; e < 32; e += 8) {
+                        uint4 hi, lo;
+                        split_pair(__uint_as_float(r[e]) * inv, __uint_as_float(r[e + 1]) * inv, hi.x, lo.x);
+                        split_pair(__uint_as_float(r[e + 2]) * inv, __uint_as_float(r[e + 3]) * inv, hi.y, lo.y);
+                        split_pair(__uint_as_float(r[e + 4]) * inv, __uint_as_float(r[e + 5]) * inv, hi.z, lo.z);
+                        split_pair(__uint_as_float(r[e + 6]) * inv, __uint_as_float(r[e + 7]) * inv, hi.w, lo.w);
+                        if (live) {
+                            uint8_t *dst = q_gen + trow * 256 + (((half * 8 + c * 4 + (e >> 3)) ^ (trow & 15)) << 4);
+                            *reinterpret_cast<uint4 *>(dst) = hi;
+                            *reinterpret_cast<uint4 *>(dst + 2 * qchunk) = lo;
                         }
-                    } else if (live) {
-                        // lanes are rows: 512 contiguous bytes per store
-#pragma unroll
-                        for (int e = 0; e < 32; e += 4)
-                            *reinterpret_cast<uint4 *>(pdst + ((size_t)(half * 16 + c * 8 + (e >> 2)) * a.rows8 + trow) * 4) = make_uint4(r[e], r[e + 1], r[e + 2], r[e + 3]);
                     }
+                } else if (live) {
+                    // lanes are rows: 512 contiguous bytes per store
+#pragma unroll
+                    for (int e = 0; e < 32; e += 4)
+                        *reinterpret_cast<uint4 *>(pdst + ((size_t)(half * 16 + c * 8 + (e >> 2)) * a.rows8 + trow) * 4) = make_uint4(r[e], r[e + 1], r[e + 2], r[e + 3]);
                 }
-            }
+            };
+            if (!(ok = add_group(s_cnt - 1, 1.f, it.n_tiles <= GROUP<PLANES>, true, put))) break;
             tc_fence_before();
             if (single) {
                 float unused;
@@ -546,18 +644,20 @@ int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool sli
     a.subs = (QR + a.rows_sub - 1) / a.rows_sub;
     fill_work(m, a, layer_ord, layer_ord2, streams, batch, M);
     const int grid = work_grid(m);
-    const size_t q_bytes = (size_t)a.rows8 * 512, smem_max = 229000;
+    const int planes = QR > 128 ? 3 : 2;
+    const size_t q_bytes = (size_t)a.rows8 * 256 * planes, smem_max = 229000;
     a.ring_slots = (int)((smem_max - 1024 - q_bytes) / SLOT_BYTES);
     if (a.ring_slots > AT_MAX_SLOTS) a.ring_slots = AT_MAX_SLOTS;
     const size_t smem = 1024 + q_bytes + (size_t)a.ring_slots * SLOT_BYTES;
     static bool attr_done[64];
     if (first_use_on_device(attr_done)) {
-        CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
+        CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
+        CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
     }
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     pdl_config(cfg, attr, dim3(grid), dim3(AT_THREADS), smem, st);
-    CUDA_TRY(cudaLaunchKernelEx(&cfg, attention_tc_kernel, cm.k, cm.v, cm2->k, cm2->v, a));
+    CUDA_TRY(cudaLaunchKernelEx(&cfg, planes == 3 ? attention_tc_kernel<3> : attention_tc_kernel<2>, cm.k, cm.v, cm2->k, cm2->v, a));
     LAUNCH_CHECK();
     return VIASD_OK;
 }

@@ -159,3 +159,50 @@ def test_one_sweep_of_many_rows_is_the_two_passes(batch, nodes):
             assert torch.equal(w, t)
     assert vb.get_stats(eng.model).device_status == 0 and int(res.n_acc.sum()) == 0
     assert (launches[0] < launches[1]) == (2 * batch * (nodes + 1) > 128)
+
+
+# ---------------------------------------------------------------------------------------------
+# precision of attention with many query rows per kv head
+# ---------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("nodes,ctx", [(63, 900), (32, 2500)])
+def test_attention_of_many_rows_is_as_precise_as_fp32(nodes, ctx):
+    """256 and 132 query rows per kv head, on a model whose logits are the normalised attention output: one layer, embeddings
+    that are exact in bf16 and small, an identity as output projection and head, no feed-forward.  The output goes through
+    two bf16 pairs (2.2e-6 each, rms); fp32 arithmetic adds 1e-6, queries and weights as pairs would add 3e-6 and more."""
+    vb = _vb()
+    H, Hkv, hd, M, B = 8, 2, 128, nodes + 1, 2
+    d, V, ff, N = H * hd, H * hd, 128, nodes
+    g = torch.Generator(device="cuda").manual_seed(7)
+    rnd = lambda *shape, s=1.0: (torch.randn(*shape, device="cuda", generator=g) * s).bfloat16()
+    eye, zero, ones = torch.eye(d, device="cuda").bfloat16(), torch.zeros(ff, d, device="cuda").bfloat16(), torch.ones(d, device="cuda")
+    wq, wk, wv = rnd(H * hd, d, s=0.04), rnd(Hkv * hd, d, s=0.04), rnd(Hkv * hd, d, s=0.04)
+    embed = rnd(V, d, s=2.0 ** -14)
+    layer = dict(wq=wq, wk=wk, wv=wv, wo=eye, wg=zero, wu=zero, wd=zero.T.contiguous(), norm1=ones, norm2=ones)
+    max_ctx = ctx + M + 5
+    cfg = vb.make_config(1, d, H, Hkv, hd, ff, V, "bf16", B, max_ctx, M, rms_eps=0.0)
+    ws = torch.empty(vb.workspace_bytes(cfg, 1), dtype=torch.uint8, device="cuda")
+    model = vb.init_model(cfg, embed, eye, ones, [layer], [1], ws)
+    kc, vc = rnd(1, B, Hkv, max_ctx, hd, s=1.3), rnd(1, B, Hkv, max_ctx, hd, s=1.3)
+    ints = lambda *s: torch.randint(0, V, s, dtype=torch.int32, device="cuda", generator=g)
+    pending, tok = ints(B), ints(B, N)
+    cache = vb.make_cache(kc, vc, kc.clone(), vc.clone(), torch.full((B,), ctx, dtype=torch.int32, device="cuda"), pending)
+    parent = torch.arange(-1, N - 1, dtype=torch.int32, device="cuda")
+    logits = torch.empty(B, M, V, device="cuda")
+    vb.full_forward(model, cache, vb.make_draft(tok, parent, parent, 0, None), logits)
+    torch.cuda.synchronize()
+    assert vb.get_stats(model).device_status == 0
+    e = embed[torch.cat([pending[:, None], tok], 1).long()].double()
+    a = e * torch.rsqrt((e * e).mean(-1, keepdim=True))
+    q = (a @ wq.double().T).view(B, M, H, hd)
+    pos = (ctx + torch.arange(M, device="cuda")).double()[:, None] * 1e4 ** (-2 * torch.arange(hd // 2, device="cuda").double() / hd)
+    c, s = torch.cos(pos)[None, :, None], torch.sin(pos)[None, :, None]
+    q = torch.cat([q[..., :64] * c - q[..., 64:] * s, q[..., 64:] * c + q[..., :64] * s], -1)
+    n = ctx + M                                                # the block's own rows as the cache holds them
+    keys, values = kc[0, :, :, :n].double().repeat_interleave(H // Hkv, 1), vc[0, :, :, :n].double().repeat_interleave(H // Hkv, 1)
+    score = torch.einsum("bmhd,bhkd->bhmk", q, keys) / hd ** 0.5
+    hidden = torch.ones(M, n, dtype=torch.bool, device="cuda").triu(ctx + 1)
+    out = torch.einsum("bhmk,bhkd->bmhd", score.masked_fill(hidden, -np.inf).softmax(-1), values).reshape(B, M, d)
+    h = e + out
+    want = h * torch.rsqrt((h * h).mean(-1, keepdim=True))
+    rel = float((logits.double() - want).norm() / want.norm())
+    assert rel < 4.2e-6, rel
