@@ -58,6 +58,7 @@ struct Workspace {                      // pointers into the caller's workspace 
     TreeInfo *tree;                     // [max_batch]: every sequence has its own draft tree (copies when the call shares one)
     DeviceStats *stats;
     float *accept_scratch;              // [3][B, judges + 1, 64] row statistics
+    float *accept_fold;                 // [B, judges + 1, vocab] residuals of a position with many rejections (sampling)
     float *gemm_scratch;                // partial tiles of split GEMM work (tcgen05 kernel)
     int *gemm_counters;                 // per-tile arrival counters, zero between launches
     size_t n_counters;

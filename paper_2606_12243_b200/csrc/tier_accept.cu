@@ -12,9 +12,9 @@
 // it is: a row-statistics kernel (one CTA per logits row, all rows at once, one sweep) leaves each row's maximum, argmax
 // and softmax denominator, and the walk starts by fetching the tree and every node's two logits at once, so that a test is
 // arithmetic on shared memory.  Only a rejection in sampling mode (residual, Eq. A.3) and the final draw sweep the
-// vocabulary: one sweep and one exchange among the cluster's CTAs each.  The residuals are not written out: an element is
-// worked out from the logits by replaying the rejections so far (a handful of scalars), in the arithmetic of Eq. A.3 round
-// by round.  CTAs exchange their sums by storing them into each other's shared memory before one cluster barrier; every
+// vocabulary: one sweep and one exchange among the cluster's CTAs each.  An element of a residual is worked out from the logits
+// by replaying the rejections so far (a handful of scalars), in the arithmetic of Eq. A.3 round by round; every FOLD of them at
+// one position are written out and the replay starts from there, so that a star of many children stays linear.  CTAs exchange their sums by storing them into each other's shared memory before one cluster barrier; every
 // CTA adds them in the same order, so all of them walk the same way.
 #include "common.cuh"
 #include <string.h>
@@ -27,6 +27,10 @@ constexpr int MAX_TEAM = 16;
 constexpr int MAXJ = VIASD_MAX_JUDGES;    // verifiers that may judge a drafted token (the last one is q); 2 for three tiers
 constexpr int KINDS = MAXJ + 1;           // distributions kept per position: the proposal and the judges
 constexpr int ACC_TEAM = 8;               // CTAs per sequence in sampling mode (a portable cluster size)
+// Rejections at one position that are replayed per element before they are written out.  Rejected children of one position,
+// us, all written out as they come / all replayed / eight at a time: 63, vocabulary 128256 933 / 1264 / 457, 8000 495 / 1167 /
+// 373, 1024 195 / - / 194; 12, vocabulary 128256 218 / 138 / 109.
+constexpr int FOLD = 8;
 
 // ---- counter-based uniforms -------------------------------------------------------------------
 __device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
@@ -238,6 +242,8 @@ struct AcceptArgs {
     RowStats rs;
     const float *judges[KINDS];              // [1..n_judges]: each judge's logits [B, M, V], weakest first, q last
     const float *drafter;                    // [B, R, V]
+    float *fold;                             // [B, KINDS, V]: numerators with the rejections folded in, each thread's own
+    int vec;                                 // all rows are 16-byte aligned: sweeps take 16 bytes at a time
     int n_judges;
     const int *draft_tok, *prow, *parent;    // [B, N], [N], [N]
     unsigned char *tier;                     // [B, N]
@@ -269,6 +275,8 @@ struct Walk {                                  // per CTA: everything the walk r
     int first_child[RS_STRIDE], next_sibling[RS_STRIDE], tok[RS_STRIDE], prow[RS_STRIDE], tier[RS_STRIDE];
     int judged[RS_STRIDE], path[RS_STRIDE];
     float xj[RS_STRIDE], x0[RS_STRIDE];        // logit of the node's token in its judge's row and in its drafter row
+    float jv[2][RS_STRIDE], pv[2][RS_STRIDE];  // numerators of the token of each child of this position, after the rejections so far
+                                               // (alternate positions: the test that ended the last one may still be reading)
     float mx[KINDS][RS_STRIDE], z[KINDS][RS_STRIDE];
     int arg[KINDS][RS_STRIDE];
     Rejection rej[RS_STRIDE];
@@ -300,10 +308,12 @@ __device__ __forceinline__ float2 team_exchange(float2 v, float2 none, Team &tm)
     return lane < (int)tm.size ? slot[lane] : none;
 }
 
-// f(i, x, y) for this CTA's share of a row's indices i; x, y: the values of two rows there (y: 0 when b is null)
+// f(x, y, i) for this CTA's share of a row's indices, N at a time from i on; x, y: the values of two rows there (y: 0 when b
+// is null)
+// (which thread gets an index depends on `vec`, the vocabulary and the team only: what a thread writes there it reads again)
 template <typename F>
-__device__ __forceinline__ void sweep_rows(const float *a, const float *b, int V, const Team &tm, F f) {
-    if ((V & 3) == 0 && ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0) {
+__device__ __forceinline__ void sweep_rows(const float *a, const float *b, int V, bool vec, const Team &tm, F f) {
+    if (vec) {
         const float4 *a4 = reinterpret_cast<const float4 *>(a), *b4 = reinterpret_cast<const float4 *>(b);
         const int n4 = V >> 2, per = (n4 + (int)tm.size - 1) / (int)tm.size, lo = (int)tm.rank * per, hi = min(n4, lo + per);
         // eight loads in flight, then a rolled loop over pieces of four values (indexed, so they pass through local memory): a
@@ -321,24 +331,31 @@ __device__ __forceinline__ void sweep_rows(const float *a, const float *b, int V
             const int n = min(4, (hi - i0 + ACC_THREADS - 1) / ACC_THREADS);
 #pragma unroll 1
             for (int j = 0; j < n; ++j) {
-                const int i = 4 * (i0 + j * ACC_THREADS);
-                const float4 u = x[j], v = y[j];
-                f(i, u.x, v.x); f(i + 1, u.y, v.y); f(i + 2, u.z, v.z); f(i + 3, u.w, v.w);
+                const float u[4] = {x[j].x, x[j].y, x[j].z, x[j].w}, v[4] = {y[j].x, y[j].y, y[j].z, y[j].w};
+                f(u, v, 4 * (i0 + j * ACC_THREADS));
             }
         }
     } else {
-        for (int i = tm.rank * ACC_THREADS + threadIdx.x; i < V; i += tm.size * ACC_THREADS) f(i, a[i], b ? b[i] : 0.f);
+        for (int i = tm.rank * ACC_THREADS + threadIdx.x; i < V; i += tm.size * ACC_THREADS) {
+            const float u[1] = {a[i]}, v[1] = {b ? b[i] : 0.f};
+            f(u, v, i);
+        }
     }
 }
 
-// Numerators at token i after the rejections so far: the judge of tier t (starting from jt) and the proposal (from pr).
+// Numerators at tokens i, i + 1, ... after the rejections so far: the judge of tier t (starting from jt) and the proposal (pr).
 // Eq. A.3 round by round: the rejecting judge becomes its residual against the proposal (kept as it is if the residual
 // vanishes); the rejected token leaves the proposal.
-__device__ __forceinline__ void replay(const Rejection *rej, int n, int i, int t, float &jt, float &pr) {
+template <int N>
+__device__ __forceinline__ void replay(const Rejection *rej, int n, int i, int t, float (&jt)[N], float (&pr)[N]) {
     for (int k = 0; k < n; ++k) {
         const Rejection r = rej[k];
-        if (r.t == t && r.sj >= 0.f) jt = fmaxf(0.f, jt * r.sj - pr * r.sp);
-        if (i == r.v) pr = 0.f;
+        if (r.t == t && r.sj >= 0.f) {
+#pragma unroll
+            for (int e = 0; e < N; ++e) jt[e] = fmaxf(0.f, jt[e] * r.sj - pr[e] * r.sp);
+        }
+#pragma unroll
+        for (int e = 0; e < N; ++e) pr[e] = i + e == r.v ? 0.f : pr[e];
     }
 }
 
@@ -409,22 +426,41 @@ accept_kernel(AcceptArgs a) {
         if (b == 0 && tid == 0) atomicAdd(&a.stats->steps, 1ull);
     }
 
+    // What rejections at this position have been folded into the arrays of a.fold: the first `n_fold`, those of the judges in
+    // `folded` (bit t; bit 0: the proposal's array is in use).
+    int n_fold = 0;
+    unsigned folded = 0;
+    auto fold_row = [&](int k) { return a.fold + ((size_t)b * KINDS + k) * V; };
+    auto judge_row = [&](int t, int cur) -> const float * { return folded >> t & 1 ? fold_row(t) : a.judges[t] + ((size_t)b * M + cur) * V; };
+    auto proposal_row = [&](const float *r0) -> const float * { return folded & 1 ? fold_row(0) : r0; };
+    // the judge's and the proposal's numerators from i on after n_rej rejections, from what judge_row and proposal_row hold there
+    auto numerators = [&](int t, int i, const auto &xt, float mxt, const auto &x0, float mx0, int n_rej, auto &jt, auto &pr) {
+        constexpr int N = sizeof(jt) / sizeof(float);
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            jt[e] = folded >> t & 1 ? xt[e] : expf((xt[e] - mxt) * a.inv_temp);
+            pr[e] = folded & 1 ? x0[e] : expf((x0[e] - mx0) * a.inv_temp);
+        }
+        replay(w.rej + n_fold, n_rej - n_fold, i, t, jt, pr);
+    };
+
     // argmax_v (log weight(v) - log(-log u_v)): a draw from the judge of tier t at block row `cur` after n_rej rejections
     auto draw = [&](int t, int cur, const float *r0, float mx0, int n_rej) -> int {
         const float *rt = a.judges[t] + ((size_t)b * M + cur) * V;
         const float mxt = w.mx[t][cur];
         MaxIdx best = no_idx();
-        sweep_rows(rt, n_rej ? r0 : nullptr, V, tm, [&](int i, float xt, float x0) {
-            float jt = 1.f, lw = (xt - mxt) * a.inv_temp;         // log weight; through the residuals once there are any
-            if (n_rej) {
-                jt = expf(lw);
-                float pr = expf((x0 - mx0) * a.inv_temp);
-                replay(w.rej, n_rej, i, t, jt, pr);
-                lw = logf(jt);
+        sweep_rows(n_rej ? judge_row(t, cur) : rt, n_rej ? proposal_row(r0) : nullptr, V, a.vec, tm, [&](const auto &xt, const auto &x0, int i) {
+            constexpr int N = sizeof(xt) / sizeof(float);
+            float jt[N], pr[N];
+            if (n_rej) numerators(t, i, xt, mxt, x0, mx0, n_rej, jt, pr);
+#pragma unroll
+            for (int e = 0; e < N; ++e) {
+                // log weight; through the residuals once there are any
+                const float lw = n_rej ? logf(jt[e]) : (xt[e] - mxt) * a.inv_temp;
+                const float u = unit_f32(k_gum, ((unsigned long long)cur << 32) + (unsigned long long)(i + e));
+                MaxIdx c; c.v = !n_rej || jt[e] > 0.f ? lw - logf(-logf(u)) : -INFINITY; c.i = i + e;
+                best = better(best, c);
             }
-            const float u = unit_f32(k_gum, ((unsigned long long)cur << 32) + (unsigned long long)i);
-            MaxIdx c; c.v = jt > 0.f ? lw - logf(-logf(u)) : -INFINITY; c.i = i;
-            best = better(best, c);
         });
         best = block_argmax(best, shm);
         if (tm.size > 1) {
@@ -435,14 +471,14 @@ accept_kernel(AcceptArgs a) {
         return best.i == 0x7fffffff ? 0 : best.i;
     };
 
-    int cur = 0, n_acc = 0, corr = -1, corr_src = 0, parity = 0, draw_t = 0, n_rej = 0;
+    int cur = 0, n_acc = 0, corr = -1, corr_src = 0, parity = 0, draw_t = 0, n_rej = 0, pos = 0;
     const float *r0 = nullptr;                                   // the drafter row of this position and its maximum
     float mx0 = 0.f;
-    const float scale2 = a.inv_temp * LOG2E;
     bool needs_q = false;
     while (true) {
         int c = w.first_child[cur];
-        n_rej = 0;
+        n_rej = n_fold = 0;
+        folded = 0;
         r0 = nullptr;
         if (c < 0) {                                             // leaf: whole path accepted
             if (a.emit_bonus && a.probe) { needs_q = true; break; }
@@ -475,16 +511,20 @@ accept_kernel(AcceptArgs a) {
                     r0 = a.drafter + ((size_t)b * a.R + row0) * V;
                     mx0 = w.mx[0][row0];
                     Z[0] = w.z[0][row0];
+                    pos ^= 1;
+                    for (int n = tid; n < N; n += ACC_THREADS) {      // (of the children of this row; the others' are not used)
+                        // a child that names another drafter row than its elder sibling is still tested against that sibling's
+                        const float x0 = w.prow[n] == row0 ? w.x0[n] : r0[w.tok[n]];
+                        w.jv[pos][n] = expf((w.xj[n] - w.mx[w.tier[n]][cur]) * a.inv_temp);
+                        w.pv[pos][n] = expf((x0 - mx0) * a.inv_temp);
+                    }
+                    __syncthreads();
                 }
 #pragma unroll
                 for (int k = 1; k < KINDS; ++k) if (k == t) Zt = Z[k];
                 const float u = unit_f32(k_acc, (unsigned long long)c);
-                // (a child that names another drafter row than its elder sibling is still tested against that sibling's)
-                const float x0 = w.prow[c] == row0 ? w.x0[c] : r0[v];
-                float pv = expf((x0 - mx0) * a.inv_temp), jv = expf((w.xj[c] - mxt) * a.inv_temp);
-                replay(w.rej, n_rej, v, t, jv, pv);
-                const float lp = logf(pv / Z[0]);
-                const float lj = logf(jv / Zt);
+                const float lp = logf(w.pv[pos][c] / Z[0]);
+                const float lj = logf(w.jv[pos][c] / Zt);
                 pass = (logf(u) + a.log1m_alpha + lp) < lj;       // u < j(v) / ((1 - alpha) p(v)), Eq. A.2
             }
             if (pass) {
@@ -497,13 +537,36 @@ accept_kernel(AcceptArgs a) {
             if (sampling) {
                 // the masses of the judge's residual and of the proposal without the rejected token
                 const float sj = a.inv_beta / Zt, sp = 1.f / Z[0];
-                const float *rt = a.judges[t] + ((size_t)b * M + cur) * V;
+                if (n_rej - n_fold == FOLD) {
+                    // the judges that have rejected, the proposal with the last of them (all start from its old values)
+                    unsigned write = 0;
+                    for (int k = 0; k < n_rej; ++k) write |= 1u << w.rej[k].t;
+                    for (int k = 1; k <= J; ++k) {
+                        if (!(write >> k & 1)) continue;
+                        const bool last = write >> (k + 1) == 0;
+                        float *to = fold_row(k), *to0 = fold_row(0);
+                        const float mxk = w.mx[k][cur];
+                        sweep_rows(judge_row(k, cur), proposal_row(r0), V, a.vec, tm, [&](const auto &xt, const auto &x0, int i) {
+                            constexpr int N = sizeof(xt) / sizeof(float);
+                            float jt[N], pr[N];
+                            numerators(k, i, xt, mxk, x0, mx0, n_rej, jt, pr);
+#pragma unroll
+                            for (int e = 0; e < N; ++e) { to[i + e] = jt[e]; if (last) to0[i + e] = pr[e]; }
+                        });
+                    }
+                    folded |= write | 1u;
+                    n_fold = n_rej;
+                }
                 float s = 0.f, z = 0.f;
-                sweep_rows(rt, r0, V, tm, [&](int i, float xt, float x0) {
-                    float jt = ex2((xt - mxt) * scale2), pr = ex2((x0 - mx0) * scale2);
-                    replay(w.rej, n_rej, i, t, jt, pr);
-                    s += fmaxf(0.f, jt * sj - pr * sp);
-                    z += i == v ? 0.f : pr;
+                sweep_rows(judge_row(t, cur), proposal_row(r0), V, a.vec, tm, [&](const auto &xt, const auto &x0, int i) {
+                    constexpr int N = sizeof(xt) / sizeof(float);
+                    float jt[N], pr[N];
+                    numerators(t, i, xt, mxt, x0, mx0, n_rej, jt, pr);
+#pragma unroll
+                    for (int e = 0; e < N; ++e) {
+                        s += fmaxf(0.f, jt[e] * sj - pr[e] * sp);
+                        z += i + e == v ? 0.f : pr[e];
+                    }
                 });
                 s = block_sum(s, sh[2 * parity]);
                 z = block_sum(z, sh[2 * parity + 1]);
@@ -513,8 +576,15 @@ accept_kernel(AcceptArgs a) {
                     s = warp_sum(got.x);
                     z = warp_sum(got.y);
                 }
-                if (tid == 0) w.rej[n_rej] = Rejection{t, v, s > 0.f ? sj : -1.f, sp};
+                const Rejection r{t, v, s > 0.f ? sj : -1.f, sp};
+                if (tid == 0) w.rej[n_rej] = r;
                 ++n_rej;
+                for (int n = tid; n < N; n += ACC_THREADS) {
+                    float jt[1] = {w.jv[pos][n]}, pr[1] = {w.pv[pos][n]};
+                    replay(&r, 1, w.tok[n], w.tier[n], jt, pr);
+                    w.jv[pos][n] = jt[0];
+                    w.pv[pos][n] = pr[0];
+                }
 #pragma unroll
                 for (int k = 1; k < KINDS; ++k) if (k == t && s > 0.f) Z[k] = s;
                 if (z > 0.f) Z[0] = z;
@@ -634,6 +704,10 @@ int launch_accept(const viasd_model *m, const viasd_draft *d, const viasd_params
     for (int k = 1; k < KINDS; ++k) a.judges[k] = k <= js.n ? js.logits[k - 1] : nullptr;
     a.n_judges = js.n;
     a.drafter = d->drafter_logits;
+    a.fold = m->ws.accept_fold;
+    uintptr_t rows16 = (uintptr_t)a.drafter;
+    for (int k = 1; k <= js.n; ++k) rows16 |= (uintptr_t)a.judges[k];
+    a.vec = m->cfg.vocab % 4 == 0 && (rows16 & 15) == 0;
     a.draft_tok = d->draft_tok; a.prow = d->prow; a.parent = d->parent; a.tier = r->tier; a.conf = r->conf; a.tree = m->ws.tree;
     a.do_tier = do_tier ? 1 : 0; a.conf_source = p->conf_source;
     a.cuts = tier_cuts(js);

@@ -206,3 +206,46 @@ def test_attention_of_many_rows_is_as_precise_as_fp32(nodes, ctx):
     want = h * torch.rsqrt((h * h).mean(-1, keepdim=True))
     rel = float((logits.double() - want).norm() / want.norm())
     assert rel < 4.2e-6, rel
+
+
+# ---------------------------------------------------------------------------------------------
+# many rejections at one position
+# ---------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("vocab,team,nodes,alpha,beta", [(4099, 1, 40, 0.0, 1.0), (4100, 1, 25, 0.1, 0.8), (33000, 8, 40, 0.0, 1.0), (20003, 2, 17, 0.0, 1.3)])
+def test_star_of_rejected_children(vocab, team, nodes, alpha, beta):
+    """A star of children, all unlikely under their judges, half of them judged by either: the rejections of one position are
+    written out every eighth time and replayed between; vocabularies of every alignment, one CTA and several.  The last
+    child is likely, so that a test after many rejections passes too.  Decisions against the oracle under the margin rule."""
+    from oracle import tiers
+    from tests import parity_util as PU
+    vb = _vb()
+    base = W.get("mini_8b_tree")
+    wl = replace(base, batch=4, ctx=8, parent=tuple([-1] * nodes), shape=replace(base.shape, vocab=vocab, n_layers=1), n_routed=1)
+    eng = _engine(wl)
+    vb.set_option(eng.model, "accept_team", team)
+    si = eng.inputs
+    rng = np.random.default_rng(vocab)
+    B, M, V = wl.batch, wl.rows, vocab
+    near = np.repeat(si.drafter_logits[:, :1], M, axis=1)
+    slim = (near + rng.standard_normal((B, M, V))).astype(np.float32)
+    full = (near + rng.standard_normal((B, M, V))).astype(np.float32)
+    for b in range(B):
+        for n in range(nodes):
+            d = 12.0 if n == nodes - 1 and b % 2 else -6.0
+            slim[b, 0, si.draft_tok[b, n]] += d
+            full[b, 0, si.draft_tok[b, n]] += d
+    d = tiers.tier_rule(si.drafter_logits, si.draft_tok, si.prow, 0.0, 0.0)[1].ravel()
+    lo, hi = float(np.median(d)), 1.0                          # nothing is accepted outright
+    res = vb.alloc_result(B, nodes)
+    p = eng.params(log_tau_lo=lo, log_tau_hi=hi, mode=1, alpha=alpha, beta=beta)
+    vb.tier_accept(eng.model, eng.draft, p, torch.from_numpy(slim).cuda(), torch.from_numpy(full).cuda(), 3, res)
+    torch.cuda.synchronize()
+    tier, _ = tiers.tier_rule(si.drafter_logits, si.draft_tok, si.prow, lo, hi)
+    assert np.array_equal(res.tier.cpu().numpy(), tier)
+    P = tiers.Params(mode="sampling", temperature=wl.temperature, seed=wl.seed, alpha=alpha, beta=beta)
+    seqs = tiers.resolve(si.draft_tok, wl.parent, si.prow, tier, si.drafter_logits, slim, full, P)
+    assert int(((res.judge & 3) == 2).sum()) >= 9 * B          # folded in every sequence
+    pinned, total, whole = PU.compare_resolution(seqs, res.n_acc.cpu().numpy(), res.path.cpu().numpy(), res.out_tok.cpu().numpy(),
+                                                 res.n_emit.cpu().numpy(), res.corr_src.cpu().numpy(), eps_row=2.5e-5)
+    PU.assert_pinned(f"star of {nodes}, vocabulary {vocab}", pinned, total, whole, B, 0.85, 3)
+    assert vb.get_stats(eng.model).device_status == 0 and eng.guards_intact()
