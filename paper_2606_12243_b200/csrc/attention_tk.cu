@@ -117,12 +117,6 @@ __device__ __forceinline__ bool next_item(const AttnTkArgs &a, int per, ItemSrc 
     return false;
 }
 
-__device__ __forceinline__ float ex2(float x) {            // 2^x, hardware approximation (2 ulp)
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 // MN-major operand tile with the 128-byte swizzle: 64 contiguous elements along MN per row of 128 bytes,
 // 8 rows (8 steps of the contraction) per 1024-byte group; groups `sbo` bytes apart along the contraction,
 // 64-element blocks `lbo` bytes apart along MN.

@@ -152,12 +152,6 @@ __device__ __forceinline__ size_t row_off(const AttnWork &a, const Item &i, int 
     const int g2 = i.row0 + r, hq = (int)((g2 * a.m_recip) >> 32);
     return ((size_t)(i.be * a.M + g2 - hq * a.M) * a.H + i.kvh * (a.H / a.Hkv) + hq) * HD;
 }
-__device__ __forceinline__ float ex2(float x) {            // 2^x, hardware approximation (2 ulp)
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 // x0, x1 -> packed bf16 pairs hi = bf16(x), lo = bf16(x - hi); the low half word is the even element
 __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t &hi, uint32_t &lo) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);

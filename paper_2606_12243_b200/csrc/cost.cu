@@ -19,7 +19,6 @@ namespace {
 constexpr int COST_THREADS = 512, COST_WARPS = COST_THREADS / 32, MAX_TEAM = 4;
 constexpr int BATCH = 4;                        // 16-byte loads of each row in flight per thread
 constexpr float REF_GAP = 20.f;                 // a thread's reference may be exceeded by this much (in exponent units)
-constexpr float LOG2E = 1.4426950408889634f;
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
@@ -29,6 +28,9 @@ __device__ __forceinline__ void push_f32(float *own, unsigned rank, float v) {  
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
 struct Share { unsigned rank, size; };          // this CTA's place among the CTAs of its row
+__device__ __forceinline__ void row_barrier(const Share &s) {
+    if (s.size > 1) { cluster_arrive(); cluster_wait(); } else __syncthreads();
+}
 __device__ __forceinline__ Share row_share() {
     Share s;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(s.rank));
@@ -105,32 +107,26 @@ __device__ __forceinline__ void sweep_pair(const float *a, const float *b, int V
     }
 }
 
-__device__ __forceinline__ float ex2(float x) {            // 2^x, hardware approximation (2 ulp)
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// Running maximum and denominator of one row, per thread: sum of exp((x - ref) / T); scale2 = log2(e) / T.
+// Running maximum and denominator of one row, per thread: sum of exp((x - ref) / T).
 struct Denom {
     float ref, lim, mx, s;
     __device__ __forceinline__ void init() { ref = lim = mx = -INFINITY; s = 0.f; }
     template <int N>
-    __device__ __forceinline__ void add(Count<N>, const float (&x)[4 * BATCH], float scale2, float gap) {
+    __device__ __forceinline__ void add(Count<N>, const float (&x)[4 * BATCH], ExpScale scale, float gap) {
         float bm = x[0];
 #pragma unroll
         for (int e = 1; e < N; ++e) bm = fmaxf(bm, x[e]);
         if (bm > lim) {                             // the first values, or far above the reference: rare
-            s *= ex2((ref - bm) * scale2);
+            s *= exp_scaled(ref - bm, scale);
             ref = bm;
             lim = bm + gap;
         }
         mx = fmaxf(mx, bm);
         const float r = ref == -INFINITY ? 0.f : ref;
 #pragma unroll
-        for (int e = 0; e < N; ++e) s += ex2((x[e] - r) * scale2);
+        for (int e = 0; e < N; ++e) s += exp_scaled(x[e] - r, scale);
     }
-    __device__ __forceinline__ float at(float m, float scale2) const { return ref == -INFINITY ? 0.f : s * ex2((ref - m) * scale2); }
+    __device__ __forceinline__ float at(float m, ExpScale scale) const { return ref == -INFINITY ? 0.f : s * exp_scaled(ref - m, scale); }
 };
 
 __device__ __forceinline__ float phi(float z, int smooth, float tau, float inv_tau) {
@@ -145,14 +141,13 @@ __device__ __forceinline__ float phi(float z, int smooth, float tau, float inv_t
 template <int SMOOTH>
 __global__ void __launch_bounds__(COST_THREADS, 2)
 kl_cost_kernel(float *__restrict__ cost_rows, const float *__restrict__ judge, const float *__restrict__ proposal, int rows, int V,
-               float inv_temp, float log1m_alpha, float log_beta, float tau) {
+               ExpScale scale, float inv_temp, float log1m_alpha, float log_beta, float tau) {
     __shared__ float sh_mx[2][COST_WARPS], sh_s[2][COST_WARPS], sh_c[1][COST_WARPS], part[2][4][MAX_TEAM], fin[2][MAX_TEAM];
     const Share me = row_share();
     const int lane = threadIdx.x & 31, clusters = gridDim.x / me.size;
     const bool on = lane < (int)me.size;
-    const float gap = REF_GAP / inv_temp, inv_tau = SMOOTH ? 1.f / tau : 0.f, scale2 = inv_temp * LOG2E;
-    cluster_arrive();
-    cluster_wait();                                           // every CTA of the cluster runs: its shared memory may be written
+    const float gap = REF_GAP / inv_temp, inv_tau = SMOOTH ? 1.f / tau : 0.f;
+    row_barrier(me);                                          // every CTA of the cluster runs: its shared memory may be written
     int buf = 0, before = -1;
     auto finish_before = [&]() {                              // the row before this one, by one warp of CTA 0
         if (before >= 0 && me.rank == 0 && threadIdx.x < 32) {
@@ -164,52 +159,55 @@ kl_cost_kernel(float *__restrict__ cost_rows, const float *__restrict__ judge, c
         const float *jq = judge + (size_t)row * V, *pp = proposal + (size_t)row * V;
         Denom dq, dp;
         dq.init(); dp.init();
-        sweep_pair(jq, pp, V, me, [&](auto n, const float (&q)[4 * BATCH], const float (&p)[4 * BATCH]) { dq.add(n, q, scale2, gap); dp.add(n, p, scale2, gap); });
+        sweep_pair(jq, pp, V, me, [&](auto n, const float (&q)[4 * BATCH], const float (&p)[4 * BATCH]) { dq.add(n, q, scale, gap); dp.add(n, p, scale, gap); });
         float m[2] = {dq.mx, dp.mx};
         block_combine<2>(m, sh_mx, MaxOp());                  // this CTA's maxima (-inf if it has no share) ...
-        float z[2] = {dq.at(m[0], scale2), dp.at(m[1], scale2)};
+        float z[2] = {dq.at(m[0], scale), dp.at(m[1], scale)};
         block_combine<2>(z, sh_s, SumOp());                   // ... and denominators relative to them
         if (threadIdx.x < me.size) {
             push_f32(&part[buf][0][me.rank], threadIdx.x, m[0]); push_f32(&part[buf][1][me.rank], threadIdx.x, m[1]);
             push_f32(&part[buf][2][me.rank], threadIdx.x, z[0]); push_f32(&part[buf][3][me.rank], threadIdx.x, z[1]);
         }
-        cluster_arrive();
-        cluster_wait();
+        row_barrier(me);
         finish_before();
         const float a = on ? part[buf][0][lane] : -INFINITY, b = on ? part[buf][1][lane] : -INFINITY;
         const float mq = warp_all(a, MaxOp()), mp = warp_all(b, MaxOp());
-        const float lzq = logf(warp_all(a == -INFINITY ? 0.f : part[buf][2][lane] * expf((a - mq) * inv_temp), SumOp()));
-        const float lzp = logf(warp_all(b == -INFINITY ? 0.f : part[buf][3][lane] * expf((b - mp) * inv_temp), SumOp()));
-        float acc[1] = {0.f};
+        const float zq = warp_all(a == -INFINITY ? 0.f : part[buf][2][lane] * exp_scaled(a - mq, scale), SumOp());
+        const float zp = warp_all(b == -INFINITY ? 0.f : part[buf][3][lane] * exp_scaled(b - mp, scale), SumOp());
+        // lp - lq as (p - q) / T plus a constant of the row that is worked out from small numbers, the weights' denominators
+        // outside the sums: log q and log p themselves are of the order of ten, and their last bit was the cost's error
+        // (vocabulary 152064: 7.4e-7 rms, now 2.8e-7)
+        const float shift = fmaf(mq - mp, inv_temp, logf(zq / zp)), sh1 = log1m_alpha + shift, sh2 = log_beta + shift;
+        float acc_p = 0.f, acc_q = 0.f;
         sweep_pair(jq, pp, V, me, [&](auto n, const float (&q)[4 * BATCH], const float (&p)[4 * BATCH]) {
 #pragma unroll
             for (int e = 0; e < decltype(n)::n; ++e) {
-                const float lq = (q[e] - mq) * inv_temp - lzq, lp = (p[e] - mp) * inv_temp - lzp, d = lp - lq;
-                acc[0] += ex2(lp * LOG2E) * phi(log1m_alpha + d, SMOOTH, tau, inv_tau) + ex2(lq * LOG2E) * phi(log_beta + d, SMOOTH, tau, inv_tau);
+                const float d = p[e] - q[e];
+                acc_p += exp_scaled(p[e] - mp, scale) * phi(fmaf(d, inv_temp, sh1), SMOOTH, tau, inv_tau);
+                acc_q += exp_scaled(q[e] - mq, scale) * phi(fmaf(d, inv_temp, sh2), SMOOTH, tau, inv_tau);
             }
         });
+        float acc[1] = {acc_p / zp + acc_q / zq};
         block_combine<1>(acc, sh_c, SumOp());
         if (threadIdx.x == 0) push_f32(&fin[buf][me.rank], 0, acc[0]);
     }
-    cluster_arrive();
-    if (me.rank != 0) return;                                 // (only CTA 0's shared memory is still read)
-    cluster_wait();
+    row_barrier(me);
+    if (me.rank != 0) return;
     finish_before();
 }
 
 // Region masses (Eq. B.8-B.10): per row, the mass of p = softmax(proposal / T) on the tokens the gating row places in
 // region A (d >= log tau_hi), B (log tau_lo <= d < log tau_hi) and C (below), d = l[u] - max l in fp32 exactly as the
-// tier kernel decides a drafted token.  Built like the cost kernel: maxima, then the sums.
+// tier kernel decides a drafted token.  Built like the cost kernel: maxima, then the sums.  (scale2 = log2(e) / T: the masses
+// are shares of one sum, in which a scale that is slightly off cancels.)
 __global__ void __launch_bounds__(COST_THREADS, 2)
 region_mass_kernel(float *__restrict__ mass, const float *__restrict__ gate, const float *__restrict__ proposal, int rows, int V,
-                   float inv_temp, float log_tau_hi, float log_tau_lo) {
+                   float scale2, float log_tau_hi, float log_tau_lo) {
     __shared__ float sh_mx[2][COST_WARPS], sh_s[3][COST_WARPS], part[2][2][MAX_TEAM], fin[2][3][MAX_TEAM];
     const Share me = row_share();
     const int lane = threadIdx.x & 31, clusters = gridDim.x / me.size;
     const bool on = lane < (int)me.size;
-    const float scale2 = inv_temp * LOG2E;
-    cluster_arrive();
-    cluster_wait();
+    row_barrier(me);
     int buf = 0, before = -1;
     auto finish_before = [&]() {
         if (before >= 0 && me.rank == 0 && threadIdx.x < 32) {
@@ -229,8 +227,7 @@ region_mass_kernel(float *__restrict__ mass, const float *__restrict__ gate, con
         });
         block_combine<2>(v, sh_mx, MaxOp());
         if (threadIdx.x < me.size) { push_f32(&part[buf][0][me.rank], threadIdx.x, v[0]); push_f32(&part[buf][1][me.rank], threadIdx.x, v[1]); }
-        cluster_arrive();
-        cluster_wait();
+        row_barrier(me);
         finish_before();
         const float mg = warp_all(on ? part[buf][0][lane] : -INFINITY, MaxOp()), mp = warp_all(on ? part[buf][1][lane] : -INFINITY, MaxOp());
         float m[3] = {0.f, 0.f, 0.f};
@@ -246,9 +243,8 @@ region_mass_kernel(float *__restrict__ mass, const float *__restrict__ gate, con
         block_combine<3>(m, sh_s, SumOp());
         if (threadIdx.x < 3) push_f32(&fin[buf][threadIdx.x][me.rank], 0, threadIdx.x == 0 ? m[0] : threadIdx.x == 1 ? m[1] : m[2]);
     }
-    cluster_arrive();
+    row_barrier(me);
     if (me.rank != 0) return;
-    cluster_wait();
     finish_before();
 }
 
@@ -298,6 +294,7 @@ int launch_rows(void (*kernel)(P...), int rows, int team, int (&resident)[64][MA
         resident[dev][team] = n < 1 ? 1 : n;
     }
     cfg.gridDim = dim3((rows < resident[dev][team] ? rows : resident[dev][team]) * team);
+    cfg.numAttrs = team > 1 ? 1 : 0;                          // (a CTA by itself: no cluster to set up)
     CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, args...));
     LAUNCH_CHECK();
     return VIASD_OK;
@@ -312,7 +309,7 @@ extern "C" int viasd_region_mass(const float *gate_logits, const float *proposal
     cudaStream_t st = (cudaStream_t)stream;
     static int resident[64][MAX_TEAM + 1];
     int rc = launch_rows(region_mass_kernel, rows, row_team(vocab, false), resident, st, mass, gate_logits, proposal_logits, rows, vocab,
-                         1.0f / temperature, log_tau_hi, log_tau_lo);
+                         (1.0f / temperature) * 1.44269504f, log_tau_hi, log_tau_lo);
     if (rc) return rc;
     if (mean) {
         row_sum_kernel<<<1, 1024, 0, st>>>(mean, mass, rows, 3, (float)rows);
@@ -331,7 +328,7 @@ extern "C" int viasd_kl_cost(const float *judge_logits, const float *proposal_lo
     cudaStream_t st = (cudaStream_t)stream;
     static int resident[2][64][MAX_TEAM + 1];
     int rc = launch_rows(margin ? kl_cost_kernel<1> : kl_cost_kernel<0>, rows, row_team(vocab, margin == 1), resident[margin], st, cost_rows, judge_logits,
-                         proposal_logits, rows, vocab, 1.0f / temperature, log1pf(-alpha), logf(beta), tau);
+                         proposal_logits, rows, vocab, exp_scale(temperature), 1.0f / temperature, log1pf(-alpha), logf(beta), tau);
     if (rc) return rc;
     if (cost_total) {
         row_sum_kernel<<<1, 1024, 0, st>>>(cost_total, cost_rows, rows, 1, 1.f);

@@ -145,15 +145,9 @@ tier_kernel(unsigned char *__restrict__ tier, float *__restrict__ conf, DeviceSt
 // exceeded by e^20); two sweeps read a batch's rows twice from HBM, 16 sequences' 1040 rows of 0.5 MB being far more than L2
 // holds.  Eight 16-byte loads per thread in flight: few rows are bound by what a CTA has under way.
 constexpr int RS_STRIDE = VIASD_MAX_ROWS_PER_SEQ, RS_THREADS = 512, RS_BATCH = 8;
-constexpr float RS_GAP = 20.f, LOG2E = 1.4426950408889634f;
+constexpr float RS_GAP = 20.f;
 struct RowStats { float *mx; int *arg; float *z; };       // each [B, KINDS, RS_STRIDE]
 struct RowPtrs { const float *p[KINDS]; };                // drafter logits, then each judge's
-
-__device__ __forceinline__ float ex2(float x) {            // 2^x, hardware approximation (2 ulp)
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 template <bool WANT_Z>
 struct RowAcc {
@@ -162,7 +156,7 @@ struct RowAcc {
     __device__ __forceinline__ void init() { ref = lim = -INFINITY; s = 0.f; best = no_idx(); }
     // N values from index i on, in pieces of four `step` apart
     template <int N>
-    __device__ __forceinline__ void add(const float (&x)[N], int i, int step, float scale2, float gap) {
+    __device__ __forceinline__ void add(const float (&x)[N], int i, int step, ExpScale scale, float gap) {
         float bm = x[0];
 #pragma unroll
         for (int e = 1; e < N; ++e) bm = fmaxf(bm, x[e]);
@@ -173,19 +167,19 @@ struct RowAcc {
         }
         if (!WANT_Z) return;
         if (bm > lim) {
-            s *= ex2((ref - bm) * scale2);
+            s *= exp_scaled(ref - bm, scale);
             ref = bm;
             lim = bm + gap;
         }
         const float r = ref == -INFINITY ? 0.f : ref;
 #pragma unroll
-        for (int e = 0; e < N; ++e) s += ex2((x[e] - r) * scale2);
+        for (int e = 0; e < N; ++e) s += exp_scaled(x[e] - r, scale);
     }
 };
 
 template <bool WANT_Z>
 __global__ void __launch_bounds__(RS_THREADS, 2)
-row_stats_kernel(RowStats rs, RowPtrs src, int R, int M, int V, float inv_temp, DeviceStats *stats, int clear_needs,
+row_stats_kernel(RowStats rs, RowPtrs src, int R, int M, int V, ExpScale scale, float gap, DeviceStats *stats, int clear_needs,
                  TreeInfo *tree, const int *parent, int per_seq) {
     // tree != null: no forward pass of the same call has laid the trees out, so the first CTA of each sequence does
     __shared__ float sh[RS_THREADS / 32];
@@ -200,13 +194,12 @@ row_stats_kernel(RowStats rs, RowPtrs src, int R, int M, int V, float inv_temp, 
     const int rows = kind == 0 ? R : M;
     if (!base || r >= rows) return;
     const float *row = base + ((size_t)b * rows + r) * V;
-    const float scale2 = inv_temp * LOG2E, gap = RS_GAP / inv_temp;
     RowAcc<WANT_Z> acc;
     acc.init();
     // up to three values in front of the first 16-byte boundary (an odd vocabulary), then 16-byte pieces, then the rest
     const int head = min(V, (int)((4 - ((reinterpret_cast<uintptr_t>(row) >> 2) & 3)) & 3)), n4 = (V - head) >> 2, tail = V - head - 4 * n4;
     const float4 *r4 = reinterpret_cast<const float4 *>(row + head);
-    if ((int)threadIdx.x < head) { const float x[1] = {row[threadIdx.x]}; acc.add(x, threadIdx.x, 0, scale2, gap); }
+    if ((int)threadIdx.x < head) { const float x[1] = {row[threadIdx.x]}; acc.add(x, threadIdx.x, 0, scale, gap); }
     int i0 = threadIdx.x;
 #pragma unroll 1
     for (; i0 + (RS_BATCH - 1) * RS_THREADS < n4; i0 += RS_BATCH * RS_THREADS) {
@@ -216,19 +209,19 @@ row_stats_kernel(RowStats rs, RowPtrs src, int R, int M, int V, float inv_temp, 
             const float4 v = r4[i0 + j * RS_THREADS];
             x[4 * j] = v.x; x[4 * j + 1] = v.y; x[4 * j + 2] = v.z; x[4 * j + 3] = v.w;
         }
-        acc.add(x, head + 4 * i0, 4 * RS_THREADS, scale2, gap);
+        acc.add(x, head + 4 * i0, 4 * RS_THREADS, scale, gap);
     }
 #pragma unroll 1
     for (; i0 < n4; i0 += 2 * RS_THREADS) {
         const bool two = i0 + RS_THREADS < n4;
         const float4 v = r4[i0], w = two ? r4[i0 + RS_THREADS] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         const float x[8] = {v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w};
-        acc.add(x, head + 4 * i0, 4 * RS_THREADS, scale2, gap);
+        acc.add(x, head + 4 * i0, 4 * RS_THREADS, scale, gap);
     }
-    if ((int)threadIdx.x < tail) { const float x[1] = {row[V - tail + threadIdx.x]}; acc.add(x, V - tail + threadIdx.x, 0, scale2, gap); }
+    if ((int)threadIdx.x < tail) { const float x[1] = {row[V - tail + threadIdx.x]}; acc.add(x, V - tail + threadIdx.x, 0, scale, gap); }
     const MaxIdx best = block_argmax(acc.best, shm);
     float z = 0.f;
-    if (WANT_Z) z = block_sum(acc.ref == -INFINITY ? 0.f : acc.s * ex2((acc.ref - best.v) * scale2), sh);
+    if (WANT_Z) z = block_sum(acc.ref == -INFINITY ? 0.f : acc.s * exp_scaled(acc.ref - best.v, scale), sh);
     if (threadIdx.x == 0) {
         const size_t o = ((size_t)b * KINDS + kind) * RS_STRIDE + r;
         rs.mx[o] = best.v;
@@ -254,6 +247,7 @@ struct AcceptArgs {
     DeviceStats *stats;
     int N, R, V;
     int mode, strict_break, emit_bonus;
+    ExpScale scale;
     float inv_temp, log1m_alpha, inv_beta;
     float log_acc_rel[KINDS];                // greedy gate per judging tier
     unsigned long long seed, step;
@@ -309,37 +303,44 @@ __device__ __forceinline__ float2 team_exchange(float2 v, float2 none, Team &tm)
 }
 
 // f(x, y, i) for this CTA's share of a row's indices, N at a time from i on; x, y: the values of two rows there (y: 0 when b
-// is null)
-// (which thread gets an index depends on `vec`, the vocabulary and the team only: what a thread writes there it reads again)
+// is null).  Four consecutive values to a thread, whatever the alignment, which only decides how they are loaded: what a thread
+// writes at an index it reads again.
 template <typename F>
 __device__ __forceinline__ void sweep_rows(const float *a, const float *b, int V, bool vec, const Team &tm, F f) {
-    if (vec) {
-        const float4 *a4 = reinterpret_cast<const float4 *>(a), *b4 = reinterpret_cast<const float4 *>(b);
-        const int n4 = V >> 2, per = (n4 + (int)tm.size - 1) / (int)tm.size, lo = (int)tm.rank * per, hi = min(n4, lo + per);
-        // eight loads in flight, then a rolled loop over pieces of four values (indexed, so they pass through local memory): a
-        // CTA has 16 values per thread and sweep; unrolled, their code came from a cold instruction cache (8 us a sweep), one
-        // at a time they are a chain of latencies
+    const int n4 = V >> 2, per = (n4 + (int)tm.size - 1) / (int)tm.size, lo = (int)tm.rank * per, hi = min(n4, lo + per);
+    // eight loads in flight, then a rolled loop over pieces of four values (indexed, so they pass through local memory): a
+    // CTA has 16 values per thread and sweep; unrolled, their code came from a cold instruction cache (8 us a sweep), one
+    // at a time they are a chain of latencies
 #pragma unroll 1
-        for (int i0 = lo + threadIdx.x; i0 < hi; i0 += 4 * ACC_THREADS) {
-            float4 x[4], y[4];
+    for (int i0 = lo + threadIdx.x; i0 < hi; i0 += 4 * ACC_THREADS) {
+        float4 x[4], y[4];
+        if (vec) {
+            const float4 *a4 = reinterpret_cast<const float4 *>(a), *b4 = reinterpret_cast<const float4 *>(b);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int i = min(i0 + j * ACC_THREADS, hi - 1);
                 x[j] = a4[i];
                 y[j] = b ? b4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
             }
-            const int n = min(4, (hi - i0 + ACC_THREADS - 1) / ACC_THREADS);
-#pragma unroll 1
-            for (int j = 0; j < n; ++j) {
-                const float u[4] = {x[j].x, x[j].y, x[j].z, x[j].w}, v[4] = {y[j].x, y[j].y, y[j].z, y[j].w};
-                f(u, v, 4 * (i0 + j * ACC_THREADS));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int i = 4 * min(i0 + j * ACC_THREADS, hi - 1);
+                x[j] = make_float4(a[i], a[i + 1], a[i + 2], a[i + 3]);
+                y[j] = b ? make_float4(b[i], b[i + 1], b[i + 2], b[i + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
-    } else {
-        for (int i = tm.rank * ACC_THREADS + threadIdx.x; i < V; i += tm.size * ACC_THREADS) {
-            const float u[1] = {a[i]}, v[1] = {b ? b[i] : 0.f};
-            f(u, v, i);
+        const int n = min(4, (hi - i0 + ACC_THREADS - 1) / ACC_THREADS);
+#pragma unroll 1
+        for (int j = 0; j < n; ++j) {
+            const float u[4] = {x[j].x, x[j].y, x[j].z, x[j].w}, v[4] = {y[j].x, y[j].y, y[j].z, y[j].w};
+            f(u, v, 4 * (i0 + j * ACC_THREADS));
         }
+    }
+    const int i = 4 * n4 + (int)threadIdx.x;                      // the last few of a vocabulary that is no multiple of four
+    if (tm.rank == 0 && i < V) {
+        const float u[1] = {a[i]}, v[1] = {b ? b[i] : 0.f};
+        f(u, v, i);
     }
 }
 
@@ -436,10 +437,11 @@ accept_kernel(AcceptArgs a) {
     // the judge's and the proposal's numerators from i on after n_rej rejections, from what judge_row and proposal_row hold there
     auto numerators = [&](int t, int i, const auto &xt, float mxt, const auto &x0, float mx0, int n_rej, auto &jt, auto &pr) {
         constexpr int N = sizeof(jt) / sizeof(float);
+        const bool ft = folded >> t & 1, f0 = folded & 1;
 #pragma unroll
         for (int e = 0; e < N; ++e) {
-            jt[e] = folded >> t & 1 ? xt[e] : expf((xt[e] - mxt) * a.inv_temp);
-            pr[e] = folded & 1 ? x0[e] : expf((x0[e] - mx0) * a.inv_temp);
+            jt[e] = ft ? xt[e] : exp_scaled(xt[e] - mxt, a.scale);
+            pr[e] = f0 ? x0[e] : exp_scaled(x0[e] - mx0, a.scale);
         }
         replay(w.rej + n_fold, n_rej - n_fold, i, t, jt, pr);
     };
@@ -515,8 +517,8 @@ accept_kernel(AcceptArgs a) {
                     for (int n = tid; n < N; n += ACC_THREADS) {      // (of the children of this row; the others' are not used)
                         // a child that names another drafter row than its elder sibling is still tested against that sibling's
                         const float x0 = w.prow[n] == row0 ? w.x0[n] : r0[w.tok[n]];
-                        w.jv[pos][n] = expf((w.xj[n] - w.mx[w.tier[n]][cur]) * a.inv_temp);
-                        w.pv[pos][n] = expf((x0 - mx0) * a.inv_temp);
+                        w.jv[pos][n] = exp_scaled(w.xj[n] - w.mx[w.tier[n]][cur], a.scale);
+                        w.pv[pos][n] = exp_scaled(x0 - mx0, a.scale);
                     }
                     __syncthreads();
                 }
@@ -696,8 +698,9 @@ int launch_accept(const viasd_model *m, const viasd_draft *d, const viasd_params
         src.p[0] = p->mode == 1 || (do_tier && p->conf_source == 0) ? d->drafter_logits : nullptr;
         for (int k = 1; k < KINDS; ++k) src.p[k] = k <= js.n ? js.logits[k - 1] : nullptr;
         auto kernel = p->mode == 1 ? row_stats_kernel<true> : row_stats_kernel<false>;
+        const float temperature = p->mode == 1 ? p->temperature : 1.f;
         kernel<<<dim3(rows, d->batch, js.n + 1), RS_THREADS, 0, st>>>(a.rs, src, d->n_prows, M, m->cfg.vocab,
-            p->mode == 1 ? 1.0f / p->temperature : 1.0f, m->ws.stats, do_tier ? 1 : 0, tree_ready ? nullptr : m->ws.tree, d->parent, d->per_sequence);
+            exp_scale(temperature), RS_GAP * temperature, m->ws.stats, do_tier ? 1 : 0, tree_ready ? nullptr : m->ws.tree, d->parent, d->per_sequence);
         LAUNCH_CHECK();
     }
     a.judges[0] = nullptr;
@@ -716,6 +719,7 @@ int launch_accept(const viasd_model *m, const viasd_draft *d, const viasd_params
     a.N = d->n_nodes; a.R = d->n_prows; a.V = m->cfg.vocab;
     a.mode = p->mode; a.strict_break = p->strict_break; a.emit_bonus = p->emit_bonus;
     a.inv_temp = 1.0f / p->temperature;
+    a.scale = exp_scale(p->mode == 1 ? p->temperature : 1.f);
     a.log1m_alpha = log1pf(-p->alpha);
     a.inv_beta = 1.0f / p->beta;
     // greedy gates: log_acc_rel[1] for every slim verifier, log_acc_rel[2] for q

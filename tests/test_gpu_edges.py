@@ -249,3 +249,23 @@ def test_star_of_rejected_children(vocab, team, nodes, alpha, beta):
                                                  res.n_emit.cpu().numpy(), res.corr_src.cpu().numpy(), eps_row=2.5e-5)
     PU.assert_pinned(f"star of {nodes}, vocabulary {vocab}", pinned, total, whole, B, 0.85, 3)
     assert vb.get_stats(eng.model).device_status == 0 and eng.guards_intact()
+
+
+# ---------------------------------------------------------------------------------------------
+# precision of the verification cost
+# ---------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("vocab,temperature", [(32000, 1.0), (50257, 0.7), (152064, 1.0), (152064, 1.3)])
+def test_cost_is_as_precise_as_its_sums(vocab, temperature):
+    """Relative error of a row's cost, rms over rows: the fp32 sums over its vocabulary (2e-7 to 3e-7 rms, measured; any other
+    order shows as much), not the last bit of a logarithm of the order of ten, which shifts every margin of a row (7e-7)."""
+    vb = _vb()
+    g = torch.Generator(device="cuda").manual_seed(11)
+    judge = torch.randn(64, vocab, device="cuda", generator=g) * 1.3
+    prop = judge + torch.randn(64, vocab, device="cuda", generator=g) * 0.4
+    got, _ = vb.kl_cost(judge, prop, temperature=temperature)
+    t = float(np.float32(temperature))
+    lq, lp = (judge.double() / t).log_softmax(1), (prop.double() / t).log_softmax(1)
+    d = (lp - lq).clamp(min=0)
+    want = (lp.exp() * d).sum(1) + (lq.exp() * d).sum(1)
+    err = (got.double() - want) / want
+    assert float(err.pow(2).mean().sqrt()) < 4.5e-7, float(err.pow(2).mean().sqrt())
