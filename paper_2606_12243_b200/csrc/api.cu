@@ -148,7 +148,7 @@ int run_gemm(viasd_model *m, const GemmCall &g, int rows, cudaStream_t st) {
     if (!m->use_tc) {
         GemmSegs s{{g.w[0], g.w[1], g.w[2]}, {g.n[0], g.n[1], g.n[2]}, g.count};
         return launch_gemm_rowwarp(g.x, g.x_plane, s, rows, g.k, c.dtype, g.epi, g.out_f32, g.out_act, g.act_plane,
-                                   g.ld_out, st);
+                                   g.ld_out, m->sm_count, st);
     }
     for (int row0 = 0; row0 < rows; row0 += 128) {
         const int nr = rows - row0 < 128 ? rows - row0 : 128;
@@ -716,13 +716,13 @@ int viasd_gemm(const void *x, const void *w, float *y, int rows, int n, int k, i
     cudaStream_t st = (cudaStream_t)stream;
     if (g_use_pdl < 0) { const char *e = getenv("VIASD_PDL"); g_use_pdl = (e && e[0] == '0') ? 0 : 1; }
     const char *force = getenv("VIASD_GEMM");
-    if (dtype == 0 || (force && strcmp(force, "rowwarp") == 0)) {
-        GemmSegs s{{w, nullptr, nullptr}, {n, 0, 0}, 1};
-        return launch_gemm_rowwarp(x, 0, s, rows, k, dtype, EPI_STORE, y, nullptr, 0, n, st);
-    }
     int dev = 0, sms = 0;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (dtype == 0 || (force && strcmp(force, "rowwarp") == 0)) {
+        GemmSegs s{{w, nullptr, nullptr}, {n, 0, 0}, 1};
+        return launch_gemm_rowwarp(x, 0, s, rows, k, dtype, EPI_STORE, y, nullptr, 0, n, sms, st);
+    }
     if (sms > MAX_SMS) sms = MAX_SMS;
     const size_t counter_bytes = align_up((size_t)(tc_tiles(n) + 1) * 4, 256);
     // tile counters and the status word.  By a kernel that lets the product's launch overlap it: behind a memset the product

@@ -235,7 +235,7 @@ enum GemmEpilogue { EPI_STORE = 0, EPI_ADD = 1, EPI_SWIGLU = 2, EPI_ADD_NORM = 3
 struct GemmSegs { const void *w[3]; int n[3]; int count; };
 // x_plane / act_plane: element distance between the hi and lo planes (0: single plane)
 int launch_gemm_rowwarp(const void *x, size_t x_plane, const GemmSegs &segs, int rows, int k, int dtype,
-                        int epilogue, float *out_f32, void *out_act, size_t act_plane, int ld_out, cudaStream_t st);
+                        int epilogue, float *out_f32, void *out_act, size_t act_plane, int ld_out, int sms, cudaStream_t st);
 
 // attention.cu
 int launch_attention(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, int batch, int M,

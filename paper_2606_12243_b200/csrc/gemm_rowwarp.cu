@@ -1,8 +1,10 @@
 // Generic CUDA-core GEMM y[rows, n] = x[rows, k] * W[n, k]^T for a handful of rows.
 // One warp owns FEAT output features and streams their weight rows once with 16-byte loads; the
-// activation vector it multiplies with is reused across the FEAT features from registers.  Four features where that
-// still gives every SM two CTAs; else one (two for the gate/up pair): a 256 x 256 projection is 8 CTAs of four-feature warps,
-// each a chain of dependent loads.  With a feature per warp, the loads of several k-steps in flight, no branches between
+// activation vector it multiplies with is reused across the FEAT features from registers.  Four features where that still
+// gives every SM a CTA (a 256 x 256 projection is 8 CTAs of four-feature warps, each a chain of dependent loads); below that
+// one, or two from a size on that is the lower the more rows share a weight's load.  us with 1 / 2 / 4 features, 9 rows: 1024 x
+// 1024 9.0 / 11.3 / 19.7, 2048 x 2048 29.9 / 20.9 / 39.2, 4096 x 2048 49.8 / 39.7 / 40.6, 6144 x 1024 40.0 / 28.5 / 21.9; 5 rows: 2048 x
+// 2048 14.4 / 15.7 / 24.8, 3072 x 768 11.2 / 6.6 / 12.3; 1 row: 4096 x 2048 10.7 / 12.6 / 15.1.  With a feature per warp, the loads of several k-steps in flight, no branches between
 // them, the rows' read-modify-writes side by side and launches that overlap, the 14 GEMMs of the two-layer fp32 step
 // (d = 256) take 114 us instead of 211.
 // Serves the fp32 model configuration and any shape the tensor-core kernels do not take.
@@ -153,16 +155,17 @@ gemm_rowwarp_kernel(const T *__restrict__ x, size_t x_plane, SegTable segs, int 
 
 template <typename T, int RC>
 int dispatch_epi(const T *x, size_t x_plane, const SegTable &s, int rows, int k, int n_total, int epi, float *out_f32,
-                 T *out_act, size_t act_plane, int ld_out, cudaStream_t st) {
+                 T *out_act, size_t act_plane, int ld_out, int sms, cudaStream_t st) {
     const int outs = epi == EPI_SWIGLU ? 2 * s.end[0] : n_total;            // weight rows in all
-    const bool wide = outs >= 4 * WARPS * 2 * 148;
+    const bool two = RC > 8 ? outs >= 12 * sms : RC > 4 && outs >= 16 * sms;
+    const int feat = outs >= 4 * WARPS * sms ? 4 : two || epi == EPI_SWIGLU ? 2 : 1;
 #define ROWWARP(KIND, F)                                                                                                    \
     CUDA_TRY(launch_chained(gemm_rowwarp_kernel<T, RC, KIND, F>, ((outs + F - 1) / F + WARPS - 1) / WARPS, WARPS * 32, st,   \
                             x, x_plane, s, rows, k, n_total, out_f32, out_act, act_plane, ld_out))
     switch (epi) {
-    case EPI_STORE: if (wide) ROWWARP(EPI_STORE, 4); else ROWWARP(EPI_STORE, 1); break;
-    case EPI_ADD: if (wide) ROWWARP(EPI_ADD, 4); else ROWWARP(EPI_ADD, 1); break;
-    case EPI_SWIGLU: if (wide) ROWWARP(EPI_SWIGLU, 4); else ROWWARP(EPI_SWIGLU, 2); break;
+    case EPI_STORE: if (feat == 4) ROWWARP(EPI_STORE, 4); else if (feat == 2) ROWWARP(EPI_STORE, 2); else ROWWARP(EPI_STORE, 1); break;
+    case EPI_ADD: if (feat == 4) ROWWARP(EPI_ADD, 4); else if (feat == 2) ROWWARP(EPI_ADD, 2); else ROWWARP(EPI_ADD, 1); break;
+    case EPI_SWIGLU: if (feat == 4) ROWWARP(EPI_SWIGLU, 4); else ROWWARP(EPI_SWIGLU, 2); break;
     default: return VIASD_EINVAL;
     }
 #undef ROWWARP
@@ -172,16 +175,16 @@ int dispatch_epi(const T *x, size_t x_plane, const SegTable &s, int rows, int k,
 
 template <typename T>
 int dispatch_rows(const T *x, size_t x_plane, const SegTable &s, int rows, int k, int n_total, int epi, float *out_f32,
-                  T *out_act, size_t act_plane, int ld_out, cudaStream_t st) {
-    if (rows <= 4) return dispatch_epi<T, 4>(x, x_plane, s, rows, k, n_total, epi, out_f32, out_act, act_plane, ld_out, st);
-    if (rows <= 8) return dispatch_epi<T, 8>(x, x_plane, s, rows, k, n_total, epi, out_f32, out_act, act_plane, ld_out, st);
-    return dispatch_epi<T, 12>(x, x_plane, s, rows, k, n_total, epi, out_f32, out_act, act_plane, ld_out, st);
+                  T *out_act, size_t act_plane, int ld_out, int sms, cudaStream_t st) {
+    if (rows <= 4) return dispatch_epi<T, 4>(x, x_plane, s, rows, k, n_total, epi, out_f32, out_act, act_plane, ld_out, sms, st);
+    if (rows <= 8) return dispatch_epi<T, 8>(x, x_plane, s, rows, k, n_total, epi, out_f32, out_act, act_plane, ld_out, sms, st);
+    return dispatch_epi<T, 12>(x, x_plane, s, rows, k, n_total, epi, out_f32, out_act, act_plane, ld_out, sms, st);
 }
 
 }  // namespace
 
 int launch_gemm_rowwarp(const void *x, size_t x_plane, const GemmSegs &segs, int rows, int k, int dtype,
-                        int epilogue, float *out_f32, void *out_act, size_t act_plane, int ld_out, cudaStream_t st) {
+                        int epilogue, float *out_f32, void *out_act, size_t act_plane, int ld_out, int sms, cudaStream_t st) {
     if (rows <= 0) return VIASD_OK;
     if (k % 8 != 0) return VIASD_EINVAL;
     SegTable s;
@@ -194,7 +197,7 @@ int launch_gemm_rowwarp(const void *x, size_t x_plane, const GemmSegs &segs, int
     }
     if (epilogue == EPI_SWIGLU && (segs.count != 2 || segs.n[0] != segs.n[1])) return VIASD_EINVAL;
     if (dtype == 0)
-        return dispatch_rows<float>((const float *)x, 0, s, rows, k, total, epilogue, out_f32, (float *)out_act, 0, ld_out, st);
+        return dispatch_rows<float>((const float *)x, 0, s, rows, k, total, epilogue, out_f32, (float *)out_act, 0, ld_out, sms, st);
     return dispatch_rows<__nv_bfloat16>((const __nv_bfloat16 *)x, x_plane, s, rows, k, total, epilogue, out_f32,
-                                        (__nv_bfloat16 *)out_act, act_plane, ld_out, st);
+                                        (__nv_bfloat16 *)out_act, act_plane, ld_out, sms, st);
 }

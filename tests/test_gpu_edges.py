@@ -269,3 +269,18 @@ def test_cost_is_as_precise_as_its_sums(vocab, temperature):
     want = (lp.exp() * d).sum(1) + (lq.exp() * d).sum(1)
     err = (got.double() - want) / want
     assert float(err.pow(2).mean().sqrt()) < 4.5e-7, float(err.pow(2).mean().sqrt())
+
+
+# ---------------------------------------------------------------------------------------------
+# fp32 products at the sizes where the features per warp change (148 SMs: 1776, 2368 and 4736 outputs)
+# ---------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("rows,n,k", [(9, 1775, 72), (9, 1777, 64), (5, 2367, 40), (8, 2369, 40), (13, 3001, 40), (4, 4735, 136), (9, 4738, 64)])
+def test_fp32_product_by_features_per_warp(rows, n, k):
+    vb = _vb()
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x, w = torch.randn(rows, k, device="cuda", generator=g), torch.randn(n, k, device="cuda", generator=g) * 0.05
+    y = torch.full((rows, n), float("nan"), device="cuda")
+    vb.gemm(x, w, y, torch.empty(vb.gemm_scratch_bytes(rows, n, k), dtype=torch.uint8, device="cuda"))
+    want = x.double() @ w.double().T
+    # exact products, fp32 accumulation of k terms
+    assert float((y.double() - want).abs().max()) <= 2e-6 * np.sqrt(k) * float(want.abs().max()) + 1e-6
