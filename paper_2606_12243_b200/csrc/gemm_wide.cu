@@ -428,7 +428,29 @@ int launch_gemm_wide(const TcLaunch &L, cudaStream_t st) {
     if (dual) p.n_tiles = (L.seg_n[0] + 63) / 64;                  // 64 gate and 64 up features per CTA tile
     if (p.n_tiles <= 0 || p.k_tiles <= 0) return VIASD_OK;
     const int units = ((p.n_tiles + 1) / 2) * p.k_tiles;
-    int pairs = L.sm_count / 2 < units ? L.sm_count / 2 : units;      // (148 SMs hold 74 pairs: all resident at once)
+    static int resident[64];                                       // pairs the device holds at once, asked once per device
+    int dev = 0;
+    CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return VIASD_EUNSUPPORTED;
+    if (!resident[dev]) {
+        const int most = 204 * 1024;
+        CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel<EPI_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel<EPI_ADD_NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel<EPI_QKV_ROPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel<EPI_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        cudaLaunchConfig_t q{};
+        cudaLaunchAttribute cluster[1];
+        cluster[0].id = cudaLaunchAttributeClusterDimension;
+        cluster[0].val.clusterDim.x = 2; cluster[0].val.clusterDim.y = 1; cluster[0].val.clusterDim.z = 1;
+        q.gridDim = dim3(2); q.blockDim = dim3(WTHREADS); q.dynamicSmemBytes = most; q.attrs = cluster; q.numAttrs = 1;
+        int n = 0;
+        CUDA_TRY(cudaOccupancyMaxActiveClusters(&n, gemm_wide_kernel<EPI_QKV_ROPE>, &q));
+        if (n < 1) return VIASD_EUNSUPPORTED;
+        resident[dev] = n;
+    }
+    // the finishers of a split tile wait for its other contributors: all pairs have to be resident at once
+    int pairs = L.sm_count / 2 < resident[dev] ? L.sm_count / 2 : resident[dev];
+    if (pairs > units) pairs = units;
     p.units_per_cta = (units + pairs - 1) / pairs;
     pairs = (units + p.units_per_cta - 1) / p.units_per_cta;
     const size_t xbox = (size_t)p.tt * p.nt * 128, ring = (size_t)(L.ring_kb > 0 ? L.ring_kb : 200) * 1024;
@@ -447,14 +469,6 @@ int launch_gemm_wide(const TcLaunch &L, cudaStream_t st) {
     p.tmem_cols = cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
     const size_t smem = p.stages * (size_t)WBOX + p.x_stages * xbox + 1024;
     const CUtensorMap &w0 = *L.map_w[0], &w1 = *L.map_w[L.n_seg > 1 ? 1 : 0], &w2 = *L.map_w[L.n_seg > 2 ? 2 : 0];
-    static bool attr_done[64];
-    if (first_use_on_device(attr_done)) {
-        const int most = 204 * 1024;
-        CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel<EPI_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-        CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel<EPI_ADD_NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-        CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel<EPI_QKV_ROPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-        CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel<EPI_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    }
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     pdl_config(cfg, attr, dim3(2 * pairs), dim3(WTHREADS), smem, st, !L.ordered);
