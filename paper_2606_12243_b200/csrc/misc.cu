@@ -35,8 +35,9 @@ int launch_rope_table(const viasd_model *m, cudaStream_t st) {
 // Arrival counters of the GEMMs and of attention, zero between launches.  After a wait that expired they may not be: a pass
 // that finds the status word saying so starts from clean ones (nothing before it in the stream is still running).
 struct Counters { int *gemm, *attn; int n_gemm, n_attn; };
-__device__ __forceinline__ void clear_counters_if_failed(const Counters &c, const DeviceStats *stats, int thread, int threads) {
-    if (*reinterpret_cast<const volatile int *>(&stats->device_status) != VIASD_EDEVICE) return;
+__device__ __forceinline__ int pass_status(const DeviceStats *stats) { return *reinterpret_cast<const volatile int *>(&stats->device_status); }
+__device__ __forceinline__ void clear_counters_if_failed(const Counters &c, int status, int thread, int threads) {
+    if (status != VIASD_EDEVICE) return;
     for (int i = thread; i < c.n_gemm; i += threads) c.gemm[i] = 0;
     for (int i = thread; i < c.n_attn; i += threads) c.attn[i] = 0;
 }
@@ -59,12 +60,13 @@ __device__ __forceinline__ int clamped_len(const int *len, int b, int max_ctx, i
     return c;
 }
 __device__ __forceinline__ void prep_sequence(const PrepArgs &p, int b, int *par_sh) {       // by the CTA's first warp
-    if (b == 0) clear_counters_if_failed(p.counters, p.stats, threadIdx.x, 32);
+    const int status = b == 0 ? pass_status(p.stats) : 0;        // (asked for ahead of the tree, used behind it)
     build_tree(p.tree + b, p.parent + (p.per_seq ? (size_t)b * p.N : 0), p.N, p.stats, par_sh);
     if (threadIdx.x == 0) {
         if (b == 0 && p.full_pass) p.stats->full_ran = 1;      // the full verifier's cache receives this block's rows
         p.len_eff[b] = clamped_len(p.len, b, p.max_ctx, p.N + 1, p.stats);
     }
+    clear_counters_if_failed(p.counters, status, threadIdx.x, 32);
 }
 __device__ __forceinline__ int prep_token(const PrepArgs &p, int r) {
     if (p.row_tok) return p.row_tok[r];
@@ -90,7 +92,7 @@ __global__ void prep_replay_kernel(TreeInfo *tree, int *len_eff, int *row_tok, D
                                    const int *pending, const int *draft_tok, const int *parent, int per_seq,
                                    const int *tokens, int B, int N, int G, int max_ctx, int vocab, const Counters counters, const int *run_flag) {
     RUN_FLAG_EXIT(run_flag);
-    clear_counters_if_failed(counters, stats, threadIdx.x, blockDim.x);
+    clear_counters_if_failed(counters, pass_status(stats), threadIdx.x, blockDim.x);
     const int Mx = G + N + 1;
     if (threadIdx.x == 0) stats->full_ran = 1;
     for (int b = threadIdx.x; b < B; b += blockDim.x) {
