@@ -355,6 +355,14 @@ int check_result(const viasd_result *r, int phase) {
     return VIASD_OK;
 }
 
+// what the tiers and the walk need of a draft and a result
+int check_accept(const viasd_draft *d, const viasd_result *r, int phase) {
+    if (check_result(r, phase)) return VIASD_EINVAL;
+    if (d->n_nodes < 1 || !d->prow || !d->drafter_logits || d->n_prows < 1) return VIASD_EINVAL;
+    if ((phase & 2) && d->n_prows > VIASD_MAX_ROWS_PER_SEQ) return VIASD_EINVAL;
+    return VIASD_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -488,8 +496,7 @@ static int tier_accept_set(viasd_model *m, const viasd_draft *draft, const viasd
     int rc;
     if ((rc = check_draft(m, draft)) || (rc = check_params(params))) return rc;
     if (phase < 1 || phase > 3) return VIASD_EINVAL;
-    if ((rc = check_result(result, phase))) return rc;
-    if (draft->n_nodes < 1 || !draft->prow || !draft->drafter_logits || draft->n_prows < 1) return VIASD_EINVAL;
+    if ((rc = check_accept(draft, result, phase))) return rc;
     for (int k = 1; k < js.n; ++k) if (!(js.log_tau[k] <= js.log_tau[k - 1])) return VIASD_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     if (phase == 1) {
@@ -560,7 +567,6 @@ int viasd_kv_commit_slim(viasd_model *m, viasd_cache *cache, const viasd_draft *
 static int verify_step_routed(viasd_model *m, viasd_cache *cache, const viasd_draft *draft, const viasd_params *params,
                               float *slim_logits, float *full_logits, viasd_result *result, void *stream) {
     int rc;
-    if ((rc = check_draft(m, draft)) || (rc = check_cache(cache))) return rc;
     if (!m->fused || !cache->len_full || !cache->tokens) return VIASD_EINVAL;
     const int M = draft->n_nodes + 1, G = m->cfg.max_query - M;
     if (G < 1) return VIASD_ECAPACITY;                        // no room for replayed rows: size max_query above M
@@ -591,14 +597,15 @@ int viasd_verify_step(viasd_model *m, viasd_cache *cache, const viasd_draft *dra
     int rc;
     if (!slim_logits || !full_logits) return VIASD_EINVAL;
     if ((rc = check_params(params))) return rc;
+    // whatever one of the pieces would refuse is refused before the first of them runs
+    if ((rc = check_draft(m, draft)) || (rc = check_cache(cache)) || (rc = check_accept(draft, result, 3))) return rc;
     if (params->policy == 1) return verify_step_routed(m, cache, draft, params, slim_logits, full_logits, result, stream);
     // Both verifiers in one sweep over the layers (routed layers' weights are read once for both) while the two
     // row streams together fit one launch (128 token rows, 256 where the pair kernel runs the pass); beyond
     // that a sweep would stream every routed layer twice anyway, and the passes run one after the other.
-    const int block_rows = draft ? draft->batch * (draft->n_nodes + 1) : 0;
-    const int dual_max = !m ? 0 : m->opt.dual_max_rows >= 0 ? m->opt.dual_max_rows : block_rows >= TC_WIDE_MIN_ROWS ? TC_WIDE_ROWS : 128;
-    if (m && m->fused && draft && 2 * block_rows <= dual_max) {
-        if ((rc = check_draft(m, draft)) || (rc = check_cache(cache))) return rc;
+    const int block_rows = draft->batch * (draft->n_nodes + 1);
+    const int dual_max = m->opt.dual_max_rows >= 0 ? m->opt.dual_max_rows : block_rows >= TC_WIDE_MIN_ROWS ? TC_WIDE_ROWS : 128;
+    if (m->fused && 2 * block_rows <= dual_max) {
         if ((rc = forward_sweep(m, cache, draft, 2, full_logits, slim_logits, (cudaStream_t)stream))) return rc;
         if ((rc = tier_accept_impl(m, draft, params, slim_logits, full_logits, 3, result, true, stream))) return rc;
         return viasd_kv_commit(m, cache, draft, result, stream);

@@ -284,3 +284,28 @@ def test_fp32_product_by_features_per_warp(rows, n, k):
     want = x.double() @ w.double().T
     # exact products, fp32 accumulation of k terms
     assert float((y.double() - want).abs().max()) <= 2e-6 * np.sqrt(k) * float(want.abs().max()) + 1e-6
+
+
+# ---------------------------------------------------------------------------------------------
+# a step that will be refused
+# ---------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("dual_max", [-1, 0])
+@pytest.mark.parametrize("what", ["no drafter rows", "too many drafter rows", "no place for the path"])
+def test_refused_step_runs_nothing(dual_max, what):
+    """Arguments that the walk refuses are refused before either verifier has run, in one sweep or in turn."""
+    vb = _vb()
+    wl = W.get("mini_7b")
+    eng = _engine(wl)
+    vb.set_option(eng.model, "dual_max_rows", dual_max)
+    n_prows = {"no drafter rows": 0, "too many drafter rows": 65}.get(what, eng.inputs.n_prows)
+    draft = vb.make_draft(eng.draft_tok, eng.parent, eng.prow, n_prows, eng.drafter_logits)
+    res = vb.alloc_result(wl.batch, wl.n_nodes)
+    if what == "no place for the path":
+        res.path = None
+    before = [t.clone() for t in (eng.k_full, eng.k_slim, eng.len)]
+    n0 = vb.launch_count()
+    with pytest.raises(vb.ViasdError) as e:
+        vb.verify_step(eng.model, eng.cache, draft, eng.params(conf_source=1), eng.logits_buffer(), eng.logits_buffer(), res)
+    torch.cuda.synchronize()
+    assert e.value.code == vb.VIASD_EINVAL and vb.launch_count() == n0
+    assert all(torch.equal(a, b) for a, b in zip(before, (eng.k_full, eng.k_slim, eng.len)))
