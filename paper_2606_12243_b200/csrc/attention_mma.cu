@@ -288,7 +288,10 @@ attention_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty_bar(ks));
                 if (!(ok = warp_wait(full_bar(vs), ((ck + 1) / RING) & 1, &abort_sh, a.status))) break;
-                if (any) st.accumulate(base + vs * SLOT_BYTES, r0, lane, s);
+                if (any) {
+                    if (j0 + 32 > it.k_end) zero_tile_rows(base + vs * SLOT_BYTES, HALF_BYTES, r0 + it.k_end - j0, r0 + 32, lane);   // (this warp's keys)
+                    st.accumulate(base + vs * SLOT_BYTES, r0, lane, s);
+                }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty_bar(vs));
             }

@@ -269,6 +269,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 const int g = s_cnt + t, sb = g & 1;
                 if (!(ok = warp_wait(full_bar(st), st_ph, &abort_sh, a.status))) break;
                 if (!(ok = warp_wait(pfull_bar(sb), (g >> 1) & 1, &abort_sh, a.status))) break;
+                const int live_keys = min(TKEYS, keys - t * TKEYS);
+                if (live_keys & 15) zero_tile_rows(ring + st * SLOT_BYTES, HALF_BYTES, live_keys, (live_keys + 15) & ~15, lane);
                 tc_fence_after();
                 if (elect_one()) {
                     const uint64_t vd = smem_desc_mn(ring + st * SLOT_BYTES, HALF_BYTES, 1024);

@@ -364,13 +364,16 @@ attention_tk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 if (t == 0 && o_uses > 0 && !(ok = warp_wait(ofree_bar, (o_uses - 1) & 1, &abort_sh, a.status))) break;
                 if (SPLIT && !(ok = warp_wait(fullv_bar(vslot), vphase, &abort_sh, a.status))) break;
                 if (!(ok = warp_wait(pfull_bar(sb), (g >> 1) & 1, &abort_sh, a.status))) break;
+                const uint32_t vtile = SPLIT ? ring + (uint32_t)(NK + vslot) * SLOT_BYTES : ring + (uint32_t)(2 * vslot + 1) * SLOT_BYTES;
+                const int live_keys = uniform(min(TKEYS, it.k_end - it.k_begin - t * TKEYS)), nk = (live_keys + 15) >> 4;   // nk: 16-key groups
+                if (live_keys & 15) zero_tile_rows(vtile, HALF_BYTES, live_keys, 16 * nk, lane);
                 tc_fence_after();
                 if (elect_one()) {
-                    const uint64_t vd = smem_desc_mn(SPLIT ? ring + (uint32_t)(NK + vslot) * SLOT_BYTES : ring + (uint32_t)(2 * vslot + 1) * SLOT_BYTES, HALF_BYTES, 1024);
+                    const uint64_t vd = smem_desc_mn(vtile, HALF_BYTES, 1024);
                     const uint64_t pd = smem_desc(psm + sb * 2 * QCH);
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk)                    // 16 keys per step: two 8-key groups of 1024 bytes
-                        tc_mma(tmem + TM_O, vd + kk * (2048 >> 4), pd + (kk >> 2) * (QCH >> 4) + (kk & 3) * 2, idesc_pv, (t > 0 || kk > 0) ? 1u : 0u);
+                        if (kk < nk) tc_mma(tmem + TM_O, vd + kk * (2048 >> 4), pd + (kk >> 2) * (QCH >> 4) + (kk & 3) * 2, idesc_pv, (t > 0 || kk > 0) ? 1u : 0u);
                     tc_commit(SPLIT ? emptyv_bar(vslot) : emptyk_bar(vslot));   // the slot is free once these MMAs have read it
                     tc_commit(pvdone_bar(sb));
                 }

@@ -123,6 +123,19 @@ __device__ __forceinline__ bool elect_one() {
 template <typename T>
 __device__ __forceinline__ T uniform(T x) { return (T)__shfl_sync(0xffffffffu, x, 0); }
 
+// Zeroes rows [from, to) of a K or V tile that TMA has brought (two halves of 128-byte rows, `half` bytes apart), by a warp, and
+// hands them on to the tensor cores.  Keys past the end of a sequence have weight zero, but what a cache holds there
+// may never have been written, and 0 x NaN is not 0.
+__device__ __forceinline__ void zero_tile_rows(uint32_t tile, uint32_t half, int from, int to, int lane) {
+#pragma unroll 1
+    for (int i = from * 8 + lane; i < to * 8; i += 32) {
+        asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(tile + (uint32_t)i * 16u), "r"(0) : "memory");
+        asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(tile + half + (uint32_t)i * 16u), "r"(0) : "memory");
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+}
+
 // ---- the same for a whole warp in step ---------------------------------------------------------
 // Loops that feed TMA and the tensor cores, run by all lanes of their warp with the instruction itself predicated to one
 // lane.  Inside an `if (lane == 0)` the compiler keeps addresses, coordinates and descriptors in per-thread registers and

@@ -309,3 +309,27 @@ def test_refused_step_runs_nothing(dual_max, what):
     torch.cuda.synchronize()
     assert e.value.code == vb.VIASD_EINVAL and vb.launch_count() == n0
     assert all(torch.equal(a, b) for a, b in zip(before, (eng.k_full, eng.k_slim, eng.len)))
+
+
+# ---------------------------------------------------------------------------------------------
+# caches that have never been written past the block
+# ---------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("name,nodes,kernel", [("mini_7b", 8, "mma"), ("mini_7b", 8, "tk"), ("mini_8b_tree", 26, "tc"), ("mini_8b_tree", 40, "tc"),
+                                               ("mini_32b_b3", 5, "tk"), ("mini_32b_b3", 5, "tc"), ("c1_tiny", 4, "auto")])
+@pytest.mark.parametrize("ctx", [0, 116, 245, 333])
+def test_nothing_past_the_block_is_read_into_the_result(name, nodes, kernel, ctx):
+    """NaN in every slot past the block's: same bits as with zeros there, whatever 16-, 32- or 128-key group the block ends in."""
+    vb = _vb()
+    base = W.get(name)
+    eng = _engine(replace(base, ctx=ctx, parent=W.chain(nodes), shape=replace(base.shape, n_layers=2), n_routed=1), extra_ctx=140)
+    vb.set_option(eng.model, "attention_kernel", kernel)
+    eng.len.fill_(ctx)
+    got = []
+    for fill in (0.0, float("nan")):
+        for t in (eng.k_full, eng.v_full):
+            t[:, :, :, ctx:] = fill
+        out = eng.logits_buffer()
+        vb.full_forward(eng.model, eng.cache, eng.draft, out)
+        torch.cuda.synchronize()
+        got.append(out)
+    assert torch.isfinite(got[1]).all() and torch.equal(*got)
