@@ -19,6 +19,10 @@
  *     to viasd_init_model (weights, workspace); they must outlive the handle.
  *   - All work is enqueued on the caller's stream (a cudaStream_t passed as void*); no call synchronises
  *     except viasd_init_model and viasd_get_stats.
+ *   - CTAs of one launch wait for one another inside the GPU (for a tile, or a head's keys, that several SMs share), which
+ *     needs all SMs of the device: calls of different handles, or of viasd_gemm with different scratch, on one GPU have to
+ *     be ordered after one another (one stream, or events), as those of one handle do, which share its workspace.  Two that
+ *     overlap may run out their bounded waits and end with VIASD_EDEVICE.
  *   - Every function returns 0 (VIASD_OK) or a negative error code; nothing throws, exits or traps.
  *     Conditions only the device can see (a sequence too long for the cache, a token id outside the
  *     vocabulary) are clamped to a safe value and recorded in a device status word that
@@ -211,8 +215,9 @@ int viasd_get_stats(viasd_model *m, viasd_stats *host_out, void *stream);
  * within the stated tolerances under every setting, but their last bits may change with it.
  * Errors: EINVAL (null handle, unknown option, value out of range). */
 enum {
-    VIASD_OPT_ATTENTION_KERNEL = 0,    /* 0 choose by shape (default), 1 mma.sync, 2 tcgen05 with query rows on the
-                                          TMEM lanes, 3 tcgen05 with keys on the lanes (where the shape allows) */
+    VIASD_OPT_ATTENTION_KERNEL = 0,    /* 0 choose by shape (default), 1 mma.sync (up to 16 query rows per kv head, else as
+                                          2), 2 tcgen05 with query rows on the TMEM lanes, 3 tcgen05 with keys on the lanes
+                                          (where the shape allows, else as 1) */
     VIASD_OPT_ATTENTION_SPLITS,        /* key ranges per (sequence, kv head), 1..16; 0 = cost model (default) */
     VIASD_OPT_ATTENTION_LO,            /* mma.sync kernel: hi/lo split of queries and probabilities 2 (default),
                                           queries only 1, neither 0 (fails the logit tolerance at full size) */

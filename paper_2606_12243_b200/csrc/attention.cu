@@ -222,12 +222,12 @@ static int tk_nsplit(const viasd_model *m, int batch, int M, int streams, int su
     return best;
 }
 
-// merge of the key ranges: inside the attention kernel when there is little to merge, else its own kernel
+// Attention on the tensor cores: the choice of the kernel.
 static int mma_attention(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, const void *kc2,
                          const void *vc2, int layer_ord2, int streams, int batch, int M, cudaStream_t st) {
     const viasd_config &c = m->cfg;
-    // Which kernel (VIASD_OPT_ATTENTION_KERNEL): the mma.sync kernel, tcgen05 with the query rows on the TMEM lanes, or
-    // tcgen05 with the keys on the lanes (few query rows only).  Default: keys-on-lanes where it applies, else mma.sync.
+    // VIASD_OPT_ATTENTION_KERNEL: mma.sync (up to 16 query rows per kv head), tcgen05 with the query rows on the TMEM lanes
+    // (any), or tcgen05 with the keys on the lanes (up to 32 rows per item); by default, as below.
     const int kind = m->opt.attn_kernel == 1 ? 0 : m->opt.attn_kernel == 2 ? 1 : m->opt.attn_kernel == 3 ? 2 : 3;   // 0 mma, 1 tc, 2 tk, 3 default
     const int QR = (c.n_heads / c.n_kv_heads) * M;
     // More than 32 query rows per kv head: the rows-on-lanes kernel, whose tile costs the same whatever the rows (per layer,

@@ -44,17 +44,6 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], 
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<uint32_t *>(&v);
-}
-// hi = bf16(x), lo = bf16(x - hi), both packed for two values
-__device__ __forceinline__ void split2(float x0, float x1, uint32_t &hi, uint32_t &lo) {
-    __nv_bfloat16 h0 = __float2bfloat16_rn(x0), h1 = __float2bfloat16_rn(x1);
-    hi = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-    lo = pack_bf16(x0 - __bfloat162float(h0), x1 - __bfloat162float(h1));
-}
-
 // byte offset of (row, 16-byte chunk) in a 128-byte-swizzled tile whose rows are 128 bytes
 __device__ __forceinline__ uint32_t sw128(int row, int chunk) { return (uint32_t)row * 128u + (uint32_t)((chunk ^ (row & 7)) << 4); }
 
@@ -393,14 +382,13 @@ attention_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
 
 }  // namespace
 
-// tensor maps over the caches are rebuilt only when the caller's pointers change
 int attention_tensor_supported(const viasd_model *m) { return m->cfg.dtype == 1 && m->cfg.head_dim == HD && m->use_tc; }
 int attention_mma_supported(const viasd_model *m, int M) {
     const viasd_config &c = m->cfg;
     return c.dtype == 1 && c.head_dim == HD && (c.n_heads / c.n_kv_heads) * M <= 16 && m->use_tc;
 }
 
-static int cache_maps(viasd_model *m, CacheMaps &cm, const void *kc, const void *vc, int n_layers) {
+int attention_cache_maps(const viasd_model *m, CacheMaps &cm, const void *kc, const void *vc, int n_layers) {
     if (cm.k_ptr == kc && cm.v_ptr == vc) return VIASD_OK;
     const viasd_config &c = m->cfg;
     const uint64_t rows = (uint64_t)n_layers * c.max_batch * c.n_kv_heads * c.max_ctx;
@@ -419,11 +407,11 @@ int launch_attention_mma(viasd_model *m, const void *kc, const void *vc, bool sl
     if (!attention_mma_supported(m, M)) return VIASD_EINVAL;
     CacheMaps &cm = slim ? m->cmaps_slim : m->cmaps_full;
     int rc;
-    if ((rc = cache_maps(m, cm, kc, vc, slim ? m->n_routed : c.n_layers))) return rc;
+    if ((rc = attention_cache_maps(m, cm, kc, vc, slim ? m->n_routed : c.n_layers))) return rc;
     CacheMaps *cm2 = &cm;
     if (streams == 2) {
         cm2 = &m->cmaps_slim;
-        if ((rc = cache_maps(m, *cm2, kc2, vc2, m->n_routed))) return rc;
+        if ((rc = attention_cache_maps(m, *cm2, kc2, vc2, m->n_routed))) return rc;
     }
     AttnWork a;
     a.subs = 1;

@@ -614,18 +614,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 
 }  // namespace
 
-// tensor maps over the caches are rebuilt only when the caller's pointers change
-static int cache_maps_tc(viasd_model *m, CacheMaps &cm, const void *kc, const void *vc, int n_layers) {
-    if (cm.k_ptr == kc && cm.v_ptr == vc) return VIASD_OK;
-    const viasd_config &c = m->cfg;
-    const uint64_t rows = (uint64_t)n_layers * c.max_batch * c.n_kv_heads * c.max_ctx;
-    int rc;
-    if ((rc = tc_make_map(&cm.k, kc, rows, HD, TKEYS))) return rc;
-    if ((rc = tc_make_map(&cm.v, vc, rows, HD, TKEYS))) return rc;
-    cm.k_ptr = kc; cm.v_ptr = vc;
-    return VIASD_OK;
-}
-
 // streams = 1: one cache (full or slim).  streams = 2: rows [0, batch*M) against the full cache at layer_ord and
 // rows [batch*M, 2*batch*M) against the slim cache at layer_ord2, in one launch.
 int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, const void *kc2,
@@ -633,11 +621,11 @@ int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool sli
     const viasd_config &c = m->cfg;
     CacheMaps &cm = slim ? m->cmaps_slim : m->cmaps_full;
     int rc;
-    if ((rc = cache_maps_tc(m, cm, kc, vc, slim ? m->n_routed : c.n_layers))) return rc;
+    if ((rc = attention_cache_maps(m, cm, kc, vc, slim ? m->n_routed : c.n_layers))) return rc;
     CacheMaps *cm2 = &cm;
     if (streams == 2) {
         cm2 = &m->cmaps_slim;
-        if ((rc = cache_maps_tc(m, *cm2, kc2, vc2, m->n_routed))) return rc;
+        if ((rc = attention_cache_maps(m, *cm2, kc2, vc2, m->n_routed))) return rc;
     }
     const int QR = c.n_heads / c.n_kv_heads * M;
     AttnWork a;

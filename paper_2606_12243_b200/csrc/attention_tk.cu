@@ -693,19 +693,6 @@ int attention_tk_heads_per_item(int group_heads, int M) {
         if (group_heads % hpi == 0 && hpi * M <= 32) return group_heads / hpi <= VIASD_ATTN_ITEMS_PER_KV_HEAD ? hpi : 0;
     return 0;
 }
-int attention_tk_supported(int group_heads, int M) { return attention_tk_heads_per_item(group_heads, M) > 0; }
-
-// tensor maps over the caches are rebuilt only when the caller's pointers change
-static int cache_maps_tk(viasd_model *m, CacheMaps &cm, const void *kc, const void *vc, int n_layers) {
-    if (cm.k_ptr == kc && cm.v_ptr == vc) return VIASD_OK;
-    const viasd_config &c = m->cfg;
-    const uint64_t rows = (uint64_t)n_layers * c.max_batch * c.n_kv_heads * c.max_ctx;
-    int rc;
-    if ((rc = tc_make_map(&cm.k, kc, rows, HD, TKEYS))) return rc;
-    if ((rc = tc_make_map(&cm.v, vc, rows, HD, TKEYS))) return rc;
-    cm.k_ptr = kc; cm.v_ptr = vc;
-    return VIASD_OK;
-}
 
 // streams = 1: one cache (full or slim).  streams = 2: rows [0, batch*M) against the full cache at layer_ord and
 // rows [batch*M, 2*batch*M) against the slim cache at layer_ord2, in one launch.
@@ -715,11 +702,11 @@ int launch_attention_tk(viasd_model *m, const void *kc, const void *vc, bool sli
     const viasd_config &c = m->cfg;
     CacheMaps &cm = slim ? m->cmaps_slim : m->cmaps_full;
     int rc;
-    if ((rc = cache_maps_tk(m, cm, kc, vc, slim ? m->n_routed : c.n_layers))) return rc;
+    if ((rc = attention_cache_maps(m, cm, kc, vc, slim ? m->n_routed : c.n_layers))) return rc;
     CacheMaps *cm2 = &cm;
     if (streams == 2) {
         cm2 = &m->cmaps_slim;
-        if ((rc = cache_maps_tk(m, *cm2, kc2, vc2, m->n_routed))) return rc;
+        if ((rc = attention_cache_maps(m, *cm2, kc2, vc2, m->n_routed))) return rc;
     }
     const int grp = c.n_heads / c.n_kv_heads, hpi = attention_tk_heads_per_item(grp, M);
     if (hpi == 0) return VIASD_EINVAL;

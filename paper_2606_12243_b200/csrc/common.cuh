@@ -25,7 +25,6 @@ struct TreeInfo {                       // one per sequence, rebuilt from `paren
     int depth[VIASD_MAX_ROWS_PER_SEQ];
     int first_child[VIASD_MAX_ROWS_PER_SEQ];          // per row: first child node or -1
     int next_sibling[VIASD_MAX_ROWS_PER_SEQ];         // per node: next child of the same parent or -1
-    int is_chain;
 };
 
 struct DeviceStats {
@@ -129,14 +128,11 @@ struct viasd_model {
 // the nodes in order, each a round trip through memory, took 7 us for a tree of 26 and 13 us for a chain of 63.)
 __device__ inline void build_tree(TreeInfo *tree, const int *parent, int N, DeviceStats *stats, int *par_sh) {
     const int lane = threadIdx.x & 31, M = N + 1;
-    bool chain = true;
     for (int n = lane; n < N; n += 32) {
         int p = parent[n];
         if (p != -2 && (p < -1 || p >= n)) { stats->device_status = VIASD_EDEVICE; p = -1; }
-        chain = chain && p == n - 1;
         par_sh[n] = p;
     }
-    chain = __all_sync(0xffffffffu, chain);
     __syncwarp();
     for (int i = lane; i < M; i += 32) {                     // row i is node i - 1 (row 0: the pending token)
         unsigned long long anc = 1ull << i;
@@ -156,7 +152,7 @@ __device__ inline void build_tree(TreeInfo *tree, const int *parent, int N, Devi
         tree->first_child[i] = first;
         if (i > 0) tree->next_sibling[i - 1] = next;
     }
-    if (lane == 0) { tree->is_chain = chain; tree->next_sibling[N] = -1; }
+    if (lane == 0) tree->next_sibling[N] = -1;
     __syncwarp();                                            // par_sh may be used again
 }
 
@@ -245,10 +241,11 @@ int attention_mma_supported(const viasd_model *m, int M);
 int launch_attention_mma(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, const void *kc2,
                          const void *vc2, int layer_ord2, int streams, int batch, int M, cudaStream_t st);
 int attention_tensor_supported(const viasd_model *m);
+// tensor maps over a model's caches, rebuilt only when the caller's pointers change
+int attention_cache_maps(const viasd_model *m, CacheMaps &cm, const void *kc, const void *vc, int n_layers);
 int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, const void *kc2,
                          const void *vc2, int layer_ord2, int streams, int batch, int M, cudaStream_t st);
 int attention_tk_heads_per_item(int group_heads, int M);
-int attention_tk_supported(int group_heads, int M);
 int launch_attention_tk(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, const void *kc2,
                          const void *vc2, int layer_ord2, int streams, int batch, int M, int nsplit, int fuse_merge,
                          cudaStream_t st);

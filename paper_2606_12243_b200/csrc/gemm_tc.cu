@@ -16,8 +16,8 @@
 // bit-reproducible whoever does it.  A contributor that
 // continues into the next tile never waits, so waits cannot chain.
 //
-// Warp roles (320 threads): warp 0 issues TMA loads into a ring of stages, warp 1 allocates TMEM and
-// issues tcgen05.mma, warps 2-9 read the accumulators (tcgen05.ld) and run the epilogue.  Accumulators
+// Warp roles (192 or 320 threads): warp 0 issues TMA loads into a ring of stages, warp 1 allocates TMEM and
+// issues tcgen05.mma, one or two groups of four warps read the accumulators (tcgen05.ld) and run the epilogue.  Accumulators
 // are double-buffered in TMEM so the epilogue of one tile overlaps the main loop of the next.
 // Every wait is bounded: on expiry the CTA records VIASD_EDEVICE, lets its copies land and leaves.
 #include "common.cuh"

@@ -77,10 +77,11 @@ int launch_clear_words(int *words, int n, cudaStream_t st);   // counters of a s
 // gemm_wide.cu: pairs of CTAs, up to 256 token rows; L.nt = tc_wide_th(rows), gate/up maps with 64-row boxes
 constexpr int TC_WIDE_ROWS = 256;
 // Token rows of one verifier from which a pass runs on the pair kernel (the choice may not depend on whether the other
-// verifier's rows ride along, or the one-sweep step and its pieces would differ in the last bit).  8B shapes, one-CTA /
-// pair kernel, us: 54 rows QKV 16.0 / 18.0, O 13.7 / 15.7, gate-up 45.7 / 45.5, down 29 / 30; 108 rows 19.8 / 20.1,
-// 17.0 / 17.2, 63 / 56, 36 / 32.  Whole steps: 13B batch 8 (56 rows, 112 in routed layers) 6.94 -> 6.70 ms with it, 8B
-// batch 1 (27 and 54 rows) 4.33 -> 4.51 ms.
+// verifier's rows ride along, or the one-sweep step and its pieces would differ in the last bit).  Six layers, half of
+// them routed, context 512, us, one-CTA / pair kernel: 48 rows full pass 8B 767 / 761, 7B 720 / 703, 13B 948 / 911, step 887 /
+// 826, 856 / 801, 1163 / 1072; 54 rows full pass 752 / 749, 705 / 710, 936 / 936, step 897 / 889, 885 / 833, 1243 / 1147; 64 rows full
+// pass 797 / 793, 736 / 746, 979 / 946; 81 rows 888 / 815, 860 / 769, 1160 / 1031, step 1473 / 1151, 1441 / 1160, 1938 / 1566.  With
+// 27 rows per verifier (8B batch 1, 54 in its routed layers) the step was 4.33 / 4.51 ms.
 constexpr int TC_WIDE_MIN_ROWS = 48;
 int tc_wide_th(int rows);
 int launch_gemm_wide(const TcLaunch &L, cudaStream_t st);

@@ -113,7 +113,6 @@ __global__ void prep_replay_kernel(TreeInfo *tree, int *len_eff, int *row_tok, D
             t->anc[i] = t->anc[pr] | (1ull << i);
             t->depth[i] = t->depth[pr] + 1;
         }
-        t->is_chain = 0;
         const int l = len[b] - G;
         const int c = min(max(l, 0), max_ctx - Mx);
         if (c != l) stats->device_status = VIASD_ECAPACITY;     // fewer than G committed tokens, or no room for the rows
