@@ -230,7 +230,8 @@ enum {
     VIASD_OPT_TK_GRID,                 /* keys-on-lanes attention with tiles dealt evenly: CTAs to use; 0 = one per SM */
     VIASD_OPT_TK_FLAT,                 /* keys-on-lanes attention: deal tiles 1, key ranges 0; -1 = by shape (default) */
     VIASD_OPT_GEMM_RING_KB,            /* stream-K GEMM: shared-memory ring in KB, 32..200; 0 = default (200) */
-    VIASD_OPT_GEMM_EPI_GROUPS          /* stream-K GEMM: groups of four epilogue warps, 1 or 2; 0 = by token tile */
+    VIASD_OPT_GEMM_EPI_GROUPS,         /* stream-K GEMM: groups of four epilogue warps, 1 or 2; 0 = by token tile */
+    VIASD_OPT_ONE_LAUNCH               /* 1 (default): the forward pass of a small model with few token rows is one launch; 0: never */
 };
 int viasd_set_option(viasd_model *m, int option, int value);
 

@@ -26,7 +26,7 @@ EXPORTS = ["viasd_workspace_bytes", "viasd_init_model", "viasd_full_forward", "v
            "viasd_tier_accept_n", "viasd_kv_commit_slim"]
 
 OPTIONS = {"attention_kernel": 0, "attention_splits": 1, "attention_lo": 2, "accept_team": 3, "dual_max_rows": 4,
-           "tk_grid": 5, "tk_flat": 6, "gemm_ring_kb": 7, "gemm_epi_groups": 8}
+           "tk_grid": 5, "tk_flat": 6, "gemm_ring_kb": 7, "gemm_epi_groups": 8, "one_launch": 9}
 ATTENTION_KERNELS = {"auto": 0, "mma": 1, "tc": 2, "tk": 3}
 
 TIMING_CLASSES = ["gemm", "attention", "norm", "rope", "embed", "tier_accept", "commit"]

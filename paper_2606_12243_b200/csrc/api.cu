@@ -68,6 +68,7 @@ size_t carve(const viasd_config &c, char *base, Workspace *ws) {
         w.a_head = cv.take<void>(R * c.d_model * 4);
         w.ssq_head = cv.take<float>((size_t)(c.d_model / 128 + 1) * 4 * R * 4);
         w.attn_counters = cv.take<int>(attn_counter_count(c.max_batch, c.n_heads, c.n_kv_heads) * sizeof(int));
+        w.pass_counters = cv.take<int>(small_pass_counters(c.max_batch, c.n_heads) * sizeof(int));
         w.n_counters = widest / 64 + 8;                      // (a tile of the pair kernel's gate/up launch has 64 features)
         w.gemm_counters = cv.take<int>(w.n_counters * 4);
     }
@@ -105,6 +106,7 @@ void default_options(ModelOptions &o) {
     o.tk_flat = env_int("VIASD_TK_FLAT", -1);
     o.ring_kb = env_int("VIASD_TC_RING_KB", 0);
     o.epi_groups = env_int("VIASD_TC_EPI_GROUPS", 0);
+    o.one_launch = env_int("VIASD_ONE_LAUNCH", 1);
 }
 
 int check_config(const viasd_config *c) {
@@ -299,6 +301,8 @@ int forward(viasd_model *m, const viasd_cache *cache, const viasd_draft *d, bool
     int rc;
     if ((rc = check_draft(m, d)) || (rc = check_cache(cache))) return rc;
     if (!logits) return VIASD_EINVAL;
+    if (small_pass_takes(m, cache, d->batch, d->n_nodes + 1))
+        return timed(m, VIASD_T_GEMM, st, [&] { return launch_small_pass(m, cache, d, slim ? 1 : 0, 0, logits, logits, st); });
     if (m->fused) return forward_sweep(m, cache, d, slim ? 1 : 0, slim ? nullptr : logits, slim ? logits : nullptr, st);
     const viasd_config &c = m->cfg;
     const int B = d->batch, M = d->n_nodes + 1, rows = B * M;
@@ -460,6 +464,7 @@ int viasd_init_model(const viasd_config *cfg, const viasd_weights *w, const unsi
     cudaError_t e = cudaMemset(m->ws.stats, 0, sizeof(DeviceStats));
     if (e == cudaSuccess) { const int one = 1; e = cudaMemcpy(&m->ws.stats->full_ran, &one, sizeof(int), cudaMemcpyHostToDevice); }
     if (e == cudaSuccess) e = cudaMemset(m->ws.gemm_counters, 0, m->ws.n_counters * 4);
+    if (e == cudaSuccess) e = cudaMemset(m->ws.pass_counters, 0, small_pass_counters(cfg->max_batch, cfg->n_heads) * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(m->ws.attn_counters, 0, attn_counter_count(cfg->max_batch, cfg->n_heads, cfg->n_kv_heads) * sizeof(int));
     if (e == cudaSuccess) { rc = launch_rope_table(m, 0); if (rc == VIASD_OK) e = cudaDeviceSynchronize(); }
     if (e != cudaSuccess) { g_last_cuda_error = (int)e; rc = VIASD_ECUDA; }
@@ -574,9 +579,9 @@ static int verify_step_routed(viasd_model *m, viasd_cache *cache, const viasd_dr
     int *flag = &m->ws.stats->full_ran;
     if (params->conf_source == 0) {
         if ((rc = viasd_tier_accept(m, draft, params, nullptr, nullptr, 1, result, stream))) return rc;
-        if ((rc = forward_sweep(m, cache, draft, 1, nullptr, slim_logits, st))) return rc;
+        if ((rc = forward(m, cache, draft, true, slim_logits, st))) return rc;
     } else {
-        if ((rc = forward_sweep(m, cache, draft, 1, nullptr, slim_logits, st))) return rc;
+        if ((rc = forward(m, cache, draft, true, slim_logits, st))) return rc;
         if ((rc = viasd_tier_accept(m, draft, params, slim_logits, nullptr, 1, result, stream))) return rc;
     }
     CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(int), st));
@@ -585,7 +590,12 @@ static int verify_step_routed(viasd_model *m, viasd_cache *cache, const viasd_dr
     if ((rc = timed(m, VIASD_T_TIER_ACCEPT, st, [&] { return launch_accept(m, draft, params, probe_set, result, true,
                                                                       false, st, &probe); }))) return rc;
     m->run_flag = flag;
-    rc = forward_sweep(m, cache, draft, 0, full_logits, nullptr, st, G);
+    if (small_pass_takes(m, cache, draft->batch, M + G)) {
+        rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_prep_replay(m, cache, draft, G, st); });
+        if (!rc) rc = timed(m, VIASD_T_GEMM, st, [&] { return launch_small_pass(m, cache, draft, 0, G, full_logits, nullptr, st); });
+    } else {
+        rc = forward_sweep(m, cache, draft, 0, full_logits, nullptr, st, G);
+    }
     m->run_flag = nullptr;
     if (rc) return rc;
     if ((rc = tier_accept_impl(m, draft, params, slim_logits, full_logits, 2, result, false, stream))) return rc;
@@ -605,8 +615,12 @@ int viasd_verify_step(viasd_model *m, viasd_cache *cache, const viasd_draft *dra
     // that a sweep would stream every routed layer twice anyway, and the passes run one after the other.
     const int block_rows = draft->batch * (draft->n_nodes + 1);
     const int dual_max = m->opt.dual_max_rows >= 0 ? m->opt.dual_max_rows : block_rows >= TC_WIDE_MIN_ROWS ? TC_WIDE_ROWS : 128;
-    if (m->fused && 2 * block_rows <= dual_max) {
-        if ((rc = forward_sweep(m, cache, draft, 2, full_logits, slim_logits, (cudaStream_t)stream))) return rc;
+    const bool small = small_pass_takes(m, cache, draft->batch, draft->n_nodes + 1);
+    if (small ? m->opt.dual_max_rows < 0 || 2 * block_rows <= dual_max : m->fused && 2 * block_rows <= dual_max) {
+        cudaStream_t st = (cudaStream_t)stream;
+        if (small) rc = timed(m, VIASD_T_GEMM, st, [&] { return launch_small_pass(m, cache, draft, 2, 0, full_logits, slim_logits, st); });
+        else rc = forward_sweep(m, cache, draft, 2, full_logits, slim_logits, st);
+        if (rc) return rc;
         if ((rc = tier_accept_impl(m, draft, params, slim_logits, full_logits, 3, result, true, stream))) return rc;
         return viasd_kv_commit(m, cache, draft, result, stream);
     }
@@ -647,6 +661,7 @@ int viasd_set_option(viasd_model *m, int option, int value) {
     case VIASD_OPT_TK_FLAT: if (value < -1 || value > 1) return VIASD_EINVAL; o.tk_flat = value; break;
     case VIASD_OPT_GEMM_RING_KB: if (value != 0 && (value < 32 || value > 200)) return VIASD_EINVAL; o.ring_kb = value; break;
     case VIASD_OPT_GEMM_EPI_GROUPS: if (value < 0 || value > 2) return VIASD_EINVAL; o.epi_groups = value; break;
+    case VIASD_OPT_ONE_LAUNCH: if (value != 0 && value != 1) return VIASD_EINVAL; o.one_launch = value; break;
     default: return VIASD_EINVAL;
     }
     return VIASD_OK;

@@ -63,6 +63,7 @@ struct Workspace {                      // pointers into the caller's workspace 
     int *gemm_counters;                 // per-tile arrival counters, zero between launches
     size_t n_counters;
     int *attn_counters;                 // [attn_counter_count()] key-range arrivals per (stream, sequence, kv head, group of query heads)
+    int *pass_counters;                 // [small_pass_counters()] arrivals of a pass in one launch, zero between launches
     float *ssq;                         // [(d / 128) * 4][R] partial sums of h^2 for the fused RMSNorm
     void *a_head; float *ssq_head;      // the block's own rows of `a` and `ssq`, compacted for the output head after a replay pass
 };
@@ -96,6 +97,7 @@ struct ModelOptions {
     int tk_flat;            // VIASD_OPT_TK_FLAT: deal tiles (1) or key ranges (0); -1 = by shape
     int ring_kb;            // VIASD_OPT_GEMM_RING_KB: shared-memory ring of the stream-K GEMM
     int epi_groups;         // VIASD_OPT_GEMM_EPI_GROUPS: groups of four epilogue warps; 0 = by token tile
+    int one_launch;         // VIASD_OPT_ONE_LAUNCH: a small model's forward pass as one launch
 };
 
 struct viasd_model {
@@ -232,6 +234,15 @@ struct GemmSegs { const void *w[3]; int n[3]; int count; };
 // x_plane / act_plane: element distance between the hi and lo planes (0: single plane)
 int launch_gemm_rowwarp(const void *x, size_t x_plane, const GemmSegs &segs, int rows, int k, int dtype,
                         int epilogue, float *out_f32, void *out_act, size_t act_plane, int ld_out, int sms, cudaStream_t st);
+
+// small_pass.cu -- a small model's forward pass in one launch
+constexpr int SMALL_PASS_MAX_LAYERS = 24, SMALL_PASS_MAX_ROWS = 64;      // rows: of both verifiers together
+inline size_t small_pass_counters(int max_batch, int n_heads) {         // two barriers; an attention item has 16 query rows of a kv head
+    return 2 + (size_t)2 * max_batch * n_heads * (VIASD_MAX_ROWS_PER_SEQ / 16);
+}
+bool small_pass_takes(const viasd_model *m, const viasd_cache *cache, int batch, int M);
+int launch_small_pass(viasd_model *m, const viasd_cache *cache, const viasd_draft *d, int mode, int replay, float *logits_full,
+                      float *logits_slim, cudaStream_t st);
 
 // attention.cu
 int launch_attention(viasd_model *m, const void *kc, const void *vc, bool slim, int layer_ord, int batch, int M,

@@ -517,6 +517,61 @@ def test_verify_step_with_each_attention_kernel(name, env, monkeypatch):
     _check_verify_step(name)
 
 
+# launch by launch, where a small model's pass is one launch by default
+@pytest.mark.parametrize("name", ["c1_tiny", "tiny_tree_f32", "mini_7b"])
+def test_verify_step_launch_by_launch(name, monkeypatch):
+    monkeypatch.setenv("VIASD_ONE_LAUNCH", "0")
+    _check_verify_step(name)
+
+
+def _one_launch_case(name, batch, nodes, ctx, tree=False, **shape):
+    base = W.get(name)
+    return replace(base, batch=batch, ctx=ctx, parent=W.tree26() if tree else W.chain(nodes), real_prefill=False,
+                   shape=replace(base.shape, **shape))
+
+
+@pytest.mark.parametrize("wl", [
+    _one_launch_case("c1_tiny", 1, 1, 0), _one_launch_case("c1_tiny", 3, 8, 63, d_model=192, d_ff=680),      # k no whole groups of 32
+    _one_launch_case("c1_tiny", 2, 26, 300, tree=True, n_kv_heads=2, vocab=1001),                             # grouped heads, odd vocabulary
+    _one_launch_case("c1_tiny", 5, 12, 70, head_dim=128, n_heads=2, n_kv_heads=1),                            # 65 rows: three launches
+    _one_launch_case("c1_tiny", 2, 63, 90), _one_launch_case("c1_tiny", 2, 8, 40, d_model=768, d_ff=2048),   # a verifier per launch; fewer rows per launch
+    _one_launch_case("mini_7b", 1, 1, 0), _one_launch_case("mini_7b", 1, 15, 63), _one_launch_case("mini_7b", 3, 7, 130),   # 2, 16, 24 rows
+    _one_launch_case("mini_8b_tree_greedy", 1, 26, 500, tree=True), _one_launch_case("mini_13b", 3, 6, 260, n_layers=2),
+    _one_launch_case("mini_7b", 1, 8, 200, d_model=1024, d_ff=2824)], ids=lambda w: f"{w.name}-{w.batch}x{w.rows}-{w.ctx}")
+def test_pass_in_one_launch_is_the_pass(wl):
+    """Logits and caches of a pass in one launch are those of the kernels for any model, launch by launch, within what either may
+    be off the oracle; and the step's are bit for bit those of the two passes on their own."""
+    wl = replace(wl, n_routed=min(wl.n_routed, wl.shape.n_layers))
+    vb = _vb()
+    outs = []
+    for one in (1, 0, 1):
+        eng = _engine(wl, fill_context="device")
+        eng.set_inputs(W.step_inputs(wl))
+        vb.set_option(eng.model, "one_launch", one)
+        sl, fl, res = eng.logits_buffer(), eng.logits_buffer(), vb.alloc_result(wl.batch, wl.n_nodes)
+        n0 = vb.launch_count()
+        if len(outs) < 2:
+            # nothing is accepted, so the commit moves no row
+            vb.verify_step(eng.model, eng.cache, eng.draft, eng.params(log_tau_lo=1e9, log_tau_hi=1e9, log_acc_rel=(1e9, 1e9, 1e9)), sl, fl, res)
+        else:
+            vb.full_forward(eng.model, eng.cache, eng.draft, fl)
+            vb.slim_forward(eng.model, eng.cache, eng.draft, sl)
+        torch.cuda.synchronize()
+        assert vb.get_stats(eng.model).device_status == 0
+        outs.append([t.clone() for t in (sl, fl, eng.k_full, eng.v_full, eng.k_slim, eng.v_slim)] + [vb.launch_count() - n0])
+    step, many, pieces = outs
+    assert step[-1] < many[-1]
+    for a, b in zip(step[:-1], pieces[:-1]):
+        assert torch.equal(a, b)
+    f32 = wl.shape.dtype == "f32"
+    for i, (a, b) in enumerate(zip(step[:-1], many[:-1])):
+        # twice the bound of either against the oracle; a bf16 cache value may round the other way
+        tol = (2e-4 if f32 else 6e-2) if i < 2 else (2e-4 if f32 else 2.0 ** -7 * max(1.0, float(b.abs().max())))
+        assert float((a.float() - b.float()).abs().max()) <= tol, i
+    if f32:
+        assert float((step[1] - many[1]).norm() / many[1].norm()) <= 1e-5
+
+
 # Sequences of different lengths in one batch.  The attention kernels deal key ranges or tiles to CTAs from the
 # committed lengths (the keys-on-lanes kernel cuts the tiles of all (sequence, head) pairs, laid end to end, into
 # equal ranges), so lengths that need 5, 6 and 7 tiles of 128 keys check those cuts against the oracle.  The extra
