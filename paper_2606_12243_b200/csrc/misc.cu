@@ -209,6 +209,7 @@ embed_norm_kernel(float *h, __nv_bfloat16 *a, size_t plane, float *ssq, int ssq_
     __shared__ int par_sh[VIASD_MAX_ROWS_PER_SEQ];
     const int r = (int)blockIdx.x - prep_ctas(p), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     PDL_TRIGGER();
+    PDL_WAIT();
     if (r < 0) { if (warp == 0) prep_sequence(p, blockIdx.x, par_sh); return; }
     const __nv_bfloat16 *src = E + (size_t)prep_token(p, r < rows ? r : r - rows) * d;
     embed_row(h, a, plane, ssq, ssq_stride, src, r < rows ? gain_full : gain_slim, r, d, warp, lane);
@@ -217,9 +218,9 @@ embed_norm_kernel(float *h, __nv_bfloat16 *a, size_t plane, float *ssq, int ssq_
 int launch_embed_norm(const viasd_model *m, const viasd_cache *c, const viasd_draft *d, bool full_pass, bool replay, const float *gain,
                       const float *gain_slim, int rows, cudaStream_t st) {
     const PrepArgs p = prep_args(m, c, d, full_pass, replay);
-    embed_norm_kernel<<<(replay ? 0 : d->batch) + (gain_slim ? 2 : 1) * rows, 256, 0, st>>>(
+    CUDA_TRY(launch_chained(embed_norm_kernel, (replay ? 0 : d->batch) + (gain_slim ? 2 : 1) * rows, 256, st,
         m->ws.h, (__nv_bfloat16 *)m->ws.a, m->ws.rows_alloc * m->cfg.d_model, m->ws.ssq, (int)m->ws.rows_alloc,
-        (const __nv_bfloat16 *)m->embed, gain, gain_slim, p, m->cfg.d_model, rows, m->run_flag);
+        (const __nv_bfloat16 *)m->embed, gain, gain_slim, p, m->cfg.d_model, rows, m->run_flag));
     LAUNCH_CHECK();
     return VIASD_OK;
 }
@@ -365,6 +366,7 @@ __global__ void __launch_bounds__(32 * COMMIT_WARPS) commit_kernel(const CommitA
     __shared__ int last_sh;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, M = a.N + 1;
     const int item = blockIdx.x * COMMIT_WARPS + warp, n_items = (a.L + a.Ls - a.layer0) * a.B * a.Hkv;
+    PDL_WAIT();
     const bool full_ran = a.stats->full_ran != 0;
     if (item < n_items) {
         const int g = item % a.Hkv, b = (item / a.Hkv) % a.B, layer = a.layer0 + item / (a.Hkv * a.B);
@@ -437,7 +439,7 @@ int launch_commit(const viasd_model *m, viasd_cache *c, const viasd_draft *d, co
     const bool vec = (((uintptr_t)a.kf | (uintptr_t)a.vf | (uintptr_t)a.ks | (uintptr_t)a.vs) & 15) == 0;
     auto kernel = vec ? commit_kernel<uint4> : cf.dtype == 0 ? commit_kernel<uint32_t> : commit_kernel<uint16_t>;
     a.row_vecs = vec ? cf.head_dim * (cf.dtype == 0 ? 4 : 2) / 16 : cf.head_dim;
-    kernel<<<(items + COMMIT_WARPS - 1) / COMMIT_WARPS, 32 * COMMIT_WARPS, 0, st>>>(a);
+    CUDA_TRY(launch_chained(kernel, (items + COMMIT_WARPS - 1) / COMMIT_WARPS, 32 * COMMIT_WARPS, st, a));
     LAUNCH_CHECK();
     return VIASD_OK;
 }

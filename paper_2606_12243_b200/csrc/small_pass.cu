@@ -851,6 +851,7 @@ template <typename T, int HD, int MT>
 __global__ void __launch_bounds__(SP_THREADS, 1) small_pass_kernel(const __grid_constant__ SpArgs a) {
     extern __shared__ __align__(128) uint8_t sp_smem[];
     RUN_FLAG_EXIT(a.run_flag);
+    PDL_TRIGGER();
     using P = Pass<T, HD, MT>;
     P pass(a, sp_smem);
     pass.run();

@@ -186,6 +186,8 @@ row_stats_kernel(RowStats rs, RowPtrs src, int R, int M, int V, ExpScale scale, 
     __shared__ MaxIdx shm[RS_THREADS / 32];
     const int kind = blockIdx.z, b = blockIdx.y, r = blockIdx.x;
     __shared__ int par_sh[VIASD_MAX_ROWS_PER_SEQ];
+    PDL_TRIGGER();
+    PDL_WAIT();
     if (kind == 0 && r == 0) {
         if (clear_needs && b == 0 && threadIdx.x == 0) stats->need_slim = stats->need_full = 0;
         if (tree && threadIdx.x < 32) build_tree(tree + b, parent + (per_seq ? (size_t)b * (M - 1) : 0), M - 1, stats, par_sh);
@@ -370,6 +372,8 @@ accept_kernel(AcceptArgs a) {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(tm.rank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(tm.size));
     tm.slots = slots; tm.phase = 0;
+    PDL_TRIGGER();
+    PDL_WAIT();
     const int tid = threadIdx.x;
     const int b = blockIdx.x / tm.size, N = a.N, M = N + 1, V = a.V;
     const bool sampling = a.mode == 1, writes = tm.rank == 0 && !a.probe;     // writes: this CTA stores the results
@@ -699,8 +703,8 @@ int launch_accept(const viasd_model *m, const viasd_draft *d, const viasd_params
         for (int k = 1; k < KINDS; ++k) src.p[k] = k <= js.n ? js.logits[k - 1] : nullptr;
         auto kernel = p->mode == 1 ? row_stats_kernel<true> : row_stats_kernel<false>;
         const float temperature = p->mode == 1 ? p->temperature : 1.f;
-        kernel<<<dim3(rows, d->batch, js.n + 1), RS_THREADS, 0, st>>>(a.rs, src, d->n_prows, M, m->cfg.vocab,
-            exp_scale(temperature), RS_GAP * temperature, m->ws.stats, do_tier ? 1 : 0, tree_ready ? nullptr : m->ws.tree, d->parent, d->per_sequence);
+        CUDA_TRY(launch_chained(kernel, dim3(rows, d->batch, js.n + 1), RS_THREADS, st, a.rs, src, d->n_prows, M, m->cfg.vocab,
+            exp_scale(temperature), RS_GAP * temperature, m->ws.stats, do_tier ? 1 : 0, tree_ready ? nullptr : m->ws.tree, d->parent, d->per_sequence));
         LAUNCH_CHECK();
     }
     a.judges[0] = nullptr;
@@ -736,15 +740,13 @@ int launch_accept(const viasd_model *m, const viasd_draft *d, const viasd_params
     if (team == ACC_TEAM && m->cfg.vocab >= 65536 && accept_team16_ok()) team = 16;     // every sweep of the vocabulary is shared
     { const int t = m->opt.accept_team; if (t == 1 || t == 2 || t == 4 || t == 8) team = t; }
     cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(d->batch * team);
-    cfg.blockDim = dim3(ACC_THREADS);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = team; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = team > 1 ? 1 : 0;
+    cudaLaunchAttribute attr[2];
+    pdl_config(cfg, attr, dim3(d->batch * team), dim3(ACC_THREADS), 0, st);
+    if (team > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = team; attr[cfg.numAttrs].val.clusterDim.y = 1; attr[cfg.numAttrs].val.clusterDim.z = 1;
+        ++cfg.numAttrs;
+    }
     CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_kernel, a));
     LAUNCH_CHECK();
     return VIASD_OK;
