@@ -56,7 +56,7 @@ size_t carve(const viasd_config &c, char *base, Workspace *ws) {
     w.row_tok = cv.take<int>(R * 4);
     w.tree = cv.take<TreeInfo>(sizeof(TreeInfo) * (size_t)c.max_batch);
     w.stats = cv.take<DeviceStats>(sizeof(DeviceStats));
-    w.accept_scratch = cv.take<float>((size_t)c.max_batch * 3 * (VIASD_MAX_JUDGES + 1) * VIASD_MAX_ROWS_PER_SEQ * 4);
+    w.accept_scratch = cv.take<float>((size_t)c.max_batch * 3 * (VIASD_MAX_JUDGES + 1) * VIASD_MAX_ROWS_PER_SEQ * ROW_STAT_PARTS * 4);
     w.accept_fold = cv.take<float>((size_t)c.max_batch * (VIASD_MAX_JUDGES + 1) * c.vocab * 4);
     {
         const int nt = tc_pick_nt(R < 128 ? (int)R : 128, true);

@@ -9,6 +9,7 @@
 #include "gemm_tc.cuh"
 
 #define VIASD_MAX_ROWS_PER_SEQ 64
+constexpr int ROW_STAT_PARTS = 4;       // a logits row's statistics come in at most this many parts
 // Arrival counters of the attention kernels: one per (stream, sequence, kv head, item of that kv head).  The
 // keys-on-lanes kernel deals the query heads of a kv head to at most this many items.
 #define VIASD_ATTN_ITEMS_PER_KV_HEAD 4
@@ -57,7 +58,7 @@ struct Workspace {                      // pointers into the caller's workspace 
     int *row_tok;                       // [R] token id per row
     TreeInfo *tree;                     // [max_batch]: every sequence has its own draft tree (copies when the call shares one)
     DeviceStats *stats;
-    float *accept_scratch;              // [3][B, judges + 1, 64] row statistics
+    float *accept_scratch;              // [3][B, judges + 1, 64, ROW_STAT_PARTS] row statistics
     float *accept_fold;                 // [B, judges + 1, vocab] residuals of a position with many rejections (sampling)
     float *gemm_scratch;                // partial tiles of split GEMM work (tcgen05 kernel)
     int *gemm_counters;                 // per-tile arrival counters, zero between launches

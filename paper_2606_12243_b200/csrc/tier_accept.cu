@@ -144,9 +144,14 @@ tier_kernel(unsigned char *__restrict__ tier, float *__restrict__ conf, DeviceSt
 // HBM-bound: every row once.  Maximum and denominator come from one sweep (a running reference per thread, moved when it is
 // exceeded by e^20); two sweeps read a batch's rows twice from HBM, 16 sequences' 1040 rows of 0.5 MB being far more than L2
 // holds.  Eight 16-byte loads per thread in flight: few rows are bound by what a CTA has under way.
+// A row's statistics are kept in parts, which the walk puts together.  Whole turns of two CTAs per SM take whole rows, part after
+// part; what is left over goes a part per CTA, so that one sequence's 66 rows fill the chip and the last of 1040 rows' turns is a
+// quarter as long (a part's numbers are the same either way).
 constexpr int RS_STRIDE = VIASD_MAX_ROWS_PER_SEQ, RS_THREADS = 512, RS_BATCH = 8;
 constexpr float RS_GAP = 20.f;
-struct RowStats { float *mx; int *arg; float *z; };       // each [B, KINDS, RS_STRIDE]
+struct RowStats { float *mx; int *arg; float *z; };       // each [B, KINDS, RS_STRIDE, parts]
+// (by the vocabulary: a row's sums do not depend on the call's other rows)
+int row_parts(int vocab) { return vocab >= 65536 ? ROW_STAT_PARTS : vocab >= 16384 ? 2 : 1; }
 struct RowPtrs { const float *p[KINDS]; };                // drafter logits, then each judge's
 
 template <bool WANT_Z>
@@ -177,57 +182,71 @@ struct RowAcc {
     }
 };
 
+struct RowUnits { int B, R, M, whole, parts; };           // rows: [drafter rows of all sequences, unless R is 0][judge 1's] ..., the first `whole` by a CTA each
 template <bool WANT_Z>
 __global__ void __launch_bounds__(RS_THREADS, 2)
-row_stats_kernel(RowStats rs, RowPtrs src, int R, int M, int V, ExpScale scale, float gap, DeviceStats *stats, int clear_needs,
+row_stats_kernel(RowStats rs, RowPtrs src, RowUnits un, int V, ExpScale scale, float gap, DeviceStats *stats, int clear_needs,
                  TreeInfo *tree, const int *parent, int per_seq) {
-    // tree != null: no forward pass of the same call has laid the trees out, so the first CTA of each sequence does
-    __shared__ float sh[RS_THREADS / 32];
-    __shared__ MaxIdx shm[RS_THREADS / 32];
-    const int kind = blockIdx.z, b = blockIdx.y, r = blockIdx.x;
+    // tree != null: no forward pass of the same call has laid the trees out, so the first CTAs do, one per sequence
+    constexpr int WARPS = RS_THREADS / 32;
+    __shared__ float sh_z[ROW_STAT_PARTS][WARPS];
+    __shared__ MaxIdx sh_m[ROW_STAT_PARTS][WARPS];
     __shared__ int par_sh[VIASD_MAX_ROWS_PER_SEQ];
     PDL_TRIGGER();
     PDL_WAIT();
-    if (kind == 0 && r == 0) {
-        if (clear_needs && b == 0 && threadIdx.x == 0) stats->need_slim = stats->need_full = 0;
-        if (tree && threadIdx.x < 32) build_tree(tree + b, parent + (per_seq ? (size_t)b * (M - 1) : 0), M - 1, stats, par_sh);
-    }
-    const float *base = src.p[kind];
-    const int rows = kind == 0 ? R : M;
-    if (!base || r >= rows) return;
-    const float *row = base + ((size_t)b * rows + r) * V;
-    RowAcc<WANT_Z> acc;
-    acc.init();
+    const int x = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (clear_needs && x == 0 && tid == 0) stats->need_slim = stats->need_full = 0;
+    if (tree && x < un.B && tid < 32) build_tree(tree + x, parent + (per_seq ? (size_t)x * (un.M - 1) : 0), un.M - 1, stats, par_sh);
+    const int id = x < un.whole ? x : un.whole + (x - un.whole) / un.parts;
+    const int first = x < un.whole ? 0 : (x - un.whole) % un.parts, last = x < un.whole ? un.parts : first + 1;
+    const bool drafter = id < un.B * un.R;
+    const int rows = drafter ? un.R : un.M, at = drafter ? id : id - un.B * un.R, kind = drafter ? 0 : 1 + at / (un.B * un.M);
+    const int br = drafter ? at : at % (un.B * un.M), b = br / rows, r = br - b * rows;
+    const float *row = src.p[kind] + (size_t)br * V;
     // up to three values in front of the first 16-byte boundary (an odd vocabulary), then 16-byte pieces, then the rest
     const int head = min(V, (int)((4 - ((reinterpret_cast<uintptr_t>(row) >> 2) & 3)) & 3)), n4 = (V - head) >> 2, tail = V - head - 4 * n4;
     const float4 *r4 = reinterpret_cast<const float4 *>(row + head);
-    if ((int)threadIdx.x < head) { const float x[1] = {row[threadIdx.x]}; acc.add(x, threadIdx.x, 0, scale, gap); }
-    int i0 = threadIdx.x;
+    const int per = (n4 + un.parts - 1) / un.parts;
 #pragma unroll 1
-    for (; i0 + (RS_BATCH - 1) * RS_THREADS < n4; i0 += RS_BATCH * RS_THREADS) {
-        float x[4 * RS_BATCH];
+    for (int part = first; part < last; ++part) {
+        const int end = min(n4, (part + 1) * per);               // this part's pieces
+        RowAcc<WANT_Z> acc;
+        acc.init();
+        if (part == 0 && tid < head) { const float v[1] = {row[tid]}; acc.add(v, tid, 0, scale, gap); }
+        int i0 = part * per + tid;
+#pragma unroll 1
+        for (; i0 < end; i0 += RS_BATCH * RS_THREADS) {
+            float v[4 * RS_BATCH];
+            if (i0 + (RS_BATCH - 1) * RS_THREADS < end) {
 #pragma unroll
-        for (int j = 0; j < RS_BATCH; ++j) {
-            const float4 v = r4[i0 + j * RS_THREADS];
-            x[4 * j] = v.x; x[4 * j + 1] = v.y; x[4 * j + 2] = v.z; x[4 * j + 3] = v.w;
+                for (int j = 0; j < RS_BATCH; ++j) {
+                    const float4 u = r4[i0 + j * RS_THREADS];
+                    v[4 * j] = u.x; v[4 * j + 1] = u.y; v[4 * j + 2] = u.z; v[4 * j + 3] = u.w;
+                }
+            } else {                                             // the last pieces, all in flight too (two at a time: a part of 8016 pieces took 1.5 times as long)
+#pragma unroll
+                for (int j = 0; j < RS_BATCH; ++j) {
+                    const float4 u = i0 + j * RS_THREADS < end ? r4[i0 + j * RS_THREADS] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+                    v[4 * j] = u.x; v[4 * j + 1] = u.y; v[4 * j + 2] = u.z; v[4 * j + 3] = u.w;
+                }
+            }
+            acc.add(v, head + 4 * i0, 4 * RS_THREADS, scale, gap);
         }
-        acc.add(x, head + 4 * i0, 4 * RS_THREADS, scale, gap);
+        if (part == un.parts - 1 && tid < tail) { const float v[1] = {row[V - tail + tid]}; acc.add(v, V - tail + tid, 0, scale, gap); }
+        const MaxIdx best = warp_argmax(acc.best);
+        float z = 0.f;
+        if (WANT_Z) z = warp_sum(acc.ref == -INFINITY ? 0.f : acc.s * exp_scaled(acc.ref - best.v, scale));
+        if (lane == 0) { sh_m[part][warp] = best; sh_z[part][warp] = z; }
     }
-#pragma unroll 1
-    for (; i0 < n4; i0 += 2 * RS_THREADS) {
-        const bool two = i0 + RS_THREADS < n4;
-        const float4 v = r4[i0], w = two ? r4[i0 + RS_THREADS] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-        const float x[8] = {v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w};
-        acc.add(x, head + 4 * i0, 4 * RS_THREADS, scale, gap);
-    }
-    if ((int)threadIdx.x < tail) { const float x[1] = {row[V - tail + threadIdx.x]}; acc.add(x, V - tail + threadIdx.x, 0, scale, gap); }
-    const MaxIdx best = block_argmax(acc.best, shm);
-    float z = 0.f;
-    if (WANT_Z) z = block_sum(acc.ref == -INFINITY ? 0.f : acc.s * exp_scaled(acc.ref - best.v, scale), sh);
-    if (threadIdx.x == 0) {
-        const size_t o = ((size_t)b * KINDS + kind) * RS_STRIDE + r;
+    __syncthreads();
+    if (warp >= last - first) return;
+    const int part = first + warp;                               // a warp per part
+    const MaxIdx mine = lane < WARPS ? sh_m[part][lane] : no_idx(), best = warp_argmax(mine);
+    const float z = WANT_Z ? warp_sum(mine.v == -INFINITY ? 0.f : sh_z[part][lane & (WARPS - 1)] * exp_scaled(mine.v - best.v, scale)) : 0.f;
+    if (lane == 0) {
+        const size_t o = (((size_t)b * KINDS + kind) * RS_STRIDE + r) * un.parts + part;
         rs.mx[o] = best.v;
-        rs.arg[o] = best.i == 0x7fffffff ? 0 : best.i;
+        rs.arg[o] = best.i;
         rs.z[o] = z;
     }
 }
@@ -235,6 +254,7 @@ row_stats_kernel(RowStats rs, RowPtrs src, int R, int M, int V, ExpScale scale, 
 // ---- accept kernel ----------------------------------------------------------------------------
 struct AcceptArgs {
     RowStats rs;
+    int parts;                               // of a row's statistics
     const float *judges[KINDS];              // [1..n_judges]: each judge's logits [B, M, V], weakest first, q last
     const float *drafter;                    // [B, R, V]
     float *fold;                             // [B, KINDS, V]: numerators with the rejections folded in, each thread's own
@@ -385,7 +405,19 @@ accept_kernel(AcceptArgs a) {
     const size_t st0 = (size_t)b * KINDS * RS_STRIDE;
     for (int e = tid; e < (J + 1) * RS_STRIDE; e += ACC_THREADS) {
         const int k = e / RS_STRIDE, r = e - k * RS_STRIDE;
-        if (r < (k == 0 ? a.R : M)) { w.mx[k][r] = a.rs.mx[st0 + e]; w.z[k][r] = a.rs.z[st0 + e]; w.arg[k][r] = a.rs.arg[st0 + e]; }
+        if (r >= (k == 0 ? a.R : M)) continue;
+        MaxIdx best = no_idx(), m[ROW_STAT_PARTS];
+        float z[ROW_STAT_PARTS], sum = 0.f;
+#pragma unroll
+        for (int i = 0; i < ROW_STAT_PARTS; ++i) {
+            const size_t o = (st0 + e) * a.parts + min(i, a.parts - 1);
+            m[i].v = a.rs.mx[o]; m[i].i = a.rs.arg[o]; z[i] = a.rs.z[o];
+        }
+#pragma unroll
+        for (int i = 0; i < ROW_STAT_PARTS; ++i) if (i < a.parts) best = better(best, m[i]);
+#pragma unroll
+        for (int i = 0; i < ROW_STAT_PARTS; ++i) if (i < a.parts && m[i].v != -INFINITY) sum += z[i] * exp_scaled(m[i].v - best.v, a.scale);
+        w.mx[k][r] = best.v; w.z[k][r] = sum; w.arg[k][r] = best.i == 0x7fffffff ? 0 : best.i;
     }
     for (int r = tid; r < M; r += ACC_THREADS) w.first_child[r] = a.tree[b].first_child[r];
     __syncthreads();
@@ -695,15 +727,20 @@ int launch_accept(const viasd_model *m, const viasd_draft *d, const viasd_params
     AcceptArgs a;
     {
         float *base = m->ws.accept_scratch;
-        const size_t n = (size_t)m->cfg.max_batch * KINDS * RS_STRIDE;
+        const size_t n = (size_t)m->cfg.max_batch * KINDS * RS_STRIDE * ROW_STAT_PARTS;
+        a.parts = row_parts(m->cfg.vocab);
         a.rs.mx = base; a.rs.arg = reinterpret_cast<int *>(base + n); a.rs.z = base + 2 * n;
-        const int M = d->n_nodes + 1, rows = M > d->n_prows ? M : d->n_prows;
         RowPtrs src;
         src.p[0] = p->mode == 1 || (do_tier && p->conf_source == 0) ? d->drafter_logits : nullptr;
-        for (int k = 1; k < KINDS; ++k) src.p[k] = k <= js.n ? js.logits[k - 1] : nullptr;
+        int judges = 0;
+        for (int k = 1; k < KINDS; ++k) src.p[k] = nullptr;
+        for (int k = 1; k <= js.n; ++k) if (js.logits[k - 1]) { src.p[k] = js.logits[k - 1]; judges = k; }   // (those of a probe come without q)
+        RowUnits un{d->batch, src.p[0] ? d->n_prows : 0, d->n_nodes + 1, 0, a.parts};
+        const int rows = un.B * (un.R + un.M * judges), turn = 2 * m->sm_count;
+        un.whole = a.parts > 1 ? rows / turn * turn : rows;
         auto kernel = p->mode == 1 ? row_stats_kernel<true> : row_stats_kernel<false>;
         const float temperature = p->mode == 1 ? p->temperature : 1.f;
-        CUDA_TRY(launch_chained(kernel, dim3(rows, d->batch, js.n + 1), RS_THREADS, st, a.rs, src, d->n_prows, M, m->cfg.vocab,
+        CUDA_TRY(launch_chained(kernel, un.whole + (rows - un.whole) * a.parts, RS_THREADS, st, a.rs, src, un, m->cfg.vocab,
             exp_scale(temperature), RS_GAP * temperature, m->ws.stats, do_tier ? 1 : 0, tree_ready ? nullptr : m->ws.tree, d->parent, d->per_sequence));
         LAUNCH_CHECK();
     }
