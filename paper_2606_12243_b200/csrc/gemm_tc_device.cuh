@@ -88,11 +88,25 @@ __device__ __forceinline__ void finish_row(const TcParams &p, int tile, int row,
     }
     if (EPI == EPI_SWIGLU) {
         if (HALVES) {
-            u.x = __shfl_down_sync(0xffffffffu, v.x, 16); u.y = __shfl_down_sync(0xffffffffu, v.y, 16);
-            u.z = __shfl_down_sync(0xffffffffu, v.z, 16); u.w = __shfl_down_sync(0xffffffffu, v.w, 16);
+            // lanes 0..15 have four gate features each, lanes 16..31 the matching up features: they trade two, so that every lane has
+            // two of both (with lanes 0..15 doing all four: 8B batch 4 6505 us, now 6470;
+            // prompt chunk 24.71 ms, now 24.30)
+            const bool low = lane < 16;
+            const float r0 = __shfl_xor_sync(0xffffffffu, low ? v.z : v.x, 16), r1 = __shfl_xor_sync(0xffffffffu, low ? v.w : v.y, 16);
+            const float g0 = low ? v.x : r0, g1 = low ? v.y : r1, u0 = low ? r0 : v.z, u1 = low ? r1 : v.w;
+            const int n = tile * 64 + 4 * (lane & 15) + (low ? 0 : 2);
+            if (n < p.seg_n[0]) {                                          // (d_ff is a multiple of 8)
+                const float y0 = g0 / (1.f + __expf(-g0)) * u0, y1 = g1 / (1.f + __expf(-g1)) * u1;
+                const __nv_bfloat16 h0 = __float2bfloat16_rn(y0), h1 = __float2bfloat16_rn(y1);
+                const __nv_bfloat162 l = __floats2bfloat162_rn(y0 - __bfloat162float(h0), y1 - __bfloat162float(h1));
+                __nv_bfloat16 *dst = p.out_act + (size_t)grow * p.ld_out + n;
+                put(live, dst, (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16));
+                put(live, dst + p.act_plane, *reinterpret_cast<const uint32_t *>(&l));
+            }
+            return;
         }
-        const int n = tile * (HALVES ? 64 : TILE_F) + 4 * lane;
-        if ((!HALVES || lane < 16) && n < p.seg_n[0]) {                    // (d_ff is a multiple of 8)
+        const int n = tile * TILE_F + 4 * lane;
+        if (n < p.seg_n[0]) {
             const float4 y = make_float4(v.x / (1.f + __expf(-v.x)) * u.x, v.y / (1.f + __expf(-v.y)) * u.y,
                                          v.z / (1.f + __expf(-v.z)) * u.z, v.w / (1.f + __expf(-v.w)) * u.w);
             store_pair4(live, p.out_act + (size_t)grow * p.ld_out + n, p.act_plane, y);
