@@ -754,24 +754,24 @@ int viasd_gemm(const void *x, const void *w, float *y, int rows, int n, int k, i
     int rc;
     const uint32_t wbox = tc_box_rows(n, 128);
     if ((rc = tc_make_map(&mw, w, n, k, wbox))) return rc;
-    for (int row0 = 0; row0 < rows; row0 += 128) {
-        const int nr = rows - row0 < 128 ? rows - row0 : 128;
-        const int nt = tc_pick_nt(nr, false);
-        const uint32_t xbox = tc_box_rows(rows, nt);
-        if ((rc = tc_make_map(&mx, x, rows, k, xbox))) return rc;
-        TcLaunch L;
-        memset(&L, 0, sizeof(L));
-        L.map_w[0] = &mw; L.seg_n[0] = n; L.w_box_rows[0] = wbox; L.n_seg = 1;
-        L.map_x = &mx; L.x_box_rows = xbox; L.has_lo = 0; L.lo_row_offset = 0;
-        L.rows = nr; L.row0 = row0; L.k = k; L.nt = nt; L.epi = EPI_STORE;
-        L.out_f32 = y; L.ld_out = n;
-        L.counters = (int *)scratch;
-        L.scratch = (float *)((char *)scratch + counter_bytes);
-        L.status = (int *)scratch + tc_tiles(n);                    // no handle here: an expired wait is recorded there
-        L.sm_count = sms;
-        if ((rc = launch_gemm_tc(L, st))) return rc;
-    }
-    return VIASD_OK;
+    // One launch whatever the rows (at most 256): without a lo plane 256 token columns fit the MMA, and two accumulators of them
+    // TMEM.  (Two launches of up to 128 rows streamed the weights twice: us, two / one, 129 x 4096 x 4096 27.1 / 19.6, 200 x 13824 x 5120
+    // 70.3 / 48.3, 256 x 28672 x 4096 113 / 81, 130 x 128000 x 2048 202 / 123, 256 x 512 x 16384 28.8 / 19.2, 160 x 320 x 512 17.4 / 17.5.)  A slot of 256 rows for each of MAX_SMS CTAs is what the
+    // scratch has for 128 rows and twice as many.
+    const int nt = rows > 128 ? (rows + 15) / 16 * 16 : tc_pick_nt(rows, false);
+    const uint32_t xbox = tc_box_rows(rows, nt);
+    if ((rc = tc_make_map(&mx, x, rows, k, xbox))) return rc;
+    TcLaunch L;
+    memset(&L, 0, sizeof(L));
+    L.map_w[0] = &mw; L.seg_n[0] = n; L.w_box_rows[0] = wbox; L.n_seg = 1;
+    L.map_x = &mx; L.x_box_rows = xbox; L.has_lo = 0; L.lo_row_offset = 0;
+    L.rows = rows; L.row0 = 0; L.k = k; L.nt = nt; L.epi = EPI_STORE;
+    L.out_f32 = y; L.ld_out = n;
+    L.counters = (int *)scratch;
+    L.scratch = (float *)((char *)scratch + counter_bytes);
+    L.status = (int *)scratch + tc_tiles(n);                        // no handle here: an expired wait is recorded there
+    L.sm_count = sms;
+    return launch_gemm_tc(L, st);
 }
 
 // What the last viasd_gemm call that used this scratch recorded (n as in that call): VIASD_OK, or VIASD_EDEVICE when

@@ -94,6 +94,12 @@ def test_gemm_around_the_split(rows, n, k):
     test_gemm_matches_matmul("bf16", rows, n, k)
 
 
+# bf16 products of more than 128 rows: one launch, the token tile a multiple of 16 up to 256; whole tiles and split ones
+@pytest.mark.parametrize("rows,n,k", [(128, 520, 1032), (129, 520, 1032), (192, 448, 688), (200, 20000, 776), (241, 4104, 2056), (256, 13824, 640), (256, 129, 4104)])
+def test_gemm_of_many_rows(rows, n, k):
+    test_gemm_matches_matmul("bf16", rows, n, k)
+
+
 # ---------------------------------------------------------------------------------------------
 # forward passes
 # ---------------------------------------------------------------------------------------------
