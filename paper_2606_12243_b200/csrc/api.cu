@@ -301,8 +301,9 @@ int forward(viasd_model *m, const viasd_cache *cache, const viasd_draft *d, bool
     int rc;
     if ((rc = check_draft(m, d)) || (rc = check_cache(cache))) return rc;
     if (!logits) return VIASD_EINVAL;
-    if (small_pass_takes(m, cache, d->batch, d->n_nodes + 1))
-        return timed(m, VIASD_T_GEMM, st, [&] { return launch_small_pass(m, cache, d, slim ? 1 : 0, 0, logits, logits, st); });
+    if (small_pass_takes(m, cache, d->batch, d->n_nodes + 1) &&
+        (rc = timed(m, VIASD_T_GEMM, st, [&] { return launch_small_pass(m, cache, d, slim ? 1 : 0, 0, logits, logits, st); })) != SMALL_PASS_NO_ROOM)
+        return rc;
     if (m->fused) return forward_sweep(m, cache, d, slim ? 1 : 0, slim ? nullptr : logits, slim ? logits : nullptr, st);
     const viasd_config &c = m->cfg;
     const int B = d->batch, M = d->n_nodes + 1, rows = B * M;
@@ -590,12 +591,12 @@ static int verify_step_routed(viasd_model *m, viasd_cache *cache, const viasd_dr
     if ((rc = timed(m, VIASD_T_TIER_ACCEPT, st, [&] { return launch_accept(m, draft, params, probe_set, result, true,
                                                                       false, st, &probe); }))) return rc;
     m->run_flag = flag;
+    rc = SMALL_PASS_NO_ROOM;
     if (small_pass_takes(m, cache, draft->batch, M + G)) {
         rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_prep_replay(m, cache, draft, G, st); });
         if (!rc) rc = timed(m, VIASD_T_GEMM, st, [&] { return launch_small_pass(m, cache, draft, 0, G, full_logits, nullptr, st); });
-    } else {
-        rc = forward_sweep(m, cache, draft, 0, full_logits, nullptr, st, G);
     }
+    if (rc == SMALL_PASS_NO_ROOM) rc = forward_sweep(m, cache, draft, 0, full_logits, nullptr, st, G);
     m->run_flag = nullptr;
     if (rc) return rc;
     if ((rc = tier_accept_impl(m, draft, params, slim_logits, full_logits, 2, result, false, stream))) return rc;
@@ -615,11 +616,15 @@ int viasd_verify_step(viasd_model *m, viasd_cache *cache, const viasd_draft *dra
     // that a sweep would stream every routed layer twice anyway, and the passes run one after the other.
     const int block_rows = draft->batch * (draft->n_nodes + 1);
     const int dual_max = m->opt.dual_max_rows >= 0 ? m->opt.dual_max_rows : block_rows >= TC_WIDE_MIN_ROWS ? TC_WIDE_ROWS : 128;
-    const bool small = small_pass_takes(m, cache, draft->batch, draft->n_nodes + 1);
-    if (small ? m->opt.dual_max_rows < 0 || 2 * block_rows <= dual_max : m->fused && 2 * block_rows <= dual_max) {
+    const bool small = small_pass_takes(m, cache, draft->batch, draft->n_nodes + 1), one_sweep = m->fused && 2 * block_rows <= dual_max;
+    if (small ? m->opt.dual_max_rows < 0 || 2 * block_rows <= dual_max : one_sweep) {
         cudaStream_t st = (cudaStream_t)stream;
+        rc = SMALL_PASS_NO_ROOM;
         if (small) rc = timed(m, VIASD_T_GEMM, st, [&] { return launch_small_pass(m, cache, draft, 2, 0, full_logits, slim_logits, st); });
-        else rc = forward_sweep(m, cache, draft, 2, full_logits, slim_logits, st);
+        if (rc == SMALL_PASS_NO_ROOM) {
+            if (one_sweep) rc = forward_sweep(m, cache, draft, 2, full_logits, slim_logits, st);
+            else if (!(rc = forward(m, cache, draft, true, slim_logits, st))) rc = forward(m, cache, draft, false, full_logits, st);
+        }
         if (rc) return rc;
         if ((rc = tier_accept_impl(m, draft, params, slim_logits, full_logits, 3, result, true, stream))) return rc;
         return viasd_kv_commit(m, cache, draft, result, stream);

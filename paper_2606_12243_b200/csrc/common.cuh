@@ -241,6 +241,7 @@ constexpr int SMALL_PASS_MAX_LAYERS = 24, SMALL_PASS_MAX_ROWS = 64;      // rows
 inline size_t small_pass_counters(int max_batch, int n_heads) {         // two barriers; an attention item has 16 query rows of a kv head
     return 2 + (size_t)2 * max_batch * n_heads * (VIASD_MAX_ROWS_PER_SEQ / 16);
 }
+constexpr int SMALL_PASS_NO_ROOM = 1;
 bool small_pass_takes(const viasd_model *m, const viasd_cache *cache, int batch, int M);
 int launch_small_pass(viasd_model *m, const viasd_cache *cache, const viasd_draft *d, int mode, int replay, float *logits_full,
                       float *logits_slim, cudaStream_t st);

@@ -905,7 +905,12 @@ int launch(SpArgs &a, const viasd_config &c, int rows, int grid, cudaStream_t st
     attr[0].id = cudaLaunchAttributeCooperative;                // the CTAs wait for one another: all of them are resident, or none is
     attr[0].val.cooperative = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    CUDA_TRY(cudaLaunchKernelEx(&cfg, small_pass_kernel<T, HD, MT>, a));
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, small_pass_kernel<T, HD, MT>, a);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {               // (a context with a share of the SMs only)
+        (void)cudaGetLastError();
+        return SMALL_PASS_NO_ROOM;
+    }
+    CUDA_TRY(e);
     LAUNCH_CHECK();
     return VIASD_OK;
 }
@@ -1024,7 +1029,8 @@ static int launch_group(viasd_model *m, const viasd_cache *cache, const viasd_dr
 #undef SP_LAUNCH
 }
 
-// A pass that small_pass_takes.  More sequences than a launch holds (fp32) go in groups, as many of them in each as fit with both
+// A pass that small_pass_takes; SMALL_PASS_NO_ROOM if the device does not hold its CTAs at once (nothing has been launched then, and
+// it goes launch by launch).  More sequences than a launch holds (fp32) go in groups, as many of them in each as fit with both
 // verifiers' rows, or else with one's.
 int launch_small_pass(viasd_model *m, const viasd_cache *cache, const viasd_draft *d, int mode, int replay, float *logits_full,
                       float *logits_slim, cudaStream_t st) {
