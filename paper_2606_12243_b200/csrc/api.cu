@@ -68,7 +68,7 @@ size_t carve(const viasd_config &c, char *base, Workspace *ws) {
         w.a_head = cv.take<void>(R * c.d_model * 4);
         w.ssq_head = cv.take<float>((size_t)(c.d_model / 128 + 1) * 4 * R * 4);
         w.attn_counters = cv.take<int>(attn_counter_count(c.max_batch, c.n_heads, c.n_kv_heads) * sizeof(int));
-        w.pass_counters = cv.take<int>(small_pass_counters(c.max_batch, c.n_heads) * sizeof(int));
+        w.pass_counters = cv.take<int>(small_pass_counters(c) * sizeof(int));
         w.n_counters = widest / 64 + 8;                      // (a tile of the pair kernel's gate/up launch has 64 features)
         w.gemm_counters = cv.take<int>(w.n_counters * 4);
     }
@@ -465,7 +465,7 @@ int viasd_init_model(const viasd_config *cfg, const viasd_weights *w, const unsi
     cudaError_t e = cudaMemset(m->ws.stats, 0, sizeof(DeviceStats));
     if (e == cudaSuccess) { const int one = 1; e = cudaMemcpy(&m->ws.stats->full_ran, &one, sizeof(int), cudaMemcpyHostToDevice); }
     if (e == cudaSuccess) e = cudaMemset(m->ws.gemm_counters, 0, m->ws.n_counters * 4);
-    if (e == cudaSuccess) e = cudaMemset(m->ws.pass_counters, 0, small_pass_counters(cfg->max_batch, cfg->n_heads) * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(m->ws.pass_counters, 0, small_pass_counters(*cfg) * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(m->ws.attn_counters, 0, attn_counter_count(cfg->max_batch, cfg->n_heads, cfg->n_kv_heads) * sizeof(int));
     if (e == cudaSuccess) { rc = launch_rope_table(m, 0); if (rc == VIASD_OK) e = cudaDeviceSynchronize(); }
     if (e != cudaSuccess) { g_last_cuda_error = (int)e; rc = VIASD_ECUDA; }

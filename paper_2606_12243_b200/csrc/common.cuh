@@ -64,7 +64,7 @@ struct Workspace {                      // pointers into the caller's workspace 
     int *gemm_counters;                 // per-tile arrival counters, zero between launches
     size_t n_counters;
     int *attn_counters;                 // [attn_counter_count()] key-range arrivals per (stream, sequence, kv head, group of query heads)
-    int *pass_counters;                 // [small_pass_counters()] arrivals of a pass in one launch, zero between launches
+    int *pass_counters;                 // [small_pass_counters()] arrivals of a pass in one launch
     float *ssq;                         // [(d / 128) * 4][R] partial sums of h^2 for the fused RMSNorm
     void *a_head; float *ssq_head;      // the block's own rows of `a` and `ssq`, compacted for the output head after a replay pass
 };
@@ -238,9 +238,16 @@ int launch_gemm_rowwarp(const void *x, size_t x_plane, const GemmSegs &segs, int
 
 // small_pass.cu -- a small model's forward pass in one launch
 constexpr int SMALL_PASS_MAX_LAYERS = 24, SMALL_PASS_MAX_ROWS = 64;      // rows: of both verifiers together
-inline size_t small_pass_counters(int max_batch, int n_heads) {         // two barriers; an attention item has 16 query rows of a kv head
-    return 2 + (size_t)2 * max_batch * n_heads * (VIASD_MAX_ROWS_PER_SEQ / 16);
+// Arrival counters of a launch, whole lines: two barriers, then a word per attention pair (16 query rows of a kv head, of which a
+// launch's rows make no more than this).  There are two such sets behind a line whose first word says which one the next launch
+// uses (Pass::hand_over).
+constexpr int SMALL_PASS_LINE = 32;
+inline int small_pass_set(const viasd_config &c) {
+    const int most = c.n_heads * (SMALL_PASS_MAX_ROWS / 16) + c.n_kv_heads * SMALL_PASS_MAX_ROWS;
+    const long long all = 2ll * c.max_batch * c.n_heads * (VIASD_MAX_ROWS_PER_SEQ / 16);
+    return (2 + (int)(all < most ? all : most) + SMALL_PASS_LINE - 1) / SMALL_PASS_LINE * SMALL_PASS_LINE;
 }
+inline size_t small_pass_counters(const viasd_config &c) { return SMALL_PASS_LINE + (size_t)2 * small_pass_set(c); }
 constexpr int SMALL_PASS_NO_ROOM = 1;
 bool small_pass_takes(const viasd_model *m, const viasd_cache *cache, int batch, int M);
 int launch_small_pass(viasd_model *m, const viasd_cache *cache, const viasd_draft *d, int mode, int replay, float *logits_full,

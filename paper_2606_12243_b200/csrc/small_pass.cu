@@ -61,7 +61,8 @@ struct SpArgs {
     int *len_eff;
     DeviceStats *stats;
     const int *run_flag;
-    int *barrier, *pairs;                       // two arrival counters, used in turn; arrivals of each attention pair's ranges; zero between launches
+    int *counters;                              // which set; the two sets: barriers, used in turn, and arrivals of each attention pair's ranges
+    int set_words;
     int red_bytes, w_bytes, x_bytes;            // shared memory: sums; a stage's weights; a warp's staged activations,
     int x_groups, x_rows;                       // that many groups of k (bf16) of that many rows (fp32: all groups) at a time
     SpLayer layer[SMALL_PASS_MAX_LAYERS];
@@ -146,7 +147,8 @@ struct Pass {
         int tok[SP_ROWS], pos[SP_ROWS], slot[SP_ROWS], n_ctx[SP_ROWS], seq[SP_ROWS];
         TreeInfo tree[SP_WARPS];
         int par[SP_WARPS][VIASD_MAX_ROWS_PER_SEQ];
-        int abort_flag, last;
+        int *counters;                                          // this launch's set
+        int n_bar, abort_flag, last;
     };
     struct Range { int pair, s, b, kvh, row0, rows, split, n, k0, k1; };
 
@@ -157,10 +159,9 @@ struct Pass {
     uint8_t *xbuf;                                              // this warp's staged activations, in one place with
     uint8_t *kvbuf;                                             // two K/V tiles: no stage uses both
     const int tid, warp, lane, g, c;
-    int n_bar;
 
     __device__ Pass(const SpArgs &a_, uint8_t *smem) : a(a_), sh(*reinterpret_cast<Shared *>(smem)), tid(threadIdx.x), warp(threadIdx.x >> 5),
-        lane(threadIdx.x & 31), g((threadIdx.x & 31) >> 2), c(threadIdx.x & 3), n_bar(0) {
+        lane(threadIdx.x & 31), g((threadIdx.x & 31) >> 2), c(threadIdx.x & 3) {
         red = reinterpret_cast<float *>(smem + (sizeof(Shared) + 127) / 128 * 128);
         wbuf = reinterpret_cast<uint8_t *>(red) + a.red_bytes;
         kvbuf = wbuf + a.w_bytes;
@@ -215,14 +216,23 @@ struct Pass {
     // All CTAs have arrived, and what they stored before is seen behind this; `meanwhile` runs between arrival and wait.  (A ninth
     // warp for the barriers, so that no warp's prefetch waits behind the release: 168 registers for all, mini 121 -> 127 us.)
     template <typename F> __device__ __forceinline__ void barrier(F meanwhile) {
-        int *ctr = a.barrier + (n_bar & 1);
         __syncthreads();
         // (a counter is used again two barriers later: by then every CTA has acknowledged its last use)
-        if (tid == 0) counter_arrive(ctr, gridDim.x, gridDim.x);
+        if (tid == 0) counter_arrive(sh.counters + (sh.n_bar & 1), gridDim.x, gridDim.x);
         meanwhile();
-        if (tid == 0) counter_wait(ctr, gridDim.x, gridDim.x, &sh.abort_flag, &a.stats->device_status);
-        ++n_bar;
+        if (tid == 0) counter_wait(sh.counters + (sh.n_bar++ & 1), gridDim.x, gridDim.x, &sh.abort_flag, &a.stats->device_status);
         __syncthreads();
+    }
+
+    // Behind a barrier, so that all CTAs know their set: the other one, which the launch before this one used, becomes the
+    // next launch's, from zero.  Counters come back to zero by themselves, also when a wait expires; one that is off all the same
+    // (a launch that was cut short, a stray write) costs one launch its results, not the handle.  (Cleared at a launch's head they
+    // would meet arrivals of CTAs that are further on, and by a kernel in front of it every pass would pay a launch.)
+    __device__ __forceinline__ void hand_over() {
+        if (blockIdx.x) return;
+        const int next = sh.counters == a.counters + SMALL_PASS_LINE ? 1 : 0;
+        for (int i = tid; i < a.set_words; i += SP_THREADS) a.counters[SMALL_PASS_LINE + next * a.set_words + i] = 0;
+        if (tid == 0) a.counters[0] = next;
     }
 
     // ---- the input of k-groups i0 .. i0 + n - 1 of this warp, rows r_lo .. r_lo + r_n - 1, to shared memory ----
@@ -738,7 +748,7 @@ struct Pass {
             __syncthreads();
             if (tid == 0) {
                 unsigned old;
-                asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(old) : "l"(a.pairs + it.pair), "r"(a.nsplit - 1) : "memory");
+                asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(old) : "l"(sh.counters + 2 + it.pair), "r"(a.nsplit - 1) : "memory");
                 sh.last = old == (unsigned)a.nsplit - 1;
             }
             __syncthreads();
@@ -779,7 +789,7 @@ struct Pass {
 
     // ---- what the pass needs of the draft: every CTA for itself, CTA 0 also for the kernels behind this one ----
     __device__ __forceinline__ void prepare() {
-        if (tid == 0) sh.abort_flag = 0;
+        if (tid == SP_THREADS - 1) { sh.n_bar = sh.abort_flag = 0; sh.counters = a.counters + SMALL_PASS_LINE + (__ldcg(a.counters) & 1) * a.set_words; }
         if (a.row_tok) {                                        // a replay pass: its preparation has run
             for (int r = tid; r < a.R; r += SP_THREADS) {
                 const int b = r / a.M, i = r - b * a.M, n = a.len_eff[b], at = n + i;
@@ -843,6 +853,7 @@ struct Pass {
             project<ST_DOWN>(li, rows);
             barrier([&] { if (li + 1 < a.n_layers) prefetch<ST_QKV>(sh.layer[li + 1]); else prefetch<ST_HEAD>(l); });
         }
+        hand_over();
         project<ST_HEAD>(a.n_layers, a.streams * a.R);
     }
 };
@@ -990,7 +1001,7 @@ static int launch_group(viasd_model *m, const viasd_cache *cache, const viasd_dr
     a.row_tok = replay ? m->ws.row_tok + (size_t)b0 * a.M : nullptr; a.kv_keep = replay ? cache->len_full + b0 : nullptr;
     a.full_pass = mode != 1;
     a.tree = m->ws.tree + b0; a.len_eff = m->ws.len_eff + b0; a.stats = m->ws.stats; a.run_flag = m->run_flag;
-    a.barrier = m->ws.pass_counters; a.pairs = m->ws.pass_counters + 2;
+    a.counters = m->ws.pass_counters; a.set_words = small_pass_set(c);
     a.first[0] = 0; a.first[1] = -1;
     for (int l = 0; l < c.n_layers; ++l) {
         int so = -1;

@@ -96,6 +96,44 @@ def test_expired_wait_leaves_a_usable_handle(name, batch):
     assert torch.equal(want, got) and int(counters.abs().max()) == 0
 
 
+@pytest.mark.parametrize("word", [0, 1, 2])
+@pytest.mark.parametrize("name", ["c1_tiny", "mini_7b"])
+def test_wrong_counter_of_a_pass_in_one_launch_costs_one_pass(name, word):
+    """The same for a small model's pass in one launch: a barrier's counter is off (its wait gives up, the status says so), or an
+    attention pair's (nobody merges that pair, or too early); the next pass, and the one behind it, compute what the first did."""
+    vb = _vb()
+    wl = W.get(name)
+    eng = _engine(wl)
+    out = eng.logits_buffer()
+
+    def run():
+        n0 = vb.launch_count()
+        vb.full_forward(eng.model, eng.cache, eng.draft, out)
+        torch.cuda.synchronize()
+        assert vb.launch_count() - n0 == 1
+        return out.clone()
+
+    want = run()
+    # in front of the workspace's last piece: a line that says which set is next, and two sets of whole lines
+    s, line = wl.shape, 32
+    words = 2 + min(2 * wl.batch * s.n_heads * 4, s.n_heads * 4 + s.n_kv_heads * 64)
+    words = -(-words // line) * line
+    last = 4 * (max(s.vocab, s.n_heads * s.head_dim + 2 * s.n_kv_heads * s.head_dim, s.d_ff) // 64 + 8)
+    n = 4 * (line + 2 * words)
+    at = eng.workspace.numel() - (last + 255) // 256 * 256 - (n + 255) // 256 * 256
+    counters = eng.workspace[at:at + n].view(torch.int32)
+    which = int(counters[0])
+    assert which in (0, 1) and int(counters[1:].abs().max()) == 0
+    counters[line + which * words + word] = 1 << 20            # the first arrival wraps it: one is missing
+    bad = run()
+    if word < 2:
+        assert vb.get_stats(eng.model).device_status == vb.VIASD_EDEVICE
+    else:
+        assert not torch.equal(bad, want)
+    for _ in range(2):
+        assert torch.equal(run(), want) and int(counters[1:].abs().max()) == 0
+
+
 # ---------------------------------------------------------------------------------------------
 # a node whose gate row does not exist
 # ---------------------------------------------------------------------------------------------
