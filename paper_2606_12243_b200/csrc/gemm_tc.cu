@@ -1,9 +1,9 @@
 // Weight-streaming bf16 GEMM on the 5th-generation tensor cores (tcgen05 + TMEM), fed by TMA.
 //
-//   y[rows, n] = x[rows, k] * W[n, k]^T        rows <= 128 per launch, W streamed once from HBM
+//   y[rows, n] = x[rows, k] * W[n, k]^T        W streamed once from HBM; rows <= 128 per launch, 256 of a plain product of one plane
 //
 // The operands are swapped: a tile of 128 output features is the MMA's M dimension (A operand, the
-// weights), the token rows are its N dimension (B operand, 16..128 wide).  Both are K-major in shared
+// weights), the token rows are its N dimension (B operand, 16..256 wide).  Both are K-major in shared
 // memory with the 128-byte swizzle, exactly as a 2-D TMA box of 64 bf16 x rows lands there.  The
 // activation comes as two bf16 planes hi + lo (x = hi + lo to ~16 mantissa bits); each weight tile is
 // multiplied with both, which costs tensor time the kernel has in abundance and no extra weight traffic.
@@ -568,6 +568,9 @@ int launch_clear_words(int *words, int n, cudaStream_t st) {
 }
 
 int launch_gemm_tc(const TcLaunch &L, cudaStream_t st) {
+    // the norm's factors and the rotary positions have a place per row up to 128, and two planes of more are no MMA's columns
+    const int most = L.has_lo || L.ssq_in || L.epi != EPI_STORE ? 128 : 256;
+    if (L.rows < 1 || L.rows > L.nt || L.nt > most) return VIASD_EINVAL;
     TcParams p;
     tc_fill_params(L, p);
     const bool dual = L.epi == EPI_SWIGLU;

@@ -66,3 +66,34 @@ def test_struct_layouts_match_header():
         sizes = [int(x) for x in subprocess.check_output([exe]).split()]
     mirrors = [vb.Config, vb.Weights, vb.Cache, vb.Draft, vb.Params, vb.Result, vb.Stats]
     assert sizes == [ctypes.sizeof(m) for m in mirrors]
+
+
+def test_gemm_of_more_than_128_rows_takes_nothing_per_row(lib, tmp_path):
+    """The one-CTA GEMM takes up to 256 rows of a plain product; what keeps something per row (norm factors, rotary positions), or
+    a second plane, ends at 128 and is refused above (before anything of the launch is looked at)."""
+    import subprocess
+    src = tmp_path / "t.cpp"
+    src.write_text("""
+        #include <cuda_runtime.h>
+        #include "gemm_tc.cuh"
+        extern "C" int call(int (*f)(const TcLaunch &, cudaStream_t), int rows, int nt, int has_lo, int epi, int norm) {
+            static float x[1];
+            TcLaunch L;
+            memset(&L, 0, sizeof(L));
+            L.rows = rows; L.nt = nt; L.has_lo = has_lo; L.epi = epi; L.ssq_in = norm ? x : nullptr; L.n_seg = 1; L.sm_count = 148;
+            return f(L, nullptr);                              // (no columns: a launch that is taken is empty)
+        }""")
+    so = tmp_path / "t.so"
+    subprocess.check_call(["g++", "-std=c++17", "-shared", "-fPIC", "-I/usr/local/cuda/include",
+                           "-I", os.path.join(ROOT, "paper_2606_12243_b200", "csrc"), str(src), "-o", str(so)])
+    call = ctypes.CDLL(str(so)).call
+    launch = ctypes.cast(lib["_Z14launch_gemm_tcRK8TcLaunchP11CUstream_st"], ctypes.c_void_p)
+    store, add, swiglu, add_norm, qkv_rope = range(5)
+    got = lambda *a: call(launch, *a)
+    for rows, nt in ((1, 16), (128, 128)):
+        assert [got(rows, nt, lo, epi, norm) for lo in (0, 1) for epi in range(5) for norm in (0, 1)] == [0] * 20
+    assert got(129, 144, 0, store, 0) == got(256, 256, 0, store, 0) == 0
+    for rows, nt in ((129, 144), (256, 256)):
+        assert [got(rows, nt, 0, epi, 0) for epi in (add, swiglu, add_norm, qkv_rope)] == [-1] * 4
+        assert got(rows, nt, 1, store, 0) == got(rows, nt, 0, store, 1) == -1
+    assert got(257, 272, 0, store, 0) == got(17, 16, 0, store, 0) == got(0, 16, 0, store, 0) == -1
