@@ -216,9 +216,10 @@ struct Pass {
     // All CTAs have arrived, and what they stored before is seen behind this; `meanwhile` runs between arrival and wait.  (A ninth
     // warp for the barriers, so that no warp's prefetch waits behind the release: 168 registers for all, mini 121 -> 127 us.)
     template <typename F> __device__ __forceinline__ void barrier(F meanwhile) {
+        int *ctr = sh.counters + (sh.n_bar & 1);                // (ahead of the barrier: its latency is not the arrival's)
         __syncthreads();
         // (a counter is used again two barriers later: by then every CTA has acknowledged its last use)
-        if (tid == 0) counter_arrive(sh.counters + (sh.n_bar & 1), gridDim.x, gridDim.x);
+        if (tid == 0) counter_arrive(ctr, gridDim.x, gridDim.x);
         meanwhile();
         if (tid == 0) counter_wait(sh.counters + (sh.n_bar++ & 1), gridDim.x, gridDim.x, &sh.abort_flag, &a.stats->device_status);
         __syncthreads();
