@@ -946,14 +946,74 @@ static int launch_rows(const viasd_model *m, int M) {
     return 0;
 }
 
+// How a call's sequences share launches (M: rows of one).  They form groups of n, the last one maybe smaller; a launch has a group of
+// both verifiers' rows, or as many groups of one verifier's as fit.  The cuts of a sequence's key ranges depend on its group's
+// size alone, so that they are the same whatever is launched; a last group that is cut otherwise has launches of its own.
+struct Grouping {
+    int batch, n, per_one;          // groups that a launch of one verifier's rows takes
+    bool fits_both;
+    int pairs;                      // attention pairs of a sequence
+    int part_seqs;                  // sequences of one verifier whose partial rows any launch has, at most
+    int sms, tiles; size_t part_room;
+    // as many ranges as keep the CTAs busy with both verifiers, not more than 64 keys of the cache each make, within the partial buffer
+    int ranges(int b0) const {
+        int ns = sms / (2 * (batch - b0 < n ? batch - b0 : n) * pairs);
+        if (ns > tiles) ns = tiles;
+        if (ns > SP_SPLITS) ns = SP_SPLITS;
+        if ((size_t)ns > part_room) ns = (int)part_room;
+        return ns < 1 ? 1 : ns;
+    }
+    int take(int b0, bool both) const {                             // sequences of the launch that begins with b0
+        const int most = both ? n : per_one * n, left = batch - b0;
+        if (left > most) return most;
+        const int full = left / n * n;
+        return full && full < left && ranges(b0 + full) != ranges(b0) ? full : left;
+    }
+    int launches(bool both) const {
+        int count = 0;
+        for (int b0 = 0; b0 < batch; b0 += take(b0, both)) ++count;
+        return count;
+    }
+};
+static Grouping grouping(const viasd_model *m, int batch, int M, int most) {
+    const viasd_config &c = m->cfg;
+    Grouping g;
+    g.batch = batch;
+    g.fits_both = 2 * M <= most;
+    const int rows = g.fits_both ? 2 * M : M, n = most / rows < batch ? most / rows : batch, groups = (batch + n - 1) / n;
+    // Groups of equal size, or all but the last as large as fits: whichever has fewer eights of rows (6 sequences of 7 rows as 4 + 2, not 3 + 3:
+    // 175 us, else 181), equal ones where that is the same (6 of 6 rows as 3 + 3, not 5 + 1: 224 us, else 264)
+    auto eights = [&](int size) {
+        const int full = batch / size, last = batch - full * size;
+        return full * ((size * rows + 7) / 8) + (last * rows + 7) / 8;
+    };
+    const int even = (batch + groups - 1) / groups;
+    g.n = eights(even) <= eights(n) ? even : n;
+    g.per_one = most / (g.n * M);
+    g.pairs = c.n_kv_heads * ((c.n_heads / c.n_kv_heads * M + SP_QG - 1) / SP_QG);
+    g.part_seqs = g.per_one * g.n < batch ? g.per_one * g.n : batch;
+    if (2 * g.n > g.part_seqs) g.part_seqs = 2 * g.n;
+    g.sms = m->sm_count; g.tiles = (c.max_ctx + 63) / 64;
+    g.part_room = m->ws.part_bytes / ((size_t)g.part_seqs * M * c.n_heads * (c.head_dim + 2) * sizeof(float));
+    return g;
+}
+
 // Which passes go this way.  us, this way / launch by launch (three layers, one of them routed; one step):
 //   fp32, d 256: 5 rows 90 / 177 (context 100), 132 / 335 (4000); 18 rows 136 / 267, 198 / 500; 32 rows 156 / 351, 334 / 635;
-//         four layers, 432 rows in groups 3018 / 4384 (300), 3810 / 4910 (2000); d 768, 9 rows 257 / 503
+//         d 768, 9 rows 257 / 503
 //   bf16, d 512, 4 kv heads: 5 rows 84 / 114 (100), 118 / 131 (4000); 9 rows 96 / 124, 132 / 141; 18 rows 119 / 135, 165 / 152;
 //         28 rows 137 / 143 (100), 148 / 152 (1000), 227 / 177 (4000); 1 kv head: 27 rows 134 / 146, 142 / 157, 171 / 174;
 //         four layers, context 300: d 768, 18 rows 195 / 200, 27 rows 231 / 213; d 1024, 9 rows 189 / 207
-// so fp32 always; bf16 while the rows a CTA reads (rows x the layer's columns of input, 2944 at d 512) and the tiles of keys per CTA
-// are few: then tcgen05 GEMMs and attention overtake it.
+// so fp32 always where one launch holds a verifier's rows (527 drawn shapes: none slower); bf16 while the rows a CTA reads (rows x the
+// layer's columns of input, 2944 at d 512) and the tiles of keys per CTA are few: then tcgen05 GEMMs and attention overtake it.
+// fp32 in several launches: each one more costs a layer's barriers, 17 us, which rows x columns have to win back, and attention by
+// the tile of keys.  Of 1109 drawn calls (d 64 - 1024, 1 - 64 rows per sequence, batch 2 - 64, context 70 - 4000, steps and
+// prompt chunks) 81 are slower in launches, 0.58 times as fast at worst; of the 985 on this side of the line 17 are (0.77), of
+// those on the other 22 would have gained more than a fifth.  Drawn again with groups of equal size: 5 of 516 (0.83), none.
+// d 192, d_ff 2816, 24 x 6 rows, a sequence per launch: 2310 / 1498; d 256, 16 x 27 rows 2738 / 4343 (context 300), 3365 / 4828 (2000);
+// d 768, 16 x 9 rows 1978 / 2305.  Key tiles are counted by the cache's capacity, as the lengths are on the device.
+// A launch has all weights of a stage in shared memory, the output head's too (plan): at 148 SMs fp32 of d 256 up to a vocabulary of
+// 16576, bf16 of d 512 up to 14208, of d 768 up to 9472; beyond that a model goes launch by launch.
 bool small_pass_takes(const viasd_model *m, const viasd_cache *cache, int batch, int M) {
     const viasd_config &c = m->cfg;
     const ModelOptions &o = m->opt;
@@ -963,10 +1023,15 @@ bool small_pass_takes(const viasd_model *m, const viasd_cache *cache, int batch,
     if (c.n_layers > SMALL_PASS_MAX_LAYERS) return false;
     const int most = launch_rows(m, M);
     if (most == 0) return false;
-    if (c.dtype == 1) {
-        const int rows = batch * M, qgroups = (c.n_heads / c.n_kv_heads * M + SP_QG - 1) / SP_QG;
+    const Grouping g = grouping(m, batch, M, most);
+    const long long rows = (long long)batch * M, columns = 2LL * c.d_model + c.n_heads * c.head_dim + c.d_ff;
+    if (c.dtype == 0) {
+        const long long launches = (batch + most / M - 1) / (most / M), seqs = g.take(0, false), ns = g.ranges(0), range = ns * (c.head_dim == 64 ? 64 : 32);
+        const long long tiles = (seqs * g.pairs * ns + m->sm_count - 1) / m->sm_count * ((c.max_ctx + range - 1) / range);   // of a CTA
+        if (launches > 1 && rows * columns < 59000 * (launches - 1) + 800 * launches * tiles * (c.head_dim / 64)) return false;
+    } else {
         if (2 * rows > most) return false;
-        const long long tiles = 2LL * batch * c.n_kv_heads * qgroups * ((c.max_ctx + 63) / 64), columns = 2LL * c.d_model + c.n_heads * c.head_dim + c.d_ff;
+        const long long tiles = 2LL * batch * g.pairs * ((c.max_ctx + 63) / 64);
         if (rows * columns * m->sm_count + 3 * 2944 * tiles > 36LL * 2944 * m->sm_count) return false;
         // (caches that are not aligned are refused by the path with tensor maps over them)
         if (((uintptr_t)cache->k_full | (uintptr_t)cache->v_full | (uintptr_t)cache->k_slim | (uintptr_t)cache->v_slim) & 15) return false;
@@ -976,8 +1041,8 @@ bool small_pass_takes(const viasd_model *m, const viasd_cache *cache, int batch,
 
 // Sequences b0 .. b0 + n - 1 of a pass.  mode 0: full verifier, 1: slim verifier, 2: both; replay: rows in front of every
 // sequence's own (prepared before this call)
-static int launch_group(viasd_model *m, const viasd_cache *cache, const viasd_draft *d, int b0, int n, int mode, int replay, float *logits_full,
-                        float *logits_slim, cudaStream_t st) {
+static int launch_group(viasd_model *m, const viasd_cache *cache, const viasd_draft *d, const Grouping &g, int b0, int n, int mode, int replay,
+                        float *logits_full, float *logits_slim, cudaStream_t st) {
     const viasd_config &c = m->cfg;
     SpArgs a;
     memset(&a, 0, sizeof(a));
@@ -1022,19 +1087,10 @@ static int launch_group(viasd_model *m, const viasd_cache *cache, const viasd_dr
         s.next[1] = m->final_norm;
         for (int j = i + 1; j < a.n_layers; ++j) if (a.layer[j].ord[1] >= 0) { s.next[1] = a.layer[j].n1; break; }
     }
-    // Key ranges: as many as keep the CTAs busy with both streams (the cuts may not depend on how many there are), none shorter than
-    // a tile, within the partial buffer.
-    const int qgroups = (c.n_heads / c.n_kv_heads * a.M + SP_QG - 1) / SP_QG, pairs = a.B * c.n_kv_heads * qgroups;
-    const int tiles = (c.max_ctx + 63) / 64;
-    int ns = m->sm_count / (2 * pairs);
-    if (ns > tiles) ns = tiles;
-    if (ns > SP_SPLITS) ns = SP_SPLITS;
-    const size_t per = (size_t)2 * a.R * c.n_heads * (c.head_dim + 2) * sizeof(float);
-    while (ns > 1 && per * ns > m->ws.part_bytes) --ns;
-    a.nsplit = ns < 1 ? 1 : ns;
-    a.att_items = pairs * a.nsplit;
+    a.nsplit = g.ranges(b0);
+    a.att_items = a.B * g.pairs * a.nsplit;
     a.part = m->ws.part;
-    a.part_ml = reinterpret_cast<float2 *>(m->ws.part + (size_t)2 * a.R * c.n_heads * a.nsplit * c.head_dim);
+    a.part_ml = reinterpret_cast<float2 *>(m->ws.part + (size_t)g.part_seqs * a.M * c.n_heads * a.nsplit * c.head_dim);
     const int rows = a.streams * a.R;
 #define SP_LAUNCH(T, HD, MT) launch<T, HD, MT>(a, c, rows, m->sm_count, st)
     return SP_DISPATCH(m, rows, SP_LAUNCH);
@@ -1042,23 +1098,25 @@ static int launch_group(viasd_model *m, const viasd_cache *cache, const viasd_dr
 }
 
 // A pass that small_pass_takes; SMALL_PASS_NO_ROOM if the device does not hold its CTAs at once (nothing has been launched then, and
-// it goes launch by launch).  More sequences than a launch holds (fp32) go in groups, as many of them in each as fit with both
-// verifiers' rows, or else with one's.
+// it goes launch by launch).  More sequences than a launch holds (fp32) go in groups, as many of them in each as fit: with both
+// verifiers' rows, or with one's where that makes fewer launches times layers.  (Groups of as many as would fit with both, whichever
+// were in the launch, left half of a single verifier's rows empty: 16 prompts' chunks of 17 rows were 32 launches, not 12.)
 int launch_small_pass(viasd_model *m, const viasd_cache *cache, const viasd_draft *d, int mode, int replay, float *logits_full,
                       float *logits_slim, cudaStream_t st) {
-    const int M = d->n_nodes + 1 + replay, most = launch_rows(m, M), both = most / (2 * M), one = most / M;
-    if (one < 1) return VIASD_EINVAL;
-    const bool together = mode == 2 && both > 0;
-    const int n = both > 0 ? both : one;                        // (the same for every mode: a group's key ranges depend on it)
-    for (int b0 = 0; b0 < d->batch; b0 += n) {
-        const int nb = d->batch - b0 < n ? d->batch - b0 : n;
+    const int M = d->n_nodes + 1 + replay, most = launch_rows(m, M);
+    if (most < M) return VIASD_EINVAL;
+    const Grouping g = grouping(m, d->batch, M, most);
+    const bool together = mode == 2 && g.fits_both && g.launches(true) * m->cfg.n_layers <= g.launches(false) * (m->cfg.n_layers + m->n_routed);
+    for (int b0 = 0, nb; b0 < d->batch; b0 += nb) {
+        nb = g.take(b0, together);
+        auto group = [&](int which) { return launch_group(m, cache, d, g, b0, nb, which, replay, logits_full, logits_slim, st); };
         int rc;
         if (together) {
-            if ((rc = launch_group(m, cache, d, b0, nb, 2, replay, logits_full, logits_slim, st))) return rc;
+            if ((rc = group(2))) return rc;
             continue;
         }
-        if (mode != 0 && (rc = launch_group(m, cache, d, b0, nb, 1, replay, logits_full, logits_slim, st))) return rc;
-        if (mode != 1 && (rc = launch_group(m, cache, d, b0, nb, 0, replay, logits_full, logits_slim, st))) return rc;
+        if (mode != 0 && (rc = group(1))) return rc;
+        if (mode != 1 && (rc = group(0))) return rc;
     }
     return VIASD_OK;
 }

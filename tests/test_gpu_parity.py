@@ -540,6 +540,7 @@ def _one_launch_case(name, batch, nodes, ctx, tree=False, **shape):
     _one_launch_case("c1_tiny", 1, 1, 0), _one_launch_case("c1_tiny", 3, 8, 63, d_model=192, d_ff=680),      # k no whole groups of 32
     _one_launch_case("c1_tiny", 2, 26, 300, tree=True, n_kv_heads=2, vocab=1001),                             # grouped heads, odd vocabulary
     _one_launch_case("c1_tiny", 5, 12, 70, head_dim=128, n_heads=2, n_kv_heads=1),                            # 65 rows: three launches
+    _one_launch_case("c1_tiny", 5, 20, 90), _one_launch_case("c1_tiny", 7, 16, 300, n_layers=3),              # apart: 63 and 42, 51 and 17 rows
     _one_launch_case("c1_tiny", 2, 63, 90), _one_launch_case("c1_tiny", 2, 8, 40, d_model=768, d_ff=2048),   # a verifier per launch; fewer rows per launch
     _one_launch_case("mini_7b", 1, 1, 0), _one_launch_case("mini_7b", 1, 15, 63), _one_launch_case("mini_7b", 3, 7, 130),   # 2, 16, 24 rows
     _one_launch_case("mini_8b_tree_greedy", 1, 26, 500, tree=True), _one_launch_case("mini_13b", 3, 6, 260, n_layers=2),
@@ -576,6 +577,39 @@ def test_pass_in_one_launch_is_the_pass(wl):
         assert float((a.float() - b.float()).abs().max()) <= tol, i
     if f32:
         assert float((step[1] - many[1]).norm() / many[1].norm()) <= 1e-5
+
+
+@pytest.mark.parametrize("batch,nodes,ctx,takes,shape", [
+    (16, 26, 300, True, {}), (11, 5, 4000, True, dict(d_model=192, d_ff=680)), (16, 16, 300, True, dict(n_layers=3)),
+    (24, 5, 70, False, dict(d_model=192, n_heads=2, n_kv_heads=2, d_ff=2816)), (12, 7, 300, False, dict(n_heads=2, n_kv_heads=1, d_ff=2816)),
+    (32, 24, 130, False, dict(d_model=64, n_heads=1, n_kv_heads=1, d_ff=256, vocab=512)), (4, 5, 70, True, dict(d_model=192, d_ff=680))],
+    ids=lambda v: str(v) if isinstance(v, int) else "-".join(f"{a}{b}" for a, b in v.items()) or "tiny")
+def test_fp32_batches_in_groups_where_that_gains(batch, nodes, ctx, takes, shape):
+    """More sequences than a launch holds: several launches of a pass each, unless they are so many of so few rows and columns that
+    the pass is faster launch by launch.  Step and single passes take the same route."""
+    vb = _vb()
+    wl = _one_launch_case("c1_tiny", batch, nodes, ctx, **shape)
+    eng = _engine(wl, fill_context="device", extra_ctx=82)
+    eng.set_inputs(W.step_inputs(wl))
+    sl, fl, res = eng.logits_buffer(), eng.logits_buffer(), vb.alloc_result(wl.batch, wl.n_nodes)
+
+    def launches(f, *args):
+        n0 = vb.launch_count()
+        f(eng.model, eng.cache, eng.draft, *args)
+        torch.cuda.synchronize()
+        return vb.launch_count() - n0
+
+    calls = [(vb.verify_step, eng.params(), sl, fl, res), (vb.full_forward, fl), (vb.slim_forward, sl)]
+    counts = []
+    for one in (1, 0):
+        vb.set_option(eng.model, "one_launch", one)
+        eng.len.fill_(wl.ctx)
+        counts.append([launches(*c) for c in calls])
+    assert vb.get_stats(eng.model).device_status == 0
+    if takes:
+        assert counts[0] < counts[1] and counts[0][1] == counts[0][2] <= batch
+    else:
+        assert counts[0] == counts[1]
 
 
 # Sequences of different lengths in one batch.  The attention kernels deal key ranges or tiles to CTAs from the
