@@ -592,7 +592,7 @@ static int verify_step_routed(viasd_model *m, viasd_cache *cache, const viasd_dr
                                                                       false, st, &probe); }))) return rc;
     m->run_flag = flag;
     rc = SMALL_PASS_NO_ROOM;
-    if (small_pass_takes(m, cache, draft->batch, M + G)) {
+    if (small_pass_takes(m, cache, draft->batch, M + G, true)) {
         rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_prep_replay(m, cache, draft, G, st); });
         if (!rc) rc = timed(m, VIASD_T_GEMM, st, [&] { return launch_small_pass(m, cache, draft, 0, G, full_logits, nullptr, st); });
     }

@@ -249,7 +249,7 @@ inline int small_pass_set(const viasd_config &c) {
 }
 inline size_t small_pass_counters(const viasd_config &c) { return SMALL_PASS_LINE + (size_t)2 * small_pass_set(c); }
 constexpr int SMALL_PASS_NO_ROOM = 1;
-bool small_pass_takes(const viasd_model *m, const viasd_cache *cache, int batch, int M);
+bool small_pass_takes(const viasd_model *m, const viasd_cache *cache, int batch, int M, bool replay = false);
 int launch_small_pass(viasd_model *m, const viasd_cache *cache, const viasd_draft *d, int mode, int replay, float *logits_full,
                       float *logits_slim, cudaStream_t st);
 

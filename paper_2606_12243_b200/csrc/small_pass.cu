@@ -1014,7 +1014,29 @@ static Grouping grouping(const viasd_model *m, int batch, int M, int most) {
 // d 768, 16 x 9 rows 1978 / 2305.  Key tiles are counted by the cache's capacity, as the lengths are on the device.
 // A launch has all weights of a stage in shared memory, the output head's too (plan): at 148 SMs fp32 of d 256 up to a vocabulary of
 // 16576, bf16 of d 512 up to 14208, of d 768 up to 9472; beyond that a model goes launch by launch.
-bool small_pass_takes(const viasd_model *m, const viasd_cache *cache, int batch, int M) {
+// bf16 steps of 33 - 64 rows of both verifiers (the kernel's instance for 64, whose padding and smaller stages of input tell) go this way
+// where a step's estimate is the smaller one: per layer 15.2 us and what a CTA multiplies and its tiles of keys take, against
+// 26.4 us and weights, rows and keys, fitted to 2688 drawn steps of 2 - 32 rows per verifier (median error 3 %, 7 % in a tenth).  Without it 242
+// of them are slower in one launch (0.74 at worst; d 640, two layers, 21 rows 124 / 116 us), with it 77 (0.87; drawn again: 90 of 2728, 0.86); 35 of those it
+// sends launch by launch would have gained 5 % or more.  A single pass follows the step, as both compute the same bits.
+static bool one_launch_gains(const viasd_model *m, const Grouping &g, int rows) {
+    const viasd_config &c = m->cfg;
+    auto up = [](long long a, long long b) { return (double)((a + b - 1) / b); };
+    auto units = [&](long long n) { return up(n, m->sm_count); };
+    auto chunks = [&](int k) { return up(k, KG * SP_WARPS); };
+    const int d = c.d_model, ff = c.d_ff, qd = c.n_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim, routed = m->n_routed, other = c.n_layers - routed;
+    const double products = (units((qd + 2 * kvd) / 16) + units(ff / 8)) * chunks(d) + units(d / 8) * (chunks(qd) + chunks(ff));
+    const long long pairs = (long long)g.batch * g.pairs, ns = g.ranges(0);
+    auto layer = [&](int streams) { return units(streams * pairs * ns) * (15.2 + 1.6 * up(c.max_ctx, 64 * ns)) + 0.029 * streams * rows * products; };
+    const double one = 32 + routed * layer(2) + other * layer(1) + 0.029 * 2 * rows * chunks(d) * units((c.vocab + 15) / 16) +
+                       (d > 512 ? routed * 3.1 * (d - 512) / 128 : 0);
+    const double params = (double)d * (2 * qd + 2 * kvd) + 3. * d * ff;
+    const double many = 26.4 * (c.n_layers + 1) + 0.21 * rows * (c.n_layers + routed) + 1.29e-6 * (c.n_layers * params + (double)c.vocab * d) +
+                        1e-3 * c.max_ctx * (1.52 * c.n_layers + 0.051 * pairs * (c.n_layers + routed));
+    return one <= many;
+}
+
+bool small_pass_takes(const viasd_model *m, const viasd_cache *cache, int batch, int M, bool replay) {
     const viasd_config &c = m->cfg;
     const ModelOptions &o = m->opt;
     if (!o.one_launch || (c.dtype == 1 && !m->fused)) return false;
@@ -1033,6 +1055,7 @@ bool small_pass_takes(const viasd_model *m, const viasd_cache *cache, int batch,
         if (2 * rows > most) return false;
         const long long tiles = 2LL * batch * g.pairs * ((c.max_ctx + 63) / 64);
         if (rows * columns * m->sm_count + 3 * 2944 * tiles > 36LL * 2944 * m->sm_count) return false;
+        if (!replay && rows > 16 && !one_launch_gains(m, g, (int)rows)) return false;
         // (caches that are not aligned are refused by the path with tensor maps over them)
         if (((uintptr_t)cache->k_full | (uintptr_t)cache->v_full | (uintptr_t)cache->k_slim | (uintptr_t)cache->v_slim) & 15) return false;
     }

@@ -543,7 +543,7 @@ def _one_launch_case(name, batch, nodes, ctx, tree=False, **shape):
     _one_launch_case("c1_tiny", 5, 20, 90), _one_launch_case("c1_tiny", 7, 16, 300, n_layers=3),              # apart: 63 and 42, 51 and 17 rows
     _one_launch_case("c1_tiny", 2, 63, 90), _one_launch_case("c1_tiny", 2, 8, 40, d_model=768, d_ff=2048),   # a verifier per launch; fewer rows per launch
     _one_launch_case("mini_7b", 1, 1, 0), _one_launch_case("mini_7b", 1, 15, 63), _one_launch_case("mini_7b", 3, 7, 130),   # 2, 16, 24 rows
-    _one_launch_case("mini_8b_tree_greedy", 1, 26, 500, tree=True), _one_launch_case("mini_13b", 3, 6, 260, n_layers=2),
+    _one_launch_case("mini_8b_tree_greedy", 1, 26, 500, tree=True), _one_launch_case("mini_13b", 3, 6, 260),
     _one_launch_case("mini_7b", 1, 8, 200, d_model=1024, d_ff=2824)], ids=lambda w: f"{w.name}-{w.batch}x{w.rows}-{w.ctx}")
 def test_pass_in_one_launch_is_the_pass(wl):
     """Logits and caches of a pass in one launch are those of the kernels for any model, launch by launch, within what either may
@@ -579,16 +579,24 @@ def test_pass_in_one_launch_is_the_pass(wl):
         assert float((step[1] - many[1]).norm() / many[1].norm()) <= 1e-5
 
 
-@pytest.mark.parametrize("batch,nodes,ctx,takes,shape", [
-    (16, 26, 300, True, {}), (11, 5, 4000, True, dict(d_model=192, d_ff=680)), (16, 16, 300, True, dict(n_layers=3)),
-    (24, 5, 70, False, dict(d_model=192, n_heads=2, n_kv_heads=2, d_ff=2816)), (12, 7, 300, False, dict(n_heads=2, n_kv_heads=1, d_ff=2816)),
-    (32, 24, 130, False, dict(d_model=64, n_heads=1, n_kv_heads=1, d_ff=256, vocab=512)), (4, 5, 70, True, dict(d_model=192, d_ff=680))],
-    ids=lambda v: str(v) if isinstance(v, int) else "-".join(f"{a}{b}" for a, b in v.items()) or "tiny")
-def test_fp32_batches_in_groups_where_that_gains(batch, nodes, ctx, takes, shape):
-    """More sequences than a launch holds: several launches of a pass each, unless they are so many of so few rows and columns that
-    the pass is faster launch by launch.  Step and single passes take the same route."""
+_ROUTE = lambda v: str(v) if isinstance(v, (int, str)) else "-".join(f"{a}{b}" for a, b in v.items()) or "as-is"
+
+
+@pytest.mark.parametrize("name,batch,nodes,ctx,takes,shape", [
+    # fp32, more sequences than a launch holds: several launches, unless they are many of few rows and columns
+    ("c1_tiny", 16, 26, 300, True, {}), ("c1_tiny", 11, 5, 4000, True, dict(d_model=192, d_ff=680)), ("c1_tiny", 16, 16, 300, True, dict(n_layers=3)),
+    ("c1_tiny", 4, 5, 70, True, dict(d_model=192, d_ff=680)), ("c1_tiny", 24, 5, 70, False, dict(d_model=192, n_heads=2, n_kv_heads=2, d_ff=2816)),
+    ("c1_tiny", 12, 7, 300, False, dict(n_heads=2, n_kv_heads=1, d_ff=2816)),
+    ("c1_tiny", 32, 24, 130, False, dict(d_model=64, n_heads=1, n_kv_heads=1, d_ff=256, vocab=512)),
+    # bf16, 33 to 64 rows of both verifiers: by the estimate
+    ("mini_7b", 1, 26, 300, True, {}), ("mini_7b", 2, 8, 1000, True, {}), ("mini_8b_tree_greedy", 3, 8, 300, True, {}),
+    ("mini_7b", 3, 7, 130, False, dict(n_layers=1, d_model=1024)), ("mini_7b", 1, 20, 70, False, dict(n_layers=1, d_model=1024, n_heads=1, n_kv_heads=1, d_ff=2048)),
+    ("mini_7b", 1, 26, 1000, False, dict(n_layers=1, d_model=384, n_heads=1, n_kv_heads=1, d_ff=2816, vocab=8192))], ids=_ROUTE)
+def test_passes_go_in_one_launch_where_that_gains(name, batch, nodes, ctx, takes, shape):
+    """Which way a small model's pass goes, at shapes measured on either side; the step and the single passes take the same."""
     vb = _vb()
-    wl = _one_launch_case("c1_tiny", batch, nodes, ctx, **shape)
+    wl = _one_launch_case(name, batch, nodes, ctx, **shape)
+    wl = replace(wl, n_routed=min(wl.n_routed, wl.shape.n_layers))
     eng = _engine(wl, fill_context="device", extra_ctx=82)
     eng.set_inputs(W.step_inputs(wl))
     sl, fl, res = eng.logits_buffer(), eng.logits_buffer(), vb.alloc_result(wl.batch, wl.n_nodes)
