@@ -318,7 +318,9 @@ int viasd_selftest_wait_expiry(int *status, int limit_us, long long *waited_cycl
  * accept / commit path is bracketed by one pair of CUDA events on the caller's stream (the launches inside a run
  * keep their programmatic overlap; a few thousand runs are kept, later ones are dropped).
  * viasd_get_timing: synchronises `stream`, sums the recorded intervals per kernel class into `out`
- * (VIASD_T_COUNT entries each) and clears the record. */
+ * (VIASD_T_COUNT entries each) and clears the record.  A small model's pass in one launch (VIASD_OPT_ONE_LAUNCH) counts as
+ * VIASD_T_GEMM, its embedding, norms, rotary embedding and attention included; `launches` counts the calls inside
+ * a pass that launch something, one for a product or a pass whose rows take several launches. */
 enum { VIASD_T_GEMM = 0, VIASD_T_ATTENTION, VIASD_T_NORM, VIASD_T_ROPE, VIASD_T_EMBED, VIASD_T_TIER_ACCEPT,
        VIASD_T_COMMIT, VIASD_T_COUNT };
 typedef struct { double ms[VIASD_T_COUNT]; long long launches[VIASD_T_COUNT]; long long dropped; } viasd_timing;

@@ -81,15 +81,18 @@ template <typename F>
 int timed(viasd_model *m, int cls, cudaStream_t st, F &&f) {
     KernelTimer &t = m->timer;
     if (!t.on) return f();
-    if (t.open >= 0 && t.cls[t.open] == cls) { ++t.cnt[t.open]; return f(); }     // the run goes on
-    if (t.open >= 0) { CUDA_TRY(cudaEventRecord(t.end[t.open], st)); t.open = -1; }
-    if (t.n >= KernelTimer::CAP) { ++t.dropped; return f(); }
-    const int i = t.n++;
-    t.cls[i] = cls;
-    t.cnt[i] = 1;
-    CUDA_TRY(cudaEventRecord(t.beg[i], st));
-    t.open = i;
-    return f();
+    if (t.open < 0 || t.cls[t.open] != cls) {                   // (else the run goes on)
+        if (t.open >= 0) { CUDA_TRY(cudaEventRecord(t.end[t.open], st)); t.open = -1; }
+        if (t.n >= KernelTimer::CAP) { ++t.dropped; return f(); }
+        const int i = t.n++;
+        t.cls[i] = cls;
+        t.cnt[i] = 0;
+        CUDA_TRY(cudaEventRecord(t.beg[i], st));
+        t.open = i;
+    }
+    const int run = t.open, rc = f();
+    if (rc != SMALL_PASS_NO_ROOM) ++t.cnt[run];                 // (that one has launched nothing)
+    return rc;
 }
 
 int env_int(const char *name, int dflt) { const char *e = getenv(name); return e && *e ? atoi(e) : dflt; }
@@ -182,7 +185,7 @@ int run_gemm(viasd_model *m, const GemmCall &g, int rows, cudaStream_t st) {
 // once and applied to both streams, an unrouted layer runs on the full stream only.  Results are those of the two
 // separate passes; only the weight traffic of the routed layers is shared.
 // replay > 0 (mode 0 only, routed execution policy): every sequence's block is extended in front by its last `replay`
-// committed tokens (see prep_replay_kernel); the logits written are those of the block's own rows.
+// committed tokens, as launch_prep_replay has laid them out before; the logits written are those of the block's own rows.
 int forward_sweep(viasd_model *m, const viasd_cache *cache, const viasd_draft *d, int mode, float *logits_full,
                   float *logits_slim, cudaStream_t st, int replay = 0) {
     const viasd_config &c = m->cfg;
@@ -225,7 +228,6 @@ int forward_sweep(viasd_model *m, const viasd_cache *cache, const viasd_draft *d
     auto wseg = [&](TcLaunch &L, int i, const WMap &w, int n) { L.map_w[i] = &w.map; L.seg_n[i] = n; L.w_box_rows[i] = w.box_rows; };
     const int ssq_n = (c.d_model / 128) * 4;
 
-    if (replay && (rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_prep_replay(m, cache, d, replay, st); }))) return rc;
     if ((rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_embed_norm(m, cache, d, mode != 1, replay > 0, m->norm1[layer_id(0)],
                                                                          dual ? m->norm1[m->routed[0]] : nullptr, rows, st); }))) return rc;
     for (int it = 0; it < n_run; ++it) {
@@ -591,11 +593,9 @@ static int verify_step_routed(viasd_model *m, viasd_cache *cache, const viasd_dr
     if ((rc = timed(m, VIASD_T_TIER_ACCEPT, st, [&] { return launch_accept(m, draft, params, probe_set, result, true,
                                                                       false, st, &probe); }))) return rc;
     m->run_flag = flag;
-    rc = SMALL_PASS_NO_ROOM;
-    if (small_pass_takes(m, cache, draft->batch, M + G, true)) {
-        rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_prep_replay(m, cache, draft, G, st); });
-        if (!rc) rc = timed(m, VIASD_T_GEMM, st, [&] { return launch_small_pass(m, cache, draft, 0, G, full_logits, nullptr, st); });
-    }
+    rc = timed(m, VIASD_T_EMBED, st, [&] { return launch_prep_replay(m, cache, draft, G, st); });
+    if (!rc) rc = !small_pass_takes(m, cache, draft->batch, M + G, true) ? SMALL_PASS_NO_ROOM :
+                  timed(m, VIASD_T_GEMM, st, [&] { return launch_small_pass(m, cache, draft, 0, G, full_logits, nullptr, st); });
     if (rc == SMALL_PASS_NO_ROOM) rc = forward_sweep(m, cache, draft, 0, full_logits, nullptr, st, G);
     m->run_flag = nullptr;
     if (rc) return rc;

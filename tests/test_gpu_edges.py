@@ -371,3 +371,63 @@ def test_nothing_past_the_block_is_read_into_the_result(name, nodes, kernel, ctx
         torch.cuda.synchronize()
         got.append(out)
     assert torch.isfinite(got[1]).all() and torch.equal(*got)
+
+
+# ---------------------------------------------------------------------------------------------
+# a context that does not hold the one launch of a small model's pass
+# ---------------------------------------------------------------------------------------------
+_NO_ROOM = """
+import sys
+sys.path.insert(0, {root!r})
+from dataclasses import replace
+import torch
+from paper_2606_12243_b200 import binding as vb
+vb.LIB_PATH = {lib!r}
+from paper_2606_12243_b200.engine import Engine
+from synth import workloads as W
+
+for name, policy in (("c1_tiny", 0), ("mini_7b", 0), ("mini_13b", 0), ("mini_7b", 1)):
+    wl = W.get(name)
+    outs = []
+    for one in (1, 0):
+        eng = Engine(wl, fill_context="device", max_query=wl.rows + (18 if policy else 0))
+        eng.set_inputs(W.step_inputs(wl))
+        vb.set_option(eng.model, "one_launch", one)
+        vb.set_timing(eng.model, True)
+        sl, fl, f2, s2, res = *(eng.logits_buffer().zero_() for _ in range(4)), vb.alloc_result(wl.batch, wl.n_nodes)
+        n0 = vb.launch_count()
+        vb.full_forward(eng.model, eng.cache, eng.draft, f2)
+        vb.slim_forward(eng.model, eng.cache, eng.draft, s2)
+        # (every token is the full verifier's to judge: the routed step's pass runs)
+        vb.verify_step(eng.model, eng.cache, eng.draft, eng.params(policy=policy, log_tau_lo=1e9, log_tau_hi=1e9), sl, fl, res)
+        torch.cuda.synchronize()
+        stats = vb.get_stats(eng.model)
+        assert stats.device_status == 0 and stats.full_ran
+        timing = vb.get_timing(eng.model)
+        outs.append(([vb.launch_count() - n0] + [v["launches"] for v in timing.values() if isinstance(v, dict)],
+                     [t.clone() for t in (sl, fl, f2, s2, eng.k_full, eng.v_full, eng.k_slim, eng.v_slim, eng.len, eng.pending, res.out_tok, res.n_acc)]))
+    assert outs[0][0] == outs[1][0], (name, policy, outs[0][0], outs[1][0])
+    assert all(torch.equal(a, b) for a, b in zip(outs[0][1], outs[1][1])), (name, policy)
+"""
+
+
+def test_pass_without_room_goes_launch_by_launch(tmp_path):
+    """The driver refuses the cooperative launch (in a context with a share of the SMs, say): the library with that launcher replaced by
+    one that always answers so computes, launches and counts what it does with the option off - step, single passes, routed step."""
+    import os
+    import subprocess
+    import sys
+    from paper_2606_12243_b200 import build as B
+    B.build()
+    stub, obj, lib = tmp_path / "stub.cu", tmp_path / "stub.o", tmp_path / "libviasd_no_room.so"
+    stub.write_text("""
+        #include "common.cuh"
+        bool small_pass_takes(const viasd_model *m, const viasd_cache *, int, int, bool) { return m->opt.one_launch; }
+        int launch_small_pass(viasd_model *, const viasd_cache *, const viasd_draft *, int, int, float *, float *, cudaStream_t) { return SMALL_PASS_NO_ROOM; }
+        """)
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.check_call([B.NVCC, *B.FLAGS, "-I", B.CSRC, "-c", str(stub), "-o", str(obj)])
+    others = [os.path.join(B.OBJ, f[:-3] + ".o") for f in B._sources() if f != "small_pass.cu"]
+    subprocess.check_call([B.NVCC, "-shared", "-o", str(lib), str(obj), *others, "-lcuda"])
+    code = _NO_ROOM.format(root=root, lib=str(lib))
+    subprocess.run([sys.executable, "-c", code], check=True, timeout=300, cwd=root)
