@@ -419,12 +419,13 @@ int launch_attention_mma(viasd_model *m, const void *kc, const void *vc, bool sl
     a.ring_slots = RING;
     fill_work(m, a, layer_ord, layer_ord2, streams, batch, M);
     const size_t smem = 1024 + (size_t)RING * SLOT_BYTES + (size_t)WARPS * 16 * HD * sizeof(float);
-    static bool attr_done[64];
-    if (first_use_on_device(attr_done)) {
+    static std::atomic<bool> attr_done[64];
+    if (int rc = once_on_device(attr_done, [&]() -> int {
         CUDA_TRY(cudaFuncSetAttribute(attention_mma_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         CUDA_TRY(cudaFuncSetAttribute(attention_mma_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         CUDA_TRY(cudaFuncSetAttribute(attention_mma_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    }
+        return VIASD_OK;
+    })) return rc;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     pdl_config(cfg, attr, dim3(work_grid(m)), dim3(WARPS * 32 + 32), smem, st);

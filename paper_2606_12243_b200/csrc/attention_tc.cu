@@ -639,11 +639,12 @@ int launch_attention_tc(viasd_model *m, const void *kc, const void *vc, bool sli
     a.ring_slots = (int)((smem_max - 1024 - q_bytes) / SLOT_BYTES);
     if (a.ring_slots > AT_MAX_SLOTS) a.ring_slots = AT_MAX_SLOTS;
     const size_t smem = 1024 + q_bytes + (size_t)a.ring_slots * SLOT_BYTES;
-    static bool attr_done[64];
-    if (first_use_on_device(attr_done)) {
+    static std::atomic<bool> attr_done[64];
+    if (int rc = once_on_device(attr_done, [&]() -> int {
         CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
         CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
-    }
+        return VIASD_OK;
+    })) return rc;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     pdl_config(cfg, attr, dim3(grid), dim3(AT_THREADS), smem, st);

@@ -748,12 +748,13 @@ int launch_attention_tk(viasd_model *m, const void *kc, const void *vc, bool sli
         a.nk = a.nv = 1024 + op_bytes + 3 * (size_t)(2 * SLOT_BYTES) <= 220 * 1024 ? 3 : 2;
         smem = 1024 + op_bytes + a.nk * (size_t)(2 * SLOT_BYTES);
     }
-    static bool attr_done[64];
-    if (first_use_on_device(attr_done)) {
+    static std::atomic<bool> attr_done[64];
+    if (int rc = once_on_device(attr_done, [&]() -> int {
         CUDA_TRY(cudaFuncSetAttribute(attention_tk_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024));
         CUDA_TRY(cudaFuncSetAttribute(attention_tk_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024));
         CUDA_TRY(cudaFuncSetAttribute(attention_tk_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024));
-    }
+        return VIASD_OK;
+    })) return rc;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     pdl_config(cfg, attr, dim3(grid), dim3(nr == 32 ? TK_THREADS + 128 : TK_THREADS), smem, st);

@@ -5,6 +5,7 @@
 #include <stdint.h>
 #include <stddef.h>
 #include <math.h>
+#include <atomic>
 #include "../../include/viasd.h"
 #include "gemm_tc.cuh"
 
@@ -171,14 +172,21 @@ extern unsigned long long g_launch_count;
     } while (0)
 #define LAUNCH_CHECK() do { ++g_launch_count; CUDA_TRY(cudaGetLastError()); } while (0)
 
-// cudaFuncSetAttribute applies to the current device only: remembers, per device, whether a launcher has set its
-// kernels' attributes there.  Returns true the first time it is asked about (flags, current device).
-inline bool first_use_on_device(bool (&flags)[64]) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return true;     // unknown: set them again, which is harmless
-    const bool first = !flags[dev];
-    flags[dev] = true;
-    return first;
+// A kernel's attributes belong to the current device: `set` runs on the first launch there, and none returns before it has run.  (Two
+// threads' first launches may both run it, which is harmless; if it fails, the next launch tries again.)
+template <typename F>
+inline int once_on_device(std::atomic<bool> (&done)[64], int dev, F set) {
+    const bool known = dev >= 0 && dev < 64;
+    if (known && done[dev].load(std::memory_order_acquire)) return VIASD_OK;
+    const int rc = set();
+    if (known && rc == VIASD_OK) done[dev].store(true, std::memory_order_release);
+    return rc;
+}
+template <typename F>
+inline int once_on_device(std::atomic<bool> (&done)[64], F set) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+    return once_on_device(done, dev, set);
 }
 
 // Programmatic dependent launch: a kernel launched with this configuration may begin (prologue, weight

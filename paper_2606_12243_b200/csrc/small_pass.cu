@@ -908,9 +908,11 @@ template <typename T, int HD, int MT>
 int launch(SpArgs &a, const viasd_config &c, int rows, int grid, cudaStream_t st) {
     size_t smem = 0;
     if (!plan<T, HD, MT>(c, rows, grid, a, smem)) return VIASD_EINVAL;
-    static bool attr_done[64];
-    if (first_use_on_device(attr_done))
+    static std::atomic<bool> attr_done[64];
+    if (int rc = once_on_device(attr_done, [&]() -> int {
         CUDA_TRY(cudaFuncSetAttribute(small_pass_kernel<T, HD, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SP_SMEM));
+        return VIASD_OK;
+    })) return rc;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     cfg.gridDim = dim3(grid); cfg.blockDim = dim3(SP_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;

@@ -97,3 +97,31 @@ def test_gemm_of_more_than_128_rows_takes_nothing_per_row(lib, tmp_path):
         assert [got(rows, nt, 0, epi, 0) for epi in (add, swiglu, add_norm, qkv_rope)] == [-1] * 4
         assert got(rows, nt, 1, store, 0) == got(rows, nt, 0, store, 1) == -1
     assert got(257, 272, 0, store, 0) == got(17, 16, 0, store, 0) == got(0, 16, 0, store, 0) == -1
+
+
+def test_no_launch_overtakes_the_first_ones_attributes(tmp_path):
+    """Two threads launch a kernel for the first time: the second one's launch may not go out before the kernel's shared-memory limit has
+    been raised; a failure is not remembered as done."""
+    import subprocess
+    from paper_2606_12243_b200 import build as B
+    src, exe = tmp_path / "t.cu", tmp_path / "t"
+    src.write_text("""
+        #include "common.cuh"
+        #include <chrono>
+        #include <thread>
+        static std::atomic<bool> done[64], ready(false);
+        int main() {
+            if (once_on_device(done, 3, [] { return (int)VIASD_ECUDA; }) != VIASD_ECUDA) return 1;
+            auto set = [] { std::this_thread::sleep_for(std::chrono::milliseconds(300)); ready = true; return (int)VIASD_OK; };
+            std::thread first([&] { once_on_device(done, 3, set); });
+            std::this_thread::sleep_for(std::chrono::milliseconds(100));
+            if (once_on_device(done, 3, set) != VIASD_OK || !ready) return 2;
+            first.join();
+            int again = 0;
+            once_on_device(done, 3, [&] { ++again; return (int)VIASD_OK; });        // done there,
+            once_on_device(done, 4, [&] { ++again; return (int)VIASD_OK; });        // not on another device,
+            once_on_device(done, 64, [&] { ++again; return (int)VIASD_OK; });       // and always where there is no place
+            return again == 2 ? 0 : 3;
+        }""")
+    subprocess.check_call([B.NVCC, *B.FLAGS, "-I", B.CSRC, str(src), "-o", str(exe), "-lpthread"])
+    assert subprocess.call([str(exe)]) == 0
