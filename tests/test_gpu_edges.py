@@ -42,16 +42,21 @@ def _step(eng, model, cache, batch, nodes):
 # ---------------------------------------------------------------------------------------------
 # arrays that need not be aligned beyond their element
 # ---------------------------------------------------------------------------------------------
-@pytest.mark.parametrize("name,batch,head_dim", [("c1_tiny", None, None), ("mini_7b", None, None), ("mini_7b", 8, None), ("mini_7b", None, 64)])
-def test_gains_and_caches_need_no_alignment(name, batch, head_dim):
-    """Norm gains at an odd float offset (fp32 path, one-CTA GEMM, pair GEMM from 48 rows on, unfused bf16 path), and where
-    no tensor map is built over them (fp32, head_dim 64) caches at an odd element: same bits as aligned."""
+@pytest.mark.parametrize("name,batch,head_dim,one", [("c1_tiny", None, None, 1), ("mini_7b", None, None, 1), ("mini_7b", 8, None, 1), ("mini_7b", None, 64, 1),
+                                                     ("c1_tiny", None, None, 0), ("mini_7b", None, None, 0)])
+def test_gains_and_caches_need_no_alignment(name, batch, head_dim, one, monkeypatch):
+    """Norm gains at an odd float offset (a pass in one launch, fp32 and bf16; pair GEMM from 48 rows on; unfused bf16 path; fp32 path launch
+    by launch, one-CTA GEMM), and where no tensor map is built over them (fp32, head_dim 64) caches at an odd element: same bits as
+    aligned."""
+    monkeypatch.setenv("VIASD_ONE_LAUNCH", str(one))
     vb = _vb()
     base = W.get(name)
     wl = replace(base, batch=batch or base.batch, shape=replace(base.shape, head_dim=head_dim or base.shape.head_dim))
     eng = _engine(wl)
     state = [t.clone() for t in (eng.k_full, eng.v_full, eng.k_slim, eng.v_slim, eng.len, eng.pending, eng.tokens, eng.len_full)]
+    n0 = vb.launch_count()
     want = _step(eng, eng.model, eng.cache, wl.batch, wl.n_nodes)
+    assert (vb.launch_count() - n0 == 4) == (one == 1 and batch is None and head_dim is None)      # pass, statistics, walk, commit
     layers = [{k: _shifted(v) if k.startswith("norm") else v for k, v in l.items()} for l in eng.layers]
     ws = torch.empty_like(eng.workspace)
     assert ws.data_ptr() % 256 == 0
@@ -79,8 +84,10 @@ def test_expired_wait_leaves_a_usable_handle(name, batch):
     wl = replace(base, batch=batch, shape=replace(base.shape, n_layers=1, d_model=2048, d_ff=2048), n_routed=1)
     eng = _engine(wl)
     want, got = eng.logits_buffer(), eng.logits_buffer()
+    n0 = vb.launch_count()
     vb.full_forward(eng.model, eng.cache, eng.draft, want)
     torch.cuda.synchronize()
+    assert vb.launch_count() - n0 > 1                          # (not a small model's pass in one)
     # the counters are the workspace's last piece
     s = wl.shape
     n = 4 * (max(s.vocab, s.n_heads * s.head_dim + 2 * s.n_kv_heads * s.head_dim, s.d_ff) // 64 + 8)
@@ -352,16 +359,20 @@ def test_refused_step_runs_nothing(dual_max, what):
 # ---------------------------------------------------------------------------------------------
 # caches that have never been written past the block
 # ---------------------------------------------------------------------------------------------
-@pytest.mark.parametrize("name,nodes,kernel", [("mini_7b", 8, "mma"), ("mini_7b", 8, "tk"), ("mini_8b_tree", 26, "tc"), ("mini_8b_tree", 40, "tc"),
-                                               ("mini_32b_b3", 5, "tk"), ("mini_32b_b3", 5, "tc"), ("c1_tiny", 4, "auto")])
+@pytest.mark.parametrize("name,nodes,kernel,one", [("mini_7b", 8, "mma", 1), ("mini_7b", 8, "tk", 1), ("mini_8b_tree", 26, "tc", 1), ("mini_8b_tree", 40, "tc", 1),
+                                                   ("mini_32b_b3", 5, "tk", 1), ("mini_32b_b3", 5, "tc", 1), ("c1_tiny", 4, "auto", 1), ("c1_tiny", 4, "auto", 0),
+                                                   ("mini_7b", 8, "auto", 1), ("mini_8b_tree_greedy", 5, "auto", 1)])
 @pytest.mark.parametrize("ctx", [0, 116, 245, 333])
-def test_nothing_past_the_block_is_read_into_the_result(name, nodes, kernel, ctx):
-    """NaN in every slot past the block's: same bits as with zeros there, whatever 16-, 32- or 128-key group the block ends in."""
+def test_nothing_past_the_block_is_read_into_the_result(name, nodes, kernel, one, ctx):
+    """NaN in every slot past the block's: same bits as with zeros there, whatever 16-, 32-, 64- or 128-key group the block ends in;
+    with kernel "auto" in one launch, or (one: 0) launch by launch."""
     vb = _vb()
     base = W.get(name)
     eng = _engine(replace(base, ctx=ctx, parent=W.chain(nodes), shape=replace(base.shape, n_layers=2), n_routed=1), extra_ctx=140)
     vb.set_option(eng.model, "attention_kernel", kernel)
+    vb.set_option(eng.model, "one_launch", one)
     eng.len.fill_(ctx)
+    n0 = vb.launch_count()
     got = []
     for fill in (0.0, float("nan")):
         for t in (eng.k_full, eng.v_full):
@@ -371,6 +382,7 @@ def test_nothing_past_the_block_is_read_into_the_result(name, nodes, kernel, ctx
         torch.cuda.synchronize()
         got.append(out)
     assert torch.isfinite(got[1]).all() and torch.equal(*got)
+    assert (vb.launch_count() - n0 == 2) == (kernel == "auto" and one == 1)
 
 
 # ---------------------------------------------------------------------------------------------

@@ -18,6 +18,10 @@ torch = pytest.importorskip("torch")
 FLOOR_FRAC = 0.85       # observed: 0.90 (16 sequences of the shrunken 32B shape) to 1.0
 
 
+# A small model's pass launch by launch too: through the kernels for any model
+LAUNCHES = {"VIASD_ONE_LAUNCH": "0"}
+
+
 def _floor_full(batch):
     """Least number of sequences that must be compared to their end (observed: 13 of 16, 7 of 8, else all)."""
     return -(-3 * batch // 4)
@@ -198,10 +202,12 @@ def test_forward_with_wide_query_groups(name, batch, nodes, ctx):
 
 
 # The rows-on-lanes kernel at its edges: 33+ and exactly 128 rows, a context that ends on a tile and one past it, no context,
-# each way of cutting the keys (whole pairs, k ranges per pair, tiles dealt evenly over a small grid).  Bounds as above.
+# each way of cutting the keys (whole pairs, k ranges per pair, tiles dealt evenly over a small grid).  Bounds as above.  (Without an
+# option the small ones are one launch, whose attention has the same edges.)
 @pytest.mark.parametrize("nodes,batch,ctx,env", [(8, 1, 0, {}), (15, 1, 112, {}), (15, 2, 113, {}), (31, 2, 500, {"VIASD_ATTN_NSPLIT": "1"}),
                                                  (31, 3, 700, {"VIASD_ATTN_NSPLIT": "3"}), (8, 1, 2300, {}),
-                                                 (26, 8, 700, {"VIASD_TK_GRID": "3"}), (3, 2, 300, {"VIASD_ATTN": "tc"})])
+                                                 (26, 8, 700, {"VIASD_TK_GRID": "3"}), (3, 2, 300, {"VIASD_ATTN": "tc"}),
+                                                 (8, 1, 0, LAUNCHES), (15, 1, 112, LAUNCHES), (15, 2, 113, LAUNCHES), (8, 1, 2300, LAUNCHES)])
 def test_rows_on_lanes_attention_edges(nodes, batch, ctx, env, monkeypatch):
     for k, v in env.items():
         monkeypatch.setenv(k, v)
@@ -575,8 +581,11 @@ def test_pass_in_one_launch_is_the_pass(wl):
         # twice the bound of either against the oracle; a bf16 cache value may round the other way
         tol = (2e-4 if f32 else 6e-2) if i < 2 else (2e-4 if f32 else 2.0 ** -7 * max(1.0, float(b.abs().max())))
         assert float((a.float() - b.float()).abs().max()) <= tol, i
-    if f32:
-        assert float((step[1] - many[1]).norm() / many[1].norm()) <= 1e-5
+    # bf16: about four times the largest seen, 5.7e-5, and 4.0e-4 without a context, where a new value of K or V that rounds the other way
+    # is half of what a row attends to; activations or queries without their lo parts are off by 1e-3 and more
+    for a, b in zip(step[:2], many[:2]):
+        rel = float((a - b).norm() / b.norm())
+        assert rel <= (1e-5 if f32 else 2.5e-4 if wl.ctx else 1.6e-3), rel
 
 
 _ROUTE = lambda v: str(v) if isinstance(v, (int, str)) else "-".join(f"{a}{b}" for a, b in v.items()) or "as-is"
@@ -725,7 +734,7 @@ def test_workspace_of_exactly_the_queried_size_is_enough(name):
 # as a rare difference between runs: the same step, many times, must give the same bits.
 @pytest.mark.parametrize("name,env", [("mini_7b", {}), ("mini_13b", {"VIASD_ATTN": "tk"}), ("mini_32b_b3", {"VIASD_ATTN": "tk"}),
                                       ("mini_8b_tree", {}), ("mini_8b_tree", {"VIASD_ATTN": "tk"}),
-                                      ("mini_7b", {"VIASD_ATTN": "tk", "VIASD_TK_GRID": "7"})])
+                                      ("mini_7b", {"VIASD_ATTN": "tk", "VIASD_TK_GRID": "7"}), ("mini_7b", LAUNCHES)])
 def test_repeated_verify_steps_are_bit_identical(name, env, monkeypatch):
     for k, v in env.items():
         monkeypatch.setenv(k, v)
@@ -750,11 +759,13 @@ def test_repeated_verify_steps_are_bit_identical(name, env, monkeypatch):
     assert vb.get_stats(eng.model).device_status == 0
 
 
-@pytest.mark.parametrize("name", ["mini_7b", "mini_8b_tree_greedy", "mini_13b"])
-def test_verify_step_replayed_from_a_cuda_graph_gives_the_same_bits(name):
+@pytest.mark.parametrize("name,env", [("mini_7b", {}), ("mini_8b_tree_greedy", {}), ("mini_13b", {}), ("mini_7b", LAUNCHES)])
+def test_verify_step_replayed_from_a_cuda_graph_gives_the_same_bits(name, env, monkeypatch):
     """Every launch of a step goes to the caller's stream and nothing in it synchronises or allocates, so after one
     ordinary call (which builds the tensor maps and sets the kernel attributes) a step can be captured into a CUDA graph
     - programmatic dependent launches included - and replayed: same logits, same tokens, bit for bit."""
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
     wl = W.get(name)
     vb = _vb()
     eng, st, si, model = _prepare(wl)
@@ -1164,15 +1175,17 @@ def test_expired_wait_is_reported_and_the_context_stays_usable():
 # ---------------------------------------------------------------------------------------------
 # routed execution policy: the full verifier runs only when the walk needs it
 # ---------------------------------------------------------------------------------------------
-@pytest.mark.parametrize("name,replay,alg2", [("mini_7b", 18, False), ("mini_8b_tree_greedy", 12, False), ("mini_13b", 14, False),
-                                              ("mini_13b", 14, True)])
-def test_routed_policy_emits_what_running_both_passes_emits(name, replay, alg2):
+@pytest.mark.parametrize("name,replay,alg2,env", [("mini_7b", 18, False, {}), ("mini_8b_tree_greedy", 12, False, {}), ("mini_13b", 14, False, {}),
+                                                  ("mini_13b", 14, True, {}), ("mini_7b", 18, False, LAUNCHES)])
+def test_routed_policy_emits_what_running_both_passes_emits(name, replay, alg2, env, monkeypatch):
     """A decoding loop under policy 1 (q' in every step, q only when a tier-2 node is reached before the first break,
     its cache caught up by replaying the last committed tokens) against the same loop under policy 0 and against the
     oracle, with thresholds that leave most blocks to tiers 0 and 1: same tiers, same accepted paths, same emitted
     tokens in every step; q's pass skipped in some steps and run in others; q''s cache identical, q's cache equal as
     far as it is complete and complete again after a pass of q.  alg2: the same with the slim verifier's own confidence
     as the gate and a tier-1 acceptance ending the block (Algorithm 2 as printed)."""
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
     wl = W.get(name)
     vb = _vb()
     n_steps, M = 12, wl.rows
