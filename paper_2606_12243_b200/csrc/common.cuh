@@ -214,8 +214,9 @@ inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, c
 }
 // A pass that runs only when a device flag says so (the full verifier's pass under the routed execution policy): every
 // kernel of it takes the flag's address and leaves at once when the flag is zero.  The flag is written by a kernel that
-// has completed before the pass's first kernel starts (the pass opens with ordinary, fully ordered launches), so
-// reading it ahead of the dependency wait is safe.
+// has completed before the pass's first kernel starts: that one, prep_replay_kernel, is an ordinary launch, and of the chained
+// ones behind it (the embedding among them) none starts before it has ended.  So reading the flag ahead of the dependency
+// wait is safe.
 #define RUN_FLAG_EXIT(ptr) do { if ((ptr) != nullptr && *reinterpret_cast<const volatile int *>(ptr) == 0) return; } while (0)
 #define PDL_WAIT() asm volatile("griddepcontrol.wait;" ::: "memory")
 #define PDL_TRIGGER() asm volatile("griddepcontrol.launch_dependents;" ::: "memory")

@@ -89,8 +89,7 @@ __device__ __forceinline__ void finish_row(const TcParams &p, int tile, int row,
     if (EPI == EPI_SWIGLU) {
         if (HALVES) {
             // lanes 0..15 have four gate features each, lanes 16..31 the matching up features: they trade two, so that every lane has
-            // two of both (with lanes 0..15 doing all four: 8B batch 4 6505 us, now 6470;
-            // prompt chunk 24.71 ms, now 24.30)
+            // two of both (with lanes 0..15 doing all four: prompt chunk 24.71 ms, now 24.30; steps of many rows within their runs' spread)
             const bool low = lane < 16;
             const float r0 = __shfl_xor_sync(0xffffffffu, low ? v.z : v.x, 16), r1 = __shfl_xor_sync(0xffffffffu, low ? v.w : v.y, 16);
             const float g0 = low ? v.x : r0, g1 = low ? v.y : r1, u0 = low ? r0 : v.z, u1 = low ? r1 : v.w;

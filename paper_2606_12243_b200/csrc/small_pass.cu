@@ -16,7 +16,8 @@
 //
 // bf16 models: mma.sync m16n8k16, weights exact, activations as bf16 pairs hi + lo as in the kernels for large models (a unit
 // is too small for a tcgen05 tile: 8 features against 128 lanes).  fp32 models: CUDA cores, fp32 throughout.  A row's results do
-// not depend on the rows beside it, nor on whether one or both verifiers' rows are in the launch.
+// not depend on whether one or both verifiers' rows are in the launch, nor on the values of other rows; on how many there are only by
+// the key ranges of its attention (Grouping::ranges).
 //
 // One step, launches before / one launch: two fp32 layers of d 256, 5 rows 145 / 69 us; four bf16 layers of d 512, 9 rows 164 / 120.
 // What bounds it now (cycles per stage): stores to arrival 1000, arrival to exit 1000, activations from L2 700 - 2400 (every CTA
@@ -957,7 +958,8 @@ struct Grouping {
     int pairs;                      // attention pairs of a sequence
     int part_seqs;                  // sequences of one verifier whose partial rows any launch has, at most
     int sms, tiles; size_t part_room;
-    // as many ranges as keep the CTAs busy with both verifiers, not more than 64 keys of the cache each make, within the partial buffer
+    // as many ranges as keep the CTAs busy with both verifiers, one per 64 keys of the cache's capacity at most, within the partial buffer;
+    // of a short context (they are cut on the device, at whole 32s) some are half a tile, or empty and merged as nothing
     int ranges(int b0) const {
         int ns = sms / (2 * (batch - b0 < n ? batch - b0 : n) * pairs);
         if (ns > tiles) ns = tiles;

@@ -9,8 +9,8 @@
 // token: children of the current row are tried in index order; tier-0 children are taken at once, tier-1 children are
 // judged by q', tier-2 children by q.  The first row where no child passes ends the walk and the strongest judge that
 // rejected there emits the replacement token.  The walk is sequential over depth, so everything that can be known before
-// it is: a row-statistics kernel (one CTA per logits row, all rows at once, one sweep) leaves each row's maximum, argmax
-// and softmax denominator, and the walk starts by fetching the tree and every node's two logits at once, so that a test is
+// it is: a row-statistics kernel (a CTA per logits row, or per part of one, one sweep) leaves each row's maximum, argmax
+// and softmax denominator, in parts, and the walk starts by fetching the tree and every node's two logits at once, so that a test is
 // arithmetic on shared memory.  Only a rejection in sampling mode (residual, Eq. A.3) and the final draw sweep the
 // vocabulary: one sweep and one exchange among the cluster's CTAs each.  An element of a residual is worked out from the logits
 // by replaying the rejections so far (a handful of scalars), in the arithmetic of Eq. A.3 round by round; every FOLD of them at
@@ -139,7 +139,8 @@ tier_kernel(unsigned char *__restrict__ tier, float *__restrict__ conf, DeviceSt
 }
 
 // ---- row statistics ---------------------------------------------------------------------------
-// grid (rows, B, 1 + judges): kind 0 = drafter rows [B, R, V], kind k = judge k's rows [B, M, V] (the last judge is q).
+// One-dimensional grid over rows, kind by kind, and parts (RowUnits): kind 0 = drafter rows [B, R, V], kind k = judge k's rows
+// [B, M, V] (the last judge is q).
 // Per row: max, argmax (lowest index on ties) and, when wanted, sum exp((l - max) / T).
 // HBM-bound: every row once.  Maximum and denominator come from one sweep (a running reference per thread, moved when it is
 // exceeded by e^20); two sweeps read a batch's rows twice from HBM, 16 sequences' 1040 rows of 0.5 MB being far more than L2
