@@ -231,7 +231,7 @@ enum {
     VIASD_OPT_TK_FLAT,                 /* keys-on-lanes attention: deal tiles 1, key ranges 0; -1 = by shape (default) */
     VIASD_OPT_GEMM_RING_KB,            /* stream-K GEMM: shared-memory ring in KB, 32..200; 0 = default (200) */
     VIASD_OPT_GEMM_EPI_GROUPS,         /* stream-K GEMM: groups of four epilogue warps, 1 or 2; 0 = by token tile */
-    VIASD_OPT_ONE_LAUNCH               /* 1 (default): the forward pass of a small model with few token rows is one launch; 0: never */
+    VIASD_OPT_ONE_LAUNCH               /* 1 (default): a small model's forward pass is one launch (fp32 batches: a few) where that is the faster way; 0: never */
 };
 int viasd_set_option(viasd_model *m, int option, int value);
 

@@ -547,6 +547,8 @@ def _one_launch_case(name, batch, nodes, ctx, tree=False, **shape):
     _one_launch_case("c1_tiny", 2, 26, 300, tree=True, n_kv_heads=2, vocab=1001),                             # grouped heads, odd vocabulary
     _one_launch_case("c1_tiny", 5, 12, 70, head_dim=128, n_heads=2, n_kv_heads=1),                            # 65 rows: three launches
     _one_launch_case("c1_tiny", 5, 20, 90), _one_launch_case("c1_tiny", 7, 16, 300, n_layers=3),              # apart: 63 and 42, 51 and 17 rows
+    _one_launch_case("c1_tiny", 6, 5, 200), _one_launch_case("c1_tiny", 6, 6, 200), _one_launch_case("c1_tiny", 11, 5, 700, d_model=192),      # 3 + 3, 4 + 2, 4 + 4 + 3
+    _one_launch_case("c1_tiny", 9, 3, 130, head_dim=128, n_kv_heads=2, vocab=1001),                            # 8 + 1
     _one_launch_case("c1_tiny", 2, 63, 90), _one_launch_case("c1_tiny", 2, 8, 40, d_model=768, d_ff=2048),   # a verifier per launch; fewer rows per launch
     _one_launch_case("mini_7b", 1, 1, 0), _one_launch_case("mini_7b", 1, 15, 63), _one_launch_case("mini_7b", 3, 7, 130),   # 2, 16, 24 rows
     _one_launch_case("mini_8b_tree_greedy", 1, 26, 500, tree=True), _one_launch_case("mini_13b", 3, 6, 260),
